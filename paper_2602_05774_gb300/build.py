@@ -1,6 +1,6 @@
 """Build the CUDA library libvsd.so (sm_103a) in-tree.
 
-Three translation units are compiled in parallel with nvcc and linked into
+The translation units of csrc are compiled in parallel with nvcc and linked into
 paper_2602_05774_gb300/_build/libvsd.so against the shared CUDA runtime (so
 the process shares one runtime with PyTorch).  No CMake.
 """
@@ -15,7 +15,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libvsd.so")
-SOURCES = ["vsd_api.cu", "vsd_kernels_f32.cu", "vsd_kernels_bf16.cu", "vsd_noalloc.cu",
+SOURCES = ["vsd_api.cu", "vsd_kernels_f32.cu", "vsd_kernels_bf16.cu", "vsd_tree_f32.cu",
+           "vsd_tree_bf16.cu", "vsd_noalloc.cu",
            "vsd_lmhead.cu", "vsd_lmhead_bwd.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]

@@ -247,6 +247,20 @@ __device__ __forceinline__ void ring_init(Ring* rg, uint64_t timeout_ns) {
     __syncthreads();
 }
 
+// Dynamic shared memory: [Ring (vector rows)] [chunk table].
+template <bool VEC>
+__device__ __forceinline__ void smem_views(unsigned char* dsm, Ring*& rg, float4*& tab,
+                                           uint64_t timeout_ns) {
+    if (VEC) {
+        rg = reinterpret_cast<Ring*>(dsm);
+        tab = reinterpret_cast<float4*>(dsm + sizeof(Ring));
+        ring_init(rg, timeout_ns);
+    } else {
+        rg = nullptr;
+        tab = reinterpret_cast<float4*>(dsm);
+    }
+}
+
 // Bounded wait on a slot; false (and the timeout status bit) if it ran out.
 __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, int* status,
                                           uint64_t timeout_ns) {
@@ -581,8 +595,8 @@ __device__ __forceinline__ Located table_locate(const float4* tab, int nch, int 
 // and return the first token of positive mass whose running mass exceeds tc
 // (the chunk-frame threshold); if none does, the last token with mass; -1 if
 // the chunk has no mass.  Only tokens of positive mass can be returned, so
-// masked positions (at or beyond V) never are.  mass(fx, fy) gives a token's
-// mass.
+// masked positions (at or beyond V) never are.  mass(fx, fy, v) gives token
+// v's mass.
 template <typename T, bool NEED_X, bool NEED_Y, class Mass>
 __device__ __forceinline__ int rescan_regs(const uint4 (&bx)[kLoads], const uint4 (&by)[kLoads],
                                            int ch, float tc, const Mass& mass, int lane) {
@@ -599,7 +613,8 @@ __device__ __forceinline__ int rescan_regs(const uint4 (&bx)[kLoads], const uint
         int lastpos = -1;
 #pragma unroll
         for (int e = 0; e < PV; ++e) {
-            m[e] = mass(NEED_X ? fx[e] : 0.f, NEED_Y ? fy[e] : 0.f);
+            m[e] = mass(NEED_X ? fx[e] : 0.f, NEED_Y ? fy[e] : 0.f,
+                        (int)base + k * 32 * PV + lane * PV + e);
             run += m[e];
             if (m[e] > 0.f) lastpos = e;
         }
@@ -643,16 +658,16 @@ __device__ __forceinline__ int warp_rescan(const T* x, const T* y, int64_t V, in
 
 struct MassX {
     float mm, c;
-    __device__ float operator()(float fx, float) const { return mass_rel(fx, mm, c); }
+    __device__ float operator()(float fx, float, int) const { return mass_rel(fx, mm, c); }
 };
 struct MassY {
     float mm, c;
-    __device__ float operator()(float, float fy) const { return mass_rel(fy, mm, c); }
+    __device__ float operator()(float, float fy, int) const { return mass_rel(fy, mm, c); }
 };
 // Residual mass max(0, p(v) - q(v)) with p and q normalised by 1/Z factors.
 struct MassRes {
     float mx, my, izx, izy, c;
-    __device__ float operator()(float fx, float fy) const {
+    __device__ float operator()(float fx, float fy, int) const {
         const float p = ex2((fy - my) * c) * izy;
         const float q = ex2((fx - mx) * c) * izx;
         return fmaxf(p - q, 0.f);

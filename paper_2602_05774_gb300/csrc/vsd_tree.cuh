@@ -17,8 +17,9 @@
 //                each node's gradient terms (sums over its subtree).
 //   k_tree_grad  one block per row: grad = g q(v) minus the sparse terms of
 //                the row's children (their tokens and corrected tokens).
-//   k_tree_seq   one block per tree: the sequential sibling rule along the
-//                accepted path, with one read of a row per rejected sibling.
+//   k_tree_seq_rows / k_tree_seq   the sequential sibling rule: one block per
+//                row decides which of the row's children is accepted, one block
+//                per tree follows the decisions along the accepted path.
 #pragma once
 
 #include "vsd_passes.cuh"
@@ -49,7 +50,7 @@ struct __align__(16) TreeCoef {
 static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 
 // ------------------------------------------------------------ k_tree_rows
-template <typename T, bool VEC, bool EM>
+template <typename T, bool VEC>
 __device__ void tree_row_children(const Problem<T>& P, int r, Ring* rg, float4* tab, int* s_any) {
     const int N = P.N;
     const int64_t V = P.V;
@@ -66,10 +67,8 @@ __device__ void tree_row_children(const Problem<T>& P, int r, Ring* rg, float4* 
     // the target's table for the draws from p (each warp, identical values)
     float My = 0.f;
     TableSum Sy{0, 0, 0.0};
-    if (EM) {
-        My = table_max(tab, P.nch, 1, lane);
-        Sy = table_sum(tab, P.nch, 1, frame_of(My), c, lane);
-    }
+    My = table_max(tab, P.nch, 1, lane);
+    Sy = table_sum(tab, P.nch, 1, frame_of(My), c, lane);
     int k = 0;
     for (int n = u + 1; n < N; ++n) {
         if (__ldg(par + n) != u) continue;
@@ -89,7 +88,7 @@ __device__ void tree_row_children(const Problem<T>& P, int r, Ring* rg, float4* 
             token_logs(x, y, tok, rec, P.ts.invTd, &nr.lq, &nr.la);
         }
         nr.acc = nr.la > -INFINITY && __ldg(P.u_accept + n0 + n) <= expf(nr.la);
-        if (EM && !rec.flags) {
+        if (!rec.flags) {
             int zp = warp_sample<T, VEC>(x, y, V, tab, P.nch, 1, My, Sy,
                                          __ldg(P.u_correct + n0 + n), c, lane, pol);
             if (zp >= V) zp = -1;
@@ -102,7 +101,7 @@ __device__ void tree_row_children(const Problem<T>& P, int r, Ring* rg, float4* 
         }
     }
     __syncthreads();
-    if (!EM || !*s_any || rec.flags) return;
+    if (!*s_any || rec.flags) return;
     // a child is rejected: the residual max(0, p - q) of the row, and each
     // rejected child's draw from it (or from p if it has no mass)
     const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
@@ -131,7 +130,7 @@ __device__ void tree_row_children(const Problem<T>& P, int r, Ring* rg, float4* 
     }
 }
 
-template <typename T, bool VEC, bool EM>
+template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_tree_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
@@ -148,15 +147,14 @@ __global__ void __launch_bounds__(kThreads) k_tree_rows(Problem<T> P) {
     const int r = blockIdx.x;
     row_pass<T, VEC, true, kNoToken, true>(P, r, rg, tab, sh);
     __syncthreads();
-    tree_row_children<T, VEC, EM>(P, r, rg, tab, &s_any);
-    if (threadIdx.x == 0 && P.tout.row_stats)
-        reinterpret_cast<float4*>(P.tout.row_stats)[r] = ld_cg(P.rstats + r);
+    tree_row_children<T, VEC>(P, r, rg, tab, &s_any);
 }
 
 // ------------------------------------------------------------ shared helpers
 struct TreeShared2 {
     int par[1024];
     int depth[1024];
+    short anc[1024];
     unsigned char pacc[1024];
     int maxd;
 };
@@ -175,15 +173,39 @@ __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
     }
     const int bad = __syncthreads_or(badl);
     if (bad) return false;
-    if (threadIdx.x == 0) {
-        sh.depth[0] = 0;
-        int maxd = 0;
-        for (int n = 1; n < N; ++n) {
-            sh.depth[n] = sh.depth[sh.par[n]] + 1;
-            maxd = max(maxd, sh.depth[n]);
-        }
-        sh.maxd = maxd;
+    // depths by pointer doubling: depth[n] steps from n to anc[n]
+    for (int n = threadIdx.x; n < N; n += kThreads) {
+        sh.depth[n] = n ? 1 : 0;
+        sh.anc[n] = (short)(n ? sh.par[n] : 0);
     }
+    if (threadIdx.x == 0) sh.maxd = 0;
+    for (;;) {
+        __syncthreads();
+        short a[1024 / kThreads];
+        int d[1024 / kThreads];
+        int more = 0;
+#pragma unroll
+        for (int k = 0; k < 1024 / kThreads; ++k) {
+            const int n = threadIdx.x + k * kThreads;
+            if (n >= N) break;
+            a[k] = sh.anc[sh.anc[n]];
+            d[k] = sh.depth[n] + sh.depth[sh.anc[n]];
+            more |= a[k] != 0;
+        }
+        more = __syncthreads_or(more);
+#pragma unroll
+        for (int k = 0; k < 1024 / kThreads; ++k) {
+            const int n = threadIdx.x + k * kThreads;
+            if (n >= N) break;
+            sh.anc[n] = a[k];
+            sh.depth[n] = d[k];
+        }
+        if (!more) break;
+    }
+    __syncthreads();
+    int md = 0;
+    for (int n = threadIdx.x; n < N; n += kThreads) md = max(md, sh.depth[n]);
+    atomicMax(&sh.maxd, md);
     __syncthreads();
     return true;
 }
@@ -203,7 +225,7 @@ struct TreeEmShared {
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_tree_em(Problem<T> P, vsd_tree_em_outputs o) {
-    extern __shared__ __align__(16) unsigned char dsm[];
+    extern __shared__ __align__(128) unsigned char dsm[];
     TreeEmShared& sh = *reinterpret_cast<TreeEmShared*>(dsm);
     const int N = P.N, b = blockIdx.x, n0 = b * N;
     const bool ok = tree_load<T>(P, b, sh.t);
@@ -474,55 +496,335 @@ __global__ void __launch_bounds__(kThreads) k_tree_grad(Problem<T> P, G* grad) {
     }
 }
 
-// ------------------------------------------------------------ k_tree_seq
-// The sequential sibling rule (lossless multi-draft) along the accepted path
-// of one tree.  At node u with children c_1 .. c_m (node order) child i is
-// accepted with probability min(1, p_i(t_i)/q_i(t_i)); after a rejection
-// p_{i+1} = norm(max(0, p_i - q_i)) (p_i kept if that has no mass) and
-// q_{i+1} = q_i without t_i, renormalised.  p_i at a point follows the
-// recursion from the row's p and q and the normalisers found so far; each
-// normaliser is one read of the row (chunk sums of max(0, p_i - q_i), summed
-// exactly), and after the last rejection the correction token is drawn from
-// that table.
-struct SeqState {
-    int nrem;              // children tried so far at this node
-    int rem[1024];         // their tokens (removed from q)
-    double S[1024];        // S[j]: normaliser of p_{j+2} (0: p kept)
-    double Qs[1024];       // Qs[j]: remaining draft mass before the (j+1)-th child
+// ------------------------------------------------------------ sequential rule
+// The sequential sibling rule (lossless multi-draft) at a node u with children
+// c_1 .. c_m (node order): child i is accepted with probability
+// min(1, p_i(t_i)/q_i(t_i)); after a rejection p_{i+1} = norm(max(0, p_i - q_i))
+// (p_i kept if that has no mass) and q_{i+1} = q_i without t_i, renormalised.
+//
+// Which child of u is accepted first, and the correction token if none is,
+// depend on u's row, its children and their uniforms alone, so every row is
+// decided where it is read (k_tree_seq_rows, one block per row); the walk
+// along the accepted path then only follows the rows' decisions (k_tree_seq).
+//
+// Every q_i is the same q but for a factor 1/Q_i (Q_i: the draft mass not yet
+// removed), and max(0, max(0, p - a q) - b q) = max(0, p - (a + b) q) for
+// a, b >= 0, so with p_i = P_i / T_i
+//   P_i(v) = max(0, p(v) - A_i q(v)),  A_{i+1} = A_i + T_i / Q_i,  T_i = sum P_i
+// and a removed token keeps the A of the step that removed it.  Each rejected
+// child therefore costs one read of the row (from L2, where the row pass left
+// it) with one multiply-add more than the plain residual, however many
+// siblings went before it.
+struct SeqCtl {
+    int m;          // children of the row's node
+    int next;       // the accepted child (node index), -1 so far
+    int out;        // the correction token
+    double A, T, Q; // A_i, T_i, Q_i of the child tried next
+    double An;      // A_{i+1}
+    float ah, al;   // A_{i+1} in two floats
 };
+// Per child of the row's node, in node order (dynamic shared memory, sized by
+// the tree's nodes).
+struct SeqKids {
+    double* p;      // p and q of its token at the row
+    double* q;
+    float2* A;      // the A its token keeps once removed, in two floats
+    int* tok;
+    int* kid;       // its node
+};
+inline size_t seq_smem_bytes(int N) { return (size_t)N * 32; }
+__device__ __forceinline__ SeqKids seq_kids(unsigned char* base, int N) {
+    SeqKids s;
+    s.p = reinterpret_cast<double*>(base);
+    s.q = s.p + N;
+    s.A = reinterpret_cast<float2*>(s.q + N);
+    s.tok = reinterpret_cast<int*>(s.A + N);
+    s.kid = s.tok + N;
+    return s;
+}
+
+__device__ __forceinline__ float2 two_floats(double a) {
+    const float h = (float)a;
+    return make_float2(h, (float)(a - (double)h));
+}
+// max(0, p - A q): the products are exact inside the multiply-adds, so A in
+// two floats loses nothing of the double.
+__device__ __forceinline__ float seq_mass(float p, float q, float ah, float al) {
+    return fmaxf(fmaf(-al, q, fmaf(-ah, q, p)), 0.f);
+}
+
+// The masses of one row after some rejections: A for every token but the
+// first `nrem` children's, which keep their own.
+struct SeqMass {
+    MassRes mr;
+    float ah, al;
+    const int* tok;
+    const float2* A;
+    int nrem;
+    // (the first of equal tokens is the one that was removed)
+    __device__ float operator()(float fx, float fy, int v) const {
+        const float p = ex2((fy - mr.my) * mr.c) * mr.izy;
+        const float q = ex2((fx - mr.mx) * mr.c) * mr.izx;
+        for (int j = 0; j < nrem; ++j)
+            if (tok[j] == v) return seq_mass(p, q, A[j].x, A[j].y);
+        return seq_mass(p, q, ah, al);
+    }
+};
+
+// Sum of the masses of one chunk (warp).
+template <typename T>
+__device__ __forceinline__ float seq_chunk(const uint4 (&bx)[kLoads], const uint4 (&by)[kLoads],
+                                           int ch, const SeqMass& sm, int lane) {
+    constexpr int PV = Traits<T>::kPerVec, NP = PV / 2, CE = chunk_elems<T>();
+    bool some = false;  // a removed token lies in this chunk
+    for (int j = lane; j < sm.nrem; j += 32) some |= (unsigned)(sm.tok[j] - ch * CE) < (unsigned)CE;
+    float acc = 0.f;
+    if (__any_sync(0xffffffffu, some)) {
+#pragma unroll
+        for (int k = 0; k < kLoads; ++k) {
+            float fx[PV], fy[PV];
+            unpack<T>(bx[k], fx);
+            unpack<T>(by[k], fy);
+#pragma unroll
+            for (int e = 0; e < PV; ++e)
+                acc += sm(fx[e], fy[e], ch * CE + k * 32 * PV + lane * PV + e);
+        }
+        return warp_sum(acc);
+    }
+    const MassRes& mr = sm.mr;
+    const uint64_t mx2 = f2(mr.mx, mr.mx), my2 = f2(mr.my, mr.my), c2 = f2(mr.c, mr.c);
+    const uint64_t izx2 = f2(mr.izx, mr.izx), izy2 = f2(mr.izy, mr.izy);
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+        uint64_t px[NP], py[NP];
+        vec_pairs<T>(bx[k], px);
+        vec_pairs<T>(by[k], py);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            float q0, q1, p0, p1;
+            f2split(f2mul(f2_mass(px[i], mx2, c2), izx2), q0, q1);
+            f2split(f2mul(f2_mass(py[i], my2, c2), izy2), p0, p1);
+            acc += seq_mass(p0, q0, sm.ah, sm.al) + seq_mass(p1, q1, sm.ah, sm.al);
+        }
+    }
+    return warp_sum(acc);
+}
+
+// One read of row r: tab[ch].y = the chunk sums of its masses (block).
+template <typename T, bool VEC>
+__device__ void seq_stream(const Problem<T>& P, int r, Ring* rg, float4* tab, const SeqMass& sm) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t V = P.V;
+    const T* x = P.draft + (int64_t)r * V;
+    const T* y = P.target + (int64_t)r * V;
+    const uint64_t pol = policy_evict_normal();
+    if constexpr (VEC) {
+        ring_stream<T, true>(rg, x, y, V, 0, P.nch, pol, pol, P.status,
+                             [&](int ch, const uint4 (&bx)[kLoads], const uint4 (&by)[kLoads]) {
+                                 const float t = seq_chunk<T>(bx, by, ch, sm, lane);
+                                 if (lane == 0) tab[ch] = make_float4(0.f, t, 0.f, 0.f);
+                             });
+    } else {
+        for (int ch = warp; ch < P.nch; ch += kWarps) {
+            uint4 bx[kLoads], by[kLoads];
+            load_chunk<T, VEC>(x, V, ch, lane, pol, bx);
+            load_chunk<T, VEC>(y, V, ch, lane, pol, by);
+            const float t = seq_chunk<T>(bx, by, ch, sm, lane);
+            if (lane == 0) tab[ch] = make_float4(0.f, t, 0.f, 0.f);
+        }
+    }
+    __syncthreads();
+}
+
+// Inverse-CDF draw from the masses whose chunk sums are in tab (warp; -1 if
+// there is no mass).
+template <typename T, bool VEC>
+__device__ int seq_draw(const Problem<T>& P, int r, const float4* tab, const TableSum& S, float u,
+                        const SeqMass& sm, int lane) {
+    const Located loc = table_locate(tab, P.nch, 0, 0.f, P.ts.c, S, u, lane);
+    if (loc.ch < 0) return -1;
+    return warp_rescan<T, VEC, true, true>(P.draft + (int64_t)r * P.V, P.target + (int64_t)r * P.V,
+                                           P.V, loc.ch, loc.tc, sm, lane, policy_evict_normal());
+}
+
+// The decision at node u = row r (block, after the row's pass): tries its
+// children in turn.  Per tried child tnode[].lq = alpha, .acc, .zp = 1 (0 for
+// the others), for every child .la; tlist[r] = the accepted child, 0 if u has
+// no children, -1 if all were rejected, with the correction token in
+// es.corr[r].
+template <typename T, bool VEC>
+__device__ void tree_seq_row(const Problem<T>& P, int r, Ring* rg, float4* tab, SeqCtl& ct,
+                             const SeqKids& s) {
+    const int N = P.N, b = r / N, u = r - b * N, n0 = b * N;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t V = P.V;
+    const int32_t* par = P.parent + (int64_t)n0;
+    const float c = P.ts.c;
+    const RowRec rec = ld_cg(P.rows + r);
+    if (warp == 0) {  // the children, in node order
+        int m = 0;
+        for (int g = u + 1; g < N; g += 32) {
+            const bool is = g + lane < N && __ldg(par + g + lane) == u;
+            const unsigned bal = __ballot_sync(0xffffffffu, is);
+            if (is) s.kid[m + __popc(bal & ((1u << lane) - 1u))] = g + lane;
+            m += __popc(bal);
+        }
+        if (lane == 0) {
+            ct.m = m;
+            ct.next = m ? -1 : 0;
+            ct.out = -1;
+            ct.A = 0.0;
+            ct.T = ct.Q = 1.0;
+        }
+    }
+    __syncthreads();
+    const int m = ct.m;
+    for (int i = threadIdx.x; i < m; i += kThreads) {
+        const int n = n0 + s.kid[i], tok = __ldg(P.given_tokens + n);
+        TreeNodeRec nr;
+        nr.la = -INFINITY;
+        nr.lq = 0.f;
+        nr.acc = nr.zp = 0;
+        nr.lq_zp = nr.la_zp = nr.lq_zr = nr.la_zr = 0.f;
+        nr.zr = -1;
+        nr.pad[0] = nr.pad[1] = nr.pad[2] = 0;
+        double p = 0.0, q = 0.0;
+        if (tok < 0 || tok >= V) {
+            atomicOr(P.status, VSD_STATUS_BAD_TOKEN);
+        } else if (!rec.flags) {
+            const float xv = elem_value(P.draft + (int64_t)r * V, tok);
+            const float yv = elem_value(P.target + (int64_t)r * V, tok);
+            float lq;
+            token_logs_vals(xv, yv, rec, P.ts.invTd, &lq, &nr.la);
+            p = exp(((double)yv - rec.my) * P.ts.invTd - rec.lzy);
+            q = exp(((double)xv - rec.mx) * P.ts.invTd - rec.lzx);
+        }
+        s.tok[i] = tok;
+        s.p[i] = p;
+        s.q[i] = q;
+        P.tnode[n] = nr;
+    }
+    __syncthreads();
+    const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
+    for (int i = 0; i < m; ++i) {
+        if (threadIdx.x == 0) {
+            const int n = n0 + s.kid[i], t = s.tok[i];
+            int before = -1;  // the earlier sibling that removed t, if any
+            for (int j = 0; j < i && before < 0; ++j)
+                if (s.tok[j] == t) before = j;
+            const double Q = ct.Q, A = ct.A, Tm = ct.T;
+            double alpha = 0.0;
+            if (!rec.flags && t >= 0 && t < V) {
+                const double At = before >= 0 ? (double)s.A[before].x + (double)s.A[before].y : A;
+                const double pi = fmax(0.0, s.p[i] - At * s.q[i]) / Tm;
+                const double qi = before >= 0 || !(Q > 0.0) ? 0.0 : s.q[i] / Q;
+                alpha = qi > 0.0 ? fmin(1.0, pi / qi) : (pi > 0.0 ? 1.0 : 0.0);
+            }
+            const bool a = __ldg(P.u_accept + n) <= alpha && !rec.flags;
+            P.tnode[n].lq = (float)alpha;
+            P.tnode[n].acc = a ? 1 : 0;
+            P.tnode[n].zp = 1;
+            if (a) ct.next = s.kid[i];
+            ct.An = A + (Q > 0.0 ? Tm / Q : 0.0);
+            const float2 h = two_floats(ct.An);
+            ct.ah = h.x;
+            ct.al = h.y;
+            if (before < 0) ct.Q = Q - s.q[i];
+        }
+        __syncthreads();
+        if (ct.next > 0) break;
+        if (!rec.flags) {
+            // T_{i+1} (one read of the row); the draw after the last rejection
+            const float uc = __ldg(P.u_correct + n0 + s.kid[i]);
+            const SeqMass sm{mr, ct.ah, ct.al, s.tok, s.A, i};
+            seq_stream<T, VEC>(P, r, rg, tab, sm);
+            if (warp == 0) {
+                const TableSum Rt = table_sum(tab, P.nch, 0, 0.f, c, lane);
+                // (no mass left: p_i is kept, and the draw is from it)
+                const int tok = i < m - 1 ? -1
+                                : Rt.Z > 0.0 ? seq_draw<T, VEC>(P, r, tab, Rt, uc, sm, lane)
+                                             : -2;
+                if (lane == 0) {
+                    if (Rt.Z > 0.0 && Rt.Z < INFINITY) {
+                        ct.A = ct.An;
+                        ct.T = Rt.Z;
+                    }
+                    s.A[i] = two_floats(ct.A);
+                    ct.out = tok;
+                }
+            }
+            __syncthreads();
+            if (ct.out == -2) {
+                const float2 h = two_floats(ct.A);
+                const SeqMass keep{mr, h.x, h.y, s.tok, s.A, i};
+                __syncthreads();
+                seq_stream<T, VEC>(P, r, rg, tab, keep);
+                if (warp == 0) {
+                    const TableSum Pt = table_sum(tab, P.nch, 0, 0.f, c, lane);
+                    const int tok =
+                        Pt.Z > 0.0 ? seq_draw<T, VEC>(P, r, tab, Pt, uc, keep, lane) : -1;
+                    if (lane == 0) ct.out = tok;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        P.tlist[r] = ct.next;
+        P.es.corr[r] = ct.out;
+    }
+}
+
+// One block per node row (a leaf's row only for the statistics output; the
+// row the bonus token needs is then read by k_tree_seq).
+// What bounds it: the row reads and row tails (3840 rows of 2 x 64 KB), and
+// the reads after a rejection, which come from L2.  64 trees of 60 nodes,
+// V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
+// block per tree, in an fp64 recursion per element over the earlier siblings.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kThreads) k_tree_seq_rows(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ RowShared sh;
+    __shared__ SeqCtl ct;
+    Ring* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    const SeqKids kids = seq_kids(reinterpret_cast<unsigned char*>(tab + P.nch), P.N);
+    const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
+    int need = P.tout.row_stats != nullptr;
+    for (int n = u + 1 + threadIdx.x; n < N && !need; n += kThreads)
+        need = __ldg(P.parent + (int64_t)b * N + n) == u;
+    if (!__syncthreads_or(need)) {
+        if (threadIdx.x == 0) P.tlist[r] = 0;
+        return;
+    }
+    row_pass<T, VEC, true, kNoToken, false>(P, r, rg, tab, sh);
+    __syncthreads();
+    if (threadIdx.x == 0 && P.tout.row_stats)
+        reinterpret_cast<float4*>(P.tout.row_stats)[r] = ld_cg(P.rstats + r);
+    tree_seq_row<T, VEC>(P, r, rg, tab, ct, kids);
+}
 
 struct TreeSeqShared {
     TreeShared2 t;
-    SeqState st;
-    int kids[1024];
-    int nk;
-    int cur, out_tok, leaf_bonus;
+    double lk[1024];
+    float la[1024];
+    int next[1024];
+    unsigned char on[1024];  // on the accepted path
+    int best, lastkid;
 };
 
-// p_i(v) and q_i(v) for the (i+1)-th child (i = children rejected so far),
-// from the row's own p(v), q(v).
-__device__ __forceinline__ void seq_point(const SeqState& st, int i, int64_t v, double p,
-                                          double q, double& pi, double& qi) {
-    pi = p;
-    bool removed = false;
-    for (int j = 0; j < i; ++j) {
-        const double qj = removed ? 0.0 : (st.Qs[j] > 0.0 ? q / st.Qs[j] : 0.0);
-        if (st.S[j] > 0.0) pi = fmax(0.0, pi - qj) / st.S[j];
-        removed |= st.rem[j] == v;
-    }
-    qi = removed ? 0.0 : (st.Qs[i] > 0.0 ? q / st.Qs[i] : 0.0);
-}
-
+// One block per tree: the accepted path, and every node's outputs.
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    TreeSeqShared& sh = *reinterpret_cast<TreeSeqShared*>(dsm);
-    float4* tab = reinterpret_cast<float4*>(dsm + sizeof(TreeSeqShared));
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ RowShared rsh;
+    Ring* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    TreeSeqShared& sh = *reinterpret_cast<TreeSeqShared*>(tab + P.nch);
     const int N = P.N, b = blockIdx.x, n0 = b * N;
-    const int64_t V = P.V;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const vsd_tree_outputs& o = P.tout;
-    const float c = P.ts.c;
     if (!tree_load<T>(P, b, sh.t)) {
         for (int n = threadIdx.x; n < N; n += kThreads) {
             o.alpha[n0 + n] = 0.f;
@@ -540,224 +842,57 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
         return;
     }
     for (int n = threadIdx.x; n < N; n += kThreads) {
-        o.alpha[n0 + n] = n ? 0.f : 1.f;
-        o.accept[n0 + n] = n ? 0 : 1;
-        o.path_accept[n0 + n] = n ? 0 : 1;
-        o.corr_tokens[n0 + n] = -1;
-    }
-    if (threadIdx.x == 0) {  // log kappa: the path validity (Eq. 2) of every node
-        double* lk = sh.st.S;  // (scratch before the walk)
-        lk[0] = 0.0;
-        o.logkappa[n0] = 0.f;
-        for (int n = 1; n < N; ++n) {
-            lk[n] = lk[sh.t.par[n]] + (double)ld_cg(&P.tnode[n0 + n].la);
-            o.logkappa[n0 + n] = (float)lk[n];
-        }
-        sh.cur = 0;
-        sh.out_tok = -1;
-    }
-    __syncthreads();
-    for (;;) {
-        const int u = sh.cur;
-        // the children of u, in node order
-        if (threadIdx.x == 0) {
-            int m = 0;
-            for (int n = u + 1; n < N; ++n)
-                if (sh.t.par[n] == u) sh.kids[m++] = n;
-            sh.nk = m;
-            sh.st.nrem = 0;
-        }
-        __syncthreads();
-        const int m = sh.nk;
-        if (m == 0) break;
-        const int ru = n0 + u;
-        const RowRec rec = ld_cg(P.rows + ru);
-        const T* x = P.draft + (int64_t)ru * V;
-        const T* y = P.target + (int64_t)ru * V;
-        int next = -1;
-        for (int i = 0; i < m; ++i) {
-            const int ch = sh.kids[i];
-            if (threadIdx.x == 0) {
-                const int t = __ldg(P.given_tokens + n0 + ch);
-                double alpha = 0.0;
-                if (!rec.flags && t >= 0 && t < V) {
-                    if (i == 0) sh.st.Qs[0] = 1.0;
-                    const double p = exp(((double)elem_value(y, t) - rec.my) * P.ts.invTd - rec.lzy);
-                    const double q = exp(((double)elem_value(x, t) - rec.mx) * P.ts.invTd - rec.lzx);
-                    double pi, qi;
-                    seq_point(sh.st, i, t, p, q, pi, qi);
-                    alpha = qi > 0.0 ? fmin(1.0, pi / qi) : (pi > 0.0 ? 1.0 : 0.0);
-                }
-                const bool a = __ldg(P.u_accept + n0 + ch) <= alpha && !rec.flags;
-                o.alpha[n0 + ch] = (float)alpha;
-                o.accept[n0 + ch] = a ? 1 : 0;
-                sh.st.rem[i] = t;
-                if (a) {
-                    o.path_accept[n0 + ch] = 1;
-                    sh.cur = ch;
-                    sh.st.nrem = -1;  // accepted
-                } else {
-                    sh.st.nrem = i + 1;
-                    const double q_t = (t >= 0 && t < V && !rec.flags)
-                        ? exp(((double)elem_value(x, t) - rec.mx) * P.ts.invTd - rec.lzx) : 0.0;
-                    // the remaining draft mass once t_i is removed (t_i not removed before)
-                    bool before = false;
-                    for (int j = 0; j < i; ++j) before |= sh.st.rem[j] == t;
-                    sh.st.Qs[i + 1] = sh.st.Qs[i] - (before ? 0.0 : q_t);
-                }
-            }
-            __syncthreads();
-            if (sh.st.nrem < 0) {
-                next = sh.cur;
-                break;
-            }
-            if (rec.flags) continue;
-            // the normaliser of p_{i+2}: chunk sums of max(0, p_{i+1} - q_{i+1})
-            // (one read of the row); the draw after the last rejection
-            const int ii = i + 1;  // children rejected so far
-            for (int chn = warp; chn < P.nch; chn += kWarps) {
-                const uint64_t pol = policy_evict_normal();
-                uint4 bx[kLoads], by[kLoads];
-                load_chunk<T, VEC>(x, V, chn, lane, pol, bx);
-                load_chunk<T, VEC>(y, V, chn, lane, pol, by);
-                float acc = 0.f;
-#pragma unroll
-                for (int k = 0; k < kLoads; ++k) {
-                    float fx[Traits<T>::kPerVec], fy[Traits<T>::kPerVec];
-                    unpack<T>(bx[k], fx);
-                    unpack<T>(by[k], fy);
-#pragma unroll
-                    for (int e = 0; e < Traits<T>::kPerVec; ++e) {
-                        const int64_t v = (int64_t)chn * chunk_elems<T>() +
-                                          k * 32 * Traits<T>::kPerVec + lane * Traits<T>::kPerVec + e;
-                        if (v >= V) continue;
-                        const double p = (double)(ex2((fy[e] - rec.my) * c) * rec.izy);
-                        const double q = (double)(ex2((fx[e] - rec.mx) * c) * rec.izx);
-                        double pi, qi;
-                        seq_point(sh.st, ii - 1, v, p, q, pi, qi);
-                        acc += (float)fmax(0.0, pi - qi);
-                    }
-                }
-                acc = warp_sum(acc);
-                if (lane == 0) tab[chn] = make_float4(0.f, acc, 0.f, 0.f);
-            }
-            __syncthreads();
-            if (warp == 0) {
-                const TableSum Rt = table_sum(tab, P.nch, 0, 0.f, c, lane);
-                if (lane == 0) sh.st.S[ii - 1] = Rt.Z > 0.0 && Rt.Z < INFINITY ? Rt.Z : 0.0;
-                if (i == m - 1) {  // every child rejected: the correction token
-                    const float uc = __ldg(P.u_correct + n0 + ch);
-                    int tok = -1;
-                    if (Rt.Z > 0.0) {
-                        const Located loc = table_locate(tab, P.nch, 0, 0.f, c, Rt, uc, lane);
-                        if (loc.ch >= 0) {  // rescan the chunk in token order
-                            float carry = 0.f;
-                            const int64_t base = (int64_t)loc.ch * chunk_elems<T>();
-                            int last = -1;
-                            for (int64_t v0 = base; v0 < base + chunk_elems<T>() && tok < 0; v0 += 32) {
-                                const int64_t v = v0 + lane;
-                                float mv = 0.f;
-                                if (v < V) {
-                                    const double p = (double)(ex2((elem_value(y, v) - rec.my) * c) * rec.izy);
-                                    const double q = (double)(ex2((elem_value(x, v) - rec.mx) * c) * rec.izx);
-                                    double pi, qi;
-                                    seq_point(sh.st, ii - 1, v, p, q, pi, qi);
-                                    mv = (float)fmax(0.0, pi - qi);
-                                }
-                                const float incl = carry + warp_incl_scan(mv, lane);
-                                const unsigned hit = __ballot_sync(0xffffffffu, mv > 0.f && incl > loc.tc);
-                                const unsigned pos = __ballot_sync(0xffffffffu, mv > 0.f);
-                                if (hit) tok = (int)(v0 + __ffs(hit) - 1);
-                                else if (pos) last = (int)(v0 + 31 - __clz(pos));
-                                carry = __shfl_sync(0xffffffffu, incl, 31);
-                            }
-                            if (tok < 0) tok = last;
-                        }
-                    } else {  // no residual mass: keep the last target distribution
-                        tok = -2;
-                    }
-                    if (lane == 0) sh.out_tok = tok;
-                }
-            }
-            __syncthreads();
-            if (i == m - 1) {
-                if (sh.out_tok == -2) {
-                    // p_{m+1} = p_m: draw from it with the same uniform (a
-                    // pass over the row's masses p_m, as above)
-                    for (int chn = warp; chn < P.nch; chn += kWarps) {
-                        const uint64_t pol = policy_evict_normal();
-                        uint4 bx[kLoads], by[kLoads];
-                        load_chunk<T, VEC>(x, V, chn, lane, pol, bx);
-                        load_chunk<T, VEC>(y, V, chn, lane, pol, by);
-                        float acc = 0.f;
-#pragma unroll
-                        for (int k = 0; k < kLoads; ++k) {
-                            float fx[Traits<T>::kPerVec], fy[Traits<T>::kPerVec];
-                            unpack<T>(bx[k], fx);
-                            unpack<T>(by[k], fy);
-#pragma unroll
-                            for (int e = 0; e < Traits<T>::kPerVec; ++e) {
-                                const int64_t v = (int64_t)chn * chunk_elems<T>() +
-                                                  k * 32 * Traits<T>::kPerVec +
-                                                  lane * Traits<T>::kPerVec + e;
-                                if (v >= V) continue;
-                                const double p = (double)(ex2((fy[e] - rec.my) * c) * rec.izy);
-                                const double q = (double)(ex2((fx[e] - rec.mx) * c) * rec.izx);
-                                double pi, qi;
-                                seq_point(sh.st, ii - 1, v, p, q, pi, qi);
-                                acc += (float)pi;
-                            }
-                        }
-                        acc = warp_sum(acc);
-                        if (lane == 0) tab[chn] = make_float4(0.f, acc, 0.f, 0.f);
-                    }
-                    __syncthreads();
-                    if (warp == 0) {
-                        const TableSum Pt = table_sum(tab, P.nch, 0, 0.f, c, lane);
-                        const float uc = __ldg(P.u_correct + n0 + ch);
-                        int tok = -1;
-                        if (Pt.Z > 0.0) {
-                            const Located loc = table_locate(tab, P.nch, 0, 0.f, c, Pt, uc, lane);
-                            if (loc.ch >= 0) {
-                                float carry = 0.f;
-                                const int64_t base = (int64_t)loc.ch * chunk_elems<T>();
-                                int last = -1;
-                                for (int64_t v0 = base; v0 < base + chunk_elems<T>() && tok < 0; v0 += 32) {
-                                    const int64_t v = v0 + lane;
-                                    float mv = 0.f;
-                                    if (v < V) {
-                                        const double p = (double)(ex2((elem_value(y, v) - rec.my) * c) * rec.izy);
-                                        const double q = (double)(ex2((elem_value(x, v) - rec.mx) * c) * rec.izx);
-                                        double pi, qi;
-                                        seq_point(sh.st, ii - 1, v, p, q, pi, qi);
-                                        mv = (float)pi;
-                                    }
-                                    const float incl = carry + warp_incl_scan(mv, lane);
-                                    const unsigned hit = __ballot_sync(0xffffffffu, mv > 0.f && incl > loc.tc);
-                                    const unsigned pos = __ballot_sync(0xffffffffu, mv > 0.f);
-                                    if (hit) tok = (int)(v0 + __ffs(hit) - 1);
-                                    else if (pos) last = (int)(v0 + 31 - __clz(pos));
-                                    carry = __shfl_sync(0xffffffffu, incl, 31);
-                                }
-                                if (tok < 0) tok = last;
-                            }
-                        }
-                        if (lane == 0) sh.out_tok = tok;
-                    }
-                    __syncthreads();
-                }
-                if (threadIdx.x == 0) o.corr_tokens[n0 + ch] = sh.out_tok;
-            }
-        }
-        if (next < 0) break;  // every child rejected: the path ends at u
-        __syncthreads();
+        sh.next[n] = P.tlist[n0 + n];
+        sh.la[n] = n ? P.tnode[n0 + n].la : 0.f;
+        sh.on[n] = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        const int best = sh.cur;
+        int u = 0;
+        sh.on[0] = 1;
+        while (sh.next[u] > 0) {  // (a child comes after its parent)
+            u = sh.next[u];
+            sh.on[u] = 1;
+        }
+        sh.best = u;
+        sh.lastkid = 0;
+        sh.lk[0] = 0.0;
+    }
+    // log kappa: the path validity (Eq. 2) of every node, level by level
+    for (int l = 1; l <= sh.t.maxd; ++l) {
+        __syncthreads();
+        for (int n = threadIdx.x; n < N; n += kThreads)
+            if (sh.t.depth[n] == l) sh.lk[n] = sh.lk[sh.t.par[n]] + (double)sh.la[n];
+    }
+    __syncthreads();
+    const int best = sh.best;
+    for (int n = threadIdx.x; n < N; n += kThreads) {
+        const int pn = n ? sh.t.par[n] : 0;
+        float alpha = n ? 0.f : 1.f;
+        int acc = n ? 0 : 1;
+        if (n && sh.on[pn] && P.tnode[n0 + n].zp) {  // tried
+            alpha = P.tnode[n0 + n].lq;
+            acc = P.tnode[n0 + n].acc;
+        }
+        o.alpha[n0 + n] = alpha;
+        o.accept[n0 + n] = acc ? 1 : 0;
+        o.path_accept[n0 + n] = sh.on[n];
+        o.logkappa[n0 + n] = (float)sh.lk[n];
+        o.corr_tokens[n0 + n] = -1;
+        if (n && pn == best) atomicMax(&sh.lastkid, n);
+    }
+    __syncthreads();
+    const bool leaf = sh.lastkid == 0;
+    if (leaf && !P.tout.row_stats) {  // the leaf's row, for the bonus token
+        row_pass<T, VEC, true, kNoToken, false>(P, n0 + best, rg, tab, rsh);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
         o.deepest[b] = best;
         o.accept_len[b] = sh.t.depth[best];
-        o.bonus[b] = sh.nk > 0 ? sh.out_tok : ld_cg(P.rows + n0 + best).ps;
+        const int tok = leaf ? ld_cg(P.rows + n0 + best).ps : P.es.corr[n0 + best];
+        if (!leaf) o.corr_tokens[n0 + sh.lastkid] = tok;
+        o.bonus[b] = tok;
     }
 }
 

@@ -114,3 +114,31 @@ def test_tree_em_bad_tree_is_flagged(vsd):
     for b in (0, 2):
         assert g["loss"][b].item() == good["loss"][b].item()
         assert torch.equal(g["grad"][12 * b:12 * (b + 1)], good["grad"][12 * b:12 * (b + 1)])
+
+
+@pytest.mark.parametrize("V,dtype", [(300, "f32"), (1032, "bf16"), (2049, "bf16"), (1025, "f32")])
+def test_tree_sequential_many_siblings(vsd, oracle, V, dtype):
+    """Rows with more children than a warp has lanes, among them repeated
+    tokens, nearly all rejected: every rejection changes what the next child is
+    tested against, and the removed tokens keep the mass they had."""
+    from paper_2602_05774_gb300 import inputs
+    B, m = 4, 37
+    N = 1 + m + 3
+    g = torch.Generator().manual_seed(V)
+    p = inputs.linear_problem(B, N, 1, V, dtype, "gauss", seed=V, draft_sigma=1.0,
+                              noise_sigma=1.0)
+    par = torch.tensor([-1] + [0] * m + [1, 1, 2], dtype=torch.int32).view(1, N).repeat(B, 1)
+    rows = (torch.arange(B).view(B, 1) * N + par.clamp(min=0).long()).view(-1)
+    # tokens the draft likes better than the target does are rejected
+    top = (p["draft"].float() - 0.8 * p["target"].float()).topk(m, dim=1).indices.to(torch.int32)
+    tokens = top[rows, (torch.arange(N).repeat(B) - 1).clamp(0, m - 1)].view(B, N)
+    tokens[:, 9], tokens[:, 35] = tokens[:, 3], tokens[:, 2]  # repeated siblings
+    ua = 1.0 - torch.rand(B, N, generator=g) * 0.02
+    uc = torch.rand(B, N, generator=g)
+    orc = oracle.tree(_np32(p["draft"]), _np32(p["target"]), 1.0, par.numpy(), tokens.numpy(),
+                      _np32(ua), _np32(uc), rule=1)
+    assert orc["corr_tokens"][:, m].max() >= 0  # every sibling of some row tried
+    got = vsd.verify_tree(p["draft"].cuda(), p["target"].cuda(), par.cuda(), tokens.cuda(),
+                          ua.cuda(), uc.cuda(), 1.0, rule=vsd.TREE_SEQUENTIAL)
+    torch.cuda.synchronize()
+    compare_tree_sequential(got, orc)
