@@ -176,6 +176,17 @@ template <> __device__ __forceinline__ float vec_max<__nv_bfloat16>(const uint4&
     return fmaxf(__low2float(m), __high2float(m));
 }
 
+// Programmatic dependent launch: let the next kernel's blocks start once every
+// block of this grid has come here (or ended); wait for the previous kernel of
+// the stream to complete.  Every kernel of a chain waits, so each one follows
+// all those before it.
+__device__ __forceinline__ void grid_launch_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- TMA / mbarrier
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);

@@ -59,4 +59,23 @@ static cudaError_t prep(K kernel, size_t smem) {
     return ensure_dyn_smem(reinterpret_cast<const void*>(kernel), smem);
 }
 
+// Launch `kern` as a programmatic dependent of the stream's previous kernel: its
+// blocks may become resident while that kernel's last ones still run, and wait
+// in grid_wait() until it has completed and its writes are visible.
+template <typename... P, typename... A>
+static cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem,
+                                cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 }  // namespace vsd

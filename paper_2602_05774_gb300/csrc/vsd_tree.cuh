@@ -5,11 +5,10 @@
 //   k_tree_rows  one block per node row u: the row pass (tables, statistics,
 //                the target's argmax, a draw from p with u's uniform), then
 //                for every child x of u its token's test at u's row (Eq. 1,
-//                each branch alone) and, for the EM, the draws a corrected
-//                path may take at x: from p with x's uniform (below a
-//                rejection) and from the residual norm(max(0, p - q)) (the
-//                first rejection; one more read of the row when a child is
-//                rejected).
+//                each branch alone).
+//   k_tree_draws one block per row with children: the draws their corrected
+//                paths take there, from the residual norm(max(0, p - q)) at
+//                the first rejection, from p below it.
 //   k_tree_em    one block per tree: the accepted paths, the corrected path
 //                z' of every node, the log-kappa sums along the root paths
 //                (Eq. 2), o~ and o' (Algorithm 2), beta and zeta over the nodes
@@ -31,7 +30,7 @@ struct __align__(16) TreeNodeRec {
     float la;      // log alpha of x's token at its parent's row (the branch alone)
     float lq;      // log q of that token
     int acc;       // u_accept <= alpha
-    int zp;        // draw from p at the parent's row with x's u_correct
+    int zp;        // draw from p at the parent's row with x's u_correct (-1: none)
     float lq_zp, la_zp;
     int zr;        // residual draw at the parent's row with x's u_correct (-1: none)
     float lq_zr, la_zr;
@@ -50,104 +49,144 @@ struct __align__(16) TreeCoef {
 static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 
 // ------------------------------------------------------------ k_tree_rows
-template <typename T, bool VEC>
-__device__ void tree_row_children(const Problem<T>& P, int r, Ring* rg, float4* tab, int* s_any) {
-    const int N = P.N;
-    const int64_t V = P.V;
-    const int b = r / N, u = r - b * N, n0 = b * N;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int32_t* par = P.parent + (int64_t)n0;
-    const T* x = P.draft + (int64_t)r * V;
-    const T* y = P.target + (int64_t)r * V;
-    const float c = P.ts.c;
-    const uint64_t pol = policy_evict_normal();
-    const RowRec rec = ld_cg(P.rows + r);
-    if (threadIdx.x == 0) *s_any = 0;
-    __syncthreads();
-    // the target's table for the draws from p (each warp, identical values)
-    float My = 0.f;
-    TableSum Sy{0, 0, 0.0};
-    My = table_max(tab, P.nch, 1, lane);
-    Sy = table_sum(tab, P.nch, 1, frame_of(My), c, lane);
-    int k = 0;
-    for (int n = u + 1; n < N; ++n) {
-        if (__ldg(par + n) != u) continue;
-        if (k++ % kWarps != warp) continue;
-        TreeNodeRec nr;
-        nr.la = -INFINITY;
-        nr.lq = -INFINITY;
-        nr.zp = -1;
-        nr.lq_zp = nr.la_zp = -INFINITY;
-        nr.zr = -1;
-        nr.lq_zr = nr.la_zr = -INFINITY;
-        nr.pad[0] = nr.pad[1] = nr.pad[2] = 0;
-        const int tok = __ldg(P.given_tokens + n0 + n);
-        if (tok < 0 || tok >= V) {
-            if (lane == 0) atomicOr(P.status, VSD_STATUS_BAD_TOKEN);
-        } else if (!rec.flags) {
-            token_logs(x, y, tok, rec, P.ts.invTd, &nr.lq, &nr.la);
-        }
-        nr.acc = nr.la > -INFINITY && __ldg(P.u_accept + n0 + n) <= expf(nr.la);
-        if (!rec.flags) {
-            int zp = warp_sample<T, VEC>(x, y, V, tab, P.nch, 1, My, Sy,
-                                         __ldg(P.u_correct + n0 + n), c, lane, pol);
-            if (zp >= V) zp = -1;
-            nr.zp = zp;
-            if (zp >= 0) token_logs(x, y, zp, rec, P.ts.invTd, &nr.lq_zp, &nr.la_zp);
-        }
-        if (lane == 0) {
-            P.tnode[n0 + n] = nr;
-            if (!nr.acc) *s_any = 1;
-        }
-    }
-    __syncthreads();
-    if (!*s_any || rec.flags) return;
-    // a child is rejected: the residual max(0, p - q) of the row, and each
-    // rejected child's draw from it (or from p if it has no mass)
-    const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
-    stream_residual<T, VEC>(rg, x, y, V, 0, P.nch, tab, mr, P.status);
-    __syncthreads();
-    const TableSum Rt = table_sum(tab, P.nch, 0, 0.f, c, lane);
-    k = 0;
-    for (int n = u + 1; n < N; ++n) {
-        if (__ldg(par + n) != u) continue;
-        if (k++ % kWarps != warp) continue;
-        TreeNodeRec nr = P.tnode[n0 + n];  // written by this warp above
-        if (nr.acc) continue;
-        int zr = -1;
-        if (Rt.Z > 0.0) {
-            const Located loc =
-                table_locate(tab, P.nch, 0, 0.f, c, Rt, __ldg(P.u_correct + n0 + n), lane);
-            if (loc.ch >= 0)
-                zr = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane, pol);
-            if (zr >= V) zr = -1;
-        } else {
-            zr = nr.zp;  // no residual mass: the draw from p with the same uniform
-        }
-        nr.zr = zr;
-        if (zr >= 0) token_logs(x, y, zr, rec, P.ts.invTd, &nr.lq_zr, &nr.la_zr);
-        if (lane == 0) P.tnode[n0 + n] = nr;
-    }
-}
-
+// One block per node row: the row pass, then each child's token tested at the
+// row (one thread per child: Eq. 1, each branch alone), and the row's chunk
+// table kept in global memory for the draws.
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_tree_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    __shared__ int s_any;
-    Ring* rg = nullptr;
+    Ring* rg;
     float4* tab;
-    if (VEC) {
-        rg = reinterpret_cast<Ring*>(dsm);
-        tab = reinterpret_cast<float4*>(dsm + sizeof(Ring));
-        ring_init(rg, P.timeout_ns);
-    } else {
-        tab = reinterpret_cast<float4*>(dsm);
-    }
-    const int r = blockIdx.x;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
+    const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
+    const int64_t V = P.V;
     row_pass<T, VEC, true, kNoToken, true>(P, r, rg, tab, sh);
     __syncthreads();
-    tree_row_children<T, VEC>(P, r, rg, tab, &s_any);
+    const RowRec rec = ld_cg(P.rows + r);
+    int kids = 0;
+    for (int n = u + 1 + threadIdx.x; n < N; n += kThreads) {
+        if (__ldg(P.parent + n0 + n) != u) continue;
+        kids = 1;
+        TreeNodeRec nr;
+        nr.la = nr.lq = -INFINITY;
+        nr.zp = nr.zr = -1;
+        nr.lq_zp = nr.la_zp = nr.lq_zr = nr.la_zr = -INFINITY;
+        nr.pad[0] = nr.pad[1] = nr.pad[2] = 0;
+        const int tok = __ldg(P.given_tokens + n0 + n);
+        if (tok < 0 || tok >= V)
+            atomicOr(P.status, VSD_STATUS_BAD_TOKEN);
+        else if (!rec.flags)
+            token_logs(P.draft + (int64_t)r * V, P.target + (int64_t)r * V, tok, rec, P.ts.invTd,
+                       &nr.lq, &nr.la);
+        nr.acc = nr.la > -INFINITY && __ldg(P.u_accept + n0 + n) <= expf(nr.la);
+        P.tnode[n0 + n] = nr;
+    }
+    if (__syncthreads_or(kids))
+        for (int ch = threadIdx.x; ch < P.nch; ch += kThreads)
+            P.gtab[(int64_t)r * P.nch_ws + ch] = tab[ch];
+}
+
+// ------------------------------------------------------------ k_tree_draws
+// One block per row with children: the corrected tokens its children may
+// need, and no others.  On an accepted path a rejected child draws from the
+// row's residual max(0, p - q) (one more read of the row; from p if that has
+// no mass); below a rejection every child draws from p, for which the row's
+// chunk table and one chunk suffice.  Whether u is on an accepted path follows
+// from the acceptance bits of its ancestors, which are all known here; only
+// these few rows are read twice (64 trees of 60 nodes: about 300 of 3840).
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ int s_par[1024], s_path;
+    Ring* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
+    const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int kids = 0;
+    for (int n = threadIdx.x; n < N; n += kThreads) {
+        const int pn = __ldg(P.parent + n0 + n);
+        s_par[n] = pn;
+        kids |= n > u && pn == u;
+    }
+    grid_wait();
+    if (!__syncthreads_or(kids)) return;
+    if (threadIdx.x == 0) {
+        int path = 1, x = u;
+        while (x > 0 && path > 0) {
+            const int pn = s_par[x];
+            path = pn < 0 || pn >= x ? -1 : ld_cg(&P.tnode[n0 + x].acc) != 0;  // -1: a bad tree
+            x = pn;
+        }
+        s_path = path;
+    }
+    __syncthreads();
+    const int path = s_path;
+    const RowRec rec = ld_cg(P.rows + r);
+    if (path < 0 || rec.flags) return;
+    const int64_t V = P.V;
+    const T* x = P.draft + (int64_t)r * V;
+    const T* y = P.target + (int64_t)r * V;
+    const float c = P.ts.c;
+    const uint64_t pol = policy_evict_normal();
+    const double invT = P.ts.invTd;
+    // f(n) for the children that need a draw, shared out among the warps
+    auto each_child = [&](auto&& f) {
+        int k = 0;
+        for (int n = u + 1; n < N; ++n)
+            if (s_par[n] == u && !(path && ld_cg(&P.tnode[n0 + n].acc)) && k++ % kWarps == warp)
+                f(n0 + n);
+    };
+    if (path) {
+        int rej = 0;
+        for (int n = u + 1 + threadIdx.x; n < N; n += kThreads)
+            rej |= s_par[n] == u && !ld_cg(&P.tnode[n0 + n].acc);
+        if (!__syncthreads_or(rej)) return;
+        const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
+        stream_residual<T, VEC>(rg, x, y, V, 0, P.nch, tab, mr, P.status);
+        __syncthreads();
+        const TableSum Rt = table_sum(tab, P.nch, 0, 0.f, c, lane);
+        if (Rt.Z > 0.0) {
+            each_child([&](int n) {
+                const Located loc =
+                    table_locate(tab, P.nch, 0, 0.f, c, Rt, __ldg(P.u_correct + n), lane);
+                if (loc.ch < 0) return;
+                const int z = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane,
+                                                              pol);
+                if (z < 0 || z >= V) return;
+                float lq, la;
+                token_logs(x, y, z, rec, invT, &lq, &la);
+                if (lane == 0) {
+                    P.tnode[n].zr = z;
+                    P.tnode[n].lq_zr = lq;
+                    P.tnode[n].la_zr = la;
+                }
+            });
+            return;
+        }
+        __syncthreads();  // no residual mass: draws from p with the same uniforms
+    }
+    for (int ch = threadIdx.x; ch < P.nch; ch += kThreads)
+        tab[ch] = ld_cg(P.gtab + (int64_t)r * P.nch_ws + ch);
+    __syncthreads();
+    const float My = table_max(tab, P.nch, 1, lane);
+    const TableSum Sy = table_sum(tab, P.nch, 1, frame_of(My), c, lane);
+    each_child([&](int n) {
+        const int z = warp_sample<T, VEC>(x, y, V, tab, P.nch, 1, My, Sy, __ldg(P.u_correct + n), c,
+                                          lane, pol);
+        if (z < 0 || z >= V) return;
+        float lq, la;
+        token_logs(x, y, z, rec, invT, &lq, &la);
+        if (lane == 0) {
+            TreeNodeRec* nr = P.tnode + n;
+            (path ? nr->zr : nr->zp) = z;
+            (path ? nr->lq_zr : nr->lq_zp) = lq;
+            (path ? nr->la_zr : nr->la_zp) = la;
+        }
+    });
 }
 
 // ------------------------------------------------------------ shared helpers
@@ -211,25 +250,242 @@ __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
 }
 
 // ------------------------------------------------------------ k_tree_em
-// The M-step of one tree, in double precision on one thread (a tree has at
-// most 1024 nodes; the arithmetic follows the proposals in node order, so the
-// result does not depend on scheduling).  Scratch per node in shared memory.
+// The M-step of one tree, in double precision, by one block: the sums along
+// the root paths go level by level (a node adds its term to its parent's sum),
+// the subtree sums back up level by level (a node adds its children's sums in
+// descending node order), and what belongs to one node or one depth is taken
+// in parallel.  The order of every sum is fixed, so the result does not depend
+// on scheduling.  (On one thread per tree the fp64 latency of this pass was
+// 578 us of a call's 873 at 64 trees of 60 nodes; the whole call now takes 252.)
 struct TreeEmShared {
     TreeShared2 t;
     double lk[1024], lkc[1024], lkr[1024], lqt[1024], lqz[1024];
-    double st[1024], sz[1024];   // subtree sums of the gradient terms
+    union {
+        struct {
+            float la[1024], laz[1024], lar[1024], lq[1024];  // the nodes' own terms
+        } e;
+        struct {
+            double st[1024], sz[1024];  // CAR logits, then subtree sums of the gradient terms
+        } m;
+    };
     float w[1024][4];            // o~, o', beta, zeta
     float lqzn[1024];            // log q of z'_x at its parent's row
     int z[1024];                 // corrected token z'_x
+    unsigned char acc[1024];
+    short first[1024], last[1024];  // a node's first and last child (0: none)
+    double red[kWarps][2];
 };
+
+// Sum over the block in a fixed order; every thread returns it.
+__device__ __forceinline__ double2 block_sum(double2 v, double (*red)[2]) {
+    v.x = warp_sum(v.x);
+    v.y = warp_sum(v.y);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5][0] = v.x;
+        red[threadIdx.x >> 5][1] = v.y;
+    }
+    __syncthreads();
+    double2 s = make_double2(0.0, 0.0);
+    for (int w = 0; w < kWarps; ++w) {
+        s.x += red[w][0];
+        s.y += red[w][1];
+    }
+    return s;
+}
+
+template <typename T>
+__device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o, int b,
+                              TreeEmShared& sh) {
+    const int N = P.N, n0 = b * N, tid = threadIdx.x;
+    const int warp = tid >> 5, lane = tid & 31;
+    const int* par = sh.t.par;
+    const int* depth = sh.t.depth;
+    const int maxd = sh.t.maxd;
+    for (int n = tid; n < N; n += kThreads) {
+        sh.acc[n] = n ? P.tnode[n0 + n].acc != 0 : 1;
+        sh.first[n] = sh.last[n] = 0;
+    }
+    // accepted paths
+    for (int l = 0; l <= maxd; ++l) {
+        __syncthreads();
+        for (int n = tid; n < N; n += kThreads)
+            if (depth[n] == l) sh.t.pacc[n] = n ? sh.acc[n] && sh.t.pacc[par[n]] : 1;
+    }
+    __syncthreads();
+    // the E-step per node (R15): z' and the node's terms of the sums
+    for (int n = tid; n < N; n += kThreads) {
+        if (n == 0) {
+            sh.lk[0] = sh.lkc[0] = sh.lkr[0] = sh.lqt[0] = sh.lqz[0] = 0.0;
+            sh.z[0] = -1;
+            sh.lqzn[0] = 0.f;
+            continue;
+        }
+        const int a = par[n];
+        const TreeNodeRec nr = ld_cg_rec(P.tnode + n0 + n);
+        const RowRec ra = ld_cg(P.rows + n0 + a);
+        int zc;
+        float lqz, laz;
+        if (sh.t.pacc[n]) {
+            zc = __ldg(P.given_tokens + n0 + n); lqz = nr.lq; laz = nr.la;
+        } else if (sh.t.pacc[a]) {  // the first rejection on the path: the residual
+            zc = nr.zr; lqz = nr.lq_zr; laz = nr.la_zr;
+        } else {                    // below a rejection: the draw from p
+            zc = nr.zp; lqz = nr.lq_zp; laz = nr.la_zp;
+        }
+        if (zc < 0) { lqz = -INFINITY; laz = -INFINITY; }
+        sh.z[n] = zc;
+        sh.lqzn[n] = lqz;
+        sh.e.la[n] = nr.la;
+        sh.e.laz[n] = laz;
+        sh.e.lar[n] = (ra.flags || ra.ref < 0) ? -INFINITY : ra.la_ref;
+        sh.e.lq[n] = nr.lq;
+        if (o.logq_tok) o.logq_tok[n0 + n] = nr.lq;
+    }
+    for (int l = 1; l <= maxd; ++l) {
+        __syncthreads();
+        for (int n = tid; n < N; n += kThreads) {
+            if (depth[n] != l) continue;
+            const int a = par[n];
+            sh.lk[n] = sh.lk[a] + (double)sh.e.la[n];
+            sh.lkc[n] = sh.lkc[a] + (double)sh.e.laz[n];
+            sh.lkr[n] = sh.lkr[a] + (double)sh.e.lar[n];
+            sh.lqt[n] = sh.lqt[a] + (double)sh.e.lq[n];
+            sh.lqz[n] = sh.lqz[a] + (double)sh.lqzn[n];
+        }
+    }
+    __syncthreads();
+    // o~, o' (Algorithm 2 with w(depth): w(l) = w_base^l, trees may be deeper
+    // than the host's table of w), N_b, the CAR logits
+    double2 Nb = make_double2(0.0, 0.0);
+    for (int n = 1 + tid; n < N; n += kThreads) {
+        const double wl = pow(P.w_base, (double)depth[n]);
+        const bool ot = sh.lk[n] >= sh.lkr[n];
+        const bool op = ot || sh.lkc[n] >= sh.lkr[n];
+        sh.w[n][0] = ot ? 1.f : 0.f;
+        sh.w[n][1] = op ? (float)wl : 0.f;
+        if (op) Nb.x += wl;
+        sh.m.st[n] = (P.zeta_mode == 0 ? exp(sh.lqt[n]) : sh.lqt[n]) * P.inv_tau;
+    }
+    Nb = block_sum(Nb, sh.red);
+    // beta (leave-one-out) and zeta (softmax of q(z~)/tau, or log q in
+    // zeta_mode 1) over the nodes of each depth: one warp per depth.  (All o'
+    // of a depth are equal or 0, so the sums behind beta are exact.)
+    for (int l = 1 + warp; l <= maxd; l += kWarps) {
+        double num = 0.0, den = 0.0, cmax = -INFINITY;
+        for (int n = 1 + lane; n < N; n += 32) {
+            if (depth[n] != l) continue;
+            const double op = sh.w[n][1];
+            num += op * sh.w[n][0];
+            den += op;
+            cmax = fmax(cmax, sh.m.st[n]);
+        }
+        num = warp_sum(num);
+        den = warp_sum(den);
+#pragma unroll
+        for (int k = 16; k; k >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, k));
+        double zs = 0.0;
+        for (int n = 1 + lane; n < N; n += 32) {
+            if (depth[n] != l) continue;
+            const double ez = exp(sh.m.st[n] - cmax);
+            sh.m.st[n] = ez;
+            zs += ez;
+        }
+        zs = warp_sum(zs);
+        for (int n = 1 + lane; n < N; n += 32) {
+            if (depth[n] != l) continue;
+            const double op = sh.w[n][1];
+            const double d1 = den - op, n1 = num - op * sh.w[n][0];
+            sh.w[n][2] = d1 > 0.0 ? (float)(n1 / d1) : 0.f;
+            sh.w[n][3] = (float)(sh.m.st[n] / zs);
+        }
+    }
+    __syncthreads();
+    // the objective (Eq. advance) and each proposal's gradient terms; the
+    // nodes' first and last children
+    double2 J = make_double2(0.0, 0.0);
+    for (int n = tid; n < N; n += kThreads) {
+        double st = 0.0, sz = 0.0;
+        if (n) {
+            const double ot = sh.w[n][0], op = sh.w[n][1];
+            const double bz = (double)sh.w[n][2] * (double)sh.w[n][3];
+            if (op != 0.0) {
+                const double lqn = ot > 0.0 ? sh.lqt[n] : sh.lqz[n];
+                J.x += op * (lqn - bz * sh.lqt[n]);
+                st = op * (ot - bz);
+                sz = op * (1.0 - ot);
+            }
+            bool f = true, z = true;
+            for (int k = par[n] + 1; k < n && f; ++k) f = par[k] != par[n];
+            for (int k = n + 1; k < N && z; ++k) z = par[k] != par[n];
+            if (f) sh.first[par[n]] = (short)n;
+            if (z) sh.last[par[n]] = (short)n;
+        }
+        sh.m.st[n] = st;
+        sh.m.sz[n] = sz;
+    }
+    J = block_sum(J, sh.red);
+    // subtree sums (the proposals whose path goes through a node)
+    for (int l = maxd - 1; l >= 0; --l) {
+        for (int a = tid; a < N; a += kThreads) {
+            if (depth[a] != l || !sh.last[a]) continue;
+            double st = sh.m.st[a], sz = sh.m.sz[a];
+            for (int n = sh.last[a]; n >= sh.first[a]; --n)
+                if (par[n] == a) {
+                    st += sh.m.st[n];
+                    sz += sh.m.sz[n];
+                }
+            sh.m.st[a] = st;
+            sh.m.sz[a] = sz;
+        }
+        __syncthreads();
+    }
+    const double scale = Nb.x > 0.0 ? 1.0 / ((double)P.B * Nb.x * P.ts.Td) : 0.0;
+    if (tid == 0) o.loss[b] = Nb.x > 0.0 ? (float)(-J.x / Nb.x) : 0.f;
+    for (int x = tid; x < N; x += kThreads) {
+        if (x) {
+            TreeCoef cf;
+            cf.t = __ldg(P.given_tokens + n0 + x);
+            cf.ct = (float)(sh.m.st[x] * scale);
+            cf.z = sh.z[x];
+            cf.cz = (float)(sh.m.sz[x] * scale);
+            if (cf.z == cf.t) {
+                cf.ct = (float)((sh.m.st[x] + sh.m.sz[x]) * scale);
+                cf.z = -1;
+                cf.cz = 0.f;
+            }
+            P.tcoef[n0 + x] = cf;
+        }
+        float g = 0.f;  // the row's dense factor: its children's, in node order
+        if (sh.last[x])
+            for (int n = sh.first[x]; n <= sh.last[x]; ++n)
+                if (par[n] == x) g += (float)((sh.m.st[n] + sh.m.sz[n]) * scale);
+        P.tg[n0 + x] = g;
+        if (o.corr_tokens) o.corr_tokens[n0 + x] = sh.z[x];
+        if (o.weights)
+            reinterpret_cast<float4*>(o.weights)[n0 + x] =
+                x ? make_float4(sh.w[x][0], sh.w[x][1], sh.w[x][2], sh.w[x][3])
+                  : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (o.logq_tok && x == 0) o.logq_tok[n0] = 0.f;
+        if (o.logq_corr) o.logq_corr[n0 + x] = sh.lqzn[x];
+        if (o.logkappa) o.logkappa[n0 + x] = (float)sh.lk[x];
+        if (o.logkappa_corr) o.logkappa_corr[n0 + x] = (float)sh.lkc[x];
+        if (o.logkappa_ref) o.logkappa_ref[n0 + x] = (float)sh.lkr[x];
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_tree_em(Problem<T> P, vsd_tree_em_outputs o) {
     extern __shared__ __align__(128) unsigned char dsm[];
     TreeEmShared& sh = *reinterpret_cast<TreeEmShared*>(dsm);
     const int N = P.N, b = blockIdx.x, n0 = b * N;
+    grid_launch_next();
     const bool ok = tree_load<T>(P, b, sh.t);
-    if (!ok) {
+    grid_wait();
+    if (ok) {
+        if (threadIdx.x == 0) P.tbad[b] = 0;
+        tree_em_nodes<T>(P, o, b, sh);
+    } else {
         for (int n = threadIdx.x; n < N; n += kThreads) {
             P.tcoef[n0 + n] = TreeCoef{-1, 0.f, -1, 0.f};
             P.tg[n0 + n] = 0.f;
@@ -241,129 +497,6 @@ __global__ void __launch_bounds__(kThreads) k_tree_em(Problem<T> P, vsd_tree_em_
             atomicOr(P.status, VSD_STATUS_BAD_TREE);
             P.tbad[b] = 1;
             o.loss[b] = 0.f;
-        }
-    } else if (threadIdx.x == 0) {
-        P.tbad[b] = 0;
-        const int* par = sh.t.par;
-        const int* depth = sh.t.depth;
-        // the E-step per node (R15): accepted paths, z', the sums along the paths
-        sh.t.pacc[0] = 1;
-        sh.lk[0] = sh.lkc[0] = sh.lkr[0] = sh.lqt[0] = sh.lqz[0] = 0.0;
-        sh.z[0] = -1;
-        sh.lqzn[0] = 0.f;
-        for (int x = 1; x < N; ++x) {
-            const int a = par[x];
-            const TreeNodeRec nr = ld_cg_rec(P.tnode + n0 + x);
-            const RowRec ra = ld_cg(P.rows + n0 + a);
-            const int tok = __ldg(P.given_tokens + n0 + x);
-            const bool pa = nr.acc && sh.t.pacc[a];
-            sh.t.pacc[x] = pa;
-            int zc;
-            float lqz, laz;
-            if (pa) {
-                zc = tok; lqz = nr.lq; laz = nr.la;
-            } else if (sh.t.pacc[a]) {  // the first rejection on the path: the residual
-                zc = nr.zr; lqz = nr.lq_zr; laz = nr.la_zr;
-            } else {                    // below a rejection: the draw from p
-                zc = nr.zp; lqz = nr.lq_zp; laz = nr.la_zp;
-            }
-            if (zc < 0) { lqz = -INFINITY; laz = -INFINITY; }
-            sh.z[x] = zc;
-            sh.lqzn[x] = lqz;
-            const double lar = (ra.flags || ra.ref < 0) ? -INFINITY : (double)ra.la_ref;
-            sh.lk[x] = sh.lk[a] + (double)nr.la;
-            sh.lkc[x] = sh.lkc[a] + (double)laz;
-            sh.lkr[x] = sh.lkr[a] + lar;
-            sh.lqt[x] = sh.lqt[a] + (double)nr.lq;
-            sh.lqz[x] = sh.lqz[a] + (double)lqz;
-        }
-        // o~, o' (Algorithm 2 with w(depth))
-        double Nb = 0.0;
-        for (int n = 1; n < N; ++n) {
-            // w(l) = w_base^l at the node's depth (trees may be deeper than the
-            // host's table of w)
-            const double wl = pow(P.w_base, (double)depth[n]);
-            const bool ot = sh.lk[n] >= sh.lkr[n];
-            const bool op = ot || sh.lkc[n] >= sh.lkr[n];
-            sh.w[n][0] = ot ? 1.f : 0.f;
-            sh.w[n][1] = op ? (float)wl : 0.f;
-            Nb += op ? wl : 0.0;
-        }
-        // beta (leave-one-out) and zeta (softmax of q(z~)/tau, or log q in
-        // zeta_mode 1) over the nodes of each depth
-        for (int l = 1; l <= sh.t.maxd; ++l) {
-            double num = 0.0, den = 0.0, cmax = -INFINITY;
-            for (int n = 1; n < N; ++n) {
-                if (depth[n] != l) continue;
-                const double op = sh.w[n][1];
-                num += op * sh.w[n][0];
-                den += op;
-                const double cq = (P.zeta_mode == 0 ? exp(sh.lqt[n]) : sh.lqt[n]) * P.inv_tau;
-                cmax = fmax(cmax, cq);
-            }
-            double zs = 0.0;
-            for (int n = 1; n < N; ++n) {
-                if (depth[n] != l) continue;
-                const double cq = (P.zeta_mode == 0 ? exp(sh.lqt[n]) : sh.lqt[n]) * P.inv_tau;
-                zs += exp(cq - cmax);
-            }
-            for (int n = 1; n < N; ++n) {
-                if (depth[n] != l) continue;
-                const double op = sh.w[n][1];
-                const double d1 = den - op, n1 = num - op * sh.w[n][0];
-                sh.w[n][2] = d1 > 0.0 ? (float)(n1 / d1) : 0.f;
-                const double cq = (P.zeta_mode == 0 ? exp(sh.lqt[n]) : sh.lqt[n]) * P.inv_tau;
-                sh.w[n][3] = (float)(exp(cq - cmax) / zs);
-            }
-        }
-        // the objective (Eq. advance), each proposal's terms, subtree sums
-        // (the proposals whose path goes through a node)
-        double J = 0.0;
-        for (int n = 0; n < N; ++n) sh.st[n] = sh.sz[n] = 0.0;
-        for (int n = 1; n < N; ++n) {
-            const double ot = sh.w[n][0], op = sh.w[n][1];
-            const double bz = (double)sh.w[n][2] * (double)sh.w[n][3];
-            if (op == 0.0) continue;
-            const double lqn = ot > 0.0 ? sh.lqt[n] : sh.lqz[n];
-            J += op * (lqn - bz * sh.lqt[n]);
-            sh.st[n] += op * (ot - bz);
-            sh.sz[n] += op * (1.0 - ot);
-        }
-        for (int n = N - 1; n >= 1; --n) {  // children come after their parents
-            sh.st[par[n]] += sh.st[n];
-            sh.sz[par[n]] += sh.sz[n];
-        }
-        const double scale = Nb > 0.0 ? 1.0 / ((double)P.B * Nb * P.ts.Td) : 0.0;
-        for (int n = 0; n < N; ++n) P.tg[n0 + n] = 0.f;
-        o.loss[b] = Nb > 0.0 ? (float)(-J / Nb) : 0.f;
-        for (int x = 1; x < N; ++x) {
-            TreeCoef cf;
-            cf.t = __ldg(P.given_tokens + n0 + x);
-            cf.ct = (float)(sh.st[x] * scale);
-            cf.z = sh.z[x];
-            cf.cz = (float)(sh.sz[x] * scale);
-            if (cf.z == cf.t) {
-                cf.ct = (float)((sh.st[x] + sh.sz[x]) * scale);
-                cf.z = -1;
-                cf.cz = 0.f;
-            }
-            P.tcoef[n0 + x] = cf;
-            P.tg[n0 + par[x]] += (float)((sh.st[x] + sh.sz[x]) * scale);
-        }
-    }
-    __syncthreads();
-    if (ok) {
-        for (int n = threadIdx.x; n < N; n += kThreads) {
-            if (o.corr_tokens) o.corr_tokens[n0 + n] = sh.z[n];
-            if (o.weights)
-                reinterpret_cast<float4*>(o.weights)[n0 + n] =
-                    n ? make_float4(sh.w[n][0], sh.w[n][1], sh.w[n][2], sh.w[n][3])
-                      : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (o.logq_tok) o.logq_tok[n0 + n] = n ? ld_cg(&P.tnode[n0 + n].lq) : 0.f;
-            if (o.logq_corr) o.logq_corr[n0 + n] = sh.lqzn[n];
-            if (o.logkappa) o.logkappa[n0 + n] = (float)sh.lk[n];
-            if (o.logkappa_corr) o.logkappa_corr[n0 + n] = (float)sh.lkc[n];
-            if (o.logkappa_ref) o.logkappa_ref[n0 + n] = (float)sh.lkr[n];
         }
     }
     if (threadIdx.x == 0) {
@@ -378,121 +511,106 @@ __global__ void __launch_bounds__(kThreads) k_tree_em(Problem<T> P, vsd_tree_em_
 // ------------------------------------------------------------ k_tree_grad
 // Row r of the gradient: g q(v) minus the sparse terms of r's children.  The
 // terms are merged by token in a fixed order (sorted by token, then by child)
-// so that the sums do not depend on scheduling.
-constexpr int kTreeMaxTerms = 2048;
-struct TreeGradShared {
-    int tok[kTreeMaxTerms];
-    float cf[kTreeMaxTerms];
-    int skey[kTreeMaxTerms];
-    float scf[kTreeMaxTerms];
-    int n, nu;
+// so that the sums do not depend on scheduling.  The dense part is written
+// first, eight 16-byte vectors in flight per thread (a row without one is
+// written as zeros and not read); then one thread per merged term writes its
+// element.  What bounds it: the rows' reads and writes (64 trees of 60 nodes,
+// V = 32000: 246 MB written, about half of the draft rows read).
+struct TreeGradTerm {
+    int tok, key;  // token; 2 n for node n's own token, 2 n + 1 for its corrected one
+    float cf;
 };
+inline size_t tree_grad_smem_bytes(int N) { return (size_t)N * 4 * sizeof(TreeGradTerm); }
 
 template <typename T, bool VEC, typename G>
 __global__ void __launch_bounds__(kThreads) k_tree_grad(Problem<T> P, G* grad) {
-    __shared__ TreeGradShared sh;
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ int s_n, s_nu;
     constexpr int PV = Traits<T>::kPerVec;
     const int N = P.N, r = blockIdx.x, b = r / N, u = r - b * N, n0 = b * N;
+    TreeGradTerm* tm = reinterpret_cast<TreeGradTerm*>(dsm);  // [2 N] as gathered, then merged
+    TreeGradTerm* srt = tm + 2 * N;                           // [2 N] sorted
     const int64_t V = P.V;
     G* g = grad + (int64_t)r * V;
     const T* x = P.draft + (int64_t)r * V;
     const int32_t* par = P.parent + (int64_t)n0;
-    if (threadIdx.x == 0) sh.n = 0;
+    if (threadIdx.x == 0) s_n = s_nu = 0;
+    grid_wait();
     __syncthreads();
     const bool bad = ld_cg(P.tbad + b) != 0;
     if (!bad) {  // the children's terms
         for (int n = u + 1 + threadIdx.x; n < N; n += kThreads) {
             if (__ldg(par + n) != u) continue;
             const TreeCoef cf = ld_cg_rec(P.tcoef + n0 + n);
-            const int slot = atomicAdd(&sh.n, cf.z >= 0 ? 2 : 1);
-            // (order fixed below by the sort key: token, then child index)
-            sh.tok[slot] = cf.t;
-            sh.cf[slot] = cf.ct;
-            sh.skey[slot] = 2 * n;
-            if (cf.z >= 0) {
-                sh.tok[slot + 1] = cf.z;
-                sh.cf[slot + 1] = cf.cz;
-                sh.skey[slot + 1] = 2 * n + 1;
-            }
+            const int slot = atomicAdd(&s_n, cf.z >= 0 ? 2 : 1);
+            tm[slot] = TreeGradTerm{cf.t, 2 * n, cf.ct};
+            if (cf.z >= 0) tm[slot + 1] = TreeGradTerm{cf.z, 2 * n + 1, cf.cz};
         }
     }
-    __syncthreads();
-    const int n = sh.n;
-    // rank sort by (token, key) into scf/skey order: entry i goes to its rank
-    __shared__ int rk_tok[kTreeMaxTerms];
-    for (int i = threadIdx.x; i < n; i += kThreads) {
-        int rank = 0;
-        for (int j = 0; j < n; ++j)
-            rank += sh.tok[j] < sh.tok[i] || (sh.tok[j] == sh.tok[i] && sh.skey[j] < sh.skey[i]);
-        rk_tok[rank] = sh.tok[i];
-        sh.scf[rank] = sh.cf[i];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {  // merge equal tokens, in order
-        int m = 0;
-        for (int i = 0; i < n; ++i) {
-            if (m > 0 && sh.tok[m - 1] == rk_tok[i]) {
-                sh.cf[m - 1] += sh.scf[i];
-            } else {
-                sh.tok[m] = rk_tok[i];
-                sh.cf[m] = sh.scf[i];
-                ++m;
-            }
-        }
-        sh.nu = m;
-    }
-    __syncthreads();
-    const int nu = sh.nu;
-    // the first merged term at or after token v (binary search)
-    auto first_at = [&](int64_t v) {
-        int lo = 0, hi = nu;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if ((int64_t)sh.tok[mid] < v) lo = mid + 1; else hi = mid;
-        }
-        return lo;
-    };
     const float gr = bad ? 0.f : ld_cg(P.tg + r);
     const RowRec rec = ld_cg(P.rows + r);
-    const float gq = (nu == 0 && gr == 0.f) ? 0.f : gr * rec.izx;
+    __syncthreads();
+    const int nt = s_n;
+    const float gq = (nt == 0 && gr == 0.f) ? 0.f : gr * rec.izx;
     const float mx = rec.mx, c = P.ts.c;
     const bool dense = gq != 0.f && isfinite(mx);
+    for (int i = threadIdx.x; i < nt; i += kThreads) {  // rank sort by (token, key)
+        int rank = 0;
+        for (int j = 0; j < nt; ++j)
+            rank += tm[j].tok < tm[i].tok || (tm[j].tok == tm[i].tok && tm[j].key < tm[i].key);
+        srt[rank] = tm[i];
+    }
     if constexpr (VEC) {
+        constexpr int U = 8, NP = PV / 2;
         const uint64_t pol = policy_evict_first();
         const int nvec = (int)(V / PV);
-        for (int i = threadIdx.x; i < nvec; i += kThreads) {
-            const int64_t v0 = (int64_t)i * PV;
-            float o[PV];
+        const uint64_t mx2 = f2(mx, mx), c2 = f2(c, c), gq2 = f2(gq, gq);
+        for (int i0 = threadIdx.x; i0 < nvec; i0 += kThreads * U) {
+            uint4 buf[U];
             if (dense) {
-                float f[PV];
-                unpack<T>(ld_stream(x + v0, pol), f);
 #pragma unroll
-                for (int e = 0; e < PV; ++e) o[e] = gq * ex2((f[e] - mx) * c);
-            } else {
-#pragma unroll
-                for (int e = 0; e < PV; ++e) o[e] = 0.f;
+                for (int k = 0; k < U; ++k)
+                    if (i0 + k * kThreads < nvec)
+                        buf[k] = ld_stream(x + (int64_t)(i0 + k * kThreads) * PV, pol);
             }
-            if (nu) {
-                for (int k = first_at(v0); k < nu && sh.tok[k] < v0 + PV; ++k) {
 #pragma unroll
-                    for (int e = 0; e < PV; ++e)
-                        if (v0 + e == sh.tok[k]) o[e] -= sh.cf[k];
+            for (int k = 0; k < U; ++k) {
+                const int i = i0 + k * kThreads;
+                if (i >= nvec) break;
+                float o[PV];
+                if (dense) {
+                    uint64_t pr[NP];
+                    vec_pairs<T>(buf[k], pr);
+#pragma unroll
+                    for (int q = 0; q < NP; ++q)
+                        f2split(f2mul(gq2, f2_mass(pr[q], mx2, c2)), o[2 * q], o[2 * q + 1]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < PV; ++e) o[e] = 0.f;
                 }
+                grad_store<T, G, PV>(g, (int64_t)i * PV, o, pol);
             }
-            grad_store<T, G, PV>(g, v0, o, pol);
         }
     } else {
         for (int64_t v = threadIdx.x; v < V; v += kThreads) {
-            float val = dense ? gq * ex2((elem_value(x, v) - mx) * c) : 0.f;
-            if (nu) {
-                const int k = first_at(v);
-                if (k < nu && sh.tok[k] == v) val -= sh.cf[k];
-            }
+            const float val = dense ? gq * ex2((elem_value(x, v) - mx) * c) : 0.f;
             if constexpr (sizeof(G) == 2)
                 g[v] = __float2bfloat16_rn(val);
             else
                 g[v] = val;
         }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nt; i += kThreads) {  // a token's first term sums them, in order
+        const int t = srt[i].tok;
+        if ((i && srt[i - 1].tok == t) || t < 0 || t >= V) continue;
+        float cf = srt[i].cf;
+        for (int j = i + 1; j < nt && srt[j].tok == t; ++j) cf += srt[j].cf;
+        const float val = (dense ? gq * ex2((elem_value(x, t) - mx) * c) : 0.f) - cf;
+        if constexpr (sizeof(G) == 2)
+            g[t] = __float2bfloat16_rn(val);
+        else
+            g[t] = val;
     }
 }
 

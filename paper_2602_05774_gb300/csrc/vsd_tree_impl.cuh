@@ -189,17 +189,24 @@ cudaError_t Launch<VSD_T>::tree_em(const Problem<VSD_T>& P, bool vec,
     if (e) return e;
     rows<<<P.R, kThreads, smem, s>>>(P);
     if ((e = cudaGetLastError())) return e;
+    auto draws = vec ? k_tree_draws<VSD_T, true> : k_tree_draws<VSD_T, false>;
+    if ((e = prep(draws, smem))) return e;
+    if ((e = launch_after(draws, P.R, kThreads, smem, s, P))) return e;
     if ((e = prep(k_tree_em<VSD_T>, sizeof(TreeEmShared)))) return e;
-    k_tree_em<VSD_T><<<P.B, kThreads, sizeof(TreeEmShared), s>>>(P, o);
-    if ((e = cudaGetLastError())) return e;
-#define VSD_TGRAD(V_, G_) \
-    k_tree_grad<VSD_T, V_, G_><<<P.R, kThreads, 0, s>>>(P, reinterpret_cast<G_*>(grad))
+    if ((e = launch_after(k_tree_em<VSD_T>, P.B, kThreads, sizeof(TreeEmShared), s, P, o)))
+        return e;
+    const size_t gsm = tree_grad_smem_bytes(P.N);
+#define VSD_TGRAD(V_, G_)                                                           \
+    do {                                                                            \
+        if ((e = prep(k_tree_grad<VSD_T, V_, G_>, gsm))) return e;                  \
+        return launch_after(k_tree_grad<VSD_T, V_, G_>, P.R, kThreads, gsm, s, P,   \
+                            reinterpret_cast<G_*>(grad));                           \
+    } while (0)
     if (vec && grad_bf16) VSD_TGRAD(true, __nv_bfloat16);
     else if (vec) VSD_TGRAD(true, float);
     else if (grad_bf16) VSD_TGRAD(false, __nv_bfloat16);
     else VSD_TGRAD(false, float);
 #undef VSD_TGRAD
-    return cudaGetLastError();
 }
 
 }  // namespace vsd

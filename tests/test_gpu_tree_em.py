@@ -142,3 +142,30 @@ def test_tree_sequential_many_siblings(vsd, oracle, V, dtype):
                           ua.cuda(), uc.cuda(), 1.0, rule=vsd.TREE_SEQUENTIAL)
     torch.cuda.synchronize()
     compare_tree_sequential(got, orc)
+
+
+@pytest.mark.parametrize("N,deep,V,dtype", [(129, 3, 517, "f32"), (300, 40, 264, "bf16"),
+                                            (1024, 200, 33, "f32")])
+def test_tree_em_large_trees_match_oracle(vsd, oracle, N, deep, V, dtype):
+    """More nodes than a block has threads, many more depths than it has
+    warps, single children and rows with dozens of them."""
+    from paper_2602_05774_gb300 import inputs
+    B = 2
+    g = torch.Generator().manual_seed(N)
+    p = inputs.linear_problem(B, N, 1, V, dtype, "gauss", seed=N, noise_sigma=0.2)
+    par = torch.empty(B, N, dtype=torch.int32)
+    for b in range(B):
+        for n in range(N):  # a chain, then anywhere below
+            par[b, n] = n - 1 if n <= deep else int(torch.randint(0, n, (1,), generator=g)) // 4
+    rows = (torch.arange(B).view(B, 1) * N + par.clamp(min=0).long()).view(-1)
+    top = p["draft"].float().topk(8, dim=1).indices.to(torch.int32)
+    tokens = top[rows, torch.randint(0, 8, (B * N,), generator=g)].view(B, N)
+    tokens[:, 0] = 0
+    ua, uc = torch.rand(B, N, generator=g), torch.rand(B, N, generator=g)
+    orc = oracle.tree_em(_np32(p["draft"]), _np32(p["target"]), 1.0, par.numpy(),
+                         tokens.numpy(), _np32(ua), _np32(uc))
+    prm = vsd.params(grad_dtype=torch.float32)
+    got = vsd.tree_estep_mstep(p["draft"].cuda(), p["target"].cuda(), par.cuda(), tokens.cuda(),
+                               ua.cuda(), uc.cuda(), 1.0, prm=prm)
+    torch.cuda.synchronize()
+    compare_tree_em(got, orc, B, N, V, grad_dtype="f32")
