@@ -45,11 +45,19 @@ constexpr int kSegChunks = VSD_SEG_CHUNKS;
 #define VSD_GRAD_SEG_CHUNKS 16
 #endif
 constexpr int kGradSegChunks = VSD_GRAD_SEG_CHUNKS;
-// Longest row (in chunks) whose tail the streaming warps run themselves.
-#ifndef VSD_STREAM_TAIL_CHUNKS
-#define VSD_STREAM_TAIL_CHUNKS 48
-#endif
-constexpr int kStreamTailChunks = VSD_STREAM_TAIL_CHUNKS;
+// The E-step + M-step runs as two kernels (vsd_staged.cuh) unless rows are long
+// (more chunks than kStagedChunks), their gradient is written and both logit
+// blocks take more than kStagedBytes: then the persistent kernel's overlap of
+// gradients with later rows is worth more than its claims cost.  Measured on
+// GB300, us per call, persistent / two kernels:
+//   V=32000 bf16 (32 chunks):  R=64 57 / 49, R=768 119 / 83, R=4096 320 / 258
+//   V=64000 bf16 (63 chunks):  R=768 169 / 120, R=4096 (1.05 GB) 430 / 413
+//   V=128256 bf16 (126):       R=64 113 / 82, R=512 (0.26 GB) 193 / 158,
+//                              R=2048 (1.05 GB) 364 / 422, R=4096 640 / 710
+//   V=64000 float32 (125):     R=512 (0.26 GB) 175 / 139, R=2048 (1.05 GB) 343 / 386
+//   no gradient, V=128256 bf16: R=1024 185 / 172, R=4096 470 / 419
+constexpr int kStagedChunks = 64;
+constexpr size_t kStagedBytes = (size_t)512 << 20;
 
 // Upper bounds of the chunk count and segment count of a row over both logit
 // dtypes (the smaller float32 chunk gives the larger count).
@@ -246,8 +254,6 @@ Problem<T> make_problem(const void* draft, const void* target, const vsd_layout&
     P.path_A = at<int>(ws, w.path_A);
     // the tree layout has no E-step view and no path lengths: their arrays
     // hold its residual lists and its nodes' log alpha
-    P.stream_tails = 0;
-    P.resq_sem = 1;
     P.tnode = L.parent ? at<TreeNodeRec>(ws, w.tnode) : nullptr;
     P.tcoef = L.parent ? at<TreeCoef>(ws, w.tcoef) : nullptr;
     P.tg = L.parent ? at<float>(ws, w.tg) : nullptr;
@@ -424,27 +430,21 @@ vsd_status fused_impl(const void* draft, const void* target, vsd_layout L, float
     P.out = *out;
     const size_t gelem = P.grad_bf16 ? 2 : 4;
     const bool vec = vec_ok(draft, target, out->grad, L.V, sizeof(T), gelem);
-    const int per_sm = Launch<T>::fused_blocks_per_sm(P, vec, P.grad_bf16);
-    // rows of one short segment: the streaming warps run the row tails
-    // themselves (three warps at once) instead of leaving them to the
-    // control warp, which would otherwise bound the kernel
-    P.stream_tails = (P.nseg == 1 && P.nch <= kStreamTailChunks) ? 1 : 0;
-    // Residual claims: short rows through the counting semaphore (claims in
-    // parallel: the per-prefix chain bounds those launches), long rows by one
-    // compare-and-swap on the queue head (one round trip fewer per claim:
-    // there the claims of the streaming jobs bound it).  Measured on GB300:
-    // V=32000 0.107 vs 0.136 ms, V=128256 0.669 vs 0.642 ms.
-    P.resq_sem = P.stream_tails;
     P.xtab_given = xtab_given ? 1 : 0;
     // no dense gradient asked for: no gradient jobs (the M-step's coefficients
     // stay in the workspace for vsd_lmhead_backward)
     if (!out->grad) P.gnseg = 0;
+    cudaError_t e = clear ? clear_counters(ws, L, s) : cudaSuccess;
+    if (e != cudaSuccess) return from_cuda(e);
+    // (the test hook of the bounded gradient waits needs the kernel that waits)
+    if (!P.inject_wait_fault && (P.nch <= kStagedChunks || !out->grad ||
+                                 2 * sizeof(T) * (size_t)P.R * (size_t)P.V <= kStagedBytes))
+        return from_cuda(Launch<T>::staged(P, vec, out->grad, P.grad_bf16, s));
+    const int per_sm = Launch<T>::fused_blocks_per_sm(P, vec, P.grad_bf16);
     const int64_t tickets = (int64_t)P.R * (P.nseg + P.gnseg);
     int ctas = per_sm * num_sms();
     if ((int64_t)ctas > tickets) ctas = (int)tickets;
-    cudaError_t e = clear ? clear_counters(ws, L, s) : cudaSuccess;
-    if (e == cudaSuccess) e = Launch<T>::fused(P, vec, out->grad, P.grad_bf16, ctas, s);
-    return from_cuda(e);
+    return from_cuda(Launch<T>::fused(P, vec, out->grad, P.grad_bf16, ctas, s));
 }
 
 }  // namespace

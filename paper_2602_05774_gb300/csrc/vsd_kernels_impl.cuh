@@ -114,7 +114,6 @@ constexpr int kSlots = VSD_SLOTS;  // jobs handed to the streaming warps ahead o
 // warps have finished that job.
 __device__ __forceinline__ int bar_full(int s) { return 1 + s; }
 __device__ __forceinline__ int bar_done(int s) { return 1 + kSlots + s; }
-constexpr int kStreamBar = 1 + 2 * kSlots;  // the streaming warps among themselves
 __device__ __forceinline__ void named_sync(int id) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(kFusedThreads) : "memory");
 }
@@ -151,20 +150,14 @@ __device__ bool claim_job(const Problem<T>& P, bool wait, int& g, Job& j) {
         // per kind of work
         const int tk = *(volatile int*)P.ticket;
         const int rdy = g < B ? ld_acquire(P.ready + g) : 0;
-        int it = -1, av;
-        if (P.resq_sem) {  // short rows: claims must not queue (the chain bounds the kernel)
-            av = *(volatile int*)P.resq_avail > 0;
-            if (av)
-                it = take_residual(P.resq_head, P.resq_avail, P.resq_flag, P.resq, P.status,
-                                   P.timeout_ns);
-        } else {  // long rows: one compare-and-swap, fewer round trips per claim
-            const int h = *(volatile int*)P.resq_head;
-            const int tl = *(volatile int*)P.resq_tail;
-            av = h < tl;
-            if (av && atomicCAS(P.resq_head, h, h + 1) == h) {
-                it = wait_flag(P.resq_flag + h, P.status, P.timeout_ns) ? ld_cg(P.resq + h) : -2;
-                if (it == -2) atomicOr(P.status, VSD_STATUS_TIMEOUT);
-            }
+        int it = -1;
+        // (one compare-and-swap on the queue's head)
+        const int h = *(volatile int*)P.resq_head;
+        const int tl = *(volatile int*)P.resq_tail;
+        const bool av = h < tl;
+        if (av && atomicCAS(P.resq_head, h, h + 1) == h) {
+            it = wait_flag(P.resq_flag + h, P.status, P.timeout_ns) ? ld_cg(P.resq + h) : -2;
+            if (it == -2) atomicOr(P.status, VSD_STATUS_TIMEOUT);
         }
         if (it == -2) return true;  // a wait ran out: end
         if (it >= 0) {
@@ -273,7 +266,7 @@ __device__ void post_job(const Problem<T>& P, const EStepView& E, const Job& j, 
     if (j.kind == kJobRow) {
         const int r = j.r;
         if (!warp_count_last(P.row_seg_cnt + r, nseg, lane)) return;
-        if (!P.stream_tails) row_tail_warp<T, VEC, KL>(P, r, tab, cs.rb, lane);
+        row_tail_warp<T, VEC, KL>(P, r, tab, cs.rb, lane);
         __syncwarp();
         const int path = r / D;
         if (!warp_count_last(P.path_cnt + path, D, lane)) return;
@@ -285,7 +278,7 @@ __device__ void post_job(const Problem<T>& P, const EStepView& E, const Job& j, 
             if (lane == 0) {  // queue the residual row's segments
                 P.path_A[path] = A;
                 publish_residuals(P.resq_tail, P.resq_avail, P.resq_flag, P.resq, path * nseg,
-                                  nseg, P.resq_sem != 0);
+                                  nseg, false);
             }
         } else {
             finish_path_warp<T>(P, E, path, A, -1, false, 0.f, 0.f, cs, lane);
@@ -365,7 +358,6 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
     __shared__ CtlShared cs;
     __shared__ Job slots[kSlots];
     __shared__ KlRec kslot[kSlots];  // VSD (KL): the top-K terms of a gradient job's row
-    __shared__ RowShared rsh;
     Ring* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
@@ -394,11 +386,6 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
                                                 j.c1, rtab, P.ts.c,
                                                 P.gnseg ? policy_evict_last() : policy_evict_first(),
                                                 policy_evict_first(), P.status);
-                if (P.stream_tails) {  // short rows: the tail here, three draws at once
-                    asm volatile("bar.sync %0, %1;" ::"r"(kStreamBar), "r"(kThreads) : "memory");
-                    row_tail<T, VEC, true, kSampleToken, true, kStreamBar, KL>(
-                        P, j.r, rtab, rsh, VEC ? &rg->data[kWarps - 1][0][0][0] : nullptr);
-                }
             } else if (j.kind == kJobResidual) {
                 // row A's table was consumed by its row tail: reuse it
                 stream_residual<T, VEC>(rg, x, P.target + (int64_t)j.r * V, V, j.c0, j.c1,

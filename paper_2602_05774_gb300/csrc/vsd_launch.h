@@ -35,6 +35,9 @@ template <typename T> struct Launch {
     // the fused persistent E-step + M-step kernel
     static cudaError_t fused(const Problem<T>& P, bool vec, void* grad, bool grad_bf16,
                              int ctas, cudaStream_t s);
+    // the E-step + M-step in two kernels (rows with paths and M-steps; gradient)
+    static cudaError_t staged(const Problem<T>& P, bool vec, void* grad, bool grad_bf16,
+                              cudaStream_t s);
     // resident blocks per SM of the fused kernel
     static int fused_blocks_per_sm(const Problem<T>& P, bool vec, bool grad_bf16);
 };

@@ -153,7 +153,6 @@ struct Problem {
     float4* gtab;                 // [R][nch_ws] per-chunk tables of each row
     int* row_seg_cnt;             // [R] segments of a row completed
     int* res_seg_cnt;             // [B*K] residual segments of a path completed
-    int stream_tails;             // fused kernel: the streaming warps run the row tails
     int greedy;                   // T = 0: every decision takes the argmax limit of
                                   // Eq. 1's distributions; ts holds temperature 1,
                                   // the M-step's
@@ -172,8 +171,7 @@ struct Problem {
     int* resq_flag;               // item written
     int* resq_head;               // next item to take
     int* resq_tail;               // next free slot
-    int* resq_avail;              // items published and not yet reserved (may dip below 0)
-    int resq_sem;                 // fused kernel claims residual items through resq_avail
+    int* resq_avail;              // trees: items published and not yet reserved (may dip below 0)
     // outputs (device, caller-owned; null = not written)
     vsd_linear_outputs out;
     vsd_tree_outputs tout;
@@ -896,11 +894,9 @@ template <typename T, bool VEC>
 __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch, uint4* buf,
                           int npair, bool ok, int lane);
 
-// The per-row work once the row's chunk table tab[0..nch) is complete
-// (block, or with BAR > 0 the kThreads threads 0 .. kThreads-1 that meet at
-// named barrier BAR): warps 0, 1 and 2 take the three tasks at once, warp 0
-// then writes the record.
-template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, int BAR = 0, bool KL = false>
+// The per-row work once the row's chunk table tab[0..nch) is complete (block):
+// warps 0, 1 and 2 take the three tasks at once, warp 0 then writes the record.
+template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool KL = false>
 __device__ void row_tail(const Problem<T>& P, int r, const float4* tab, RowShared& sh,
                          uint4* klbuf = nullptr) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -912,10 +908,7 @@ __device__ void row_tail(const Problem<T>& P, int r, const float4* tab, RowShare
         // is cleared by row_finish)
         kl_select<T, VEC>(P, r, tab, P.nch, klbuf, 2, true, lane);
     }
-    if (BAR == 0)
-        __syncthreads();
-    else
-        asm volatile("bar.sync %0, %1;" ::"r"(BAR), "r"(kThreads) : "memory");
+    __syncthreads();
     if (warp == 0) {
         RowTask ty = sh.t[1];
         if (!HAS_Y) ty = RowTask{0.f, TableSum{0, 0, 0.0}, -1};
@@ -1521,6 +1514,7 @@ struct WeightsShared {
     float rz[64];                // 1 / that sum
     float beta[64][3];           // leave-one-out beta for (o', o~) = (w, 1), (w, 0), (0, 0)
     float cmax[64];              // zeta_mode 0: exp(lmax) / tau
+    long long jn[kWarps][2];     // J and N of a block's warps
 };
 
 // x 2^E rounded toward zero, |x| clamped to 2^20 (a non-finite log-probability
@@ -1538,27 +1532,35 @@ __device__ __forceinline__ float from_fixed(long long q, int E) {
     return ldexpf(hi + lo, -E);
 }
 
-// f(e) for the entries e = lane, lane + 32, ... < ne, four at a time so that
-// their independent loads and double-precision chains overlap.
-template <class F>
+// The M-step of a prefix is run by NT threads: a warp (32) or a whole block.
+template <int NT> __device__ __forceinline__ void group_sync() {
+    if constexpr (NT == 32)
+        __syncwarp();
+    else
+        __syncthreads();
+}
+// f(e) for the entries e = lane, lane + NT, ... < ne, a warp's four at a time
+// so that their independent loads and double-precision chains overlap.
+template <int NT, class F>
 __device__ __forceinline__ void each_entry(int ne, int lane, F&& f) {
-    for (int e0 = lane; e0 < ne; e0 += 128) {
+    constexpr int U = NT == 32 ? 4 : 1;
+    for (int e0 = lane; e0 < ne; e0 += NT * U) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = e0 + 32 * u;
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + NT * u;
             if (e < ne) f(e);
         }
     }
 }
 
-// Load the tile of positions [d0, d0 + nd) of prefix b (warp).  TERMS: the
+// Load the tile of positions [d0, d0 + nd) of prefix b (NT threads).  TERMS: the
 // per-entry terms written by the forward sweep (from wscr) instead of the
 // scores.
-template <typename T, bool TERMS>
+template <typename T, bool TERMS, int NT>
 __device__ __forceinline__ void mstep_tile(const Problem<T>& P, const EStepView& E, int b, int d0,
                                            int nd, WeightsShared& sh, int lane) {
     const int K = P.K, D = P.D;
-    each_entry(K * nd, lane, [&](int e) {
+    each_entry<NT>(K * nd, lane, [&](int e) {
         const int s = e / nd, r = (b * K + s) * D + d0 + (e - s * nd);
         sh.tok[e] = ld_cg(E.tok + r);
         sh.corr[e] = ld_cg(E.corr + r);
@@ -1574,36 +1576,36 @@ __device__ __forceinline__ void mstep_tile(const Problem<T>& P, const EStepView&
             sh.lqcz[e] = ld_cg(E.lq_corr + r);
         }
     });
-    __syncwarp();
+    group_sync<NT>();
 }
 
-// M-step of prefix b by one warp (K <= 256, D <= 64).  Writes coef[] for the
+// M-step of prefix b by NT threads, `lane` among them (K <= 256, D <= 64).  Writes coef[] for the
 // prefix's rows, the optional weights table and loss_out[b].  No dependent
 // double-precision chains (GB300's FP64 latency would dominate): sums over l
 // and over entries are exact 64-bit fixed-point sums of float terms, the CAR
 // weights come from exact differences of those sums, and every reduction is
 // exact, so the result does not depend on the order of the entries.
-template <typename T>
-__device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, float* weights_out,
+template <typename T, int NT>
+__device__ void weights_group(const Problem<T>& P, const EStepView& E, int b, float* weights_out,
                              float* loss_out, WeightsShared& sh, int lane) {
     const int K = P.K, D = P.D;
     const int dt = max(1, min(D, kMTile / K));
     const bool one_tile = dt >= D;
     const float inv_tau = P.inv_tau_f;
-    for (int s = lane; s < K; s += 32) sh.lqt[s] = sh.lqc[s] = 0;
+    for (int s = lane; s < K; s += NT) sh.lqt[s] = sh.lqc[s] = 0;
     long long Jq = 0, Nq = 0;  // this lane's parts of J and N (fixed point, 2^-24)
     for (int d0 = 0; d0 < D; d0 += dt) {
         const int nd = min(dt, D - d0);
         const int ne = K * nd;
-        mstep_tile<T, false>(P, E, b, d0, nd, sh, lane);
+        mstep_tile<T, false, NT>(P, E, b, d0, nd, sh, lane);
         // running sums of log q over l, per proposal: the fixed-point terms
         // for every entry at once, then integer adds along l
-        each_entry(ne, lane, [&](int e) {
+        each_entry<NT>(ne, lane, [&](int e) {
             sh.elqt[e] = to_fixed(sh.lq[e], kLqE);
             sh.elqc[e] = to_fixed(sh.lqcz[e], kLqE);
         });
-        __syncwarp();
-        for (int s = lane; s < K; s += 32) {
+        group_sync<NT>();
+        for (int s = lane; s < K; s += NT) {
             long long a = sh.lqt[s], q = sh.lqc[s];
             for (int dd = 0; dd < nd; ++dd) {
                 const int e = s * nd + dd;
@@ -1615,15 +1617,15 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
             sh.lqt[s] = a;
             sh.lqc[s] = q;
         }
-        for (int dd = lane; dd < nd; dd += 32) {
+        for (int dd = lane; dd < nd; dd += NT) {
             sh.n1[dd] = sh.n0[dd] = 0;
             sh.lmax[dd] = (long long)0x8000000000000000ull;
             sh.zs[dd] = 0;
         }
-        __syncwarp();
+        group_sync<NT>();
         // per position: the counts behind beta and the largest running log q,
         // gathered from every entry at once with shared-memory integer atomics
-        each_entry(ne, lane, [&](int e) {
+        each_entry<NT>(ne, lane, [&](int e) {
             const int dd = e % nd;
             // Algorithm 2 scores z~ (o~); Algorithm 1 keeps z~ if it passes,
             // else z', so o' = w(l) when either passes
@@ -1634,20 +1636,20 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
             }
             atomicMax(&sh.lmax[dd], sh.elqt[e]);
         });
-        __syncwarp();
+        group_sync<NT>();
         if (P.zeta_mode == 0)  // exp(lmax) / tau, with the float split hi + lo of lmax
-            for (int dd = lane; dd < nd; dd += 32) {
+            for (int dd = lane; dd < nd; dd += NT) {
                 const long long m = sh.lmax[dd];
                 const float hi = from_fixed(m, kLqE);
                 const float lo = from_fixed(m - to_fixed(hi, kLqE), kLqE);
                 sh.cmax[dd] = expf(hi) * (1.f + lo) * inv_tau;
             }
-        __syncwarp();
+        group_sync<NT>();
         // CAR weights (Eq. zeta) relative to the proposal with the largest
         // logit: exp((Q_s - Q_max) / tau) with Q = q(z~_{1:l}) (zeta_mode 0:
         // Q_s - Q_max = Q_max expm1(d)) or Q = log q(z~_{1:l}) (zeta_mode 1:
         // Q_s - Q_max = d), d = the exact difference of the running sums
-        each_entry(ne, lane, [&](int e) {
+        each_entry<NT>(ne, lane, [&](int e) {
             const int dd = e % nd;
             const float d = from_fixed(sh.elqt[e] - sh.lmax[dd], kLqE);
             const float arg = P.zeta_mode == 0 ? sh.cmax[dd] * expm1f(d) : d * inv_tau;
@@ -1657,10 +1659,10 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
             const long long z = fixed_prod(ez, 1.f, 40);
             if (z) atomicAdd(&sh.zs[dd], (unsigned long long)z);
         });
-        __syncwarp();
+        group_sync<NT>();
         // per position, in parallel: 1 / sum, and beta (Eq. beta, leave-one-out:
         // o' is w(l) or 0, so both of its sums are w(l) times a count)
-        for (int dd = lane; dd < nd; dd += 32) {
+        for (int dd = lane; dd < nd; dd += NT) {
             const int n1 = sh.n1[dd], n0 = sh.n0[dd];
             const float zs = (float)(long long)sh.zs[dd] * 0x1p-40f;
             sh.rz[dd] = zs > 0.f ? 1.f / zs : 0.f;
@@ -1668,10 +1670,10 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
             sh.beta[dd][1] = n0 - 1 > 0 ? (float)n1 / (float)(n0 - 1) : 0.f;
             sh.beta[dd][2] = n0 > 0 ? (float)n1 / (float)n0 : 0.f;
         }
-        __syncwarp();
+        group_sync<NT>();
         // per entry, in parallel: zeta, the objective terms (Eq. advance) and
         // the per-l gradient terms o'(o~ - beta zeta), o'(1 - o~)
-        each_entry(ne, lane, [&](int e) {
+        each_entry<NT>(ne, lane, [&](int e) {
             const int s = e / nd, dd = e - s * nd, d = d0 + dd;
             const bool otb = sh.ot[e], opb = otb || sh.pc[e];
             const float w = P.wlf[d];
@@ -1694,21 +1696,35 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
                 *wo = make_float4(otb ? 1.f : 0.f, opb ? w : 0.f, beta, zeta);
             }
         });
-        __syncwarp();
+        group_sync<NT>();
     }
-    const float J = from_fixed(warp_sum_ll(Jq), 24), N = from_fixed(warp_sum_ll(Nq), 24);
+    Jq = warp_sum_ll(Jq);
+    Nq = warp_sum_ll(Nq);
+    if constexpr (NT > 32) {  // across the warps (integer sums: any order)
+        if ((lane & 31) == 0) {
+            sh.jn[lane >> 5][0] = Jq;
+            sh.jn[lane >> 5][1] = Nq;
+        }
+        group_sync<NT>();
+        Jq = Nq = 0;
+        for (int w = 0; w < NT / 32; ++w) {
+            Jq += sh.jn[w][0];
+            Nq += sh.jn[w][1];
+        }
+    }
+    const float J = from_fixed(Jq, 24), N = from_fixed(Nq, 24);
     const float scale = N > 0.f ? 1.f / ((float)P.B * N * P.ts.T) : 0.f;
     // suffix sums over l, from the last tile back (lqt, lqc now hold c0, c1)
-    for (int s = lane; s < K; s += 32) sh.lqt[s] = sh.lqc[s] = 0;
+    for (int s = lane; s < K; s += NT) sh.lqt[s] = sh.lqc[s] = 0;
     for (int d0 = ((D - 1) / dt) * dt; d0 >= 0; d0 -= dt) {
         const int nd = min(dt, D - d0);
         if (!one_tile) {
-            __syncwarp();
-            mstep_tile<T, true>(P, E, b, d0, nd, sh, lane);
+            group_sync<NT>();
+            mstep_tile<T, true, NT>(P, E, b, d0, nd, sh, lane);
         }
         // integer adds along l from the end, then every entry's coefficients
         // at once
-        for (int s = lane; s < K; s += 32) {
+        for (int s = lane; s < K; s += NT) {
             long long c0 = sh.lqt[s], c1 = sh.lqc[s];
             for (int dd = nd - 1; dd >= 0; --dd) {
                 const int e = s * nd + dd;
@@ -1720,8 +1736,8 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
             sh.lqt[s] = c0;
             sh.lqc[s] = c1;
         }
-        __syncwarp();
-        each_entry(K * nd, lane, [&](int e) {
+        group_sync<NT>();
+        each_entry<NT>(K * nd, lane, [&](int e) {
             const int s = e / nd, dd = e - s * nd;
             const long long c0 = sh.et0[e], c1 = sh.elqc[e];
             Coef cf;
@@ -1744,18 +1760,27 @@ __device__ void weights_warp(const Problem<T>& P, const EStepView& E, int b, flo
     float klterm = 0.f;
     if (P.kl_topk) {  // VSD (KL): + kl_weight (1/K) sum of the prefix's rows' top-K terms
         double sk = 0.0;
-        for (int i = lane; i < K * D; i += 32) sk += (double)ld_cg(&P.klr[b * K * D + i].loss);
+        if (lane < 32)
+            for (int i = lane; i < K * D; i += 32) sk += (double)ld_cg(&P.klr[b * K * D + i].loss);
         klterm = (float)(P.kl_weight / (double)K * warp_sum(sk));
     }
     if (lane == 0) loss_out[b] = (N > 0.f ? -J / N : 0.f) + klterm;
 }
 
-// The M-step by a block: warp 0 runs weights_warp (the same bits as the fused
-// kernel's control warp).
+// The M-step by one warp.
+template <typename T>
+__device__ __forceinline__ void weights_warp(const Problem<T>& P, const EStepView& E, int b,
+                                             float* weights_out, float* loss_out,
+                                             WeightsShared& sh, int lane) {
+    weights_group<T, 32>(P, E, b, weights_out, loss_out, sh, lane);
+}
+
+// The M-step by a block (the same bits as by a warp: every sum is an integer
+// sum).
 template <typename T>
 __device__ void weights_pass(const Problem<T>& P, const EStepView& E, int b, float* weights_out,
                              float* loss_out, WeightsShared& sh) {
-    if ((threadIdx.x >> 5) == 0) weights_warp<T>(P, E, b, weights_out, loss_out, sh, threadIdx.x & 31);
+    weights_group<T, kThreads>(P, E, b, weights_out, loss_out, sh, threadIdx.x);
 }
 
 // Mean of loss[0..B) into loss[B], summed in order (one thread).
@@ -1795,7 +1820,7 @@ __device__ __forceinline__ void grad_store(G* g, int64_t v0, const float (&o)[PV
 // e1 are multiples of the vector width.
 template <typename T, bool VEC, typename G>
 __device__ void grad_pass_range(const Problem<T>& P, int r, int64_t e0, int64_t e1,
-                                const float4* rstats, G* grad, const KlRec* kl = nullptr) {
+                                const float4* rstats, G* grad) {
     constexpr int PV = Traits<T>::kPerVec;
     constexpr int U = 8;  // vectors per batch per thread (two batches in flight)
     const int64_t V = P.V;
@@ -1854,13 +1879,10 @@ __device__ void grad_pass_range(const Problem<T>& P, int r, int64_t e0, int64_t 
             for (int u = 0; u < U; ++u) cur[u] = nxt[u];
         }
     } else {
-        const int nkl = kl ? min(max(kl->n, 0), kMaxKlTop) : 0;
         for (int64_t v = e0 + threadIdx.x; v < e1; v += kThreads) {
             float val = gq * ex2((elem_value(x, v) - mx) * c);
             if (v == cf.t0) val -= cf.c0;
             if (v == cf.t1) val -= cf.c1;
-            for (int k = 0; k < nkl; ++k)
-                if (v == kl->tok[k]) val += kl->coef[k];
             if constexpr (sizeof(G) == 2)
                 g[v] = __float2bfloat16_rn(val);
             else
@@ -1880,8 +1902,28 @@ __device__ void stream_grad(Ring* rg, const Problem<T>& P, int r, int c0, int c1
     constexpr int CE = chunk_elems<T>();
     const int64_t V = P.V;
     if constexpr (!VEC) {
-        grad_pass_range<T, VEC, G>(P, r, (int64_t)c0 * CE, min(V, (int64_t)c1 * CE), P.rstats,
-                                   grad, kl);
+        const T* x = P.draft + (int64_t)r * V;
+        G* g = grad + (int64_t)r * V;
+        const RowRec rec = ld_cg(P.rows + r);
+        const Coef cf = ld_cg(P.coef + r);
+        const float gq = cf.g * rec.izx;  // g / Z
+        const bool dense = !(cf.g == 0.f && isfinite(rec.mx));
+        const int nkl = KL ? min(max(kl->n, 0), kMaxKlTop) : 0;
+        const int64_t e1 = min(V, (int64_t)c1 * CE);
+        for (int64_t v = (int64_t)c0 * CE + threadIdx.x; v < e1; v += kThreads) {
+            // (rounded steps: no contraction into a fused multiply-add)
+            float o = dense ? __fmul_rn(
+                                  ex2(__fmul_rn(__fsub_rn(elem_value(x, v), rec.mx), P.ts.c)), gq)
+                            : 0.f;
+            if (v == cf.t0) o = __fsub_rn(o, cf.c0);
+            if (v == cf.t1) o = __fsub_rn(o, cf.c1);
+            for (int k = 0; k < nkl; ++k)
+                if (v == kl->tok[k]) o = __fadd_rn(o, kl->coef[k]);
+            if constexpr (sizeof(G) == 2)
+                g[v] = __float2bfloat16_rn(o);
+            else
+                g[v] = o;
+        }
     } else {
         constexpr int NP = PV / 2;
         const int lane = threadIdx.x & 31;

@@ -1,0 +1,186 @@
+// vsd_staged.cuh -- the E-step + M-step in two kernels, for short rows:
+//
+//   k_em_rows  one block per row: the row pass (draws, statistics, the top-K
+//              term of VSD (KL)).  The block completing a path's last row runs
+//              the path (accepted length, residual draw, log-kappa sums), the
+//              block completing a prefix's last path its M-step.  No block
+//              waits for another.
+//   k_em_grad  the gradient rows, as a programmatic dependent launch.
+//
+// Against the persistent kernel (k_fused) this gives up the overlap of one
+// prefix's gradient with another's rows, and wins what claiming and handing
+// over jobs costs: there a row's chain (claim, tail, path, M-step, publication,
+// gradient claims) runs on one control warp per block while rows are short.
+// Same results bit for bit.
+#pragma once
+
+#include "vsd_grid.cuh"
+#include "vsd_launch.h"
+
+namespace vsd {
+
+// Dynamic shared memory: [ring][chunk table]; the M-step's scratch reuses the
+// ring's data (vector rows) or follows the table.
+inline size_t staged_smem_bytes(int nch, bool vec) {
+    return stream_smem_bytes(nch, vec) + (vec ? 0 : sizeof(WeightsShared));
+}
+
+template <typename T, bool VEC, bool KL>
+__global__ void __launch_bounds__(kThreads) k_em_rows(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ union {
+        RowShared row;
+        PathShared path;
+    } sh;
+    __shared__ int s_last;
+    static_assert(sizeof(WeightsShared) <= sizeof(Ring::data), "the M-step's scratch fits the ring");
+    Ring* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
+    const int r = blockIdx.x, D = P.D, K = P.K, nch = P.nch;
+    const int64_t V = P.V;
+    const T* x = P.draft + (int64_t)r * V;
+    const T* y = P.target + (int64_t)r * V;
+    bool both = true;
+    if constexpr (VEC) {
+        if (P.xtab_given) {  // the LM head wrote the draft's half of the table
+            const float4* rtab = P.gtab + (int64_t)r * P.nch_ws;
+            for (int ch = threadIdx.x; ch < nch; ch += kThreads)
+                reinterpret_cast<float2*>(tab + ch)[0] =
+                    __ldcg(reinterpret_cast<const float2*>(rtab + ch));
+            stream_target_tables<T>(rg, y, V, 0, nch, tab, P.ts.c, policy_evict_first(), P.status);
+            both = false;
+        }
+    }
+    if (both)
+        stream_tables<T, VEC, true>(rg, x, y, V, 0, nch, tab, P.ts.c,
+                                    P.gnseg ? policy_evict_last() : policy_evict_first(),
+                                    policy_evict_first(), P.status);
+    __syncthreads();
+    row_tail<T, VEC, true, kSampleToken, true, KL>(
+        P, r, tab, sh.row, VEC ? &rg->data[kWarps - 1][0][0][0] : nullptr);
+    // the last of n blocks to arrive at a counter
+    auto last_of = [&](int* cnt, int n) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(cnt, 1) == n - 1;
+            if (s_last) __threadfence();
+        }
+        __syncthreads();
+        return s_last != 0;
+    };
+    const int path = r / D;
+    if (!last_of(P.path_cnt + path, D)) return;
+    path_head<T>(P, path, sh.path);
+    __syncthreads();
+    const int A = sh.path.A, rA = path * D + A;
+    int resid = -1;
+    // (T = 0: the residual is the target's argmax, the row's p-draw)
+    if (A < D && !sh.path.rec.flags && !P.greedy)
+        resid = residual_draw<T, VEC>(P, rA, sh.path.rec, __ldg(P.u_correct + rA), rg, tab,
+                                      &sh.path.resid);
+    path_epilogue<T>(P, path, A, resid);
+    const int prefix = path / K;
+    if (!last_of(P.prefix_cnt + prefix, K)) return;
+    WeightsShared* ws = VEC ? reinterpret_cast<WeightsShared*>(rg->data)
+                            : reinterpret_cast<WeightsShared*>(tab + nch);
+    const EStepView E{P.es.tok, P.es.corr, P.es.lq_tok, P.es.lq_corr,
+                      P.es.lk, P.es.lkc, P.es.lkr};
+    weights_group<T, kThreads>(P, E, prefix, P.out.weights, P.out.loss, *ws, threadIdx.x);
+    if (last_of(P.prefix_done, P.B) && threadIdx.x == 0) loss_mean(P.out.loss, P.B);
+}
+
+// The gradient of one segment of a row (block; nseg segments a row): the dense
+// part g q(v) from eight 16-byte vectors in flight per thread (a row without
+// one is not read), then the elements with sparse terms, one thread each, in
+// the order of the persistent kernel's gradient jobs.
+template <typename T, bool VEC, typename G, bool KL>
+__global__ void __launch_bounds__(kThreads) k_em_grad(Problem<T> P, G* grad, int nseg) {
+    __shared__ KlRec kl;
+    constexpr int PV = Traits<T>::kPerVec, NP = PV / 2, U = 8;
+    const int r = blockIdx.x / nseg, seg = blockIdx.x - r * nseg;
+    const int64_t V = P.V;
+    const T* x = P.draft + (int64_t)r * V;
+    G* g = grad + (int64_t)r * V;
+    const float c = P.ts.c;
+    // segments are whole batches of the block's vectors
+    const int nvec = (int)((V + PV - 1) / PV);
+    const int per = ((nvec + nseg - 1) / nseg + kThreads - 1) / kThreads * kThreads;
+    const int i0 = seg * per, i1 = min(nvec, i0 + per);
+    grid_wait();
+    const RowRec rec = ld_cg(P.rows + r);
+    const Coef cf = ld_cg(P.coef + r);
+    if (KL) {
+        if (threadIdx.x < sizeof(KlRec) / 16)
+            reinterpret_cast<int4*>(&kl)[threadIdx.x] =
+                __ldcg(reinterpret_cast<const int4*>(P.klr + r) + threadIdx.x);
+    }
+    const float mx = rec.mx, gq = cf.g * rec.izx;  // g / Z
+    const bool dense = !(cf.g == 0.f && isfinite(mx));
+    if constexpr (VEC) {
+        const uint64_t pol = policy_evict_first();
+        const uint64_t mx2 = f2(mx, mx), c2 = f2(c, c), gq2 = f2(gq, gq);
+        for (int ib = i0 + threadIdx.x; ib < i1; ib += kThreads * U) {
+            uint4 buf[U];
+            if (dense) {
+#pragma unroll
+                for (int k = 0; k < U; ++k)
+                    if (ib + k * kThreads < i1)
+                        buf[k] = ld_stream(x + (int64_t)(ib + k * kThreads) * PV, pol);
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const int i = ib + k * kThreads;
+                if (i >= i1) break;
+                float o[PV];
+                if (dense) {
+                    uint64_t pr[NP];
+                    vec_pairs<T>(buf[k], pr);
+#pragma unroll
+                    for (int q = 0; q < NP; ++q)
+                        f2split(f2mul(f2_mass(pr[q], mx2, c2), gq2), o[2 * q], o[2 * q + 1]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < PV; ++e) o[e] = 0.f;
+                }
+                grad_store<T, G, PV>(g, (int64_t)i * PV, o, pol);
+            }
+        }
+    } else {
+        const int64_t e1 = min(V, (int64_t)i1 * PV);
+        for (int64_t v = (int64_t)i0 * PV + threadIdx.x; v < e1; v += kThreads) {
+            const float val =
+                dense ? __fmul_rn(ex2(__fmul_rn(__fsub_rn(elem_value(x, v), mx), c)), gq) : 0.f;
+            if constexpr (sizeof(G) == 2)
+                g[v] = __float2bfloat16_rn(val);
+            else
+                g[v] = val;
+        }
+    }
+    __syncthreads();
+    // the elements with sparse terms: t0, t1, the top-K tokens
+    const int nkl = KL ? min(max(kl.n, 0), kMaxKlTop) : 0;
+    if ((int)threadIdx.x < 2 + nkl) {
+        const int j = (int)threadIdx.x - 2;
+        const int t = j >= 0 ? kl.tok[j] : threadIdx.x ? cf.t1 : cf.t0;
+        const bool mine = t >= i0 * PV && t < (int64_t)i1 * PV && t < V &&
+                          !(threadIdx.x >= 1 && t == cf.t0) && !(threadIdx.x >= 2 && t == cf.t1);
+        if (mine) {
+            // (rounded steps: no contraction into a fused multiply-add)
+            float o = dense ? __fmul_rn(ex2(__fmul_rn(__fsub_rn(elem_value(x, t), mx), c)), gq)
+                            : 0.f;
+            if (t == cf.t0) o = __fsub_rn(o, cf.c0);
+            if (t == cf.t1) o = __fsub_rn(o, cf.c1);
+            for (int k = 0; k < nkl; ++k)
+                if (t == kl.tok[k]) o = __fadd_rn(o, kl.coef[k]);
+            if constexpr (sizeof(G) == 2)
+                g[t] = __float2bfloat16_rn(o);
+            else
+                g[t] = o;
+        }
+    }
+}
+
+}  // namespace vsd

@@ -1,0 +1,82 @@
+"""The E-step + M-step as two kernels (short rows, small batches, no gradient)
+and as the persistent kernel (long rows with a gradient): against the oracle at
+the edges of the first, and against each other bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from tests.parity import compare_linear, mstep_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def vsd():
+    from paper_2602_05774_gb300 import build, vsd as v
+    build.build_library()
+    v.load()
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    return v
+
+
+def _call(vsd, p, T, prm, **kw):
+    return vsd.estep_mstep(p["draft"], p["target"], p["u_draft"], p["u_accept"], p["u_correct"],
+                           p["K"], p["D"], T, prm=prm, **kw)
+
+
+@pytest.mark.parametrize("B,K,D,V,dtype,grad,kl", [
+    (1, 1, 1, 65544, "bf16", "bf16", 0.0),   # one row in many gradient segments, ragged last chunk
+    (1, 2, 1, 65537, "f32", "f32", 0.5),     # the same, rows not 16-byte aligned
+    (2, 256, 1, 40, "f32", "bf16", 0.0),     # the most proposals
+    (1, 5, 64, 24, "f32", "f32", 0.0),       # the deepest paths
+    (2, 30, 17, 264, "bf16", "f32", 0.5),    # an M-step of several tiles
+    (3, 3, 5, 8200, "bf16", "bf16", 0.5),    # top-K terms across gradient segments
+])
+def test_two_kernels_match_oracle(vsd, oracle, B, K, D, V, dtype, grad, kl):
+    from paper_2602_05774_gb300 import inputs
+    prob = inputs.linear_problem(B, K, D, V, dtype, "gauss", seed=V + K)
+    f = lambda t: t.float().numpy()  # noqa: E731
+    orc = oracle.linear(f(prob["draft"]), f(prob["target"]), 1.0, f(prob["u_draft"]),
+                        f(prob["u_accept"]), f(prob["u_correct"]), K, D, kl_weight=kl, kl_topk=10)
+    p = {k: (v.cuda() if torch.is_tensor(v) else v) for k, v in prob.items()}
+    prm = vsd.params(grad_dtype=torch.float32 if grad == "f32" else torch.bfloat16, kl_weight=kl)
+    ws = vsd.new_workspace(vsd.layout(B, K, D, V), "cuda")
+    got = _call(vsd, p, 1.0, prm, workspace=ws)
+    torch.cuda.synchronize()
+    assert vsd.device_status(ws) == (0, 0)
+    compare_linear(got, orc, B, K, D, V, 1.0, grad_dtype=grad, kl=kl != 0,
+                   mstep_inputs=mstep_inputs(prob, kl_weight=kl, kl_topk=10) if kl
+                   else mstep_inputs(prob))
+
+
+@pytest.mark.parametrize("V,R,dtype,kind,kl,T", [
+    (70000, 2048, "bf16", "spiked", 0.0, 1.0),
+    (140000, 1024, "bf16", "zipf", 0.3, 0.7),   # two row segments
+    (70001, 1024, "f32", "gauss", 0.3, 1.0),    # rows not 16-byte aligned
+    (70000, 2048, "bf16", "spiked", 0.3, 0.0),  # greedy
+])
+def test_persistent_kernel_equals_two_kernels(vsd, V, R, dtype, kind, kl, T):
+    """A batch above the dispatch's size runs on the persistent kernel, each
+    half of it on the two kernels: every result equal bit for bit (halving the
+    batch doubles the gradient, an exact factor)."""
+    from paper_2602_05774_gb300 import inputs
+    K, D = 8, 8
+    B = R // (K * D)
+    p = inputs.linear_problem(B, K, D, V, dtype, kind, "cuda", seed=V)
+    prm = vsd.params(like=p["draft"], kl_weight=kl)
+    whole = _call(vsd, p, T, prm)
+    none = _call(vsd, p, T, prm, grad=False)
+    for n in none:
+        if n != "grad":
+            assert torch.equal(whole[n], none[n]), n
+    h = R // 2
+    for i in range(2):
+        q = dict(p, **{k: p[k][i * h:(i + 1) * h] for k in
+                       ("draft", "target", "u_draft", "u_accept", "u_correct")})
+        part = _call(vsd, q, T, prm)
+        assert torch.equal(whole["loss"][i * B // 2:(i + 1) * B // 2], part["loss"][:-1])
+        a, b = whole["grad"][i * h:(i + 1) * h], part["grad"]
+        assert torch.equal(2 * a, b)
+        for n in ("tokens", "corr_tokens", "logkappa", "weights", "row_stats"):
+            m = whole[n].view(2, -1)[i]
+            assert torch.equal(m, part[n].reshape(-1)), n
