@@ -358,6 +358,18 @@ vsd_status vsd_lmhead_backward(const void* hidden, const void* weight, int32_t H
                                const vsd_params* params, float* d_hidden, float* d_weight,
                                void* ws, size_t ws_bytes, void* stream);
 
+/* vsd_lmhead_backward with scratch memory of the caller's: with at least 2*R*V
+ * bytes (16-byte aligned, device) G is written there once as bf16, the same
+ * values, and both products read it, which is faster (R=4096, H=4096, V=32000:
+ * G made on chip for every tile of both products bounds the call without it).
+ * scratch NULL or smaller: exactly vsd_lmhead_backward.  Its contents are
+ * undefined afterwards; it may be reused once the call's work has completed. */
+vsd_status vsd_lmhead_backward_scratch(const void* hidden, const void* weight, int32_t H,
+                                       const void* draft_logits, vsd_layout layout, float T,
+                                       const vsd_params* params, float* d_hidden,
+                                       float* d_weight, void* ws, size_t ws_bytes, void* scratch,
+                                       size_t scratch_bytes, void* stream);
+
 /* The greedy reference of Algorithm 2 from its own rows: the oracle's z-bar
  * is drawn from the greedy target policy, so its validity log kappa(z-bar)
  * needs the draft and target distributions along z-bar, which the caller

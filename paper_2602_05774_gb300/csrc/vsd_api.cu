@@ -641,11 +641,21 @@ vsd_status vsd_lmhead_backward(const void* hidden, const void* weight, int32_t H
                                const void* draft_logits, vsd_layout layout, float T,
                                const vsd_params* params, float* d_hidden, float* d_weight,
                                void* ws, size_t ws_bytes, void* stream) {
+    return vsd_lmhead_backward_scratch(hidden, weight, H, draft_logits, layout, T, params,
+                                       d_hidden, d_weight, ws, ws_bytes, nullptr, 0, stream);
+}
+
+vsd_status vsd_lmhead_backward_scratch(const void* hidden, const void* weight, int32_t H,
+                                       const void* draft_logits, vsd_layout layout, float T,
+                                       const vsd_params* params, float* d_hidden,
+                                       float* d_weight, void* ws, size_t ws_bytes, void* scratch,
+                                       size_t scratch_bytes, void* stream) {
     if (!layout_ok(layout) || layout.parent) return VSD_ERR_INVALID_ARG;
     const int64_t R = rows_of(layout);
     if (R > (1 << 30) || !lmhead_shape_ok(hidden, weight, draft_logits, (int)R, layout.V, H))
         return VSD_ERR_INVALID_ARG;
-    if (((uintptr_t)d_hidden | (uintptr_t)d_weight) & 15) return VSD_ERR_INVALID_ARG;
+    if (((uintptr_t)d_hidden | (uintptr_t)d_weight | (uintptr_t)scratch) & 15)
+        return VSD_ERR_INVALID_ARG;
     vsd_status st = check_temperature(T, true);
     if (st) return st;
     const vsd_params p = params ? *params : default_params(VSD_BF16);
@@ -653,12 +663,22 @@ vsd_status vsd_lmhead_backward(const void* hidden, const void* weight, int32_t H
     if ((st = check_ws(layout, ws, ws_bytes))) return st;
     if (!d_hidden && !d_weight) return VSD_OK;
     const WsLayout w = ws_layout(layout);
-    cudaError_t e = lmhead_backward(
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const uint64_t timeout = p.wait_timeout_ns ? p.wait_timeout_ns : kDefaultTimeoutNs;
+    if (scratch && scratch_bytes >= 2 * (size_t)R * (size_t)layout.V) {
+        Problem<__nv_bfloat16> P =
+            make_problem<__nv_bfloat16>(draft_logits, nullptr, layout, T, ws);
+        set_params(P, p);
+        cudaError_t e = Launch<__nv_bfloat16>::grad_rows(P, true, scratch, true, s);
+        if (e == cudaSuccess)
+            e = lmhead_backward_dense(hidden, weight, scratch, (int)R, layout.V, H, d_hidden,
+                                      d_weight, at<int>(ws, w.status), timeout, s);
+        return from_cuda(e);
+    }
+    return from_cuda(lmhead_backward(
         hidden, weight, draft_logits, (int)R, layout.V, H, T, at<RowRec>(ws, w.rows),
         at<Coef>(ws, w.coef), p.kl_weight != 0.0 ? at<KlRec>(ws, w.klr) : nullptr,
-        at<void>(ws, w.bfac), d_hidden, d_weight, at<int>(ws, w.status), p.wait_timeout_ns ? p.wait_timeout_ns : kDefaultTimeoutNs,
-        static_cast<cudaStream_t>(stream));
-    return from_cuda(e);
+        at<void>(ws, w.bfac), d_hidden, d_weight, at<int>(ws, w.status), timeout, s));
 }
 
 vsd_status vsd_reference_logkappa(const void* ref_draft, const void* ref_target, vsd_dtype dtype,

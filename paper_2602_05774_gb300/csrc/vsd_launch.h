@@ -38,6 +38,10 @@ template <typename T> struct Launch {
     // the E-step + M-step in two kernels (rows with paths and M-steps; gradient)
     static cudaError_t staged(const Problem<T>& P, bool vec, void* grad, bool grad_bf16,
                               cudaStream_t s);
+    // the gradient rows from the records and coefficients that an E-step + M-step
+    // left in the workspace (a programmatic dependent launch)
+    static cudaError_t grad_rows(const Problem<T>& P, bool vec, void* grad, bool grad_bf16,
+                                 cudaStream_t s);
     // resident blocks per SM of the fused kernel
     static int fused_blocks_per_sm(const Problem<T>& P, bool vec, bool grad_bf16);
 };
@@ -81,5 +85,9 @@ cudaError_t lmhead_backward(const void* hidden, const void* weight, const void* 
                             int V, int H, float T, const RowRec* rows, const Coef* coef,
                             const KlRec* klr, void* fac_scratch, float* d_hidden,
                             float* d_weight, int* status, uint64_t timeout_ns, cudaStream_t s);
+// The same products from G itself, bf16 [R][V].
+cudaError_t lmhead_backward_dense(const void* hidden, const void* weight, const void* G, int R,
+                                  int V, int H, float* d_hidden, float* d_weight, int* status,
+                                  uint64_t timeout_ns, cudaStream_t s);
 
 }  // namespace vsd

@@ -43,6 +43,7 @@
 
 #include "vsd.h"
 #include "vsd_launch.h"
+#include "vsd_gemm2.cuh"
 #include "vsd_tc.cuh"
 
 namespace vsd_bwd {
@@ -129,20 +130,6 @@ __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity, Bars*
 __device__ __forceinline__ bool wait_phase_warp(uint64_t* bar, uint32_t parity, Bars* sb,
                                                 int* status) {
     return __all_sync(0xffffffffu, wait_phase(bar, parity, sb, status));
-}
-
-// Shared-memory descriptor of an MN-major bf16 operand in the 128-byte
-// swizzle: 8-row K groups of 128-byte rows (64 MN elements) 1024 bytes apart
-// (stride byte offset), 64-element MN blocks `lbo` bytes apart (leading byte
-// offset), descriptor version 1, swizzle mode 2.
-__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
 }
 
 // Shared-memory descriptor of a K-major bf16 tile with 32-element (64-byte)
@@ -643,6 +630,51 @@ cudaError_t lmhead_backward(const void* hidden, const void* weight, const void* 
     if (e == cudaSuccess && d_weight)  // G^T . hidden
         e = launch_bwd<vsd_bwd::kDWeight, VSD_BWD_NT, VSD_BWD_KB_DW>(
             logits, hidden, R, fac, klr, c, R, V, H, d_weight, status, timeout_ns, s);
+    return e;
+}
+
+namespace {
+
+// out[M][N] = A . B on CTA pairs, B stored [K][N], A [K][M] (AMN) or [M][K].
+template <bool AMN>
+cudaError_t gemm_f32(const void* a, const void* b, int M, int N, int K, float* out, int* status,
+                     uint64_t timeout_ns, cudaStream_t s) {
+    using namespace vsd_g2;
+    CUtensorMap ta, tb;
+    const bool ok = (AMN ? make_map_box(&ta, a, K, M, 64, BK, 128)
+                         : make_map_box(&ta, a, M, K, BK, BM, 128)) &&
+                    make_map_box(&tb, b, K, N, 64, BK, 128);
+    if (!ok) return cudaErrorInvalidValue;
+    auto kern = k_gemm2<AMN, true, StoreF32>;
+    cudaError_t e = ensure_dyn_smem((const void*)kern, kSmemBytes);
+    if (e != cudaSuccess) return e;
+    const int ntn = (N + BN - 1) / BN, pairs = device_sm_count() / 2;
+    const long long tiles = (long long)((M + 2 * BM - 1) / (2 * BM)) * ntn;
+    const int nk = (K + BK - 1) / BK;
+    // the rows that hold shared tiles (the last ones) start from zero
+    const int whole = nk > 1 ? SplitOrder::whole_tiles(tiles, pairs) : (int)tiles;
+    if (whole < tiles) {
+        const size_t row0 = (size_t)(whole / ntn) * 2 * BM;
+        e = cudaMemsetAsync(out + row0 * N, 0, ((size_t)M - row0) * N * sizeof(float), s);
+        if (e != cudaSuccess) return e;
+    }
+    const long long items = whole + 2 * (tiles - whole);
+    const int grid = 2 * (int)(items < pairs ? items : pairs);
+    kern<<<grid, vsd_g2::kThreads, kSmemBytes, s>>>(ta, tb, M, N, K, StoreF32{out, M, N}, status,
+                                                    timeout_ns);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t lmhead_backward_dense(const void* hidden, const void* weight, const void* G, int R,
+                                  int V, int H, float* d_hidden, float* d_weight, int* status,
+                                  uint64_t timeout_ns, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (d_hidden)  // G . W: A = G as it lies, B = W [V][H]
+        e = gemm_f32<false>(G, weight, R, H, V, d_hidden, status, timeout_ns, s);
+    if (e == cudaSuccess && d_weight)  // G^T . hidden: A = G^T from G [R][V], B = hidden [R][H]
+        e = gemm_f32<true>(G, hidden, V, H, R, d_weight, status, timeout_ns, s);
     return e;
 }
 

@@ -8,6 +8,10 @@
 namespace vsd {
 
 template <>
+cudaError_t Launch<VSD_T>::grad_rows(const Problem<VSD_T>& P, bool vec, void* grad,
+                                     bool grad_bf16, cudaStream_t s);
+
+template <>
 cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad, bool grad_bf16,
                                   cudaStream_t s) {
     const size_t smem = staged_smem_bytes(P.nch, vec);
@@ -18,6 +22,13 @@ cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad,
     if (e) return e;
     rows<<<P.R, kThreads, smem, s>>>(P);
     if ((e = cudaGetLastError()) || !grad) return e;
+    return grad_rows(P, vec, grad, grad_bf16, s);
+}
+
+template <>
+cudaError_t Launch<VSD_T>::grad_rows(const Problem<VSD_T>& P, bool vec, void* grad,
+                                     bool grad_bf16, cudaStream_t s) {
+    const bool kl = P.kl_topk != 0;
     // Gradient segments: a row each, or, where that leaves SMs short of blocks
     // (8 per SM keep about 64 KB in flight), several, of one batch of loads at
     // least.

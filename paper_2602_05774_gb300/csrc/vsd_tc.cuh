@@ -49,6 +49,20 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
     return d;
 }
 
+// Shared-memory descriptor of an MN-major bf16 operand in the 128-byte
+// swizzle: 8-row K groups of 128-byte rows (64 MN elements) 1024 bytes apart
+// (stride byte offset), 64-element MN blocks `lbo` bytes apart (leading byte
+// offset), descriptor version 1, swizzle mode 2.
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
 // Instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, both
 // K-major, an M x N tile.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {

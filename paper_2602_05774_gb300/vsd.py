@@ -24,7 +24,8 @@ SYMBOLS = ("vsd_workspace_bytes", "vsd_sample_paths", "vsd_verify_paths",
            "vsd_weighted_loss_fwd_bwd", "vsd_estep_mstep", "vsd_device_status",
            "vsd_status_string", "vsd_version", "vsd_estep_mstep_noalloc",
            "vsd_noalloc_device_status", "vsd_lmhead_logits", "vsd_lmhead_estep_mstep",
-           "vsd_reference_logkappa", "vsd_tree_estep_mstep", "vsd_lmhead_backward")
+           "vsd_reference_logkappa", "vsd_tree_estep_mstep", "vsd_lmhead_backward",
+           "vsd_lmhead_backward_scratch")
 NOALLOC_SCRATCH_BYTES = 32 << 20
 
 
@@ -110,6 +111,9 @@ def _lib():
                                                C.POINTER(LinearOutputs), vp, C.c_size_t, vp]
         lib.vsd_lmhead_backward.argtypes = [vp, vp, C.c_int32, vp, Layout, C.c_float,
                                             C.POINTER(Params), vp, vp, vp, C.c_size_t, vp]
+        lib.vsd_lmhead_backward_scratch.argtypes = [vp, vp, C.c_int32, vp, Layout, C.c_float,
+                                                    C.POINTER(Params), vp, vp, vp, C.c_size_t,
+                                                    vp, C.c_size_t, vp]
         lib.vsd_device_status.argtypes = [vp, vp, C.POINTER(C.c_int32)]
         lib.vsd_noalloc_device_status.argtypes = [vp, C.POINTER(C.c_int32)]
         lib.vsd_reference_logkappa.argtypes = [vp, vp, C.c_int, C.c_int32, C.c_int32, C.c_int32,
@@ -124,7 +128,8 @@ def _lib():
                      "vsd_estep_mstep", "vsd_device_status", "vsd_estep_mstep_noalloc",
                      "vsd_noalloc_device_status", "vsd_reference_logkappa",
                      "vsd_tree_estep_mstep",
-                     "vsd_lmhead_logits", "vsd_lmhead_estep_mstep", "vsd_lmhead_backward"):
+                     "vsd_lmhead_logits", "vsd_lmhead_estep_mstep", "vsd_lmhead_backward",
+                     "vsd_lmhead_backward_scratch"):
             getattr(lib, name).restype = C.c_int
         _LIB = lib
     return _LIB
@@ -482,10 +487,15 @@ def lmhead_backward(hidden, weight, draft_logits, K, D, T, workspace, prm=None,
             res[name] = torch.empty(*shape, dtype=torch.float32, device=dev)
         elif want is not False and want is not None:
             res[name] = want
-    _check(_lib().vsd_lmhead_backward(_ptr(hidden), _ptr(weight), H, _ptr(draft_logits), lay,
-                                      float(T), C.byref(prm), _ptr(res.get("d_hidden")),
-                                      _ptr(res.get("d_weight")), _ptr(workspace),
-                                      workspace.numel(), _stream(dev)), "vsd_lmhead_backward")
+    try:  # G in bf16, from the caching allocator; without room for it G is made on chip
+        scratch = torch.empty(R * V, dtype=torch.bfloat16, device=dev) if res else None
+    except torch.OutOfMemoryError:
+        scratch = None
+    _check(_lib().vsd_lmhead_backward_scratch(
+        _ptr(hidden), _ptr(weight), H, _ptr(draft_logits), lay, float(T), C.byref(prm),
+        _ptr(res.get("d_hidden")), _ptr(res.get("d_weight")), _ptr(workspace), workspace.numel(),
+        _ptr(scratch), 2 * R * V if scratch is not None else 0, _stream(dev)),
+        "vsd_lmhead_backward")
     return res
 
 

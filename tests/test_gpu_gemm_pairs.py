@@ -1,0 +1,63 @@
+"""The LM head's backward on CTA pairs from a gradient in scratch memory, at the
+edges of its tiles (256 x 256, K blocks of 64, the last tiles' K shared by two
+pairs), and without scratch (the gradient made on chip): every output within
+the fp32 summation bound K 2^-24 sum |a_k b_k| of the float64 product of the
+written bf16 gradient."""
+import ctypes as C
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def vsd():
+    from paper_2602_05774_gb300 import build, vsd as v
+    build.build_library()
+    v.load()
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    return v
+
+
+SHAPES = [  # B, K, D, V, H
+    (1, 1, 1, 8, 8),          # one row
+    (1, 5, 1, 264, 136),
+    (3, 17, 5, 520, 264),     # R = 255
+    (2, 16, 8, 1032, 256),    # R = 256, H = one tile
+    (1, 257, 1, 72, 520),     # R = 257 would need K > 256: see below
+    (20, 16, 8, 264, 2056),   # d_hidden: 10 x 9 tiles, whole ones and shared ones
+]
+
+
+@pytest.mark.parametrize("scratch", [True, False])
+@pytest.mark.parametrize("B,K,D,V,H", SHAPES)
+def test_backward_tiles_within_bound(vsd, B, K, D, V, H, scratch):
+    from paper_2602_05774_gb300 import inputs
+    if K > 256:
+        B, K = K, 1  # R = 257 as prefixes
+    R = B * K * D
+    p = inputs.lmhead_problem(B, K, D, V, H, "cuda", seed=V + H)
+    x = inputs.linear_problem(B, K, D, V, "bf16", "gauss", "cuda", seed=R)
+    ws = vsd.new_workspace(vsd.layout(B, K, D, V), "cuda")
+    prm = vsd.params(like=x["draft"])
+    fw = vsd.estep_mstep(x["draft"], x["target"], x["u_draft"], x["u_accept"], x["u_correct"], K,
+                         D, 1.0, prm=prm, workspace=ws)
+    G, h, w = fw["grad"].double(), p["hidden"].double(), p["weight"].double()
+    if scratch:
+        bw = vsd.lmhead_backward(p["hidden"], p["weight"], x["draft"], K, D, 1.0, ws, prm=prm)
+    else:
+        bw = dict(d_hidden=torch.empty(R, H, device="cuda"),
+                  d_weight=torch.empty(V, H, device="cuda"))
+        ptr = lambda t: C.c_void_p(t.data_ptr())  # noqa: E731
+        code = vsd.load().vsd_lmhead_backward(
+            ptr(p["hidden"]), ptr(p["weight"]), H, ptr(x["draft"]), vsd.layout(B, K, D, V), 1.0,
+            C.byref(prm), ptr(bw["d_hidden"]), ptr(bw["d_weight"]), ptr(ws), ws.numel(),
+            C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert code == 0
+    torch.cuda.synchronize()
+    assert vsd.device_status(ws) == (0, 0)
+    for name, a, b in (("d_hidden", G, w), ("d_weight", G.t(), h)):
+        bound = a.shape[1] * 2.0 ** -24 * (a.abs() @ b.abs()) + 1e-30
+        err = (bw[name].double() - a @ b).abs()
+        assert bool((err <= bound).all()), "%s off by %g" % (name, float((err - bound).max()))
