@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include "vsd.h"
+#include "vsd_grid.cuh"
 #include "vsd_launch.h"
 
 namespace vsd {
@@ -284,7 +285,7 @@ void set_params(Problem<T>& P, const vsd_params& p) {
 }
 
 cudaError_t clear_counters(void* ws, const vsd_layout& L, cudaStream_t s) {
-    return cudaMemsetAsync(ws, 0, ws_layout(L).zero_end, s);
+    return clear_words(ws, ws_layout(L).zero_end, s);
 }
 
 bool vec_ok(const void* a, const void* b, const void* g, int V, size_t elem, size_t gelem) {

@@ -17,7 +17,16 @@ constexpr int kLoads = 4;                // 16-byte vectors per lane per chunk p
 #ifndef VSD_STAGES
 #define VSD_STAGES 2
 #endif
-constexpr int kStages = VSD_STAGES;      // TMA ring depth per warp (chunks in flight)
+constexpr int kStages = VSD_STAGES;      // TMA ring depth per warp, persistent kernel
+// The same, one block per row: 16 KB of ring let eight blocks share an SM, so
+// that more rows stream while others are in their tails (64 heads of 64 rows,
+// V = 32000: LM head + E/M step 846 us with two stages and six blocks, 828 with
+// one; ten or twelve blocks spill and gain nothing).
+#ifndef VSD_ROW_STAGES
+#define VSD_ROW_STAGES 1
+#endif
+constexpr int kRowStages = VSD_ROW_STAGES;
+constexpr int kRowBlocks = 8;
 constexpr double kLog2e = 1.4426950408889634073599246810019;
 constexpr double kLn2 = 0.69314718055994530941723212145818;
 
@@ -92,6 +101,15 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 }
 __device__ __forceinline__ void st_release(int* p, int v) {
     asm volatile("st.release.gpu.global.b32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
+}
+
+// Add to a counter, releasing this thread's earlier writes (and, after a
+// barrier, its block's) and acquiring those released by earlier adds.
+__device__ __forceinline__ int atomic_add_acq_rel(int* p, int v) {
+    int r;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;"
+                 : "=r"(r) : "l"(p), "r"(v) : "memory");
+    return r;
 }
 
 __device__ __forceinline__ uint64_t global_timer_ns() {
@@ -239,6 +257,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
+// Close a group of this thread's cp.async copies; wait for all groups but the
+// last one closed.
+__device__ __forceinline__ void cp_async_commit() {
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void cp_async_wait_1() {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- packed f32x2
 // Blackwell executes two float32 add/sub/mul in one instruction on a 64-bit
 // register pair; each lane of the pair is an ordinary IEEE round-to-nearest op.
@@ -320,6 +347,21 @@ __device__ __forceinline__ float warp_sum(float v) {
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// Sum, and inclusive prefix sum, of the first n lanes' values (the other lanes
+// hold 0 for the sum): the steps that would add nothing are left out, the
+// rounding is that of the whole warp's.
+__device__ __forceinline__ double warp_sum_n(double v, int n) {
+    for (int o = 16; o; o >>= 1)
+        if (o < n) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double warp_incl_scan_n(double v, int lane, int n) {
+    for (int o = 1; o < n; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
     return v;
 }
 // Inclusive prefix sum over the lanes of a warp.

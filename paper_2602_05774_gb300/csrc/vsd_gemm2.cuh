@@ -318,6 +318,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const int c = blockIdx.x >> 1, nc = gridDim.x >> 1;
+    // (a dependent E-step takes up the SMs that run out of tiles)
+    vsd::grid_launch_next();
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&sb->full[s], 1);

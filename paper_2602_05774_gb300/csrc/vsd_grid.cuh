@@ -59,6 +59,21 @@ static cudaError_t prep(K kernel, size_t smem) {
     return ensure_dyn_smem(reinterpret_cast<const void*>(kernel), smem);
 }
 
+// The call's counters (n bytes of the workspace, a multiple of 16) to zero, as a
+// kernel, so that the first kernel of the call can be its programmatic
+// dependent and read its rows meanwhile (a memset's completion costs the call
+// about 2 us before its first kernel starts).
+static __global__ void __launch_bounds__(256) k_clear(uint4* p, int n) {
+    grid_launch_next();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < n) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+static inline cudaError_t clear_words(void* ws, size_t bytes, cudaStream_t s) {
+    const int n = (int)(bytes / 16);
+    k_clear<<<(n + 255) / 256, 256, 0, s>>>(static_cast<uint4*>(ws), n);
+    return cudaGetLastError();
+}
+
 // Launch `kern` as a programmatic dependent of the stream's previous kernel: its
 // blocks may become resident while that kernel's last ones still run, and wait
 // in grid_wait() until it has completed and its writes are visible.

@@ -12,9 +12,10 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
     const int r = blockIdx.x;
     row_pass<T, VEC, false, kSampleToken, false>(P, r, rg, tab, sh);
     if (threadIdx.x == 0) {
@@ -31,9 +32,10 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_rows_verify(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
     row_pass<T, VEC, true, kGivenToken, true>(P, blockIdx.x, rg, tab, sh);
 }
 
@@ -43,9 +45,10 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_ref_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
     row_pass<T, VEC, true, kNoToken, true>(P, blockIdx.x, rg, tab, sh);
 }
 
@@ -54,6 +57,7 @@ __global__ void __launch_bounds__(kThreads) k_ref_rows(Problem<T> P) {
 template <typename T>
 __global__ void k_ref_scan(Problem<T> P, float* out) {
     const int b = blockIdx.x, lane = threadIdx.x & 31;
+    grid_wait();
     double carry = 0.0;
     for (int d0 = 0; d0 < P.D; d0 += 32) {
         const int d = d0 + lane;
@@ -72,9 +76,10 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_paths(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ PathShared sh;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_wait();
     path_pass<T, VEC>(P, blockIdx.x, rg, tab, sh);
 }
 
@@ -83,6 +88,8 @@ __global__ void __launch_bounds__(kThreads)
     k_weights(Problem<T> P, EStepView E, float* weights, float* loss) {
     __shared__ WeightsShared sh;
     __shared__ int last;
+    grid_launch_next();
+    grid_wait();
     weights_pass<T>(P, E, blockIdx.x, weights, loss, sh);
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -97,6 +104,7 @@ __global__ void __launch_bounds__(kThreads)
 
 template <typename T, bool VEC, typename G>
 __global__ void __launch_bounds__(kThreads) k_grad(Problem<T> P, const float4* rstats, G* grad) {
+    grid_wait();
     grad_pass<T, VEC, G>(P, blockIdx.x, rstats, grad);
 }
 
@@ -358,9 +366,10 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
     __shared__ CtlShared cs;
     __shared__ Job slots[kSlots];
     __shared__ KlRec kslot[kSlots];  // VSD (KL): the top-K terms of a gradient job's row
-    Ring* rg;
+    Ring<kStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < kWarps) {  // ------------------------------- streaming warps
         for (int i = 0;; ++i) {
@@ -447,90 +456,83 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
 // ------------------------------------------------------------ launchers
 template <>
 cudaError_t Launch<VSD_T>::sample(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
     if (vec) {
         cudaError_t e = prep(k_sample<VSD_T, true>, smem);
         if (e) return e;
-        k_sample<VSD_T, true><<<P.R, kThreads, smem, s>>>(P);
+        return launch_after(k_sample<VSD_T, true>, P.R, kThreads, smem, s, P);
     } else {
         cudaError_t e = prep(k_sample<VSD_T, false>, smem);
         if (e) return e;
-        k_sample<VSD_T, false><<<P.R, kThreads, smem, s>>>(P);
+        return launch_after(k_sample<VSD_T, false>, P.R, kThreads, smem, s, P);
     }
-    return cudaGetLastError();
 }
 
 template <>
 cudaError_t Launch<VSD_T>::rows_verify(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
     auto kern = vec ? k_rows_verify<VSD_T, true> : k_rows_verify<VSD_T, false>;
     cudaError_t e = prep(kern, smem);
     if (e) return e;
-    kern<<<P.R, kThreads, smem, s>>>(P);
-    return cudaGetLastError();
+    return launch_after(kern, P.R, kThreads, smem, s, P);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::reference(const Problem<VSD_T>& P, bool vec, float* out,
                                      cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
     auto kern = vec ? k_ref_rows<VSD_T, true> : k_ref_rows<VSD_T, false>;
     cudaError_t e = prep(kern, smem);
     if (e) return e;
-    kern<<<P.R, kThreads, smem, s>>>(P);
-    e = cudaGetLastError();
-    if (e) return e;
-    k_ref_scan<VSD_T><<<P.B, 32, 0, s>>>(P, out);
-    return cudaGetLastError();
+    if ((e = launch_after(kern, P.R, kThreads, smem, s, P))) return e;
+    return launch_after(k_ref_scan<VSD_T>, P.B, 32, 0, s, P, out);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::paths(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
     const int npaths = P.B * P.K;
     if (vec) {
         cudaError_t e = prep(k_paths<VSD_T, true>, smem);
         if (e) return e;
-        k_paths<VSD_T, true><<<npaths, kThreads, smem, s>>>(P);
+        return launch_after(k_paths<VSD_T, true>, npaths, kThreads, smem, s, P);
     } else {
         cudaError_t e = prep(k_paths<VSD_T, false>, smem);
         if (e) return e;
-        k_paths<VSD_T, false><<<npaths, kThreads, smem, s>>>(P);
+        return launch_after(k_paths<VSD_T, false>, npaths, kThreads, smem, s, P);
     }
-    return cudaGetLastError();
 }
 
 template <>
 cudaError_t Launch<VSD_T>::weights(const Problem<VSD_T>& P, const EStepView& E, float* weights,
                                    float* loss, cudaStream_t s) {
-    k_weights<VSD_T><<<P.B, kThreads, 0, s>>>(P, E, weights, loss);
-    return cudaGetLastError();
+    return launch_after(k_weights<VSD_T>, P.B, kThreads, 0, s, P, E, weights, loss);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::grad(const Problem<VSD_T>& P, bool vec, const float4* rstats,
                                 void* grad, bool grad_bf16, cudaStream_t s) {
-#define VSD_GRAD(V_, G_) \
-    k_grad<VSD_T, V_, G_><<<P.R, kThreads, 0, s>>>(P, rstats, reinterpret_cast<G_*>(grad))
+#define VSD_GRAD(V_, G_)                                                        \
+    return launch_after(k_grad<VSD_T, V_, G_>, P.R, kThreads, 0, s, P, rstats, \
+                        reinterpret_cast<G_*>(grad))
     if (vec && grad_bf16) VSD_GRAD(true, __nv_bfloat16);
-    else if (vec) VSD_GRAD(true, float);
-    else if (grad_bf16) VSD_GRAD(false, __nv_bfloat16);
-    else VSD_GRAD(false, float);
+    if (vec) VSD_GRAD(true, float);
+    if (grad_bf16) VSD_GRAD(false, __nv_bfloat16);
+    VSD_GRAD(false, float);
 #undef VSD_GRAD
-    return cudaGetLastError();
 }
 
 template <>
 cudaError_t Launch<VSD_T>::fused(const Problem<VSD_T>& P, bool vec, void* grad, bool grad_bf16,
                                  int ctas, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kStages>(P.nch, vec);
     const bool kl = P.kl_topk != 0;
 #define VSD_FUSED(V_, G_, KL_)                                                         \
     do {                                                                               \
         cudaError_t e = prep(k_fused<VSD_T, V_, G_, KL_>, smem);                       \
         if (e) return e;                                                               \
-        k_fused<VSD_T, V_, G_, KL_><<<ctas, kFusedThreads, smem, s>>>(                 \
-            P, reinterpret_cast<G_*>(grad));                                           \
+        return launch_after(k_fused<VSD_T, V_, G_, KL_>, ctas, kFusedThreads, smem, s, \
+                            P, reinterpret_cast<G_*>(grad));                           \
     } while (0)
 #define VSD_FUSED_KL(V_, G_)                 \
     do {                                     \
@@ -548,7 +550,7 @@ cudaError_t Launch<VSD_T>::fused(const Problem<VSD_T>& P, bool vec, void* grad, 
 
 template <>
 int Launch<VSD_T>::fused_blocks_per_sm(const Problem<VSD_T>& P, bool vec, bool grad_bf16) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kStages>(P.nch, vec);
     const bool kl = P.kl_topk != 0;
 #define VSD_K(V_, G_) (kl ? reinterpret_cast<const void*>(k_fused<VSD_T, V_, G_, true>) \
                           : reinterpret_cast<const void*>(k_fused<VSD_T, V_, G_, false>))

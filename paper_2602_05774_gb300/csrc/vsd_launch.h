@@ -58,10 +58,10 @@ cudaError_t ensure_dyn_smem(const void* kernel, size_t smem);
 int blocks_per_sm(const void* kernel, int threads, size_t smem);
 
 inline size_t table_smem_bytes(int nch) { return (size_t)nch * sizeof(float4); }
-// Dynamic shared memory of a streaming kernel: the TMA ring (vector rows
-// only) followed by the chunk table.
-inline size_t stream_smem_bytes(int nch, bool vec) {
-    return (vec ? sizeof(Ring) : 0) + table_smem_bytes(nch);
+// Dynamic shared memory of a streaming kernel: the TMA ring of S stages (vector
+// rows only; at least MIN bytes) followed by the chunk table.
+template <int S, size_t MIN = 0> inline size_t stream_smem_bytes(int nch, bool vec) {
+    return (vec ? ring_bytes<S, MIN>() : 0) + table_smem_bytes(nch);
 }
 
 // The draft LM head on the tensor cores (vsd_lmhead.cu): logits = hidden .

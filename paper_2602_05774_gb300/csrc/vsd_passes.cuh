@@ -208,21 +208,21 @@ __device__ __forceinline__ float2 chunk_stats(const uint4 (&buf)[kLoads], float 
 }
 
 // --------------------------------------------------------------- TMA ring
-// Every warp owns kStages slots, each holding one chunk of the draft row and
+// Every warp owns S slots, each holding one chunk of the draft row and
 // one of the target row.  The warp's lane 0 issues 1-D bulk copies (TMA) up
-// to kStages chunks ahead; all lanes wait on the slot's mbarrier, read their
+// to S chunks ahead; all lanes wait on the slot's mbarrier, read their
 // own vectors, and the slot is refilled once the warp has read it.  Each warp
 // produces and consumes its own slots, so no block-wide synchronisation is
 // involved.  A stream of one row only (no target) uses the same memory as
-// 2 kStages single-chunk slots, so it keeps as many bytes in flight.  Each
+// 2 S single-chunk slots, so it keeps as many bytes in flight.  Each
 // layout has its own barriers and its own count of consumed chunks (pos2 for
 // two rows, pos1 for one; slot = pos % stages, phase = (pos / stages) & 1),
 // which persist across calls; a call consumes every chunk it issues, so the
 // two layouts never hold a buffer at the same time.
-struct Ring {
-    uint4 data[kWarps][kStages][2][kLoads * 32];
-    uint64_t bar2[kWarps][kStages];
-    uint64_t bar1[kWarps][2 * kStages];
+template <int S> struct Ring {
+    uint4 data[kWarps][S][2][kLoads * 32];
+    uint64_t bar2[kWarps][S];
+    uint64_t bar1[kWarps][2 * S];
     int pos2[kWarps];
     int pos1[kWarps];
     int broken[kWarps];  // a wait ran out: no further waits or copies in this block
@@ -231,12 +231,13 @@ struct Ring {
 
 // Every thread of the block calls it; warps beyond the streaming warps (the
 // fused kernel's control warp) own no ring slots.
-__device__ __forceinline__ void ring_init(Ring* rg, uint64_t timeout_ns) {
+template <int S>
+__device__ __forceinline__ void ring_init(Ring<S>* rg, uint64_t timeout_ns) {
     if (threadIdx.x == 0) rg->timeout_ns = timeout_ns;
     if ((threadIdx.x & 31) == 0 && (threadIdx.x >> 5) < kWarps) {
         const int w = threadIdx.x >> 5;
-        for (int st = 0; st < kStages; ++st) mbar_init(&rg->bar2[w][st], 1);
-        for (int st = 0; st < 2 * kStages; ++st) mbar_init(&rg->bar1[w][st], 1);
+        for (int st = 0; st < S; ++st) mbar_init(&rg->bar2[w][st], 1);
+        for (int st = 0; st < 2 * S; ++st) mbar_init(&rg->bar1[w][st], 1);
         rg->pos2[w] = 0;
         rg->pos1[w] = 0;
         rg->broken[w] = 0;
@@ -245,13 +246,17 @@ __device__ __forceinline__ void ring_init(Ring* rg, uint64_t timeout_ns) {
     __syncthreads();
 }
 
-// Dynamic shared memory: [Ring (vector rows)] [chunk table].
-template <bool VEC>
-__device__ __forceinline__ void smem_views(unsigned char* dsm, Ring*& rg, float4*& tab,
+// Dynamic shared memory: [Ring (vector rows only), or MIN bytes if that is
+// more][chunk table].
+template <int S, size_t MIN = 0> __host__ __device__ constexpr size_t ring_bytes() {
+    return sizeof(Ring<S>) > MIN ? sizeof(Ring<S>) : (MIN + 127) / 128 * 128;
+}
+template <bool VEC, size_t MIN = 0, int S>
+__device__ __forceinline__ void smem_views(unsigned char* dsm, Ring<S>*& rg, float4*& tab,
                                            uint64_t timeout_ns) {
     if (VEC) {
-        rg = reinterpret_cast<Ring*>(dsm);
-        tab = reinterpret_cast<float4*>(dsm + sizeof(Ring));
+        rg = reinterpret_cast<Ring<S>*>(dsm);
+        tab = reinterpret_cast<float4*>(dsm + ring_bytes<S, MIN>());
         ring_init(rg, timeout_ns);
     } else {
         rg = nullptr;
@@ -277,13 +282,13 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, int* s
 // ... < ch1) of row x (and y) through the ring; consume(ch, bx, by) gets each
 // chunk in registers (positions at or beyond V read as -inf).  Rows must be
 // 16-byte aligned with V * sizeof(T) a multiple of 16.
-template <typename T, bool HAS_Y, class Consume>
-__device__ __forceinline__ void ring_stream(Ring* rg, const T* x, const T* y, int64_t V, int ch0,
+template <typename T, bool HAS_Y, int S, class Consume>
+__device__ __forceinline__ void ring_stream(Ring<S>* rg, const T* x, const T* y, int64_t V, int ch0,
                                             int ch1, uint64_t polx, uint64_t poly, int* status,
                                             Consume&& consume) {
     constexpr int PV = Traits<T>::kPerVec;
     constexpr int CE = chunk_elems<T>();
-    constexpr int NS = HAS_Y ? kStages : 2 * kStages;
+    constexpr int NS = HAS_Y ? S : 2 * S;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint64_t* bars = HAS_Y ? rg->bar2[warp] : rg->bar1[warp];
     int* posp = HAS_Y ? &rg->pos2[warp] : &rg->pos1[warp];
@@ -353,8 +358,8 @@ __device__ __forceinline__ void ring_stream(Ring* rg, const T* x, const T* y, in
 // filling tab[c] = (max_x, sum_x, max_y, sum_y) for each chunk c (tab is a
 // shared-memory table or a row's table in global memory).  Warps take chunks
 // round-robin and keep the next chunks' loads in flight.
-template <typename T, bool VEC, bool HAS_Y>
-__device__ __forceinline__ void stream_tables(Ring* rg, const T* x, const T* y, int64_t V, int ch0,
+template <typename T, bool VEC, bool HAS_Y, int S>
+__device__ __forceinline__ void stream_tables(Ring<S>* rg, const T* x, const T* y, int64_t V, int ch0,
                                               int ch1, float4* tab, float c, uint64_t polx,
                                               uint64_t poly, int* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -397,8 +402,8 @@ __device__ __forceinline__ void stream_tables(Ring* rg, const T* x, const T* y, 
 // The target half of a row's chunk table when the draft half is given (the LM
 // head's epilogue wrote it): tab[ch].zw = (max, sum) of target chunk ch, for
 // ch in [ch0, ch1), one streaming read of the target row through the ring.
-template <typename T>
-__device__ __forceinline__ void stream_target_tables(Ring* rg, const T* y, int64_t V, int ch0,
+template <typename T, int S>
+__device__ __forceinline__ void stream_target_tables(Ring<S>* rg, const T* y, int64_t V, int ch0,
                                                      int ch1, float4* tab, float c, uint64_t pol,
                                                      int* status) {
     const int lane = threadIdx.x & 31;
@@ -589,6 +594,42 @@ __device__ __forceinline__ Located table_locate(const float4* tab, int nch, int 
     return Located{last, INFINITY};
 }
 
+// Chunk ch of a row into a shared-memory buffer with cp.async (warp; rows
+// 16-byte aligned).  Vectors at or beyond V are not read.
+template <typename T>
+__device__ __forceinline__ void chunk_async(uint4* buf, const T* row, int64_t V, int ch,
+                                            int lane) {
+    constexpr int PV = Traits<T>::kPerVec;
+    const int64_t base = (int64_t)ch * chunk_elems<T>() + lane * PV;
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+        const int64_t v0 = base + (int64_t)k * 32 * PV;
+        cp_async16(buf + k * 32 + lane, row + (v0 < V ? v0 : 0), v0 < V);
+    }
+}
+// The chunk in registers as load_chunk gives it (positions at or beyond V
+// read as -inf).
+template <typename T>
+__device__ __forceinline__ void chunk_from_smem(const uint4* buf, int64_t V, int ch, int lane,
+                                                uint4 (&b)[kLoads]) {
+    constexpr int PV = Traits<T>::kPerVec;
+    const int64_t base = (int64_t)ch * chunk_elems<T>() + lane * PV;
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k)
+        b[k] = base + (int64_t)k * 32 * PV < V
+                   ? buf[k * 32 + lane]
+                   : make_uint4(Traits<T>::kNegInf, Traits<T>::kNegInf, Traits<T>::kNegInf,
+                                Traits<T>::kNegInf);
+}
+// Logit v of a buffer holding chunk ch.
+__device__ __forceinline__ float smem_elem(const uint4* buf, int ch, int v, const float*) {
+    return reinterpret_cast<const float*>(buf)[v - ch * chunk_elems<float>()];
+}
+__device__ __forceinline__ float smem_elem(const uint4* buf, int ch, int v, const __nv_bfloat16*) {
+    return __bfloat162float(
+        reinterpret_cast<const __nv_bfloat16*>(buf)[v - ch * chunk_elems<__nv_bfloat16>()]);
+}
+
 // Scan chunk ch (in registers: bx, by as load_chunk gives them) in token order
 // and return the first token of positive mass whose running mass exceeds tc
 // (the chunk-frame threshold); if none does, the last token with mass; -1 if
@@ -644,14 +685,87 @@ __device__ __forceinline__ int rescan_regs(const uint4 (&bx)[kLoads], const uint
     return last;
 }
 
-// rescan_regs on chunk ch loaded from global memory.
+// The same on the chunk in shared memory (bx, by: buffers that chunk_async
+// filled), one vector per lane at a time: a quarter of the code, which runs
+// once per draw and is fetched more slowly than it executes.
+template <typename T, bool NEED_X, bool NEED_Y, class Mass>
+__device__ __forceinline__ int rescan_smem(const uint4* bx, const uint4* by, int64_t V, int ch,
+                                           float tc, const Mass& mass, int lane) {
+    constexpr int PV = Traits<T>::kPerVec;
+    float carry = 0.f;
+    int last = -1;
+    const int base = ch * chunk_elems<T>();
+#pragma unroll 1
+    for (int k = 0; k < kLoads; ++k) {
+        const int v0 = base + k * 32 * PV + lane * PV;
+        const bool in = v0 < V;  // (V is a whole number of vectors)
+        float fx[PV], fy[PV], m[PV];
+        if (NEED_X) unpack<T>(bx[k * 32 + lane], fx);
+        if (NEED_Y) unpack<T>(by[k * 32 + lane], fy);
+        float run = 0.f;
+        int lastpos = -1;
+#pragma unroll
+        for (int e = 0; e < PV; ++e) {
+            m[e] = in ? mass(NEED_X ? fx[e] : 0.f, NEED_Y ? fy[e] : 0.f, v0 + e) : 0.f;
+            run += m[e];
+            if (m[e] > 0.f) lastpos = e;
+        }
+        const float incl = warp_incl_scan(run, lane);
+        float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) excl = 0.f;
+        int epos = -1;
+        float acc = carry + excl;
+#pragma unroll
+        for (int e = 0; e < PV; ++e) {
+            acc += m[e];
+            if (epos < 0 && m[e] > 0.f && acc > tc) epos = e;
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, epos >= 0);
+        if (hit) {
+            const int L = __ffs(hit) - 1;
+            return base + k * 32 * PV + L * PV + __shfl_sync(0xffffffffu, epos, L);
+        }
+        const unsigned pos = __ballot_sync(0xffffffffu, lastpos >= 0);
+        if (pos) {
+            const int L = 31 - __clz(pos);
+            last = base + k * 32 * PV + L * PV + __shfl_sync(0xffffffffu, lastpos, L);
+        }
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    return last;
+}
+
+// A warp's two chunk buffers for rescans: its own ring slots (no copy of its
+// stream is in flight then), null on the scalar path.
+template <int S> __device__ __forceinline__ uint4* warp_chunks(Ring<S>* rg) {
+    return rg ? &rg->data[threadIdx.x >> 5][0][0][0] : nullptr;
+}
+
+// Both rows' chunk ch into a warp's buffers (x first), one round trip.
+template <typename T>
+__device__ __forceinline__ void load_chunk_pair(uint4* buf, const T* x, const T* y, int64_t V,
+                                                int ch, int lane) {
+    __syncwarp();
+    if (x) chunk_async<T>(buf, x, V, ch, lane);
+    if (y) chunk_async<T>(buf + kLoads * 32, y, V, ch, lane);
+    cp_async_wait_all();
+    __syncwarp();
+}
+
+// Rescan of chunk ch from global memory, through the warp's buffers (rows
+// aligned) or registers.
 template <typename T, bool VEC, bool NEED_X, bool NEED_Y, class Mass>
 __device__ __forceinline__ int warp_rescan(const T* x, const T* y, int64_t V, int ch, float tc,
-                                           const Mass& mass, int lane, uint64_t pol) {
-    uint4 bx[kLoads], by[kLoads];
-    if (NEED_X) load_chunk<T, VEC>(x, V, ch, lane, pol, bx);
-    if (NEED_Y) load_chunk<T, VEC>(y, V, ch, lane, pol, by);
-    return rescan_regs<T, NEED_X, NEED_Y>(bx, by, ch, tc, mass, lane);
+                                           const Mass& mass, int lane, uint64_t pol, uint4* buf) {
+    if constexpr (VEC) {
+        load_chunk_pair<T>(buf, NEED_X ? x : nullptr, NEED_Y ? y : nullptr, V, ch, lane);
+        return rescan_smem<T, NEED_X, NEED_Y>(buf, buf + kLoads * 32, V, ch, tc, mass, lane);
+    } else {
+        uint4 bx[kLoads], by[kLoads];
+        if (NEED_X) load_chunk<T, VEC>(x, V, ch, lane, pol, bx);
+        if (NEED_Y) load_chunk<T, VEC>(y, V, ch, lane, pol, by);
+        return rescan_regs<T, NEED_X, NEED_Y>(bx, by, ch, tc, mass, lane);
+    }
 }
 
 struct MassX {
@@ -677,13 +791,12 @@ struct MassRes {
 template <typename T, bool VEC>
 __device__ __forceinline__ int warp_sample(const T* x, const T* y, int64_t V, const float4* tab,
                                            int nch, int comp, float M, const TableSum& S, float u,
-                                           float c, int lane, uint64_t pol) {
+                                           float c, int lane, uint64_t pol, uint4* buf) {
     const Located loc = table_locate(tab, nch, comp, frame_of(M), c, S, u, lane);
     if (loc.ch < 0) return -1;
     const float mm = frame_of(tab_ms(tab[loc.ch], comp).x);
-    if (comp == 0)
-        return warp_rescan<T, VEC, true, false>(x, y, V, loc.ch, loc.tc, MassX{mm, c}, lane, pol);
-    return warp_rescan<T, VEC, false, true>(x, y, V, loc.ch, loc.tc, MassY{mm, c}, lane, pol);
+    return warp_rescan<T, VEC, true, false>(comp == 0 ? x : y, nullptr, V, loc.ch, loc.tc,
+                                            MassX{mm, c}, lane, pol, buf);
 }
 
 // First chunk whose target maximum equals the row max M (warp; -1 if none).
@@ -722,15 +835,28 @@ __device__ __forceinline__ int first_max_regs(const uint4 (&by)[kLoads], int ch,
     return -1;
 }
 
-// Lowest index whose target logit equals the row max M (warp).
-template <typename T, bool VEC>
-__device__ __forceinline__ int warp_first_max(const T* y, int64_t V, const float4* tab, int nch,
-                                              float M, int lane, uint64_t pol, int comp = 1) {
-    const int ch = table_first_max(tab, nch, M, comp);
-    if (ch < 0) return -1;
-    uint4 by[kLoads];
-    load_chunk<T, VEC>(y, V, ch, lane, pol, by);
-    return first_max_regs<T>(by, ch, M);
+// The same on the chunk in shared memory.
+template <typename T>
+__device__ __forceinline__ int first_max_smem(const uint4* by, int64_t V, int ch, float M) {
+    constexpr int PV = Traits<T>::kPerVec;
+    const int lane = threadIdx.x & 31;
+    const int base = ch * chunk_elems<T>();
+#pragma unroll 1
+    for (int k = 0; k < kLoads; ++k) {
+        const int v0 = base + k * 32 * PV + lane * PV;
+        float f[PV];
+        unpack<T>(by[k * 32 + lane], f);
+        int e0 = PV;
+#pragma unroll
+        for (int e = PV - 1; e >= 0; --e)
+            if (f[e] == M) e0 = e;
+        const unsigned hit = __ballot_sync(0xffffffffu, v0 < V && e0 < PV);
+        if (hit) {
+            const int L = __ffs(hit) - 1;
+            return base + k * 32 * PV + L * PV + __shfl_sync(0xffffffffu, e0, L);
+        }
+    }
+    return -1;
 }
 
 __device__ __forceinline__ bool row_ok(float M, double Z) {
@@ -756,52 +882,103 @@ __device__ __forceinline__ void token_logs(const T* x, const T* y, int v, const 
 // --------------------------------------------------------------- row pass
 enum XMode { kNoToken = 0, kSampleToken = 1, kGivenToken = 2 };
 
-// One of the row's three table-driven results (warp; every lane returns the
-// same values): which = 0 the draft statistics and z~ (drawn from q with
+// One of the row's three table-driven results (warp; lane 0 returns them all):
+// which = 0 the draft statistics and z~ (drawn from q with
 // u_draft, or read from given_tokens), 1 the target statistics and the draw
-// from p with u_correct, 2 the lowest-index argmax of the target.
+// from p with u_correct, 2 the lowest-index argmax of the target.  xv, yv: the
+// token's logits; lz: ln of the total.
 struct RowTask {
     float M;
     TableSum S;
     int tok;
+    float xv, yv;
+    double lz;
 };
-template <typename T, bool VEC, int XMODE>
+template <typename T, bool VEC, bool HAS_Y, int XMODE>
 __device__ __forceinline__ RowTask row_task(const Problem<T>& P, int r, const float4* tab,
-                                            int which, int lane) {
+                                            int which, int lane, uint4* buf) {
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
-    const T* y = P.target + (int64_t)r * V;
+    const T* y = HAS_Y ? P.target + (int64_t)r * V : nullptr;
     const float c = P.ts.c;
-    const uint64_t pol = policy_evict_normal();
+    const int comp = which == 0 ? 0 : 1;
     RowTask t;
-    t.M = table_max(tab, P.nch, which == 0 ? 0 : 1, lane);
-    t.S = TableSum{0, 0, 0.0};
     t.tok = -1;
-    if (which == 2) {
-        if (t.M > -INFINITY) t.tok = warp_first_max<T, VEC>(y, V, tab, P.nch, t.M, lane, pol);
-        if (t.tok >= V) t.tok = -1;
-        return t;
-    }
-    t.S = table_sum(tab, P.nch, which, frame_of(t.M), c, lane);
-    if (which == 0) {
-        if (XMODE == kSampleToken) {
-            if (row_ok(t.M, t.S.Z))
-                t.tok = P.greedy ? warp_first_max<T, VEC>(x, V, tab, P.nch, t.M, lane, pol, 0)
-                                 : warp_sample<T, VEC>(x, y, V, tab, P.nch, 0, t.M, t.S,
-                                                       __ldg(P.u_draft + r), c, lane, pol);
-            if (t.tok >= V) t.tok = -1;
-        } else if (XMODE == kGivenToken) {
-            t.tok = __ldg(P.given_tokens + r);
+    t.xv = t.yv = 0.f;
+    t.lz = 0.0;
+    // (asked for early: its latency is hidden behind the table's)
+    const float* up = which == 0 ? P.u_draft : P.u_correct;
+    const bool drawn = which == 0 ? XMODE == kSampleToken : which == 1;
+    const float u = drawn && up ? __ldg(up + r) : 0.f;
+    int given = -1;
+    if (XMODE == kGivenToken && which == 0) {
+        given = __ldg(P.given_tokens + r);
+        if (given >= 0 && given < V) {
+            t.xv = elem_value(x, given);
+            if (HAS_Y) t.yv = elem_value(y, given);
         }
+    }
+    t.M = table_max(tab, P.nch, comp, lane);
+    t.S = TableSum{0, 0, 0.0};
+    Located loc{-1, 0.f};
+    if (which == 2) {
+        if (t.M > -INFINITY) loc.ch = table_first_max(tab, P.nch, t.M);
     } else {
+        t.S = table_sum(tab, P.nch, comp, frame_of(t.M), c, lane);
         // (no uniforms for the p-draw: the reference rows of
         // vsd_reference_logkappa need only the argmax)
-        if (row_ok(t.M, t.S.Z) && (P.greedy || P.u_correct))
-            t.tok = P.greedy ? warp_first_max<T, VEC>(y, V, tab, P.nch, t.M, lane, pol)
-                             : warp_sample<T, VEC>(x, y, V, tab, P.nch, 1, t.M, t.S,
-                                                   __ldg(P.u_correct + r), c, lane, pol);
-        if (t.tok >= V) t.tok = -1;
+        if (drawn && row_ok(t.M, t.S.Z) && (P.greedy || up)) {
+            if (P.greedy)
+                loc.ch = table_first_max(tab, P.nch, t.M, comp);
+            else
+                loc = table_locate(tab, P.nch, comp, frame_of(t.M), c, t.S, u, lane);
+        }
     }
+    const bool first = which == 2 || P.greedy;
+    if constexpr (VEC) {
+        // both rows' chunk in one round trip: the draw's, and the logits of the
+        // token it returns; the logarithm of the total meanwhile
+        __syncwarp();
+        if (loc.ch >= 0) {
+            chunk_async<T>(buf, x, V, loc.ch, lane);
+            if (HAS_Y) chunk_async<T>(buf + kLoads * 32, y, V, loc.ch, lane);
+        }
+        if (which != 2 && lane == 0) t.lz = log(t.S.Z);  // (lane 0 hands the task on)
+        cp_async_wait_all();
+        __syncwarp();
+        if (loc.ch >= 0) {
+            const uint4* z = comp == 0 ? buf : buf + kLoads * 32;
+            if (first) {
+                t.tok = first_max_smem<T>(z, V, loc.ch, t.M);
+            } else {
+                const float mm = frame_of(tab_ms(tab[loc.ch], comp).x);
+                t.tok = rescan_smem<T, true, false>(z, z, V, loc.ch, loc.tc, MassX{mm, c}, lane);
+            }
+            if (t.tok >= 0) {
+                t.xv = smem_elem(buf, loc.ch, t.tok, x);
+                if (HAS_Y) t.yv = smem_elem(buf + kLoads * 32, loc.ch, t.tok, y);
+            }
+        }
+    } else {
+        if (which != 2 && lane == 0) t.lz = log(t.S.Z);
+        if (loc.ch >= 0) {
+            const T* zr = comp == 0 ? x : y;
+            uint4 z[kLoads];
+            load_chunk<T, VEC>(zr, V, loc.ch, lane, policy_evict_normal(), z);
+            if (first) {
+                t.tok = first_max_regs<T>(z, loc.ch, t.M);
+            } else {
+                const float mm = frame_of(tab_ms(tab[loc.ch], comp).x);
+                t.tok = rescan_regs<T, true, false>(z, z, loc.ch, loc.tc, MassX{mm, c}, lane);
+            }
+            if (t.tok >= V) t.tok = -1;
+            if (t.tok >= 0) {
+                t.xv = elem_value(x, t.tok);
+                if (HAS_Y) t.yv = elem_value(y, t.tok);
+            }
+        }
+    }
+    if (XMODE == kGivenToken && which == 0) t.tok = given;
     return t;
 }
 
@@ -818,11 +995,8 @@ __device__ __forceinline__ void row_finish(const Problem<T>& P, int r, const Row
     const bool okx = row_ok(tx.M, tx.S.Z);
     const bool oky = HAS_Y ? row_ok(ty.M, ty.S.Z) : true;
     const bool ok = okx && oky;
-    // the two logarithms at once, on lanes 0 and 1
-    const double lz = log(lane == 0 ? tx.S.Z : ty.S.Z);
-    const double lzx0 = __shfl_sync(0xffffffffu, lz, 0), lzy0 = __shfl_sync(0xffffffffu, lz, 1);
-    const double lzx = okx ? lzx0 : 0.0;
-    const double lzy = (HAS_Y && oky) ? lzy0 : 0.0;
+    const double lzx = okx ? tx.lz : 0.0;
+    const double lzy = (HAS_Y && oky) ? ty.lz : 0.0;
     const int tok = XMODE == kNoToken ? -1 : tx.tok;
     const bool tok_ok = tok >= 0 && tok < V;
     float lq = -INFINITY, la = -INFINITY;
@@ -896,67 +1070,29 @@ __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch
 
 // The per-row work once the row's chunk table tab[0..nch) is complete (block):
 // warps 0, 1 and 2 take the three tasks at once, warp 0 then writes the record.
-template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool KL = false>
+template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool KL = false, int S>
 __device__ void row_tail(const Problem<T>& P, int r, const float4* tab, RowShared& sh,
-                         uint4* klbuf = nullptr) {
+                         Ring<S>* rg) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0 || (HAS_Y && (warp == 1 || (ARGMAX && warp == 2)))) {
-        const RowTask t = row_task<T, VEC, XMODE>(P, r, tab, warp, lane);
+        const RowTask t = row_task<T, VEC, HAS_Y, XMODE>(P, r, tab, warp, lane, warp_chunks(rg));
         if (lane == 0) sh.t[warp] = t;
     } else if (KL && HAS_Y && warp == 3) {
         // VSD (KL): the top-K term on the fourth warp (an invalid row's term
         // is cleared by row_finish)
-        kl_select<T, VEC>(P, r, tab, P.nch, klbuf, 2, true, lane);
+        kl_select<T, VEC>(P, r, tab, P.nch, warp_chunks(rg), true, lane);
     }
     __syncthreads();
     if (warp == 0) {
         RowTask ty = sh.t[1];
-        if (!HAS_Y) ty = RowTask{0.f, TableSum{0, 0, 0.0}, -1};
+        if (!HAS_Y) ty = RowTask{0.f, TableSum{0, 0, 0.0}, -1, 0.f, 0.f, 0.0};
         const int ref = (HAS_Y && ARGMAX) ? sh.t[2].tok : -1;
-        const T* x = P.draft + (int64_t)r * P.V;
-        const T* y = HAS_Y ? P.target + (int64_t)r * P.V : nullptr;
         row_finish<T, HAS_Y, XMODE, ARGMAX>(P, r, sh.t[0], ty, ref, lane,
-                                            [&](int, int v, float& xv, float& yv) {
-                                                xv = elem_value(x, v);
-                                                yv = HAS_Y ? elem_value(y, v) : 0.f;
+                                            [&](int w, int, float& xv, float& yv) {
+                                                xv = sh.t[w].xv;
+                                                yv = sh.t[w].yv;
                                             });
     }
-}
-
-// Chunk ch of a row into a shared-memory buffer with cp.async (warp; rows
-// 16-byte aligned).  Vectors at or beyond V are not read.
-template <typename T>
-__device__ __forceinline__ void chunk_async(uint4* buf, const T* row, int64_t V, int ch,
-                                            int lane) {
-    constexpr int PV = Traits<T>::kPerVec;
-    const int64_t base = (int64_t)ch * chunk_elems<T>() + lane * PV;
-#pragma unroll
-    for (int k = 0; k < kLoads; ++k) {
-        const int64_t v0 = base + (int64_t)k * 32 * PV;
-        cp_async16(buf + k * 32 + lane, row + (v0 < V ? v0 : 0), v0 < V);
-    }
-}
-// The chunk in registers as load_chunk gives it (positions at or beyond V
-// read as -inf).
-template <typename T>
-__device__ __forceinline__ void chunk_from_smem(const uint4* buf, int64_t V, int ch, int lane,
-                                                uint4 (&b)[kLoads]) {
-    constexpr int PV = Traits<T>::kPerVec;
-    const int64_t base = (int64_t)ch * chunk_elems<T>() + lane * PV;
-#pragma unroll
-    for (int k = 0; k < kLoads; ++k)
-        b[k] = base + (int64_t)k * 32 * PV < V
-                   ? buf[k * 32 + lane]
-                   : make_uint4(Traits<T>::kNegInf, Traits<T>::kNegInf, Traits<T>::kNegInf,
-                                Traits<T>::kNegInf);
-}
-// Logit v of a buffer holding chunk ch.
-__device__ __forceinline__ float smem_elem(const uint4* buf, int ch, int v, const float*) {
-    return reinterpret_cast<const float*>(buf)[v - ch * chunk_elems<float>()];
-}
-__device__ __forceinline__ float smem_elem(const uint4* buf, int ch, int v, const __nv_bfloat16*) {
-    return __bfloat162float(
-        reinterpret_cast<const __nv_bfloat16*>(buf)[v - ch * chunk_elems<__nv_bfloat16>()]);
 }
 
 // --------------------------------------------------------------- VSD (KL)
@@ -968,15 +1104,16 @@ __device__ __forceinline__ float smem_elem(const uint4* buf, int ch, int v, cons
 //
 // Only a chunk whose target maximum reaches the Kt-th largest chunk maximum
 // can hold a selected token (Kt chunk maxima are that large, so the Kt-th
-// largest logit is too).  The warp reads those chunks of both rows in
-// increasing order, skipping a chunk whose maximum cannot beat the current
-// Kt-th entry, and keeps the running list sorted by (logit desc, index asc)
-// in lanes 0 .. Kt-1.  buf stages npair chunk pairs in shared memory (null:
-// loads into registers, one pair at a time).  ok = false (an invalid row)
+// largest logit is too), and only a logit that reaches it is one.  The warp
+// reads those chunks of the target row in increasing order, two in flight,
+// skipping a chunk whose maximum cannot beat the current Kt-th entry, and
+// keeps the running list sorted by (logit desc, index asc) in lanes 0 .. Kt-1;
+// the tokens' draft logits are read at the end.  buf: two chunk buffers in
+// shared memory (null: loads into registers).  ok = false (an invalid row)
 // writes an empty term.
 template <typename T, bool VEC>
 __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch, uint4* buf,
-                          int npair, bool ok, int lane) {
+                          bool ok, int lane) {
     constexpr int PV = Traits<T>::kPerVec;
     constexpr int CE = chunk_elems<T>();
     constexpr unsigned FULL = 0xffffffffu;
@@ -1024,27 +1161,24 @@ __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch
         tch = bc;
         tk = bv;
     }
-    float lv = -INFINITY, lx = 0.f;  // lane i < Kt: entry i (target logit, draft logit, index)
+    float lv = -INFINITY;  // lane i < Kt: entry i (target logit, index)
     int li = 0x7fffffff;
     int cnt = 0;
     float thv = -INFINITY;
     int thi = 0x7fffffff;
-    auto insert = [&](float v, int idx, float xv) {
+    auto insert = [&](float v, int idx) {
         const bool above = lane < cnt && (lv > v || (lv == v && li < idx));
         const int pos = __popc(__ballot_sync(FULL, above));
         if (pos >= Kt) return;
         const float pv = __shfl_up_sync(FULL, lv, 1);
         const int pi = __shfl_up_sync(FULL, li, 1);
-        const float px = __shfl_up_sync(FULL, lx, 1);
         if (lane > pos) {
             lv = pv;
             li = pi;
-            lx = px;
         }
         if (lane == pos) {
             lv = v;
             li = idx;
-            lx = xv;
         }
         cnt = min(cnt + 1, Kt);
         if (cnt == Kt) {
@@ -1052,63 +1186,65 @@ __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch
             thi = __shfl_sync(FULL, li, Kt - 1);
         }
     };
-    auto scan_chunk = [&](int ch, const uint4 (&bx)[kLoads], const uint4 (&by)[kLoads]) {
+    // one vector per lane: most hold no logit that counts
+    auto scan_vec = [&](int v0, const uint4& vec) {
+        if (!__any_sync(FULL, v0 < V && vec_max<T>(vec) >= fmaxf(tk, thv))) return;
+        float f[PV];
+        unpack<T>(vec, f);
 #pragma unroll
-        for (int k = 0; k < kLoads; ++k) {
-            float fx[PV], fy[PV];
-            unpack<T>(bx[k], fx);
-            unpack<T>(by[k], fy);
-#pragma unroll
-            for (int e = 0; e < PV; ++e) {
-                const int idx = ch * CE + k * 32 * PV + lane * PV + e;
-                const bool c = idx < V && (cnt < Kt || fy[e] > thv || (fy[e] == thv && idx < thi));
-                for (unsigned m = __ballot_sync(FULL, c); m; m &= m - 1) {
-                    const int L = __ffs(m) - 1;
-                    insert(__shfl_sync(FULL, fy[e], L), __shfl_sync(FULL, idx, L),
-                           __shfl_sync(FULL, fx[e], L));
-                }
+        for (int e = 0; e < PV; ++e) {
+            const int idx = v0 + e;
+            const bool c = idx < V && f[e] >= tk &&
+                           (cnt < Kt || f[e] > thv || (f[e] == thv && idx < thi));
+            for (unsigned m = __ballot_sync(FULL, c); m; m &= m - 1) {
+                const int L = __ffs(m) - 1;
+                insert(__shfl_sync(FULL, f[e], L), __shfl_sync(FULL, idx, L));
             }
         }
     };
-    const int np = (VEC && buf) ? max(1, min(npair, 3)) : 1;
-    const uint64_t pol = policy_evict_normal();
-    int ch0 = 0;
-    for (;;) {
-        int cand[3] = {-1, -1, -1};
-        int nc = 0;
-        while (nc < np && ch0 < nch) {
-            const int ch = ch0 + lane;
-            const float mxc = ch < nch ? tab[ch].z : -INFINITY;
-            const bool want = ch < nch && mxc >= tk && (cnt < Kt || mxc > thv);
-            unsigned bal = __ballot_sync(FULL, want);
-            while (bal && nc < np) {
-                cand[nc++] = ch0 + __ffs(bal) - 1;
-                bal &= bal - 1;
-            }
-            ch0 = bal ? ch0 + __ffs(bal) - 1 : ch0 + 32;
+    // the next chunk at or after ch that may hold a selected token (nch: none)
+    auto next_chunk = [&](int ch) {
+        for (; ch < nch; ch += 32) {
+            const int cl = ch + lane;
+            const float mxc = cl < nch ? tab[cl].z : -INFINITY;
+            const unsigned bal =
+                __ballot_sync(FULL, cl < nch && mxc >= tk && (cnt < Kt || mxc > thv));
+            if (bal) return ch + __ffs(bal) - 1;
         }
-        if (nc == 0) break;
-        if (VEC && buf) {
-            for (int j = 0; j < nc; ++j) {
-                chunk_async<T>(buf + (2 * j) * kLoads * 32, x, V, cand[j], lane);
-                chunk_async<T>(buf + (2 * j + 1) * kLoads * 32, y, V, cand[j], lane);
-            }
-            cp_async_wait_all();
+        return nch;
+    };
+    const uint64_t pol = policy_evict_normal();
+    int ch = next_chunk(0);
+    if (VEC && buf) {
+        int b = 0, nx = nch;
+        __syncwarp();
+        if (ch < nch) chunk_async<T>(buf, y, V, ch, lane);
+        cp_async_commit();
+        while (ch < nch) {
+            nx = next_chunk(ch + 1);
+            if (nx < nch) chunk_async<T>(buf + (b ^ 1) * kLoads * 32, y, V, nx, lane);
+            cp_async_commit();
+            cp_async_wait_1();
             __syncwarp();
-            for (int j = 0; j < nc; ++j) {
-                uint4 bx[kLoads], by[kLoads];
-                chunk_from_smem<T>(buf + (2 * j) * kLoads * 32, V, cand[j], lane, bx);
-                chunk_from_smem<T>(buf + (2 * j + 1) * kLoads * 32, V, cand[j], lane, by);
-                scan_chunk(cand[j], bx, by);
-            }
+            const uint4* z = buf + b * kLoads * 32;
+#pragma unroll 1
+            for (int k = 0; k < kLoads; ++k)
+                scan_vec(ch * CE + k * 32 * PV + lane * PV, z[k * 32 + lane]);
             __syncwarp();
-        } else {
-            uint4 bx[kLoads], by[kLoads];
-            load_chunk<T, VEC>(x, V, cand[0], lane, pol, bx);
-            load_chunk<T, VEC>(y, V, cand[0], lane, pol, by);
-            scan_chunk(cand[0], bx, by);
+            ch = nx;
+            b ^= 1;
+        }
+    } else {
+        while (ch < nch) {
+            uint4 by[kLoads];
+            load_chunk<T, VEC>(y, V, ch, lane, pol, by);
+#pragma unroll
+            for (int k = 0; k < kLoads; ++k)
+                scan_vec(ch * CE + k * 32 * PV + lane * PV, by[k]);
+            ch = next_chunk(ch + 1);
         }
     }
+    const float lx = lane < Kt && li < V ? elem_value(x, li) : 0.f;
     // Eq. klv on the selected tokens (fp64; the list is sorted, lane 0 holds
     // the largest target logit)
     const bool mine = lane < Kt;
@@ -1156,9 +1292,9 @@ __device__ void row_tail_warp(const Problem<T>& P, int r, float4* tab, RescanBuf
     const float4* rtab = P.gtab + (int64_t)r * P.nch_ws;
     for (int ch = lane; ch < nch; ch += 32) tab[ch] = ld_cg(rtab + ch);
     __syncwarp();
-    RowTask tx{table_max(tab, nch, 0, lane), TableSum{0, 0, 0.0}, -1};
+    RowTask tx{table_max(tab, nch, 0, lane), TableSum{0, 0, 0.0}, -1, 0.f, 0.f, 0.0};
     tx.S = table_sum(tab, nch, 0, frame_of(tx.M), c, lane);
-    RowTask ty{table_max(tab, nch, 1, lane), TableSum{0, 0, 0.0}, -1};
+    RowTask ty{table_max(tab, nch, 1, lane), TableSum{0, 0, 0.0}, -1, 0.f, 0.f, 0.0};
     ty.S = table_sum(tab, nch, 1, frame_of(ty.M), c, lane);
     Located lx{-1, 0.f}, ly{-1, 0.f};
     const int ca = ty.M > -INFINITY ? table_first_max(tab, nch, ty.M) : -1;
@@ -1205,6 +1341,11 @@ __device__ void row_tail_warp(const Problem<T>& P, int r, float4* tab, RescanBuf
         ref = first_max_regs<T>(b, ca, ty.M);
         if (ref >= V) ref = -1;
     }
+    {  // the two logarithms at once, on lanes 0 and 1
+        const double lz = log(lane == 0 ? tx.S.Z : ty.S.Z);
+        tx.lz = __shfl_sync(0xffffffffu, lz, 0);
+        ty.lz = __shfl_sync(0xffffffffu, lz, 1);
+    }
     row_finish<T, true, kSampleToken, true>(P, r, tx, ty, ref, lane,
                                             [&](int w, int v, float& xv, float& yv) {
                                                 if (VEC) {
@@ -1217,7 +1358,7 @@ __device__ void row_tail_warp(const Problem<T>& P, int r, float4* tab, RescanBuf
                                             });
     if (KL) {  // VSD (KL): the row's top-K term, staged through the rescan buffers
         __syncwarp();
-        kl_select<T, VEC>(P, r, tab, nch, rb.c[0], 3,
+        kl_select<T, VEC>(P, r, tab, nch, rb.c[0],
                           row_ok(tx.M, tx.S.Z) && row_ok(ty.M, ty.S.Z), lane);
     }
 }
@@ -1225,16 +1366,19 @@ __device__ void row_tail_warp(const Problem<T>& P, int r, float4* tab, RescanBuf
 // Streams row r of the draft (and, with HAS_Y, of the target) once, then runs
 // row_tail.  XMODE: whether z~ is drawn from q with u_draft, read from
 // given_tokens, or absent (trees).  ARGMAX: locate the greedy reference token.
-template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX>
-__device__ void row_pass(const Problem<T>& P, int r, Ring* rg, float4* tab, RowShared& sh) {
+template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, int S>
+__device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, RowShared& sh) {
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
     const T* y = HAS_Y ? P.target + (int64_t)r * V : nullptr;
     // The draft row is read again by the gradient pass: ask L2 to keep it.
     stream_tables<T, VEC, HAS_Y>(rg, x, y, V, 0, P.nch, tab, P.ts.c, policy_evict_last(),
                                  policy_evict_first(), P.status);
+    // (a programmatic dependent: what was read so far is the call's input; the
+    // workspace is written from here on)
+    grid_wait();
     __syncthreads();
-    row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh);
+    row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh, rg);
 }
 
 // --------------------------------------------------------------- residual
@@ -1264,8 +1408,8 @@ __device__ __forceinline__ float residual_chunk(const uint4 (&bx)[kLoads], const
     return warp_sum(acc);
 }
 
-template <typename T, bool VEC>
-__device__ void stream_residual(Ring* rg, const T* x, const T* y, int64_t V, int ch0, int ch1,
+template <typename T, bool VEC, int S>
+__device__ void stream_residual(Ring<S>* rg, const T* x, const T* y, int64_t V, int ch0, int ch1,
                                 float4* tab, const MassRes& mr, int* status) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t pol = policy_evict_normal();
@@ -1303,8 +1447,8 @@ __device__ void stream_residual(Ring* rg, const T* x, const T* y, int64_t V, int
 
 // Residual draw norm(max(0, p - q)) at row r with uniform u (block).  Returns
 // -1 when the residual has no mass.
-template <typename T, bool VEC>
-__device__ int residual_draw(const Problem<T>& P, int r, const RowRec& rec, float u, Ring* rg,
+template <typename T, bool VEC, int S>
+__device__ int residual_draw(const Problem<T>& P, int r, const RowRec& rec, float u, Ring<S>* rg,
                              float4* tab, int* out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t V = P.V;
@@ -1321,7 +1465,7 @@ __device__ int residual_draw(const Problem<T>& P, int r, const RowRec& rec, floa
             const Located loc = table_locate(tab, P.nch, 0, 0.f, c, Rt, u, lane);
             if (loc.ch >= 0)
                 tok = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane,
-                                                      policy_evict_normal());
+                                                      policy_evict_normal(), warp_chunks(rg));
         }
         if (tok >= V) tok = -1;
         if (lane == 0) *out = tok;
@@ -1426,15 +1570,15 @@ __device__ void path_epilogue_warp(const Problem<T>& P, int path, int A, int res
                 tkr = rec.ref >= 0 ? (double)rec.la_ref : NEG;
             }
             // prefix sums over l (Eq. 2): log kappa of z~, z' and the reference
-            const double lk = ck + warp_incl_scan(tk, lane);
-            const double lkc = ckc + warp_incl_scan(tkc, lane);
-            double lkr = ckr + warp_incl_scan(tkr, lane);
+            const int nd = min(32, D - d0);
+            const double lk = ck + warp_incl_scan_n(tk, lane, nd);
+            const double lkc = ckc + warp_incl_scan_n(tkc, lane, nd);
+            double lkr = ckr + warp_incl_scan_n(tkr, lane, nd);
+            EA += warp_sum_n(act ? (double)expf((float)lk) : 0.0, nd);  // Eq. 11
+            ck = __shfl_sync(0xffffffffu, lk, nd - 1);
+            ckc = __shfl_sync(0xffffffffu, lkc, nd - 1);
+            ckr = __shfl_sync(0xffffffffu, lkr, nd - 1);
             if (P.ref_logkappa && act) lkr = (double)__ldg(P.ref_logkappa + (int64_t)b * D + d);
-            EA += warp_sum(act ? (double)expf((float)lk) : 0.0);  // Eq. 11
-            const int lastl = min(31, D - 1 - d0);
-            ck = __shfl_sync(0xffffffffu, lk, lastl);
-            ckc = __shfl_sync(0xffffffffu, lkc, lastl);
-            ckr = __shfl_sync(0xffffffffu, ckr + warp_incl_scan(tkr, lane), lastl);
             if (act) {
                 P.es.tok[r] = rec.tok;
                 P.es.corr[r] = zc;
@@ -1474,8 +1618,8 @@ __device__ void path_epilogue(const Problem<T>& P, int path, int A, int resid) {
 
 // The whole path (block): head, the residual draw at the first rejection (one
 // more streaming read of that row), epilogue.
-template <typename T, bool VEC>
-__device__ void path_pass(const Problem<T>& P, int path, Ring* rg, float4* tab, PathShared& sh) {
+template <typename T, bool VEC, int S>
+__device__ void path_pass(const Problem<T>& P, int path, Ring<S>* rg, float4* tab, PathShared& sh) {
     const int D = P.D;
     const int r0 = path * D;
     path_head<T>(P, path, sh);
@@ -1895,8 +2039,8 @@ __device__ void grad_pass_range(const Problem<T>& P, int r, int64_t e0, int64_t 
 // streaming warps of the fused kernel).  Same arithmetic as grad_pass_range.
 // KL: the row has top-K terms (VSD (KL)) in kl; without them the loop is the
 // plain one.
-template <typename T, bool VEC, typename G, bool KL = false>
-__device__ void stream_grad(Ring* rg, const Problem<T>& P, int r, int c0, int c1, G* grad,
+template <typename T, bool VEC, typename G, bool KL = false, int S>
+__device__ void stream_grad(Ring<S>* rg, const Problem<T>& P, int r, int c0, int c1, G* grad,
                             const KlRec* kl = nullptr) {
     constexpr int PV = Traits<T>::kPerVec;
     constexpr int CE = chunk_elems<T>();
@@ -2158,8 +2302,8 @@ __device__ void tree_nodes(const Problem<T>& P, int b, TreeShared& sh) {
 // Residual row of node u of tree b (block): stream the row's residual
 // max(0, p - q) (Sec. 3) and draw each rejected child's token with the
 // child's own uniform; if the residual has no mass, a draw from p instead.
-template <typename T, bool VEC>
-__device__ void tree_residual_row(const Problem<T>& P, int b, int u, Ring* rg, float4* tab,
+template <typename T, bool VEC, int S>
+__device__ void tree_residual_row(const Problem<T>& P, int b, int u, Ring<S>* rg, float4* tab,
                                   int* s_tok) {
     const int N = P.N;
     const int64_t V = P.V;
@@ -2190,7 +2334,8 @@ __device__ void tree_residual_row(const Problem<T>& P, int b, int u, Ring* rg, f
                     table_locate(tab, nch, 0, 0.f, c, Rt, __ldg(P.u_correct + n0 + n), lane);
                 int tok = -1;
                 if (loc.ch >= 0)
-                    tok = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane, pol);
+                    tok = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane, pol,
+                                                          warp_chunks(rg));
                 if (lane == 0) o.corr_tokens[n0 + n] = tok < V ? tok : -1;
             }
     }
@@ -2199,14 +2344,15 @@ __device__ void tree_residual_row(const Problem<T>& P, int b, int u, Ring* rg, f
         stream_tables<T, VEC, false>(rg, y, nullptr, V, 0, nch, tab, c, pol, pol, P.status);
         __syncthreads();
         const float M = table_max(tab, nch, 0, lane);
-        const TableSum S = table_sum(tab, nch, 0, frame_of(M), c, lane);
+        const TableSum Sp = table_sum(tab, nch, 0, frame_of(M), c, lane);
         int k = 0;
         for (int n = u + 1; n < N; ++n) {
             if (__ldg(par + n) != u || ld_cg(o.path_accept + n0 + n)) continue;
             if (k++ % kWarps != warp) continue;
-            const int tok = row_ok(M, S.Z)
-                                ? warp_sample<T, VEC>(y, nullptr, V, tab, nch, 0, M, S,
-                                                      __ldg(P.u_correct + n0 + n), c, lane, pol)
+            const int tok = row_ok(M, Sp.Z)
+                                ? warp_sample<T, VEC>(y, nullptr, V, tab, nch, 0, M, Sp,
+                                                      __ldg(P.u_correct + n0 + n), c, lane, pol,
+                                                      warp_chunks(rg))
                                 : -1;
             if (lane == 0) o.corr_tokens[n0 + n] = tok < V ? tok : -1;
         }

@@ -12,6 +12,13 @@
 // over jobs costs: there a row's chain (claim, tail, path, M-step, publication,
 // gradient claims) runs on one control warp per block while rows are short.
 // Same results bit for bit.
+//
+// What bounds a single wave of rows (R up to 8 per SM) is the chain of one
+// path: at 768 rows of V = 32000 the row streams 11 us, its tail takes 7, the
+// path's residual draw 11, its epilogue 3, the M-step 9, the counters in
+// between 2, the gradient 14 (69 us a call; 119 on the persistent kernel).
+// Those steps run once per block and are short of instructions as much as of
+// data, so loops in them are kept rolled.
 #pragma once
 
 #include "vsd_grid.cuh"
@@ -19,55 +26,54 @@
 
 namespace vsd {
 
-// Dynamic shared memory: [ring][chunk table]; the M-step's scratch reuses the
-// ring's data (vector rows) or follows the table.
+// Dynamic shared memory: [ring][chunk table]; the M-step's scratch takes the
+// ring's place (vector rows) or follows the table.
 inline size_t staged_smem_bytes(int nch, bool vec) {
-    return stream_smem_bytes(nch, vec) + (vec ? 0 : sizeof(WeightsShared));
+    return stream_smem_bytes<kRowStages, sizeof(WeightsShared)>(nch, vec) +
+           (vec ? 0 : sizeof(WeightsShared));
 }
 
 template <typename T, bool VEC, bool KL>
-__global__ void __launch_bounds__(kThreads) k_em_rows(Problem<T> P) {
+__global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ union {
         RowShared row;
         PathShared path;
     } sh;
     __shared__ int s_last;
-    static_assert(sizeof(WeightsShared) <= sizeof(Ring::data), "the M-step's scratch fits the ring");
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC, sizeof(WeightsShared)>(dsm, rg, tab, P.timeout_ns);
     grid_launch_next();
     const int r = blockIdx.x, D = P.D, K = P.K, nch = P.nch;
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
     const T* y = P.target + (int64_t)r * V;
-    bool both = true;
+    const bool given = VEC && P.xtab_given;  // the LM head wrote the draft's half of the table
     if constexpr (VEC) {
-        if (P.xtab_given) {  // the LM head wrote the draft's half of the table
-            const float4* rtab = P.gtab + (int64_t)r * P.nch_ws;
-            for (int ch = threadIdx.x; ch < nch; ch += kThreads)
-                reinterpret_cast<float2*>(tab + ch)[0] =
-                    __ldcg(reinterpret_cast<const float2*>(rtab + ch));
+        if (given)
             stream_target_tables<T>(rg, y, V, 0, nch, tab, P.ts.c, policy_evict_first(), P.status);
-            both = false;
-        }
     }
-    if (both)
+    if (!given)
         stream_tables<T, VEC, true>(rg, x, y, V, 0, nch, tab, P.ts.c,
                                     P.gnseg ? policy_evict_last() : policy_evict_first(),
                                     policy_evict_first(), P.status);
+    // the kernel before this one (the clearing of the counters, or the LM
+    // head) has ended; what was read so far is the call's input
+    grid_wait();
+    if (given) {
+        const float4* rtab = P.gtab + (int64_t)r * P.nch_ws;
+        for (int ch = threadIdx.x; ch < nch; ch += kThreads)
+            reinterpret_cast<float2*>(tab + ch)[0] =
+                __ldcg(reinterpret_cast<const float2*>(rtab + ch));
+    }
     __syncthreads();
     row_tail<T, VEC, true, kSampleToken, true, KL>(
-        P, r, tab, sh.row, VEC ? &rg->data[kWarps - 1][0][0][0] : nullptr);
+        P, r, tab, sh.row, rg);
     // the last of n blocks to arrive at a counter
     auto last_of = [&](int* cnt, int n) {
         __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            s_last = atomicAdd(cnt, 1) == n - 1;
-            if (s_last) __threadfence();
-        }
+        if (threadIdx.x == 0) s_last = atomic_add_acq_rel(cnt, 1) == n - 1;
         __syncthreads();
         return s_last != 0;
     };
@@ -84,7 +90,7 @@ __global__ void __launch_bounds__(kThreads) k_em_rows(Problem<T> P) {
     path_epilogue<T>(P, path, A, resid);
     const int prefix = path / K;
     if (!last_of(P.prefix_cnt + prefix, K)) return;
-    WeightsShared* ws = VEC ? reinterpret_cast<WeightsShared*>(rg->data)
+    WeightsShared* ws = VEC ? reinterpret_cast<WeightsShared*>(dsm)
                             : reinterpret_cast<WeightsShared*>(tab + nch);
     const EStepView E{P.es.tok, P.es.corr, P.es.lq_tok, P.es.lq_corr,
                       P.es.lk, P.es.lkc, P.es.lkr};

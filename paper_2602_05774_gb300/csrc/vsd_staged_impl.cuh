@@ -20,8 +20,7 @@ cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad,
                     : (kl ? k_em_rows<VSD_T, false, true> : k_em_rows<VSD_T, false, false>);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
-    rows<<<P.R, kThreads, smem, s>>>(P);
-    if ((e = cudaGetLastError()) || !grad) return e;
+    if ((e = launch_after(rows, P.R, kThreads, smem, s, P)) || !grad) return e;
     return grad_rows(P, vec, grad, grad_bf16, s);
 }
 

@@ -53,10 +53,10 @@ static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 // row (one thread per child: Eq. 1, each branch alone), and the row's chunk
 // table kept in global memory for the draws.
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(kThreads) k_tree_rows(Problem<T> P) {
+__global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
     grid_launch_next();
@@ -100,7 +100,7 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ int s_par[1024], s_path;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
     grid_launch_next();
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
                     table_locate(tab, P.nch, 0, 0.f, c, Rt, __ldg(P.u_correct + n), lane);
                 if (loc.ch < 0) return;
                 const int z = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane,
-                                                              pol);
+                                                              pol, warp_chunks(rg));
                 if (z < 0 || z >= V) return;
                 float lq, la;
                 token_logs(x, y, z, rec, invT, &lq, &la);
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     const TableSum Sy = table_sum(tab, P.nch, 1, frame_of(My), c, lane);
     each_child([&](int n) {
         const int z = warp_sample<T, VEC>(x, y, V, tab, P.nch, 1, My, Sy, __ldg(P.u_correct + n), c,
-                                          lane, pol);
+                                          lane, pol, warp_chunks(rg));
         if (z < 0 || z >= V) return;
         float lq, la;
         token_logs(x, y, z, rec, invT, &lq, &la);
@@ -730,7 +730,7 @@ __device__ __forceinline__ float seq_chunk(const uint4 (&bx)[kLoads], const uint
 
 // One read of row r: tab[ch].y = the chunk sums of its masses (block).
 template <typename T, bool VEC>
-__device__ void seq_stream(const Problem<T>& P, int r, Ring* rg, float4* tab, const SeqMass& sm) {
+__device__ void seq_stream(const Problem<T>& P, int r, Ring<kRowStages>* rg, float4* tab, const SeqMass& sm) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
@@ -758,11 +758,11 @@ __device__ void seq_stream(const Problem<T>& P, int r, Ring* rg, float4* tab, co
 // there is no mass).
 template <typename T, bool VEC>
 __device__ int seq_draw(const Problem<T>& P, int r, const float4* tab, const TableSum& S, float u,
-                        const SeqMass& sm, int lane) {
+                        const SeqMass& sm, int lane, uint4* buf) {
     const Located loc = table_locate(tab, P.nch, 0, 0.f, P.ts.c, S, u, lane);
     if (loc.ch < 0) return -1;
     return warp_rescan<T, VEC, true, true>(P.draft + (int64_t)r * P.V, P.target + (int64_t)r * P.V,
-                                           P.V, loc.ch, loc.tc, sm, lane, policy_evict_normal());
+                                           P.V, loc.ch, loc.tc, sm, lane, policy_evict_normal(), buf);
 }
 
 // The decision at node u = row r (block, after the row's pass): tries its
@@ -771,7 +771,7 @@ __device__ int seq_draw(const Problem<T>& P, int r, const float4* tab, const Tab
 // no children, -1 if all were rejected, with the correction token in
 // es.corr[r].
 template <typename T, bool VEC>
-__device__ void tree_seq_row(const Problem<T>& P, int r, Ring* rg, float4* tab, SeqCtl& ct,
+__device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, float4* tab, SeqCtl& ct,
                              const SeqKids& s) {
     const int N = P.N, b = r / N, u = r - b * N, n0 = b * N;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -860,7 +860,7 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring* rg, float4* tab, 
                 const TableSum Rt = table_sum(tab, P.nch, 0, 0.f, c, lane);
                 // (no mass left: p_i is kept, and the draw is from it)
                 const int tok = i < m - 1 ? -1
-                                : Rt.Z > 0.0 ? seq_draw<T, VEC>(P, r, tab, Rt, uc, sm, lane)
+                                : Rt.Z > 0.0 ? seq_draw<T, VEC>(P, r, tab, Rt, uc, sm, lane, warp_chunks(rg))
                                              : -2;
                 if (lane == 0) {
                     if (Rt.Z > 0.0 && Rt.Z < INFINITY) {
@@ -880,7 +880,8 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring* rg, float4* tab, 
                 if (warp == 0) {
                     const TableSum Pt = table_sum(tab, P.nch, 0, 0.f, c, lane);
                     const int tok =
-                        Pt.Z > 0.0 ? seq_draw<T, VEC>(P, r, tab, Pt, uc, keep, lane) : -1;
+                        Pt.Z > 0.0 ? seq_draw<T, VEC>(P, r, tab, Pt, uc, keep, lane,
+                                                         warp_chunks(rg)) : -1;
                     if (lane == 0) ct.out = tok;
                 }
             }
@@ -900,19 +901,21 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring* rg, float4* tab, 
 // V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
 // block per tree, in an fp64 recursion per element over the earlier siblings.
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(kThreads) k_tree_seq_rows(Problem<T> P) {
+__global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
     __shared__ SeqCtl ct;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
     const SeqKids kids = seq_kids(reinterpret_cast<unsigned char*>(tab + P.nch), P.N);
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
     int need = P.tout.row_stats != nullptr;
     for (int n = u + 1 + threadIdx.x; n < N && !need; n += kThreads)
         need = __ldg(P.parent + (int64_t)b * N + n) == u;
     if (!__syncthreads_or(need)) {
+        grid_wait();
         if (threadIdx.x == 0) P.tlist[r] = 0;
         return;
     }
@@ -937,10 +940,11 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared rsh;
-    Ring* rg;
+    Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
     TreeSeqShared& sh = *reinterpret_cast<TreeSeqShared*>(tab + P.nch);
+    grid_wait();
     const int N = P.N, b = blockIdx.x, n0 = b * N;
     const vsd_tree_outputs& o = P.tout;
     if (!tree_load<T>(P, b, sh.t)) {

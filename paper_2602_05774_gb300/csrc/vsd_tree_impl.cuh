@@ -52,16 +52,17 @@ __global__ void __launch_bounds__(kThreads) k_tree_fused(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
     __shared__ int s_t, s_last, s_tok, s_cnt, s_leaf;
-    Ring* rg;
+    Ring<kStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
     // The per-node pass runs between streams: on the vector path its shared
     // memory is the ring's data (no copy is in flight then), else it follows
     // the chunk table.
-    static_assert(sizeof(TreeShared) <= sizeof(Ring::data), "TreeShared fits the ring");
+    static_assert(sizeof(TreeShared) <= sizeof(Ring<kStages>::data), "TreeShared fits the ring");
     TreeShared* tsh = VEC ? reinterpret_cast<TreeShared*>(rg->data)
                           : reinterpret_cast<TreeShared*>(tab + P.nch);
     const int N = P.N;
+    grid_wait();
     if (threadIdx.x == 0) s_t = atomicAdd(P.ticket, 1);
     __syncthreads();
     const int t = s_t;
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_fused(Problem<T> P) {
 template <>
 cudaError_t Launch<VSD_T>::tree(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
     // one block per node row, then tail blocks for the last trees' residual rows
-    const size_t smem = stream_smem_bytes(P.nch, vec) + (vec ? 0 : sizeof(TreeShared));
+    const size_t smem = stream_smem_bytes<kStages>(P.nch, vec) + (vec ? 0 : sizeof(TreeShared));
     auto kern = vec ? k_tree_fused<VSD_T, true> : k_tree_fused<VSD_T, false>;
     cudaError_t e = prep(kern, smem);
     if (e) return e;
@@ -160,35 +161,31 @@ cudaError_t Launch<VSD_T>::tree(const Problem<VSD_T>& P, bool vec, cudaStream_t 
     const long long most = (long long)P.B * (P.N - 1);  // residual rows at most
     if (tail > most) tail = most;
     if (tail < 1) tail = 1;
-    kern<<<(unsigned)(P.R + tail), kThreads, smem, s>>>(P);
-    return cudaGetLastError();
+    return launch_after(kern, (unsigned)(P.R + tail), kThreads, smem, s, P);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::tree_seq(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec) + seq_smem_bytes(P.N);
+    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec) + seq_smem_bytes(P.N);
     auto rows = vec ? k_tree_seq_rows<VSD_T, true> : k_tree_seq_rows<VSD_T, false>;
     cudaError_t e = prep(rows, smem);
     if (e) return e;
-    rows<<<P.R, kThreads, smem, s>>>(P);
-    if ((e = cudaGetLastError())) return e;
-    const size_t sm2 = stream_smem_bytes(P.nch, vec) + sizeof(TreeSeqShared);
+    if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
+    const size_t sm2 = stream_smem_bytes<kRowStages>(P.nch, vec) + sizeof(TreeSeqShared);
     auto seq = vec ? k_tree_seq<VSD_T, true> : k_tree_seq<VSD_T, false>;
     if ((e = prep(seq, sm2))) return e;
-    seq<<<P.B, kThreads, sm2, s>>>(P);
-    return cudaGetLastError();
+    return launch_after(seq, P.B, kThreads, sm2, s, P);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::tree_em(const Problem<VSD_T>& P, bool vec,
                                    const vsd_tree_em_outputs& o, void* grad, bool grad_bf16,
                                    cudaStream_t s) {
-    const size_t smem = stream_smem_bytes(P.nch, vec);
+    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
     auto rows = vec ? k_tree_rows<VSD_T, true> : k_tree_rows<VSD_T, false>;
     cudaError_t e = prep(rows, smem);
     if (e) return e;
-    rows<<<P.R, kThreads, smem, s>>>(P);
-    if ((e = cudaGetLastError())) return e;
+    if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
     auto draws = vec ? k_tree_draws<VSD_T, true> : k_tree_draws<VSD_T, false>;
     if ((e = prep(draws, smem))) return e;
     if ((e = launch_after(draws, P.R, kThreads, smem, s, P))) return e;
