@@ -27,7 +27,7 @@ constexpr uint64_t kDefaultTimeoutNs = 2000000000ull;
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
-    size_t status, ticket, prefix_done, grad_head, resq_head, resq_tail, resq_avail;
+    size_t status, ticket, prefix_done, grad_head, resq_head, resq_tail;
     size_t path_cnt, prefix_cnt, ready, grad_cnt, row_seg_cnt, res_seg_cnt, resq_flag, zero_end;
     size_t rows, rstats, es_tok, es_corr, es_lq_tok, es_lq_corr, es_lk, es_lkc, es_lkr;
     size_t coef, wscr, path_A, resq, klr, gtab, tnode, tcoef, tg, tbad, bfac, total;
@@ -98,8 +98,7 @@ WsLayout ws_layout(const vsd_layout& L) {
     w.grad_head = 768;
     w.resq_head = 1024;
     w.resq_tail = 1280;
-    w.resq_avail = 1536;
-    o = 1792;
+    o = 1792;  // (1536: a line that is no longer used)
     w.path_cnt = o; o = align256(o + 4 * npath);
     w.prefix_cnt = o; o = align256(o + 4 * (size_t)L.B);
     w.ready = o; o = align256(o + 4 * (size_t)L.B);
@@ -253,20 +252,18 @@ Problem<T> make_problem(const void* draft, const void* target, const vsd_layout&
     P.row_seg_cnt = at<int>(ws, w.row_seg_cnt);
     P.res_seg_cnt = at<int>(ws, w.res_seg_cnt);
     P.path_A = at<int>(ws, w.path_A);
-    // the tree layout has no E-step view and no path lengths: their arrays
-    // hold its residual lists and its nodes' log alpha
+    // the tree layout has no E-step view: its arrays hold the rows' accepted
+    // children (sequential rule) and the nodes' log alpha
     P.tnode = L.parent ? at<TreeNodeRec>(ws, w.tnode) : nullptr;
     P.tcoef = L.parent ? at<TreeCoef>(ws, w.tcoef) : nullptr;
     P.tg = L.parent ? at<float>(ws, w.tg) : nullptr;
     P.tbad = L.parent ? at<int>(ws, w.tbad) : nullptr;
     P.tlist = at<int>(ws, w.es_tok);
-    P.tcount = at<int>(ws, w.path_A);
     P.tla = at<float>(ws, w.es_lq_tok);
     P.resq = at<int>(ws, w.resq);
     P.resq_flag = at<int>(ws, w.resq_flag);
     P.resq_head = at<int>(ws, w.resq_head);
     P.resq_tail = at<int>(ws, w.resq_tail);
-    P.resq_avail = at<int>(ws, w.resq_avail);
     return P;
 }
 

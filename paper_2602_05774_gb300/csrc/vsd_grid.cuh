@@ -19,37 +19,14 @@ __device__ __forceinline__ bool wait_flag(const int* flag, int* status, uint64_t
     }
 }
 
-// Residual queue: producers reserve slots (resq_tail), write the items,
-// release each slot's flag and then add the items to resq_avail.  A consumer
-// reserves one published item with one atomic on resq_avail (returned at once
-// if none was left) and takes the next slot with one atomic on resq_head, so
-// claims pipeline in L2 instead of queueing behind a compare-and-swap.  The
-// slot may belong to a producer that reserved it but has not released it yet
-// (it is running, past its reservation): a bounded wait on the flag.
-// Callers look at resq_avail first.  Returns the item, -1 if none was left,
-// -2 if the wait ran out (status bit set).
-__device__ __forceinline__ int take_residual(int* head, int* avail, const int* flags,
-                                             const int* items, int* status,
-                                             uint64_t timeout_ns) {
-    if (atomicSub(avail, 1) <= 0) {
-        atomicAdd(avail, 1);
-        return -1;
-    }
-    const int h = atomicAdd(head, 1);
-    if (!wait_flag(flags + h, status, timeout_ns)) {
-        atomicOr(status, VSD_STATUS_TIMEOUT);
-        return -2;
-    }
-    return ld_cg(items + h);
-}
-
-__device__ __forceinline__ void publish_residuals(int* tail, int* avail, int* flags, int* items,
-                                                  int first, int n, bool sem) {
+// Residual queue (persistent kernel): producers reserve slots, write the items
+// and release each slot's flag.
+__device__ __forceinline__ void publish_residuals(int* tail, int* flags, int* items, int first,
+                                                  int n) {
     const int base = atomicAdd(tail, n);
     for (int i = 0; i < n; ++i) items[base + i] = first + i;
     __threadfence();
     for (int i = 0; i < n; ++i) st_release(flags + base + i, 1);
-    if (sem) atomicAdd(avail, n);
 }
 
 // Static plus dynamic shared memory above 48 KB needs the kernel's opt-in

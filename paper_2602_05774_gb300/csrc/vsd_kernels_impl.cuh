@@ -285,8 +285,7 @@ __device__ void post_job(const Problem<T>& P, const EStepView& E, const Job& j, 
         if (A < D && !flags && !P.greedy) {
             if (lane == 0) {  // queue the residual row's segments
                 P.path_A[path] = A;
-                publish_residuals(P.resq_tail, P.resq_avail, P.resq_flag, P.resq, path * nseg,
-                                  nseg, false);
+                publish_residuals(P.resq_tail, P.resq_flag, P.resq, path * nseg, nseg);
             }
         } else {
             finish_path_warp<T>(P, E, path, A, -1, false, 0.f, 0.f, cs, lane);

@@ -18,8 +18,8 @@ template <typename T> struct Launch {
     static cudaError_t reference(const Problem<T>& P, bool vec, float* out, cudaStream_t s);
     // accepted lengths, residual draws, corrected paths, log-kappa (linear)
     static cudaError_t paths(const Problem<T>& P, bool vec, cudaStream_t s);
-    // tree verification in one persistent launch: node rows, acceptance scan,
-    // residual draws, deepest node, bonus
+    // tree verification, each branch alone: node rows; then per row the residual
+    // draws, per tree the nodes' outputs and the bonus
     static cudaError_t tree(const Problem<T>& P, bool vec, cudaStream_t s);
     // tree verification with the sequential sibling rule
     static cudaError_t tree_seq(const Problem<T>& P, bool vec, cudaStream_t s);

@@ -19,11 +19,8 @@
 //                the per-row gradient coefficients.
 //   grad_pass    one streaming read of a draft row and write of its gradient:
 //                grad[v] = g q(v) - c0 [v = t0] - c1 [v = t1].
-//   tree_nodes / tree_residual_row / tree_bonus   per draft tree: acceptance
-//                per node at its parent's row, the AND-scan along parent
-//                pointers, log kappa, the deepest node; the residual draws at
-//                each accepted parent of rejected nodes (one block per such
-//                row); the bonus token.
+//   tree_children   a draft-tree row's children: acceptance of each one's token
+//                at the row.
 #pragma once
 
 #include "vsd_common.cuh"
@@ -163,15 +160,12 @@ struct Problem {
     struct TreeCoef* tcoef;       // [R] each node's gradient terms at its parent's row
     float* tg;                    // [R] each row's dense gradient factor
     int* tbad;                    // [B] the tree failed its checks
-    int* tlist;                   // tree layout: [R] residual rows of each tree (its rows' slots)
-    int* tcount;                  // tree layout: [B] length of each tree's list
+    int* tlist;                   // tree layout: [R] sequential rule: each row's accepted child
     float* tla;                   // tree layout: [R] log alpha of each node's token
-    int* resq;                    // [B*K*nseg] residual segment items (path*nseg + seg);
-                                  // trees: [B*N] positions b*N + i in the residual list
+    int* resq;                    // [B*K*nseg] residual segment items (path*nseg + seg)
     int* resq_flag;               // item written
     int* resq_head;               // next item to take
     int* resq_tail;               // next free slot
-    int* resq_avail;              // trees: items published and not yet reserved (may dip below 0)
     // outputs (device, caller-owned; null = not written)
     vsd_linear_outputs out;
     vsd_tree_outputs tout;
@@ -880,7 +874,8 @@ __device__ __forceinline__ void token_logs(const T* x, const T* y, int v, const 
 }
 
 // --------------------------------------------------------------- row pass
-enum XMode { kNoToken = 0, kSampleToken = 1, kGivenToken = 2 };
+// kStats: no token and no draw from p either, the statistics (and the argmax).
+enum XMode { kNoToken = 0, kSampleToken = 1, kGivenToken = 2, kStats = 3 };
 
 // One of the row's three table-driven results (warp; lane 0 returns them all):
 // which = 0 the draft statistics and z~ (drawn from q with
@@ -908,7 +903,7 @@ __device__ __forceinline__ RowTask row_task(const Problem<T>& P, int r, const fl
     t.lz = 0.0;
     // (asked for early: its latency is hidden behind the table's)
     const float* up = which == 0 ? P.u_draft : P.u_correct;
-    const bool drawn = which == 0 ? XMODE == kSampleToken : which == 1;
+    const bool drawn = which == 0 ? XMODE == kSampleToken : which == 1 && XMODE != kStats;
     const float u = drawn && up ? __ldg(up + r) : 0.f;
     int given = -1;
     if (XMODE == kGivenToken && which == 0) {
@@ -997,7 +992,7 @@ __device__ __forceinline__ void row_finish(const Problem<T>& P, int r, const Row
     const bool ok = okx && oky;
     const double lzx = okx ? tx.lz : 0.0;
     const double lzy = (HAS_Y && oky) ? ty.lz : 0.0;
-    const int tok = XMODE == kNoToken ? -1 : tx.tok;
+    const int tok = XMODE == kNoToken || XMODE == kStats ? -1 : tx.tok;
     const bool tok_ok = tok >= 0 && tok < V;
     float lq = -INFINITY, la = -INFINITY;
     if (lane < 3) {
@@ -2156,15 +2151,6 @@ __device__ void grad_pass(const Problem<T>& P, int r, const float4* rstats, G* g
 }
 
 // --------------------------------------------------------------- tree pass
-struct TreeShared {
-    int bad, deepest, maxdepth;
-    unsigned char acc[1024], pacc[1024], hasrej[1024];
-    int par[1024];
-    int depth[1024];
-    float la[1024];
-    double lk[1024];
-};
-
 // The children of node u of tree b at row u (block, right after the row's
 // pass, while the row is still in L2): alpha, the accept bit (Eq. 1) and log
 // alpha of each child's token, for the per-node pass; and the row's
@@ -2196,181 +2182,6 @@ __device__ void tree_children(const Problem<T>& P, int b, int u) {
         o.accept[n0 + n] = acc ? 1 : 0;
         P.tla[n0 + n] = la;
     }
-}
-
-// Tree verification, one draft tree b of N nodes per block; rows of tree b
-// are b*N .. b*N + N - 1, row n is the distribution node n's children were
-// drafted from (App. E tree).  This pass:
-//   1. every node, in parallel: alpha and the accept bit of its token against
-//      its parent's row (Eq. 1);
-//   2. in node order (parents come first): the accepted-path bit and the
-//      depth; then log kappa level by level (each node adds its log alpha to
-//      its parent's); the deepest accepted node;
-//   3. the list of residual rows (accepted nodes with a rejected child) for
-//      tree_residual_row, in tlist[b*N ..], its length in tcount[b]; the first
-//      child of the deepest accepted node (or -1) in tlist[b*N + N - 1], a
-//      slot the list never reaches (node N - 1 has no children).
-template <typename T>
-__device__ void tree_nodes(const Problem<T>& P, int b, TreeShared& sh) {
-    const int N = P.N;
-    const int n0 = b * N;
-    const int32_t* par = P.parent + (int64_t)n0;
-    const vsd_tree_outputs& o = P.tout;
-    // parents into shared memory; a tree is valid if node 0 is the root and
-    // every other node's parent precedes it
-    int badl = 0;
-    for (int n = threadIdx.x; n < N; n += kThreads) {
-        const int pn = __ldg(par + n);
-        sh.par[n] = pn;
-        badl |= n == 0 ? pn != -1 : (pn < 0 || pn >= n);
-    }
-    const int bad = __syncthreads_or(badl);
-    if (bad) {
-        if (threadIdx.x == 0) atomicOr(P.status, VSD_STATUS_BAD_TREE);
-        for (int n = threadIdx.x; n < N; n += kThreads) {
-            o.alpha[n0 + n] = 0.f;
-            o.accept[n0 + n] = 0;
-            o.path_accept[n0 + n] = 0;
-            o.logkappa[n0 + n] = -INFINITY;
-            o.corr_tokens[n0 + n] = -1;
-        }
-        if (threadIdx.x == 0) {
-            o.deepest[b] = -1;
-            o.accept_len[b] = -1;
-            o.bonus[b] = -1;
-            P.tcount[b] = 0;
-        }
-        return;
-    }
-    // 1. per node: log alpha and the accept bit from the parents' row blocks
-    for (int n = threadIdx.x; n < N; n += kThreads) {
-        sh.la[n] = n > 0 ? ld_cg(P.tla + n0 + n) : 0.f;
-        sh.acc[n] = n > 0 ? ld_cg(o.accept + n0 + n) : 1;
-        sh.hasrej[n] = 0;
-    }
-    __syncthreads();
-    // 2. accepted-path bits, depths, the deepest accepted node
-    if (threadIdx.x == 0) {
-        sh.pacc[0] = 1;
-        sh.depth[0] = 0;
-        sh.lk[0] = 0.0;
-        int deepest = 0, maxd = 0;
-        for (int n = 1; n < N; ++n) {
-            const int pn = sh.par[n];
-            sh.pacc[n] = (unsigned char)(sh.acc[n] && sh.pacc[pn]);
-            sh.depth[n] = sh.depth[pn] + 1;
-            maxd = max(maxd, sh.depth[n]);
-            if (sh.pacc[n] && sh.depth[n] > sh.depth[deepest]) deepest = n;
-        }
-        sh.deepest = deepest;
-        sh.maxdepth = maxd;
-        int first = -1;
-        for (int n = deepest + 1; n < N && first < 0; ++n)
-            if (sh.par[n] == deepest) first = n;
-        P.tlist[n0 + N - 1] = first;
-        o.alpha[n0] = 1.f;
-        o.accept[n0] = 1;
-        o.path_accept[n0] = 1;
-        o.logkappa[n0] = 0.f;
-        o.corr_tokens[n0] = -1;
-        o.deepest[b] = deepest;
-        o.accept_len[b] = sh.depth[deepest];
-    }
-    __syncthreads();
-    for (int L = 1; L <= sh.maxdepth; ++L) {  // log kappa along each branch (Eq. 2)
-        for (int n = threadIdx.x; n < N; n += kThreads)
-            if (sh.depth[n] == L) sh.lk[n] = sh.lk[sh.par[n]] + (double)sh.la[n];
-        __syncthreads();
-    }
-    for (int n = 1 + threadIdx.x; n < N; n += kThreads) {
-        o.path_accept[n0 + n] = sh.pacc[n];
-        o.logkappa[n0 + n] = (float)sh.lk[n];
-        o.corr_tokens[n0 + n] = -1;
-        const int pn = sh.par[n];
-        if (sh.pacc[pn] && !sh.pacc[n]) sh.hasrej[pn] = 1;
-    }
-    __syncthreads();
-    // 3. the residual rows, in node order
-    if (threadIdx.x == 0) {
-        int k = 0;
-        for (int u = 0; u < N; ++u)
-            if (sh.pacc[u] && sh.hasrej[u]) P.tlist[n0 + k++] = u;
-        P.tcount[b] = k;
-    }
-}
-
-// Residual row of node u of tree b (block): stream the row's residual
-// max(0, p - q) (Sec. 3) and draw each rejected child's token with the
-// child's own uniform; if the residual has no mass, a draw from p instead.
-template <typename T, bool VEC, int S>
-__device__ void tree_residual_row(const Problem<T>& P, int b, int u, Ring<S>* rg, float4* tab,
-                                  int* s_tok) {
-    const int N = P.N;
-    const int64_t V = P.V;
-    const int n0 = b * N;
-    const int nch = P.nch;
-    const int32_t* par = P.parent + (int64_t)n0;
-    const vsd_tree_outputs& o = P.tout;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float c = P.ts.c;
-    const uint64_t pol = policy_evict_normal();
-    const int r = n0 + u;
-    const RowRec rec = ld_cg(P.rows + r);
-    if (rec.flags) return;
-    const T* x = P.draft + (int64_t)r * V;
-    const T* y = P.target + (int64_t)r * V;
-    const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
-    stream_residual<T, VEC>(rg, x, y, V, 0, nch, tab, mr, P.status);
-    __syncthreads();
-    {  // every warp computes the total; the rejected children are shared out
-        const TableSum Rt = table_sum(tab, nch, 0, 0.f, c, lane);
-        if (threadIdx.x == 0) *s_tok = Rt.Z > 0.0;
-        int k = 0;
-        if (Rt.Z > 0.0)
-            for (int n = u + 1; n < N; ++n) {
-                if (__ldg(par + n) != u || ld_cg(o.path_accept + n0 + n)) continue;
-                if (k++ % kWarps != warp) continue;
-                const Located loc =
-                    table_locate(tab, nch, 0, 0.f, c, Rt, __ldg(P.u_correct + n0 + n), lane);
-                int tok = -1;
-                if (loc.ch >= 0)
-                    tok = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane, pol,
-                                                          warp_chunks(rg));
-                if (lane == 0) o.corr_tokens[n0 + n] = tok < V ? tok : -1;
-            }
-    }
-    __syncthreads();
-    if (!*s_tok) {  // no residual mass: each rejected child draws from p
-        stream_tables<T, VEC, false>(rg, y, nullptr, V, 0, nch, tab, c, pol, pol, P.status);
-        __syncthreads();
-        const float M = table_max(tab, nch, 0, lane);
-        const TableSum Sp = table_sum(tab, nch, 0, frame_of(M), c, lane);
-        int k = 0;
-        for (int n = u + 1; n < N; ++n) {
-            if (__ldg(par + n) != u || ld_cg(o.path_accept + n0 + n)) continue;
-            if (k++ % kWarps != warp) continue;
-            const int tok = row_ok(M, Sp.Z)
-                                ? warp_sample<T, VEC>(y, nullptr, V, tab, nch, 0, M, Sp,
-                                                      __ldg(P.u_correct + n0 + n), c, lane, pol,
-                                                      warp_chunks(rg))
-                                : -1;
-            if (lane == 0) o.corr_tokens[n0 + n] = tok < V ? tok : -1;
-        }
-    }
-    __syncthreads();
-}
-
-// The bonus token of tree b: the residual (or p) draw of the deepest accepted
-// node's first child, or, at a leaf, the p-draw at its row (one thread).
-template <typename T>
-__device__ void tree_bonus(const Problem<T>& P, int b) {
-    const int N = P.N;
-    const int n0 = b * N;
-    const vsd_tree_outputs& o = P.tout;
-    const int best = ld_cg(o.deepest + b);
-    if (best < 0) return;  // invalid tree: already written
-    const int child = ld_cg(P.tlist + n0 + N - 1);
-    o.bonus[b] = child >= 0 ? ld_cg(o.corr_tokens + n0 + child) : ld_cg(P.rows + n0 + best).ps;
 }
 
 }  // namespace vsd

@@ -48,6 +48,197 @@ struct __align__(16) TreeCoef {
 };
 static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 
+// ------------------------------------------------------------ verification
+// Every branch alone (VSD_TREE_INDEPENDENT), two kernels:
+//   k_tree_verify_rows  one block per node row with children (any row for the
+//                       statistics output): the row's statistics, then each
+//                       child's test;
+//   k_tree_verify       one block per row, of which most leave at once: at a
+//                       row on an accepted path the rejected children's draws
+//                       (one more read of the row), at the deepest accepted
+//                       node the bonus token (a leaf's row is read here), at
+//                       the root the outputs of the tree's nodes.
+// No block waits for another.  The row reads bound the first kernel, a few
+// dependent steps of one row the second.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1)
+    k_tree_verify_rows(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ RowShared sh;
+    Ring<kRowStages>* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    grid_launch_next();
+    const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
+    int need = P.tout.row_stats != nullptr;
+    for (int n = u + 1 + threadIdx.x; n < N && !need; n += kThreads)
+        need = __ldg(P.parent + (int64_t)b * N + n) == u;
+    if (!__syncthreads_or(need)) {
+        grid_wait();
+        return;
+    }
+    row_pass<T, VEC, true, kStats, false>(P, r, rg, tab, sh);
+    __syncthreads();
+    tree_children<T>(P, b, u);
+}
+
+// Per node of the tree (dynamic shared memory, after the chunk table).
+struct TreeVerifyNodes {
+    double* lk;  // [N] log kappa
+    int* par;
+    int* depth;  // -1: not on an accepted path (every node's at the root's block)
+    float* la;
+    unsigned char* acc;
+};
+inline size_t tree_verify_smem_bytes(int N) { return (size_t)N * 21 + 16; }
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ RowShared sh;
+    __shared__ int s_path, s_best, s_maxd, s_any, s_first;
+    Ring<kRowStages>* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const vsd_tree_outputs& o = P.tout;
+    TreeVerifyNodes t;
+    t.lk = reinterpret_cast<double*>(tab + P.nch);
+    t.par = reinterpret_cast<int*>(t.lk + N);
+    t.depth = t.par + N;
+    t.la = reinterpret_cast<float*>(t.depth + N);
+    t.acc = reinterpret_cast<unsigned char*>(t.la + N);
+    int bad = 0;
+    for (int n = tid; n < N; n += kThreads) {
+        const int pn = __ldg(P.parent + n0 + n);
+        t.par[n] = pn;
+        bad |= n == 0 ? pn != -1 : (pn < 0 || pn >= n);
+    }
+    grid_wait();
+    if (__syncthreads_or(bad)) {
+        if (u) return;
+        for (int n = tid; n < N; n += kThreads) {
+            o.alpha[n0 + n] = 0.f;
+            o.accept[n0 + n] = 0;
+            o.path_accept[n0 + n] = 0;
+            o.logkappa[n0 + n] = -INFINITY;
+            o.corr_tokens[n0 + n] = -1;
+        }
+        if (tid == 0) {
+            atomicOr(P.status, VSD_STATUS_BAD_TREE);
+            o.deepest[b] = -1;
+            o.accept_len[b] = -1;
+            o.bonus[b] = -1;
+        }
+        return;
+    }
+    for (int n = tid; n < N; n += kThreads) {
+        t.acc[n] = n ? ld_cg(o.accept + n0 + n) : 1;
+        if (u == 0) t.la[n] = n ? ld_cg(P.tla + n0 + n) : 0.f;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int x = u;
+        while (x > 0 && t.acc[x]) x = t.par[x];
+        s_path = x == 0;
+        s_best = -1;
+        s_maxd = s_any = 0;
+        s_first = N;
+    }
+    __syncthreads();
+    if (!s_path) return;
+    // each node's depth (-1 below a rejection), the deepest accepted node
+    // (lowest index on ties), u's children
+    for (int n = tid; n < N; n += kThreads) {
+        int d = 0, ok = 1;
+        for (int x = n; x > 0; x = t.par[x]) {
+            ok &= t.acc[x];
+            ++d;
+        }
+        t.depth[n] = ok ? d : -1 - d;
+        if (ok) atomicMax(&s_best, (d << 11) | (2047 - n));
+        atomicMax(&s_maxd, d);
+        if (n && t.par[n] == u) {
+            atomicMin(&s_first, n);
+            if (!t.acc[n]) s_any = 1;
+        }
+    }
+    __syncthreads();
+    const int best = 2047 - (s_best & 2047);
+    if (u == 0) {  // the nodes' outputs; log kappa along each branch (Eq. 2)
+        auto depth_of = [&](int n) { return t.depth[n] >= 0 ? t.depth[n] : -1 - t.depth[n]; };
+        for (int l = 0; l <= s_maxd; ++l) {
+            for (int n = tid; n < N; n += kThreads)
+                if (depth_of(n) == l) t.lk[n] = n ? t.lk[t.par[n]] + (double)t.la[n] : 0.0;
+            __syncthreads();
+        }
+        for (int n = tid; n < N; n += kThreads) {
+            const bool pa = t.depth[n] >= 0;
+            o.path_accept[n0 + n] = pa;
+            o.logkappa[n0 + n] = (float)t.lk[n];
+            // (a rejected child of an accepted node: its parent's block draws)
+            if (pa || t.depth[t.par[n]] < 0) o.corr_tokens[n0 + n] = -1;
+        }
+        if (tid == 0) {
+            o.alpha[n0] = 1.f;
+            o.accept[n0] = 1;
+            o.deepest[b] = best;
+            o.accept_len[b] = t.depth[best];
+        }
+    }
+    const int64_t V = P.V;
+    if (s_any) {  // the rejected children's draws from norm(max(0, p - q))
+        const RowRec rec = ld_cg(P.rows + r);
+        const T* x = P.draft + (int64_t)r * V;
+        const T* y = P.target + (int64_t)r * V;
+        const float c = P.ts.c;
+        const uint64_t pol = policy_evict_normal();
+        const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
+        TableSum R{0, 0, 0.0}, Sp{0, 0, 0.0};
+        float M = 0.f;
+        if (!rec.flags) {
+            stream_residual<T, VEC>(rg, x, y, V, 0, P.nch, tab, mr, P.status);
+            __syncthreads();
+            R = table_sum(tab, P.nch, 0, 0.f, c, lane);
+            if (!(R.Z > 0.0)) {  // no residual mass: draws from p with the same uniforms
+                __syncthreads();
+                stream_tables<T, VEC, false>(rg, y, nullptr, V, 0, P.nch, tab, c, pol, pol,
+                                             P.status);
+                __syncthreads();
+                M = table_max(tab, P.nch, 0, lane);
+                Sp = table_sum(tab, P.nch, 0, frame_of(M), c, lane);
+            }
+        }
+        int k = 0;
+        for (int n = u + 1; n < N; ++n) {
+            if (t.par[n] != u || t.acc[n] || k++ % kWarps != warp) continue;
+            const float uc = __ldg(P.u_correct + n0 + n);
+            int tok = -1;
+            if (R.Z > 0.0) {
+                const Located loc = table_locate(tab, P.nch, 0, 0.f, c, R, uc, lane);
+                if (loc.ch >= 0)
+                    tok = warp_rescan<T, VEC, true, true>(x, y, V, loc.ch, loc.tc, mr, lane, pol,
+                                                          warp_chunks(rg));
+            } else if (row_ok(M, Sp.Z)) {
+                tok = warp_sample<T, VEC>(y, nullptr, V, tab, P.nch, 0, M, Sp, uc, c, lane, pol,
+                                          warp_chunks(rg));
+            }
+            if (lane == 0) o.corr_tokens[n0 + n] = tok < V ? tok : -1;
+        }
+        __syncthreads();
+    }
+    if (u == best) {  // the token after the accepted path
+        const bool leaf = s_first == N;
+        if (leaf) {
+            row_pass<T, VEC, true, kNoToken, false>(P, r, rg, tab, sh);
+            __syncthreads();
+        }
+        if (tid == 0)
+            o.bonus[b] = leaf ? ld_cg(P.rows + r).ps : ld_cg(o.corr_tokens + n0 + s_first);
+    }
+}
+
 // ------------------------------------------------------------ k_tree_rows
 // One block per node row: the row pass, then each child's token tested at the
 // row (one thread per child: Eq. 1, each branch alone), and the row's chunk
@@ -62,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_rows(Pr
     grid_launch_next();
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
     const int64_t V = P.V;
-    row_pass<T, VEC, true, kNoToken, true>(P, r, rg, tab, sh);
+    row_pass<T, VEC, true, kStats, true>(P, r, rg, tab, sh);
     __syncthreads();
     const RowRec rec = ld_cg(P.rows + r);
     int kids = 0;
@@ -895,7 +1086,7 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, f
 }
 
 // One block per node row (a leaf's row only for the statistics output; the
-// row the bonus token needs is then read by k_tree_seq).
+// draw a leaf's bonus token needs is k_tree_seq's).
 // What bounds it: the row reads and row tails (3840 rows of 2 x 64 KB), and
 // the reads after a rejection, which come from L2.  64 trees of 60 nodes,
 // V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
@@ -919,7 +1110,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_row
         if (threadIdx.x == 0) P.tlist[r] = 0;
         return;
     }
-    row_pass<T, VEC, true, kNoToken, false>(P, r, rg, tab, sh);
+    row_pass<T, VEC, true, kStats, false>(P, r, rg, tab, sh);
     __syncthreads();
     if (threadIdx.x == 0 && P.tout.row_stats)
         reinterpret_cast<float4*>(P.tout.row_stats)[r] = ld_cg(P.rstats + r);
@@ -1005,7 +1196,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     }
     __syncthreads();
     const bool leaf = sh.lastkid == 0;
-    if (leaf && !P.tout.row_stats) {  // the leaf's row, for the bonus token
+    if (leaf) {  // the leaf's row, for the bonus token
         row_pass<T, VEC, true, kNoToken, false>(P, n0 + best, rg, tab, rsh);
         __syncthreads();
     }
