@@ -17,7 +17,7 @@
 //
 // Measured at R = 4096, H = 4096, V = 32000 (1.07 TFLOP a product, one launch
 // alone): logits 572 us (655 with one CTA per 128 x 256 tile), d_hidden 547 and
-// d_weight 572 from a gradient in memory plus 70 to write it (962 and 1205 with
+// d_weight 555 from a gradient in memory plus 70 to write it (962 and 1205 with
 // the gradient made on chip for every tile): 1.87 to 1.96 PFLOP/s, cuBLAS's
 // measured rate.  The tensor pipe bounds it.
 //
@@ -54,8 +54,12 @@ struct Bars {
     int err;
     uint32_t peer_it;         // CTA 0: stages the other CTA's producer issued
 };
-constexpr size_t kSmemBytes = 1024 /* alignment */ + kStages * kStageBytes + sizeof(Bars);
-static_assert(kSmemBytes <= 232448, "227 KB of shared memory per block");
+// [alignment][stages][the epilogue's staging][barriers]
+template <class Epi> constexpr size_t smem_bytes() {
+    static_assert(1024 + kStages * kStageBytes + Epi::kStaging + sizeof(Bars) <= 232448,
+                  "227 KB of shared memory per block");
+    return 1024 + kStages * kStageBytes + Epi::kStaging + sizeof(Bars);
+}
 
 // ---------------------------------------------------------------- PTX wrappers
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -215,29 +219,57 @@ struct SplitOrder {
 
 // ---------------------------------------------------------------- epilogues
 // fp32 output, row-major [M][N] (N a multiple of 4); a part of a tile is added.
+// Each warp stages 32 rows x 32 columns in shared memory (128-byte swizzle, two
+// buffers) and stores them by TMA: a thread's own stores, 16 bytes of a row
+// each, kept the epilogue at about 9 us a tile, longer than the main loop of a
+// small K (d_weight at R = 672, H = 2888, V = 32000: 193 us with them, 114 now).
 struct StoreF32 {
     using Order = SplitOrder;
-    float* out;
+    static constexpr int kStaging = 4 * 2 * 4096;
+    CUtensorMap map;  // boxes of 32 x 32
     int M, N;
-    struct State {};
+    struct State {
+        unsigned char* buf;  // this warp's two buffers
+        int n;               // stores issued
+    };
+    __device__ void init(State& st, unsigned char* staging, int q) const {
+        st.buf = staging + q * 2 * 4096;
+        st.n = 0;
+    }
     __device__ void begin(State&, const Work&) const {}
-    __device__ void columns(State&, const Work& w, int row, int col, uint32_t (&r)[32]) const {
-        if (row >= M || col >= N) return;
-        float* o = out + (size_t)row * N + col;
+    // (row: this lane's; the warp's first row is row - lane)
+    __device__ void columns(State& st, const Work& w, int row, int col, uint32_t (&r)[32]) const {
+        const int lane = threadIdx.x & 31, row0 = row - lane;
+        if (row0 >= M || col >= N) return;
+        unsigned char* b = st.buf + (st.n & 1) * 4096;
+        if (lane == 0)  // the store before the last has read its buffer
+            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        __syncwarp();
 #pragma unroll
         for (int v = 0; v < 8; ++v)
-            if (col + 4 * v < N) {
-                if (w.part)
-                    atomicAdd(reinterpret_cast<float4*>(o + 4 * v),
-                              make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]),
-                                          __uint_as_float(r[4 * v + 2]),
-                                          __uint_as_float(r[4 * v + 3])));
-                else
-                    *reinterpret_cast<uint4*>(o + 4 * v) =
-                        make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
-            }
+            *reinterpret_cast<uint4*>(b + lane * 128 + ((v ^ (lane & 7)) << 4)) =
+                make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+        vsd::fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+            const uint64_t m = reinterpret_cast<uint64_t>(&map);
+            if (w.part)
+                asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group"
+                             " [%0, {%1, %2}], [%3];"
+                             :: "l"(m), "r"(col), "r"(row0), "r"(smem_u32(b)) : "memory");
+            else
+                asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group"
+                             " [%0, {%1, %2}], [%3];"
+                             :: "l"(m), "r"(col), "r"(row0), "r"(smem_u32(b)) : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+        ++st.n;
     }
     __device__ void end(State&, const Work&, int) const {}
+    __device__ void finish(State&) const {  // the buffers outlive the stores
+        if ((threadIdx.x & 31) == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        __syncwarp();
+    }
 };
 
 // bf16 output, row-major [M][N] (N a multiple of 8), and, with tab, each row's
@@ -245,6 +277,7 @@ struct StoreF32 {
 // the hot path): tab[row * stride + chunk].xy = (max, sum 2^{(x - max) c}).
 struct StoreLogits {
     using Order = ChunkOrder;
+    static constexpr int kStaging = 0;
     __nv_bfloat16* out;
     int M, N;
     float4* tab;  // null: none
@@ -253,6 +286,8 @@ struct StoreLogits {
     struct State {
         float m, s;
     };
+    __device__ void init(State&, unsigned char*, int) const {}
+    __device__ void finish(State&) const {}
     __device__ void begin(State& st, const Work& w) const {
         if (w.first) {
             st.m = -INFINITY;
@@ -285,7 +320,7 @@ struct StoreLogits {
             if (col + i < N) gm = fmaxf(gm, f[i]);
         const float nm = fmaxf(st.m, gm);
         if (nm > -INFINITY) {
-            float acc = st.s * vsd::ex2((st.m - nm) * c);
+            float acc = __fmul_rn(st.s, vsd::ex2((st.m - nm) * c));  // (no contraction)
 #pragma unroll
             for (int i = 0; i < 32; ++i)
                 if (col + i < N) acc += vsd::ex2((f[i] - nm) * c);
@@ -307,11 +342,13 @@ struct StoreLogits {
 template <bool AMN, bool BMN, class Epi>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_gemm2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-            int M, int N, int K, const Epi epi, int* status, uint64_t timeout_ns) {
+            int M, int N, int K, const __grid_constant__ Epi epi, int* status,
+            uint64_t timeout_ns) {
     extern __shared__ unsigned char dsm_raw[];
     // (the same offsets in both CTAs: the dynamic shared memory starts alike)
     unsigned char* dsm = dsm_raw + ((1024u - (smem_u32(dsm_raw) & 1023u)) & 1023u);
-    Bars* sb = reinterpret_cast<Bars*>(dsm + kStages * kStageBytes);
+    unsigned char* staging = dsm + kStages * kStageBytes;
+    Bars* sb = reinterpret_cast<Bars*>(staging + Epi::kStaging);
     constexpr uint32_t kIdesc =
         idesc_bf16(2 * BM, BN) | (AMN ? (1u << 15) : 0u) | (BMN ? (1u << 16) : 0u);
     constexpr int kBox = 64 * BK * 2;  // one MN-major box: 8 KB
@@ -436,6 +473,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         int lt = 0;
         typename Epi::Order order(M, N, K, c, nc);
         typename Epi::State st;
+        epi.init(st, staging, q);
         Work w;
         for (; order.next(w); ++lt) {
             const int buf = lt & 1;
@@ -456,6 +494,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             __syncwarp();
             if (lane == 0) arrive_cluster(map_rank(&sb->acc_empty[buf], 0));
         }
+        epi.finish(st);
     }
     tc_fence_before();
     __syncthreads();

@@ -59,6 +59,18 @@ bool make_map_box(CUtensorMap* m, const void* base, int rows, int cols, int box_
            CUDA_SUCCESS;
 }
 
+bool make_map_store(CUtensorMap* m, float* base, int rows, int cols, int box) {
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
+    const cuuint32_t boxes[2] = {(cuuint32_t)box, (cuuint32_t)box};
+    const cuuint32_t estr[2] = {1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, boxes, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace vsd_lm
 
 namespace vsd {
@@ -80,7 +92,7 @@ cudaError_t lmhead_gemm(const void* hidden, const void* weight, int M, int N, in
         !vsd_lm::make_map_box(&tb, weight, N, K, vsd_g2::BK, vsd_g2::BH, 128))
         return cudaErrorInvalidValue;
     auto kern = vsd_g2::k_gemm2<false, false, vsd_g2::StoreLogits>;
-    cudaError_t e = ensure_dyn_smem((const void*)kern, vsd_g2::kSmemBytes);
+    cudaError_t e = ensure_dyn_smem((const void*)kern, vsd_g2::smem_bytes<vsd_g2::StoreLogits>());
     if (e != cudaSuccess) return e;
     const long long nunits = (long long)((M + 2 * vsd_g2::BM - 1) / (2 * vsd_g2::BM)) *
                              ((N + 1023) / 1024);
@@ -88,7 +100,7 @@ cudaError_t lmhead_gemm(const void* hidden, const void* weight, int M, int N, in
     const int grid = 2 * (int)(nunits < pairs ? nunits : pairs);
     const vsd_g2::StoreLogits epi{static_cast<__nv_bfloat16*>(logits), M, N, chunk_tab,
                                   chunk_stride, chunk_c};
-    kern<<<grid, vsd_g2::kThreads, vsd_g2::kSmemBytes, s>>>(ta, tb, M, N, K, epi, status,
+    kern<<<grid, vsd_g2::kThreads, vsd_g2::smem_bytes<vsd_g2::StoreLogits>(), s>>>(ta, tb, M, N, K, epi, status,
                                                             timeout_ns);
     return cudaGetLastError();
 }

@@ -644,9 +644,13 @@ cudaError_t gemm_f32(const void* a, const void* b, int M, int N, int K, float* o
     const bool ok = (AMN ? make_map_box(&ta, a, K, M, 64, BK, 128)
                          : make_map_box(&ta, a, M, K, BK, BM, 128)) &&
                     make_map_box(&tb, b, K, N, 64, BK, 128);
-    if (!ok) return cudaErrorInvalidValue;
+    StoreF32 epi;
+    epi.M = M;
+    epi.N = N;
+    if (!ok || !make_map_store(&epi.map, out, M, N, 32)) return cudaErrorInvalidValue;
     auto kern = k_gemm2<AMN, true, StoreF32>;
-    cudaError_t e = ensure_dyn_smem((const void*)kern, kSmemBytes);
+    const size_t smem = vsd_g2::smem_bytes<StoreF32>();
+    cudaError_t e = ensure_dyn_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     const int ntn = (N + BN - 1) / BN, pairs = device_sm_count() / 2;
     const long long tiles = (long long)((M + 2 * BM - 1) / (2 * BM)) * ntn;
@@ -660,8 +664,7 @@ cudaError_t gemm_f32(const void* a, const void* b, int M, int N, int K, float* o
     }
     const long long items = whole + 2 * (tiles - whole);
     const int grid = 2 * (int)(items < pairs ? items : pairs);
-    kern<<<grid, vsd_g2::kThreads, kSmemBytes, s>>>(ta, tb, M, N, K, StoreF32{out, M, N}, status,
-                                                    timeout_ns);
+    kern<<<grid, vsd_g2::kThreads, smem, s>>>(ta, tb, M, N, K, epi, status, timeout_ns);
     return cudaGetLastError();
 }
 

@@ -157,5 +157,9 @@ __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo, uint32_t hi) {
 // as zero (vsd_lmhead.cu).
 bool make_map_box(CUtensorMap* m, const void* base, int rows, int cols, int box_cols,
                   int box_rows, int swizzle_bytes);
+// Tensor map of a row-major float matrix [rows][cols] (cols a multiple of 4)
+// stored in box x box tiles, 128-byte swizzle in shared memory (box = 32);
+// elements beyond the matrix are not written (vsd_lmhead.cu).
+bool make_map_store(CUtensorMap* m, float* base, int rows, int cols, int box);
 
 }  // namespace vsd_lm
