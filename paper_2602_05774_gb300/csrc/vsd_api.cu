@@ -389,8 +389,7 @@ vsd_status verify_impl(const void* draft, const void* target, vsd_layout L, floa
                                                    : Launch<T>::tree(P, vec, s);
     } else {
         P.out = *out;
-        if (e == cudaSuccess) e = Launch<T>::rows_verify(P, vec, s);
-        if (e == cudaSuccess) e = Launch<T>::paths(P, vec, s);
+        if (e == cudaSuccess) e = Launch<T>::verify(P, vec, s);
     }
     return from_cuda(e);
 }

@@ -28,17 +28,6 @@ __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
     }
 }
 
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(kThreads) k_rows_verify(Problem<T> P) {
-    extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ RowShared sh;
-    Ring<kRowStages>* rg;
-    float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
-    grid_launch_next();
-    row_pass<T, VEC, true, kGivenToken, true>(P, blockIdx.x, rg, tab, sh);
-}
-
 // Rows along supplied greedy reference paths (Algorithm 2's z-bar): per row
 // the target's argmax and log min(1, p/q) there (row_pass with the argmax).
 template <typename T, bool VEC>
@@ -70,17 +59,6 @@ __global__ void k_ref_scan(Problem<T> P, float* out) {
         if (d < P.D) out[(int64_t)b * P.D + d] = (float)inc;
         carry = __shfl_sync(0xffffffffu, inc, 31);
     }
-}
-
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(kThreads) k_paths(Problem<T> P) {
-    extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ PathShared sh;
-    Ring<kRowStages>* rg;
-    float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
-    grid_wait();
-    path_pass<T, VEC>(P, blockIdx.x, rg, tab, sh);
 }
 
 template <typename T>
@@ -468,15 +446,6 @@ cudaError_t Launch<VSD_T>::sample(const Problem<VSD_T>& P, bool vec, cudaStream_
 }
 
 template <>
-cudaError_t Launch<VSD_T>::rows_verify(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
-    auto kern = vec ? k_rows_verify<VSD_T, true> : k_rows_verify<VSD_T, false>;
-    cudaError_t e = prep(kern, smem);
-    if (e) return e;
-    return launch_after(kern, P.R, kThreads, smem, s, P);
-}
-
-template <>
 cudaError_t Launch<VSD_T>::reference(const Problem<VSD_T>& P, bool vec, float* out,
                                      cudaStream_t s) {
     const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
@@ -485,21 +454,6 @@ cudaError_t Launch<VSD_T>::reference(const Problem<VSD_T>& P, bool vec, float* o
     if (e) return e;
     if ((e = launch_after(kern, P.R, kThreads, smem, s, P))) return e;
     return launch_after(k_ref_scan<VSD_T>, P.B, 32, 0, s, P, out);
-}
-
-template <>
-cudaError_t Launch<VSD_T>::paths(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
-    const int npaths = P.B * P.K;
-    if (vec) {
-        cudaError_t e = prep(k_paths<VSD_T, true>, smem);
-        if (e) return e;
-        return launch_after(k_paths<VSD_T, true>, npaths, kThreads, smem, s, P);
-    } else {
-        cudaError_t e = prep(k_paths<VSD_T, false>, smem);
-        if (e) return e;
-        return launch_after(k_paths<VSD_T, false>, npaths, kThreads, smem, s, P);
-    }
 }
 
 template <>

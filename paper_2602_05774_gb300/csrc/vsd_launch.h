@@ -12,12 +12,11 @@ namespace vsd {
 template <typename T> struct Launch {
     // z~ ~ q per row, tokens/logq/row_stats written from the row records
     static cudaError_t sample(const Problem<T>& P, bool vec, cudaStream_t s);
-    // row statistics of draft+target with given tokens (linear paths)
-    static cudaError_t rows_verify(const Problem<T>& P, bool vec, cudaStream_t s);
+    // verification of given tokens (linear paths): rows, accepted lengths, residual
+    // draws, corrected paths, log-kappa
+    static cudaError_t verify(const Problem<T>& P, bool vec, cudaStream_t s);
     // log kappa of supplied greedy reference paths: [B][D] rows -> out [B][D]
     static cudaError_t reference(const Problem<T>& P, bool vec, float* out, cudaStream_t s);
-    // accepted lengths, residual draws, corrected paths, log-kappa (linear)
-    static cudaError_t paths(const Problem<T>& P, bool vec, cudaStream_t s);
     // tree verification, each branch alone: node rows; then per row the residual
     // draws, per tree the nodes' outputs and the bonus
     static cudaError_t tree(const Problem<T>& P, bool vec, cudaStream_t s);

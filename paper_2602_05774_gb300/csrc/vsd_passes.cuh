@@ -9,7 +9,8 @@
 //                from p (used after the first rejection), the target argmax
 //                (greedy reference of Algorithm 2), and the log-probabilities
 //                of those tokens (Eq. 1 needs p and q at a token).
-//   path_pass    per proposal path: acceptance (Eq. 1), accepted length,
+//   path_head / residual_draw / path_epilogue
+//                per proposal path: acceptance (Eq. 1), accepted length,
 //                survival/expected length (Eqs. 9-11), the residual draw
 //                norm(max(0, p - q)) at the first rejection (Sec. 3; one more
 //                streaming read of that row), the corrected path z', and the
@@ -1608,23 +1609,6 @@ __device__ void path_epilogue_warp(const Problem<T>& P, int path, int A, int res
 template <typename T>
 __device__ void path_epilogue(const Problem<T>& P, int path, int A, int resid) {
     if ((threadIdx.x >> 5) == 0) path_epilogue_warp<T>(P, path, A, resid, threadIdx.x & 31);
-}
-
-
-// The whole path (block): head, the residual draw at the first rejection (one
-// more streaming read of that row), epilogue.
-template <typename T, bool VEC, int S>
-__device__ void path_pass(const Problem<T>& P, int path, Ring<S>* rg, float4* tab, PathShared& sh) {
-    const int D = P.D;
-    const int r0 = path * D;
-    path_head<T>(P, path, sh);
-    __syncthreads();
-    const int A = sh.A;
-    int resid = -1;
-    if (A < D && !sh.rec.flags)
-        resid = residual_draw<T, VEC>(P, r0 + A, sh.rec, __ldg(P.u_correct + r0 + A), rg, tab,
-                                      &sh.resid);
-    path_epilogue<T>(P, path, A, resid);
 }
 
 // --------------------------------------------------------------- weights

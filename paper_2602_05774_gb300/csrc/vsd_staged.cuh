@@ -33,7 +33,9 @@ inline size_t staged_smem_bytes(int nch, bool vec) {
            (vec ? 0 : sizeof(WeightsShared));
 }
 
-template <typename T, bool VEC, bool KL>
+// XMODE: kSampleToken the whole E-step + M-step; kGivenToken the verification
+// of given tokens, which ends with the paths.
+template <typename T, bool VEC, bool KL, int XMODE>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ union {
@@ -68,7 +70,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
                 __ldcg(reinterpret_cast<const float2*>(rtab + ch));
     }
     __syncthreads();
-    row_tail<T, VEC, true, kSampleToken, true, KL>(
+    row_tail<T, VEC, true, XMODE, true, KL>(
         P, r, tab, sh.row, rg);
     // the last of n blocks to arrive at a counter
     auto last_of = [&](int* cnt, int n) {
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
         resid = residual_draw<T, VEC>(P, rA, sh.path.rec, __ldg(P.u_correct + rA), rg, tab,
                                       &sh.path.resid);
     path_epilogue<T>(P, path, A, resid);
+    if (XMODE == kGivenToken) return;
     const int prefix = path / K;
     if (!last_of(P.prefix_cnt + prefix, K)) return;
     WeightsShared* ws = VEC ? reinterpret_cast<WeightsShared*>(dsm)

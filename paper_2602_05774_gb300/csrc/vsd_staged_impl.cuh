@@ -16,12 +16,24 @@ cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad,
                                   cudaStream_t s) {
     const size_t smem = staged_smem_bytes(P.nch, vec);
     const bool kl = P.kl_topk != 0;
-    auto rows = vec ? (kl ? k_em_rows<VSD_T, true, true> : k_em_rows<VSD_T, true, false>)
-                    : (kl ? k_em_rows<VSD_T, false, true> : k_em_rows<VSD_T, false, false>);
+    auto rows = vec ? (kl ? k_em_rows<VSD_T, true, true, kSampleToken>
+                           : k_em_rows<VSD_T, true, false, kSampleToken>)
+                    : (kl ? k_em_rows<VSD_T, false, true, kSampleToken>
+                          : k_em_rows<VSD_T, false, false, kSampleToken>);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     if ((e = launch_after(rows, P.R, kThreads, smem, s, P)) || !grad) return e;
     return grad_rows(P, vec, grad, grad_bf16, s);
+}
+
+template <>
+cudaError_t Launch<VSD_T>::verify(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
+    const size_t smem = stream_smem_bytes<kRowStages, sizeof(WeightsShared)>(P.nch, vec);
+    auto rows = vec ? k_em_rows<VSD_T, true, false, kGivenToken>
+                    : k_em_rows<VSD_T, false, false, kGivenToken>;
+    cudaError_t e = prep(rows, smem);
+    if (e) return e;
+    return launch_after(rows, P.R, kThreads, smem, s, P);
 }
 
 template <>

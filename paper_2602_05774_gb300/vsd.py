@@ -154,11 +154,11 @@ def _dtype_code(t):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(device):
-    return C.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    return torch.cuda.current_stream(device).cuda_stream
 
 
 def _need_cuda(*ts):
@@ -210,16 +210,18 @@ def _rows(x, V):
     return x.numel() // V
 
 
-def linear_outputs(B, K, D, V, device, grad_dtype=torch.bfloat16, grad=True, full=True, kl=False):
+def linear_outputs(B, K, D, V, device, grad_dtype=torch.bfloat16, grad=True, full=True, kl=False,
+                   loss=True):
     """Allocate the output tensors of the linear E-step / M-step (kl: the
-    per-row top-K terms of VSD (KL) too)."""
+    per-row top-K terms of VSD (KL) too; loss=False: the E-step's alone)."""
     R = B * K * D
     f = dict(device=device)
     o = dict(tokens=torch.empty(R, dtype=torch.int32, **f),
              accept_len=torch.empty(B * K, dtype=torch.int32, **f),
              corr_tokens=torch.empty(R, dtype=torch.int32, **f),
-             logkappa=torch.empty(R, dtype=torch.float32, **f),
-             loss=torch.empty(B + 1, dtype=torch.float32, **f))
+             logkappa=torch.empty(R, dtype=torch.float32, **f))
+    if loss:
+        o["loss"] = torch.empty(B + 1, dtype=torch.float32, **f)
     if full:
         o.update(logq_tok=torch.empty(R, dtype=torch.float32, **f),
                  alpha=torch.empty(R, dtype=torch.float32, **f),
@@ -230,8 +232,9 @@ def linear_outputs(B, K, D, V, device, grad_dtype=torch.bfloat16, grad=True, ful
                  logkappa_ref=torch.empty(R, dtype=torch.float32, **f),
                  ref_tokens=torch.empty(R, dtype=torch.int32, **f),
                  expected_len=torch.empty(B * K, dtype=torch.float32, **f),
-                 row_stats=torch.empty(R, 4, dtype=torch.float32, **f),
-                 weights=torch.empty(B, D, K, 4, dtype=torch.float32, **f))
+                 row_stats=torch.empty(R, 4, dtype=torch.float32, **f))
+        if loss:
+            o["weights"] = torch.empty(B, D, K, 4, dtype=torch.float32, **f)
     if kl:
         o["kl_loss"] = torch.empty(R, dtype=torch.float32, **f)
     if grad:
@@ -273,9 +276,7 @@ def verify_paths(draft, target, tokens, u_accept, u_correct, K, D, T, ref_logkap
     lay = layout(B, K, D, V)
     dev = draft.device
     ws = _ws(workspace, lay, dev)
-    o = linear_outputs(B, K, D, V, dev, grad=False)
-    del o["loss"], o["weights"]
-    o["tokens"] = torch.empty(R, dtype=torch.int32, device=dev)
+    o = linear_outputs(B, K, D, V, dev, grad=False, loss=False)
     st = _linear_struct(o)
     _check(_lib().vsd_verify_paths(_ptr(draft), _ptr(target), _dtype_code(draft), lay, float(T),
                                    _ptr(tokens), _ptr(u_accept), _ptr(u_correct),
