@@ -320,9 +320,10 @@ struct StoreLogits {
             if (col + i < N) gm = fmaxf(gm, f[i]);
         const float nm = fmaxf(st.m, gm);
         if (nm > -INFINITY) {
-            float acc = __fmul_rn(st.s, vsd::ex2((st.m - nm) * c));  // (no contraction)
+            // (column col < N: the first term, and the carried sum in one rounding)
+            float acc = fmaf(st.s, vsd::ex2((st.m - nm) * c), vsd::ex2((f[0] - nm) * c));
 #pragma unroll
-            for (int i = 0; i < 32; ++i)
+            for (int i = 1; i < 32; ++i)
                 if (col + i < N) acc += vsd::ex2((f[i] - nm) * c);
             st.s = acc;
             st.m = nm;
