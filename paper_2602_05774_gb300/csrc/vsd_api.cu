@@ -188,7 +188,8 @@ vsd_status check_params(const vsd_params& p) {
 template <typename T>
 void fill_wl(Problem<T>& P) {
     for (int d = 0; d < 64; ++d) {
-        P.wl[d] = d < P.D ? pow(P.w_base, (double)(d + 1)) : 0.0;
+        // (a tree's depths come from its parents: every entry)
+        P.wl[d] = d < P.D || P.N > 0 ? pow(P.w_base, (double)(d + 1)) : 0.0;
         P.wlf[d] = (float)P.wl[d];
     }
     P.inv_tau = 1.0 / P.tau_car;

@@ -334,9 +334,19 @@ template <> __device__ __forceinline__ float lane_max<__nv_bfloat16>(const uint4
 }
 
 // ---------------------------------------------------------------- warps
+// (one instruction; NaN lanes are ignored, as by fmaxf)
 __device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+// Two sums at once: lane 0 returns a's, lane 16 b's.  The pairs added are those
+// of warp_sum, so the bits are the same, for half the shuffles.
+__device__ __forceinline__ float warp_sum_pair(float a, float b, int lane) {
+    const bool hi = (lane & 16) != 0;
+    float v = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 __device__ __forceinline__ float warp_sum(float v) {

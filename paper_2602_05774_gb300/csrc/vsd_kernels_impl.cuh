@@ -70,14 +70,9 @@ __global__ void __launch_bounds__(kThreads)
     grid_wait();
     weights_pass<T>(P, E, blockIdx.x, weights, loss, sh);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(P.prefix_done, 1) == P.B - 1;
-        if (last) {
-            __threadfence();
-            loss_mean(loss, P.B);
-        }
-    }
+    if (threadIdx.x == 0) last = atomic_add_acq_rel(P.prefix_done, 1) == P.B - 1;
+    __syncthreads();
+    if (last && threadIdx.x < 32) loss_mean(loss, P.B, threadIdx.x);
 }
 
 template <typename T, bool VEC, typename G>
@@ -234,14 +229,14 @@ __device__ void finish_path_warp(const Problem<T>& P, const EStepView& E, int pa
     if (!warp_count_last(P.prefix_cnt + prefix, P.K, lane)) return;
     weights_warp<T>(P, E, prefix, P.out.weights, P.out.loss, cs.w, lane);
     __syncwarp();
+    int last = 0;
     if (lane == 0) {
         __threadfence();
         if (!P.inject_wait_fault) st_release(P.ready + prefix, 1);
-        if (atomicAdd(P.prefix_done, 1) == P.B - 1) {
-            __threadfence();
-            loss_mean(P.out.loss, P.B);
-        }
+        last = atomicAdd(P.prefix_done, 1) == P.B - 1;
+        if (last) __threadfence();
     }
+    if (__shfl_sync(0xffffffffu, last, 0)) loss_mean(P.out.loss, P.B, lane);
 }
 
 // What the control warp does after the streaming warps finished job j.

@@ -178,9 +178,10 @@ struct Problem {
 __device__ __forceinline__ float frame_of(float m) { return m == -INFINITY ? 0.f : m; }
 __device__ __forceinline__ float mass_rel(float f, float mm, float c) { return ex2((f - mm) * c); }
 
-// Chunk statistics of one tensor: (max, sum_v 2^{(v - max) c}) over the warp's chunk.
+// Chunk statistics of one tensor over the warp's chunk: its maximum m, and this
+// lane's part of sum_v 2^{(v - m) c}.
 template <typename T>
-__device__ __forceinline__ float2 chunk_stats(const uint4 (&buf)[kLoads], float c) {
+__device__ __forceinline__ float2 chunk_part(const uint4 (&buf)[kLoads], float c) {
     constexpr int NP = Traits<T>::kPerVec / 2;
     const float m = warp_max(lane_max<T>(buf));
     const float mm = frame_of(m);
@@ -199,7 +200,23 @@ __device__ __forceinline__ float2 chunk_stats(const uint4 (&buf)[kLoads], float 
     }
     float lo, hi;
     f2split(f2add(acc0, acc1), lo, hi);
-    return make_float2(m, warp_sum(lo + hi));
+    return make_float2(m, lo + hi);
+}
+// (m, sum) of one tensor's chunk.
+template <typename T>
+__device__ __forceinline__ float2 chunk_stats(const uint4 (&buf)[kLoads], float c) {
+    const float2 p = chunk_part<T>(buf, c);
+    return make_float2(p.x, warp_sum(p.y));
+}
+// (m, sum) of both rows' chunk into a table entry.
+template <typename T>
+__device__ __forceinline__ void chunk_stats_pair(const uint4 (&bx)[kLoads],
+                                                 const uint4 (&by)[kLoads], float c, float4* entry,
+                                                 int lane) {
+    const float2 px = chunk_part<T>(bx, c), py = chunk_part<T>(by, c);
+    const float v = warp_sum_pair(px.y, py.y, lane);
+    if ((lane & 15) == 0)
+        reinterpret_cast<float2*>(entry)[lane >> 4] = make_float2(lane ? py.x : px.x, v);
 }
 
 // --------------------------------------------------------------- TMA ring
@@ -361,10 +378,12 @@ __device__ __forceinline__ void stream_tables(Ring<S>* rg, const T* x, const T* 
     if constexpr (VEC) {
         ring_stream<T, HAS_Y>(rg, x, y, V, ch0, ch1, polx, poly, status,
                               [&](int ch, const uint4 (&bx)[kLoads], const uint4 (&by)[kLoads]) {
-                                  const float2 sx = chunk_stats<T>(bx, c);
-                                  float2 sy = make_float2(0.f, 0.f);
-                                  if (HAS_Y) sy = chunk_stats<T>(by, c);
-                                  if (lane == 0) tab[ch] = make_float4(sx.x, sx.y, sy.x, sy.y);
+                                  if constexpr (HAS_Y) {
+                                      chunk_stats_pair<T>(bx, by, c, tab + ch, lane);
+                                  } else {
+                                      const float2 sx = chunk_stats<T>(bx, c);
+                                      if (lane == 0) tab[ch] = make_float4(sx.x, sx.y, 0.f, 0.f);
+                                  }
                               });
         return;
     }
@@ -381,10 +400,12 @@ __device__ __forceinline__ void stream_tables(Ring<S>* rg, const T* x, const T* 
             load_chunk<T, VEC>(x, V, cn, lane, polx, nx);
             if (HAS_Y) load_chunk<T, VEC>(y, V, cn, lane, poly, ny);
         }
-        const float2 sx = chunk_stats<T>(bx, c);
-        float2 sy = make_float2(0.f, 0.f);
-        if (HAS_Y) sy = chunk_stats<T>(by, c);
-        if (lane == 0) tab[ch] = make_float4(sx.x, sx.y, sy.x, sy.y);
+        if constexpr (HAS_Y) {
+            chunk_stats_pair<T>(bx, by, c, tab + ch, lane);
+        } else {
+            const float2 sx = chunk_stats<T>(bx, c);
+            if (lane == 0) tab[ch] = make_float4(sx.x, sx.y, 0.f, 0.f);
+        }
 #pragma unroll
         for (int k = 0; k < kLoads; ++k) {
             bx[k] = nx[k];
@@ -1906,11 +1927,16 @@ __device__ void weights_pass(const Problem<T>& P, const EStepView& E, int b, flo
     weights_group<T, kThreads>(P, E, b, weights_out, loss_out, sh, threadIdx.x);
 }
 
-// Mean of loss[0..B) into loss[B], summed in order (one thread).
-__device__ __forceinline__ void loss_mean(float* loss, int B) {
+// Mean of loss[0..B) into loss[B], summed in order (one warp: 32 loads at a
+// time, where one thread's loads would each wait for the last).
+__device__ __forceinline__ void loss_mean(float* loss, int B, int lane) {
     double s = 0.0;
-    for (int b = 0; b < B; ++b) s += (double)ld_cg(loss + b);
-    loss[B] = (float)(s / (double)B);
+    for (int b0 = 0; b0 < B; b0 += 32) {
+        const float v = b0 + lane < B ? ld_cg(loss + b0 + lane) : 0.f;
+        const int n = min(32, B - b0);
+        for (int j = 0; j < n; ++j) s += (double)__shfl_sync(0xffffffffu, v, j);
+    }
+    if (lane == 0) loss[B] = (float)(s / (double)B);
 }
 
 // --------------------------------------------------------------- gradient

@@ -98,7 +98,8 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
     const EStepView E{P.es.tok, P.es.corr, P.es.lq_tok, P.es.lq_corr,
                       P.es.lk, P.es.lkc, P.es.lkr};
     weights_group<T, kThreads>(P, E, prefix, P.out.weights, P.out.loss, *ws, threadIdx.x);
-    if (last_of(P.prefix_done, P.B) && threadIdx.x == 0) loss_mean(P.out.loss, P.B);
+    if (last_of(P.prefix_done, P.B) && threadIdx.x < 32)
+        loss_mean(P.out.loss, P.B, threadIdx.x);
 }
 
 // The gradient of one segment of a row (block; nseg segments a row): the dense

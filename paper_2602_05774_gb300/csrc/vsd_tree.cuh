@@ -291,6 +291,7 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ int s_par[1024], s_path;
+    __shared__ unsigned char s_acc[1024];
     Ring<kRowStages>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
@@ -305,11 +306,14 @@ __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     }
     grid_wait();
     if (!__syncthreads_or(kids)) return;
+    for (int n = threadIdx.x; n < N; n += kThreads)
+        s_acc[n] = n ? ld_cg(&P.tnode[n0 + n].acc) != 0 : 1;
+    __syncthreads();
     if (threadIdx.x == 0) {
         int path = 1, x = u;
         while (x > 0 && path > 0) {
             const int pn = s_par[x];
-            path = pn < 0 || pn >= x ? -1 : ld_cg(&P.tnode[n0 + x].acc) != 0;  // -1: a bad tree
+            path = pn < 0 || pn >= x ? -1 : s_acc[x];  // -1: a bad tree
             x = pn;
         }
         s_path = path;
@@ -328,13 +332,13 @@ __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     auto each_child = [&](auto&& f) {
         int k = 0;
         for (int n = u + 1; n < N; ++n)
-            if (s_par[n] == u && !(path && ld_cg(&P.tnode[n0 + n].acc)) && k++ % kWarps == warp)
+            if (s_par[n] == u && !(path && s_acc[n]) && k++ % kWarps == warp)
                 f(n0 + n);
     };
     if (path) {
         int rej = 0;
         for (int n = u + 1 + threadIdx.x; n < N; n += kThreads)
-            rej |= s_par[n] == u && !ld_cg(&P.tnode[n0 + n].acc);
+            rej |= s_par[n] == u && !s_acc[n];
         if (!__syncthreads_or(rej)) return;
         const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
         stream_residual<T, VEC>(rg, x, y, V, 0, P.nch, tab, mr, P.status);
@@ -391,12 +395,12 @@ struct TreeShared2 {
 
 // Parents into shared memory and the tree's checks (parent[0] = -1, every
 // other parent precedes its node); depths.  Returns false for a bad tree.
-template <typename T>
+template <int NT, typename T>
 __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
     const int N = P.N;
     const int32_t* par = P.parent + (int64_t)b * N;
     int badl = 0;
-    for (int n = threadIdx.x; n < N; n += kThreads) {
+    for (int n = threadIdx.x; n < N; n += NT) {
         const int pn = __ldg(par + n);
         sh.par[n] = pn;
         badl |= n == 0 ? pn != -1 : (pn < 0 || pn >= n);
@@ -404,19 +408,19 @@ __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
     const int bad = __syncthreads_or(badl);
     if (bad) return false;
     // depths by pointer doubling: depth[n] steps from n to anc[n]
-    for (int n = threadIdx.x; n < N; n += kThreads) {
+    for (int n = threadIdx.x; n < N; n += NT) {
         sh.depth[n] = n ? 1 : 0;
         sh.anc[n] = (short)(n ? sh.par[n] : 0);
     }
     if (threadIdx.x == 0) sh.maxd = 0;
     for (;;) {
         __syncthreads();
-        short a[1024 / kThreads];
-        int d[1024 / kThreads];
+        short a[1024 / NT];
+        int d[1024 / NT];
         int more = 0;
 #pragma unroll
-        for (int k = 0; k < 1024 / kThreads; ++k) {
-            const int n = threadIdx.x + k * kThreads;
+        for (int k = 0; k < 1024 / NT; ++k) {
+            const int n = threadIdx.x + k * NT;
             if (n >= N) break;
             a[k] = sh.anc[sh.anc[n]];
             d[k] = sh.depth[n] + sh.depth[sh.anc[n]];
@@ -424,8 +428,8 @@ __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
         }
         more = __syncthreads_or(more);
 #pragma unroll
-        for (int k = 0; k < 1024 / kThreads; ++k) {
-            const int n = threadIdx.x + k * kThreads;
+        for (int k = 0; k < 1024 / NT; ++k) {
+            const int n = threadIdx.x + k * NT;
             if (n >= N) break;
             sh.anc[n] = a[k];
             sh.depth[n] = d[k];
@@ -434,7 +438,7 @@ __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
     }
     __syncthreads();
     int md = 0;
-    for (int n = threadIdx.x; n < N; n += kThreads) md = max(md, sh.depth[n]);
+    for (int n = threadIdx.x; n < N; n += NT) md = max(md, sh.depth[n]);
     atomicMax(&sh.maxd, md);
     __syncthreads();
     return true;
@@ -447,7 +451,10 @@ __device__ bool tree_load(const Problem<T>& P, int b, TreeShared2& sh) {
 // descending node order), and what belongs to one node or one depth is taken
 // in parallel.  The order of every sum is fixed, so the result does not depend
 // on scheduling.  (On one thread per tree the fp64 latency of this pass was
-// 578 us of a call's 873 at 64 trees of 60 nodes; the whole call now takes 252.)
+// 578 us of a call's 873 at 64 trees of 60 nodes; the whole call now takes 210,
+// this pass about 25.)
+// (256 threads are no faster at 60 nodes, 512 slower: 40.7, 40.0, 45.0 us)
+constexpr int kEmThreads = 128, kEmWarps = kEmThreads / 32;
 struct TreeEmShared {
     TreeShared2 t;
     double lk[1024], lkc[1024], lkr[1024], lqt[1024], lqz[1024];
@@ -464,8 +471,24 @@ struct TreeEmShared {
     int z[1024];                 // corrected token z'_x
     unsigned char acc[1024];
     short first[1024], last[1024];  // a node's first and last child (0: none)
-    double red[kWarps][2];
+    short prev[1024], next[1024];   // a node's siblings before and after it (0: none)
+    // per depth: proposals with o' != 0 and o~ = 1, with o' != 0; the largest
+    // CAR logit (as an ordered integer); the sum of the CAR weights
+    int n1[1024], n0[1024];
+    unsigned long long cmax[1024];
+    double zs[1024];
+    double red[kEmWarps][2];
 };
+
+// Doubles as integers of the same order (0 is below every double).
+__device__ __forceinline__ unsigned long long ordered_bits(double v) {
+    const long long b = __double_as_longlong(v);
+    return b < 0 ? ~(unsigned long long)b : (unsigned long long)b | 0x8000000000000000ull;
+}
+__device__ __forceinline__ double ordered_value(unsigned long long k) {
+    return __longlong_as_double(
+        (long long)(k >> 63 ? k & 0x7FFFFFFFFFFFFFFFull : ~k));
+}
 
 // Sum over the block in a fixed order; every thread returns it.
 __device__ __forceinline__ double2 block_sum(double2 v, double (*red)[2]) {
@@ -478,7 +501,7 @@ __device__ __forceinline__ double2 block_sum(double2 v, double (*red)[2]) {
     }
     __syncthreads();
     double2 s = make_double2(0.0, 0.0);
-    for (int w = 0; w < kWarps; ++w) {
+    for (int w = 0; w < kEmWarps; ++w) {
         s.x += red[w][0];
         s.y += red[w][1];
     }
@@ -493,19 +516,21 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
     const int* par = sh.t.par;
     const int* depth = sh.t.depth;
     const int maxd = sh.t.maxd;
-    for (int n = tid; n < N; n += kThreads) {
+    for (int n = tid; n < N; n += kEmThreads) {
         sh.acc[n] = n ? P.tnode[n0 + n].acc != 0 : 1;
         sh.first[n] = sh.last[n] = 0;
+        sh.n0[n] = sh.n1[n] = 0;
+        sh.cmax[n] = 0;
     }
     // accepted paths
     for (int l = 0; l <= maxd; ++l) {
         __syncthreads();
-        for (int n = tid; n < N; n += kThreads)
+        for (int n = tid; n < N; n += kEmThreads)
             if (depth[n] == l) sh.t.pacc[n] = n ? sh.acc[n] && sh.t.pacc[par[n]] : 1;
     }
     __syncthreads();
     // the E-step per node (R15): z' and the node's terms of the sums
-    for (int n = tid; n < N; n += kThreads) {
+    for (int n = tid; n < N; n += kEmThreads) {
         if (n == 0) {
             sh.lk[0] = sh.lkc[0] = sh.lkr[0] = sh.lqt[0] = sh.lqz[0] = 0.0;
             sh.z[0] = -1;
@@ -535,7 +560,7 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
     }
     for (int l = 1; l <= maxd; ++l) {
         __syncthreads();
-        for (int n = tid; n < N; n += kThreads) {
+        for (int n = tid; n < N; n += kEmThreads) {
             if (depth[n] != l) continue;
             const int a = par[n];
             sh.lk[n] = sh.lk[a] + (double)sh.e.la[n];
@@ -549,53 +574,51 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
     // o~, o' (Algorithm 2 with w(depth): w(l) = w_base^l, trees may be deeper
     // than the host's table of w), N_b, the CAR logits
     double2 Nb = make_double2(0.0, 0.0);
-    for (int n = 1 + tid; n < N; n += kThreads) {
-        const double wl = pow(P.w_base, (double)depth[n]);
+    for (int n = 1 + tid; n < N; n += kEmThreads) {
+        const double wl = depth[n] <= 64 ? P.wl[depth[n] - 1] : pow(P.w_base, (double)depth[n]);
         const bool ot = sh.lk[n] >= sh.lkr[n];
         const bool op = ot || sh.lkc[n] >= sh.lkr[n];
         sh.w[n][0] = ot ? 1.f : 0.f;
         sh.w[n][1] = op ? (float)wl : 0.f;
-        if (op) Nb.x += wl;
-        sh.m.st[n] = (P.zeta_mode == 0 ? exp(sh.lqt[n]) : sh.lqt[n]) * P.inv_tau;
+        const double cq = (P.zeta_mode == 0 ? exp(sh.lqt[n]) : sh.lqt[n]) * P.inv_tau;
+        sh.m.st[n] = cq;
+        const int l = depth[n] - 1;
+        atomicMax(&sh.cmax[l], ordered_bits(cq));
+        if (op) {
+            Nb.x += wl;
+            atomicAdd(&sh.n0[l], 1);
+            if (ot) atomicAdd(&sh.n1[l], 1);
+        }
     }
     Nb = block_sum(Nb, sh.red);
     // beta (leave-one-out) and zeta (softmax of q(z~)/tau, or log q in
-    // zeta_mode 1) over the nodes of each depth: one warp per depth.  (All o'
-    // of a depth are equal or 0, so the sums behind beta are exact.)
-    for (int l = 1 + warp; l <= maxd; l += kWarps) {
-        double num = 0.0, den = 0.0, cmax = -INFINITY;
-        for (int n = 1 + lane; n < N; n += 32) {
-            if (depth[n] != l) continue;
-            const double op = sh.w[n][1];
-            num += op * sh.w[n][0];
-            den += op;
-            cmax = fmax(cmax, sh.m.st[n]);
-        }
-        num = warp_sum(num);
-        den = warp_sum(den);
-#pragma unroll
-        for (int k = 16; k; k >>= 1) cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, k));
+    // zeta_mode 1) over the nodes of each depth.  All o' of a depth are w(l) or
+    // 0, so the sums behind beta are w(l) times a count, exactly; the CAR
+    // weights are made for every node at once and summed by a warp per depth.
+    for (int n = 1 + tid; n < N; n += kEmThreads)
+        sh.m.st[n] = exp(sh.m.st[n] - ordered_value(sh.cmax[depth[n] - 1]));
+    __syncthreads();
+    for (int l = 1 + warp; l <= maxd; l += kEmWarps) {
         double zs = 0.0;
-        for (int n = 1 + lane; n < N; n += 32) {
-            if (depth[n] != l) continue;
-            const double ez = exp(sh.m.st[n] - cmax);
-            sh.m.st[n] = ez;
-            zs += ez;
-        }
+        for (int n = 1 + lane; n < N; n += 32)
+            if (depth[n] == l) zs += sh.m.st[n];
         zs = warp_sum(zs);
-        for (int n = 1 + lane; n < N; n += 32) {
-            if (depth[n] != l) continue;
-            const double op = sh.w[n][1];
-            const double d1 = den - op, n1 = num - op * sh.w[n][0];
-            sh.w[n][2] = d1 > 0.0 ? (float)(n1 / d1) : 0.f;
-            sh.w[n][3] = (float)(sh.m.st[n] / zs);
-        }
+        if (lane == 0) sh.zs[l - 1] = zs;
+    }
+    __syncthreads();
+    for (int n = 1 + tid; n < N; n += kEmThreads) {
+        const int l = depth[n] - 1;
+        const double op = sh.w[n][1];
+        const double w = op != 0.0 ? op : (double)(float)(l < 64 ? P.wl[l] : pow(P.w_base, l + 1.0));
+        const double d1 = w * sh.n0[l] - op, n1 = w * sh.n1[l] - op * sh.w[n][0];
+        sh.w[n][2] = d1 > 0.0 ? (float)(n1 / d1) : 0.f;
+        sh.w[n][3] = (float)(sh.m.st[n] / sh.zs[l]);
     }
     __syncthreads();
     // the objective (Eq. advance) and each proposal's gradient terms; the
     // nodes' first and last children
     double2 J = make_double2(0.0, 0.0);
-    for (int n = tid; n < N; n += kThreads) {
+    for (int n = tid; n < N; n += kEmThreads) {
         double st = 0.0, sz = 0.0;
         if (n) {
             const double ot = sh.w[n][0], op = sh.w[n][1];
@@ -606,11 +629,14 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
                 st = op * (ot - bz);
                 sz = op * (1.0 - ot);
             }
-            bool f = true, z = true;
-            for (int k = par[n] + 1; k < n && f; ++k) f = par[k] != par[n];
-            for (int k = n + 1; k < N && z; ++k) z = par[k] != par[n];
-            if (f) sh.first[par[n]] = (short)n;
-            if (z) sh.last[par[n]] = (short)n;
+            const int a = par[n];
+            int k = n - 1, m = n + 1;
+            while (k > a && par[k] != a) --k;
+            while (m < N && par[m] != a) ++m;
+            sh.prev[n] = (short)(k > a ? k : 0);
+            sh.next[n] = (short)(m < N ? m : 0);
+            if (k <= a) sh.first[a] = (short)n;
+            if (m >= N) sh.last[a] = (short)n;
         }
         sh.m.st[n] = st;
         sh.m.sz[n] = sz;
@@ -618,14 +644,13 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
     J = block_sum(J, sh.red);
     // subtree sums (the proposals whose path goes through a node)
     for (int l = maxd - 1; l >= 0; --l) {
-        for (int a = tid; a < N; a += kThreads) {
+        for (int a = tid; a < N; a += kEmThreads) {
             if (depth[a] != l || !sh.last[a]) continue;
             double st = sh.m.st[a], sz = sh.m.sz[a];
-            for (int n = sh.last[a]; n >= sh.first[a]; --n)
-                if (par[n] == a) {
-                    st += sh.m.st[n];
-                    sz += sh.m.sz[n];
-                }
+            for (int n = sh.last[a]; n; n = sh.prev[n]) {
+                st += sh.m.st[n];
+                sz += sh.m.sz[n];
+            }
             sh.m.st[a] = st;
             sh.m.sz[a] = sz;
         }
@@ -633,7 +658,7 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
     }
     const double scale = Nb.x > 0.0 ? 1.0 / ((double)P.B * Nb.x * P.ts.Td) : 0.0;
     if (tid == 0) o.loss[b] = Nb.x > 0.0 ? (float)(-J.x / Nb.x) : 0.f;
-    for (int x = tid; x < N; x += kThreads) {
+    for (int x = tid; x < N; x += kEmThreads) {
         if (x) {
             TreeCoef cf;
             cf.t = __ldg(P.given_tokens + n0 + x);
@@ -648,9 +673,8 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
             P.tcoef[n0 + x] = cf;
         }
         float g = 0.f;  // the row's dense factor: its children's, in node order
-        if (sh.last[x])
-            for (int n = sh.first[x]; n <= sh.last[x]; ++n)
-                if (par[n] == x) g += (float)((sh.m.st[n] + sh.m.sz[n]) * scale);
+        for (int n = sh.first[x]; n; n = sh.next[n])
+            g += (float)((sh.m.st[n] + sh.m.sz[n]) * scale);
         P.tg[n0 + x] = g;
         if (o.corr_tokens) o.corr_tokens[n0 + x] = sh.z[x];
         if (o.weights)
@@ -666,18 +690,18 @@ __device__ void tree_em_nodes(const Problem<T>& P, const vsd_tree_em_outputs& o,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_tree_em(Problem<T> P, vsd_tree_em_outputs o) {
+__global__ void __launch_bounds__(kEmThreads) k_tree_em(Problem<T> P, vsd_tree_em_outputs o) {
     extern __shared__ __align__(128) unsigned char dsm[];
     TreeEmShared& sh = *reinterpret_cast<TreeEmShared*>(dsm);
     const int N = P.N, b = blockIdx.x, n0 = b * N;
     grid_launch_next();
-    const bool ok = tree_load<T>(P, b, sh.t);
+    const bool ok = tree_load<kEmThreads>(P, b, sh.t);
     grid_wait();
     if (ok) {
         if (threadIdx.x == 0) P.tbad[b] = 0;
         tree_em_nodes<T>(P, o, b, sh);
     } else {
-        for (int n = threadIdx.x; n < N; n += kThreads) {
+        for (int n = threadIdx.x; n < N; n += kEmThreads) {
             P.tcoef[n0 + n] = TreeCoef{-1, 0.f, -1, 0.f};
             P.tg[n0 + n] = 0.f;
             if (o.corr_tokens) o.corr_tokens[n0 + n] = -1;
@@ -690,13 +714,11 @@ __global__ void __launch_bounds__(kThreads) k_tree_em(Problem<T> P, vsd_tree_em_
             o.loss[b] = 0.f;
         }
     }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(P.prefix_done, 1) == P.B - 1) {
-            __threadfence();
-            loss_mean(o.loss, P.B);
-        }
-    }
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomic_add_acq_rel(P.prefix_done, 1) == P.B - 1;
+    __syncthreads();
+    if (last && threadIdx.x < 32) loss_mean(o.loss, P.B, threadIdx.x);
 }
 
 // ------------------------------------------------------------ k_tree_grad
@@ -1138,7 +1160,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     grid_wait();
     const int N = P.N, b = blockIdx.x, n0 = b * N;
     const vsd_tree_outputs& o = P.tout;
-    if (!tree_load<T>(P, b, sh.t)) {
+    if (!tree_load<kThreads>(P, b, sh.t)) {
         for (int n = threadIdx.x; n < N; n += kThreads) {
             o.alpha[n0 + n] = 0.f;
             o.accept[n0 + n] = 0;

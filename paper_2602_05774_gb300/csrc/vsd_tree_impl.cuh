@@ -48,7 +48,7 @@ cudaError_t Launch<VSD_T>::tree_em(const Problem<VSD_T>& P, bool vec,
     if ((e = prep(draws, smem))) return e;
     if ((e = launch_after(draws, P.R, kThreads, smem, s, P))) return e;
     if ((e = prep(k_tree_em<VSD_T>, sizeof(TreeEmShared)))) return e;
-    if ((e = launch_after(k_tree_em<VSD_T>, P.B, kThreads, sizeof(TreeEmShared), s, P, o)))
+    if ((e = launch_after(k_tree_em<VSD_T>, P.B, kEmThreads, sizeof(TreeEmShared), s, P, o)))
         return e;
     const size_t gsm = tree_grad_smem_bytes(P.N);
 #define VSD_TGRAD(V_, G_)                                                           \
