@@ -24,6 +24,8 @@
 //                at the row.
 #pragma once
 
+#include <type_traits>
+
 #include "vsd_common.cuh"
 
 namespace vsd {
@@ -443,6 +445,10 @@ __device__ __forceinline__ float table_max(const float4* tab, int nch, int comp,
 
 // --------------------------------------------------------------- table sums
 // The weight of chunk c in the row frame Mm is w_c = s_c 2^{(m_c - Mm) c}.
+// (Functions that several steps of a block's chain call are not inlined: such
+// steps run once per block, and a second copy of their code would be fetched
+// anew.  At 768 rows of V = 32000, 67.4 us a call with table_sum and
+// table_locate inlined, 64.7 without.)
 // Tables are summed in exact 64-bit fixed point, w_c 2^E rounded down, with E
 // set from the largest weight so that it keeps at least 50 significant bits
 // and no sum of up to 2048 weights overflows.  Integer sums are exact and do
@@ -545,7 +551,7 @@ struct TableSum {
 };
 
 // Sum of the chunk weights of one table component (warp).
-__device__ __forceinline__ TableSum table_sum(const float4* tab, int nch, int comp, float Mm,
+static __device__ __noinline__ TableSum table_sum(const float4* tab, int nch, int comp, float Mm,
                                               float c, int lane) {
     float wm = 0.f;
     bool bad = false;
@@ -580,8 +586,8 @@ struct Located {
     int ch;
     float tc;
 };
-__device__ __forceinline__ Located table_locate(const float4* tab, int nch, int comp, float Mm,
-                                                float c, const TableSum& S, float u, int lane) {
+static __device__ __noinline__ Located table_locate(const float4* tab, int nch, int comp, float Mm,
+                                                float c, TableSum S, float u, int lane) {
     const long long ti = fixed_scale(S.Zi, u);
     long long base = 0;
     int last = -1;
@@ -751,6 +757,37 @@ __device__ __forceinline__ int rescan_smem(const uint4* bx, const uint4* by, int
     return last;
 }
 
+struct MassX {
+    float mm, c;
+    __device__ float operator()(float fx, float, int) const { return mass_rel(fx, mm, c); }
+};
+struct MassY {
+    float mm, c;
+    __device__ float operator()(float, float fy, int) const { return mass_rel(fy, mm, c); }
+};
+// Residual mass max(0, p(v) - q(v)) with p and q normalised by 1/Z factors.
+struct MassRes {
+    float mx, my, izx, izy, c;
+    __device__ float operator()(float fx, float fy, int) const {
+        const float p = ex2((fy - my) * c) * izy;
+        const float q = ex2((fx - mx) * c) * izx;
+        return fmaxf(p - q, 0.f);
+    }
+};
+
+// rescan_smem for the residual's masses and for one row's own (draw_mass), in
+// one copy of the code.
+template <typename T>
+__device__ __noinline__ int rescan_mass(const uint4* bx, const uint4* by, int64_t V, int ch, float tc,
+                                        MassRes mass, int lane) {
+    return rescan_smem<T, true, true>(bx, by, V, ch, tc, mass, lane);
+}
+// The masses 2^{(y - mm) c} of a row as the residual of nothing: 1/Z is 1 for
+// the row, 0 for the other one (whose masses are finite in a valid row).
+__device__ __forceinline__ MassRes draw_mass(float mm, float c) {
+    return MassRes{mm, mm, 0.f, 1.f, c};
+}
+
 // A warp's two chunk buffers for rescans: its own ring slots (no copy of its
 // stream is in flight then), null on the scalar path.
 template <int S> __device__ __forceinline__ uint4* warp_chunks(Ring<S>* rg) {
@@ -775,7 +812,12 @@ __device__ __forceinline__ int warp_rescan(const T* x, const T* y, int64_t V, in
                                            const Mass& mass, int lane, uint64_t pol, uint4* buf) {
     if constexpr (VEC) {
         load_chunk_pair<T>(buf, NEED_X ? x : nullptr, NEED_Y ? y : nullptr, V, ch, lane);
-        return rescan_smem<T, NEED_X, NEED_Y>(buf, buf + kLoads * 32, V, ch, tc, mass, lane);
+        if constexpr (std::is_same<Mass, MassRes>::value)
+            return rescan_mass<T>(buf, buf + kLoads * 32, V, ch, tc, mass, lane);
+        else if constexpr (std::is_same<Mass, MassX>::value)
+            return rescan_mass<T>(buf, buf, V, ch, tc, draw_mass(mass.mm, mass.c), lane);
+        else
+            return rescan_smem<T, NEED_X, NEED_Y>(buf, buf + kLoads * 32, V, ch, tc, mass, lane);
     } else {
         uint4 bx[kLoads], by[kLoads];
         if (NEED_X) load_chunk<T, VEC>(x, V, ch, lane, pol, bx);
@@ -783,24 +825,6 @@ __device__ __forceinline__ int warp_rescan(const T* x, const T* y, int64_t V, in
         return rescan_regs<T, NEED_X, NEED_Y>(bx, by, ch, tc, mass, lane);
     }
 }
-
-struct MassX {
-    float mm, c;
-    __device__ float operator()(float fx, float, int) const { return mass_rel(fx, mm, c); }
-};
-struct MassY {
-    float mm, c;
-    __device__ float operator()(float, float fy, int) const { return mass_rel(fy, mm, c); }
-};
-// Residual mass max(0, p(v) - q(v)) with p and q normalised by 1/Z factors.
-struct MassRes {
-    float mx, my, izx, izy, c;
-    __device__ float operator()(float fx, float fy, int) const {
-        const float p = ex2((fy - my) * c) * izy;
-        const float q = ex2((fx - mx) * c) * izx;
-        return fmaxf(p - q, 0.f);
-    }
-};
 
 // Inverse-CDF draw from the distribution of one table component (warp).
 // S is the table total; returns the token (or -1 if the row has no mass).
@@ -969,7 +993,7 @@ __device__ __forceinline__ RowTask row_task(const Problem<T>& P, int r, const fl
                 t.tok = first_max_smem<T>(z, V, loc.ch, t.M);
             } else {
                 const float mm = frame_of(tab_ms(tab[loc.ch], comp).x);
-                t.tok = rescan_smem<T, true, false>(z, z, V, loc.ch, loc.tc, MassX{mm, c}, lane);
+                t.tok = rescan_mass<T>(z, z, V, loc.ch, loc.tc, draw_mass(mm, c), lane);
             }
             if (t.tok >= 0) {
                 t.xv = smem_elem(buf, loc.ch, t.tok, x);
