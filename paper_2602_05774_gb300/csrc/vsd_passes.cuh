@@ -937,7 +937,7 @@ struct RowTask {
 };
 template <typename T, bool VEC, bool HAS_Y, int XMODE>
 __device__ __forceinline__ RowTask row_task(const Problem<T>& P, int r, const float4* tab,
-                                            int which, int lane, uint4* buf) {
+                                            int which, int lane, uint4* buf, bool pdraw) {
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
     const T* y = HAS_Y ? P.target + (int64_t)r * V : nullptr;
@@ -949,7 +949,8 @@ __device__ __forceinline__ RowTask row_task(const Problem<T>& P, int r, const fl
     t.lz = 0.0;
     // (asked for early: its latency is hidden behind the table's)
     const float* up = which == 0 ? P.u_draft : P.u_correct;
-    const bool drawn = which == 0 ? XMODE == kSampleToken : which == 1 && XMODE != kStats;
+    const bool drawn =
+        which == 0 ? XMODE == kSampleToken : which == 1 && XMODE != kStats && pdraw;
     const float u = drawn && up ? __ldg(up + r) : 0.f;
     int given = -1;
     if (XMODE == kGivenToken && which == 0) {
@@ -1113,10 +1114,11 @@ __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch
 // warps 0, 1 and 2 take the three tasks at once, warp 0 then writes the record.
 template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool KL = false, int S>
 __device__ void row_tail(const Problem<T>& P, int r, const float4* tab, RowShared& sh,
-                         Ring<S>* rg) {
+                         Ring<S>* rg, bool pdraw = true) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0 || (HAS_Y && (warp == 1 || (ARGMAX && warp == 2)))) {
-        const RowTask t = row_task<T, VEC, HAS_Y, XMODE>(P, r, tab, warp, lane, warp_chunks(rg));
+        const RowTask t = row_task<T, VEC, HAS_Y, XMODE>(P, r, tab, warp, lane, warp_chunks(rg),
+                                                            pdraw);
         if (lane == 0) sh.t[warp] = t;
     } else if (KL && HAS_Y && warp == 3) {
         // VSD (KL): the top-K term on the fourth warp (an invalid row's term
@@ -1407,8 +1409,10 @@ __device__ void row_tail_warp(const Problem<T>& P, int r, float4* tab, RescanBuf
 // Streams row r of the draft (and, with HAS_Y, of the target) once, then runs
 // row_tail.  XMODE: whether z~ is drawn from q with u_draft, read from
 // given_tokens, or absent (trees).  ARGMAX: locate the greedy reference token.
+// pdraw = false leaves out the draw from p.
 template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, int S>
-__device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, RowShared& sh) {
+__device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, RowShared& sh,
+                         bool pdraw = true) {
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
     const T* y = HAS_Y ? P.target + (int64_t)r * V : nullptr;
@@ -1419,7 +1423,7 @@ __device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, R
     // workspace is written from here on)
     grid_wait();
     __syncthreads();
-    row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh, rg);
+    row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh, rg, pdraw);
 }
 
 // --------------------------------------------------------------- residual

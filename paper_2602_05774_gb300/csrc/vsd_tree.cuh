@@ -56,8 +56,9 @@ static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 //   k_tree_verify       one block per row, of which most leave at once: at a
 //                       row on an accepted path the rejected children's draws
 //                       (one more read of the row), at the deepest accepted
-//                       node the bonus token (a leaf's row is read here), at
-//                       the root the outputs of the tree's nodes.
+//                       node the bonus token (a leaf's row is read here, for
+//                       a draw that the first kernel leaves out), at the root
+//                       the outputs of the tree's nodes.
 // No block waits for another.  The row reads bound the first kernel, a few
 // dependent steps of one row the second.
 template <typename T, bool VEC>
@@ -70,10 +71,11 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1)
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
     grid_launch_next();
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
-    int need = P.tout.row_stats != nullptr;
-    for (int n = u + 1 + threadIdx.x; n < N && !need; n += kThreads)
-        need = __ldg(P.parent + (int64_t)b * N + n) == u;
-    if (!__syncthreads_or(need)) {
+    int kids = 0;
+    for (int n = u + 1 + threadIdx.x; n < N && !kids; n += kThreads)
+        kids = __ldg(P.parent + (int64_t)b * N + n) == u;
+    kids = __syncthreads_or(kids);
+    if (!kids && !P.tout.row_stats) {
         grid_wait();
         return;
     }
@@ -862,8 +864,10 @@ struct SeqKids {
     float2* A;      // the A its token keeps once removed, in two floats
     int* tok;
     int* kid;       // its node
+    float* ua;      // its uniforms
+    float* uc;
 };
-inline size_t seq_smem_bytes(int N) { return (size_t)N * 32; }
+inline size_t seq_smem_bytes(int N) { return (size_t)N * 40; }
 __device__ __forceinline__ SeqKids seq_kids(unsigned char* base, int N) {
     SeqKids s;
     s.p = reinterpret_cast<double*>(base);
@@ -871,6 +875,8 @@ __device__ __forceinline__ SeqKids seq_kids(unsigned char* base, int N) {
     s.A = reinterpret_cast<float2*>(s.q + N);
     s.tok = reinterpret_cast<int*>(s.A + N);
     s.kid = s.tok + N;
+    s.ua = reinterpret_cast<float*>(s.kid + N);
+    s.uc = s.ua + N;
     return s;
 }
 
@@ -1030,6 +1036,8 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, f
             p = exp(((double)yv - rec.my) * P.ts.invTd - rec.lzy);
             q = exp(((double)xv - rec.mx) * P.ts.invTd - rec.lzx);
         }
+        s.ua[i] = __ldg(P.u_accept + n);
+        s.uc[i] = __ldg(P.u_correct + n);
         s.tok[i] = tok;
         s.p[i] = p;
         s.q[i] = q;
@@ -1038,35 +1046,41 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, f
     __syncthreads();
     const MassRes mr{rec.mx, rec.my, rec.izx, rec.izy, c};
     for (int i = 0; i < m; ++i) {
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
             const int n = n0 + s.kid[i], t = s.tok[i];
             int before = -1;  // the earlier sibling that removed t, if any
             for (int j = 0; j < i && before < 0; ++j)
                 if (s.tok[j] == t) before = j;
             const double Q = ct.Q, A = ct.A, Tm = ct.T;
+            const double At = before >= 0 ? (double)s.A[before].x + (double)s.A[before].y : A;
+            // p_i, q_i at t, and A's step T_i / Q_i: three quotients on three lanes
+            const double num = lane == 0 ? fmax(0.0, s.p[i] - At * s.q[i]) : lane == 1 ? s.q[i] : Tm;
+            const double den = lane == 0 ? Tm : Q;
+            const double quo = den > 0.0 ? num / den : 0.0;
+            const double pi = __shfl_sync(0xffffffffu, quo, 0);
+            const double qi = before >= 0 ? 0.0 : __shfl_sync(0xffffffffu, quo, 1);
+            const double step = __shfl_sync(0xffffffffu, quo, 2);
             double alpha = 0.0;
-            if (!rec.flags && t >= 0 && t < V) {
-                const double At = before >= 0 ? (double)s.A[before].x + (double)s.A[before].y : A;
-                const double pi = fmax(0.0, s.p[i] - At * s.q[i]) / Tm;
-                const double qi = before >= 0 || !(Q > 0.0) ? 0.0 : s.q[i] / Q;
+            if (!rec.flags && t >= 0 && t < V)
                 alpha = qi > 0.0 ? fmin(1.0, pi / qi) : (pi > 0.0 ? 1.0 : 0.0);
+            const bool a = s.ua[i] <= alpha && !rec.flags;
+            if (lane == 0) {
+                P.tnode[n].lq = (float)alpha;
+                P.tnode[n].acc = a ? 1 : 0;
+                P.tnode[n].zp = 1;
+                if (a) ct.next = s.kid[i];
+                ct.An = A + step;
+                const float2 h = two_floats(ct.An);
+                ct.ah = h.x;
+                ct.al = h.y;
+                if (before < 0) ct.Q = Q - s.q[i];
             }
-            const bool a = __ldg(P.u_accept + n) <= alpha && !rec.flags;
-            P.tnode[n].lq = (float)alpha;
-            P.tnode[n].acc = a ? 1 : 0;
-            P.tnode[n].zp = 1;
-            if (a) ct.next = s.kid[i];
-            ct.An = A + (Q > 0.0 ? Tm / Q : 0.0);
-            const float2 h = two_floats(ct.An);
-            ct.ah = h.x;
-            ct.al = h.y;
-            if (before < 0) ct.Q = Q - s.q[i];
         }
         __syncthreads();
         if (ct.next > 0) break;
         if (!rec.flags) {
             // T_{i+1} (one read of the row); the draw after the last rejection
-            const float uc = __ldg(P.u_correct + n0 + s.kid[i]);
+            const float uc = s.uc[i];
             const SeqMass sm{mr, ct.ah, ct.al, s.tok, s.A, i};
             seq_stream<T, VEC>(P, r, rg, tab, sm);
             if (warp == 0) {
@@ -1107,8 +1121,8 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, f
     }
 }
 
-// One block per node row (a leaf's row only for the statistics output; the
-// draw a leaf's bonus token needs is k_tree_seq's).
+// One block per node row (a leaf's row only for the statistics output; the row
+// a bonus token needs is then read by k_tree_seq).
 // What bounds it: the row reads and row tails (3840 rows of 2 x 64 KB), and
 // the reads after a rejection, which come from L2.  64 trees of 60 nodes,
 // V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
@@ -1124,15 +1138,17 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_row
     grid_launch_next();
     const SeqKids kids = seq_kids(reinterpret_cast<unsigned char*>(tab + P.nch), P.N);
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
-    int need = P.tout.row_stats != nullptr;
-    for (int n = u + 1 + threadIdx.x; n < N && !need; n += kThreads)
-        need = __ldg(P.parent + (int64_t)b * N + n) == u;
-    if (!__syncthreads_or(need)) {
+    int has = 0;
+    for (int n = u + 1 + threadIdx.x; n < N && !has; n += kThreads)
+        has = __ldg(P.parent + (int64_t)b * N + n) == u;
+    has = __syncthreads_or(has);
+    if (!has && !P.tout.row_stats) {
         grid_wait();
         if (threadIdx.x == 0) P.tlist[r] = 0;
         return;
     }
-    row_pass<T, VEC, true, kStats, false>(P, r, rg, tab, sh);
+    // (a leaf's draw from p may become the bonus token)
+    row_pass<T, VEC, true, kNoToken, false>(P, r, rg, tab, sh, !has);
     __syncthreads();
     if (threadIdx.x == 0 && P.tout.row_stats)
         reinterpret_cast<float4*>(P.tout.row_stats)[r] = ld_cg(P.rstats + r);
@@ -1218,7 +1234,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     }
     __syncthreads();
     const bool leaf = sh.lastkid == 0;
-    if (leaf) {  // the leaf's row, for the bonus token
+    if (leaf && !P.tout.row_stats) {  // the leaf's row, for the bonus token
         row_pass<T, VEC, true, kNoToken, false>(P, n0 + best, rg, tab, rsh);
         __syncthreads();
     }
