@@ -90,10 +90,19 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
+def estep_kernels(R, V, elem, grad=True):
+    """The kernels one vsd_estep_mstep call launches, as the library chooses
+    them (the counters' clearing first)."""
+    chunks = -(-V // (2048 // elem))
+    if chunks <= 64 or not grad or 2 * elem * R * V <= 512 << 20:
+        return ["k_clear", "k_em_rows"] + (["k_em_grad"] if grad else [])
+    return ["k_clear", "k_fused"]
+
+
 def ncu_traffic(workload, kernel="k_fused"):
-    """DRAM bytes per launch of the roofline's kernel (k_fused; k_lmhead_bwd:
-    per backward call) from the committed ncu summary, if it was taken on the
-    current kernel sources; else None."""
+    """DRAM bytes per launch of the roofline's kernel (k_fused; k_gemm2: per
+    backward call, the gradient rows and both products) from the committed ncu
+    summary, if it was taken on the current kernel sources; else None."""
     path = os.path.join(ROOT, "profiles", "%s_%s_traffic.json" % (kernel, workload))
     try:
         d = json.load(open(path))
@@ -437,9 +446,9 @@ def run_ours(args):
         "achieved_gbs": achieved,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
-                     "kernel": "k_fused", "algorithmic_bytes_per_launch": alg,
-                     "launch_ms": launch_ms},
-        "gpu_launches": args.steps,
+                     "kernel": " + ".join(estep_kernels(R, V, elem)[1:]),
+                     "algorithmic_bytes_per_launch": alg, "launch_ms": launch_ms},
+        "gpu_launches": len(estep_kernels(R, V, elem)) * args.steps,
         "clocks": clk.summary(),
     }
     if e2e is not None:
@@ -512,8 +521,8 @@ def run_lmhead(args, train=False):
     step is vsd_lmhead_estep_mstep; the roofline is the GEMM's (tensor), timed
     on its own with CUDA events per launch.  train: the draft head's training
     step, vsd_lmhead_estep_mstep with no dense gradient, then
-    vsd_lmhead_backward (d_hidden and d_weight from the factored gradient);
-    the roofline is the backward's (tensor), timed per call."""
+    vsd_lmhead_backward_scratch (d_hidden and d_weight from a bf16 gradient in
+    scratch memory); the roofline is the backward's (tensor), timed per call."""
     import torch
     rank, world, local = dist_env()
     from paper_2602_05774_gb300 import multirank
@@ -621,17 +630,18 @@ def run_lmhead(args, train=False):
         "data": "synthetic (seeded; hidden ~N(0,1), LM-head weight ~N(0,0.02^2), spiked target)",
         "config": {"workload": "lmhead_train" if train else "lmhead", "B": B, "K": K, "D": D,
                    "V": V, "H": H, "logits": "bf16",
-                   "grad": "factored: made on chip by the backward, never in HBM" if train
+                   "grad": "factored; the backward writes it once as bf16 scratch" if train
                    else "bf16", "temperatures": [T],
                    "l2": "inputs larger than L2 (no flush)", "rows_per_gpu": R},
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak,
-                     "traffic": ncu_traffic("lmhead_train", "k_lmhead_bwd") if train else None,
+                     "traffic": ncu_traffic("lmhead_train", "k_gemm2") if train else None,
                      "peak_kind": peak_kind,
-                     "kernel": "k_lmhead_bwd (d_hidden + d_weight)" if train else "k_lmhead",
+                     "kernel": "k_em_grad + k_gemm2 (d_hidden, d_weight)" if train else "k_gemm2",
                      "flops_per_launch": flops, "launch_ms": gemm_ms},
-        # per step: GEMM, fused E/M (+ row factors, d_hidden, d_weight)
-        "gpu_launches": (5 if train else 2) * args.steps,
+        # per step: the E/M step's kernels and the GEMM (+ the gradient rows, two GEMMs)
+        "gpu_launches": (len(estep_kernels(R, V, 2, not train)) + (4 if train else 1))
+        * args.steps,
         "clocks": clk.summary(),
     }
     if e2e is not None:
@@ -800,9 +810,9 @@ def run_tree(args):
                    "rows_read": rows_read},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "peak_kind": peak_kind,
-                     "kernel": "k_tree_fused",
+                     "kernel": "k_tree_verify_rows + k_tree_verify",
                      "algorithmic_bytes_per_launch": alg, "launch_ms": launch_ms},
-        "gpu_launches": args.steps,
+        "gpu_launches": 3 * args.steps,  # and the counters' clearing
         "clocks": clk.summary(),
     }
     if e2e is not None:

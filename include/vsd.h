@@ -228,10 +228,12 @@ vsd_status vsd_weighted_loss_fwd_bwd(const void* draft, vsd_dtype dtype, vsd_lay
                                      float* weights, void* ws, size_t ws_bytes, void* stream);
 
 /* The fused E-step + M-step (Algorithm 1, both steps, for all prefixes at
- * once; Algorithm 2 as the oracle; Eqs. 1, 2, 11, beta, zeta, advance): one
- * persistent kernel runs sampling, verification, utilities, weights, loss and
- * gradient over all prefixes, with the results of vsd_sample_paths,
- * vsd_verify_paths and vsd_weighted_loss_fwd_bwd.  Arguments as for those
+ * once; Algorithm 2 as the oracle; Eqs. 1, 2, 11, beta, zeta, advance): two
+ * kernels (rows with paths and M-steps, then the gradient), or for long rows
+ * with a gradient one persistent kernel, run sampling, verification,
+ * utilities, weights, loss and gradient over all prefixes, with the results
+ * of vsd_sample_paths, vsd_verify_paths and vsd_weighted_loss_fwd_bwd; which
+ * of the two is a matter of speed only.  Arguments as for those
  * calls: draft, target [R][V] of `dtype`; u_draft, u_accept, u_correct [R];
  * ref_logkappa optional [B][D]; params NULL for the defaults (App. F:
  * w(l) = 1.05^l, tau = 0.2).  Required members of `out`: tokens, accept_len,

@@ -380,7 +380,7 @@ def weighted_loss_fwd_bwd(draft, estep, K, D, T, prm=None, workspace=None, grad=
 
 def estep_mstep(draft, target, u_draft, u_accept, u_correct, K, D, T, ref_logkappa=None,
                 prm=None, workspace=None, out=None, full=True, grad=True):
-    """The fused E-step + M-step (one persistent kernel).  Returns the outputs
+    """The fused E-step + M-step (vsd_estep_mstep).  Returns the outputs
     (grad=False: no dense gradient, for lmhead_backward on the same workspace)."""
     _need_cuda(draft, target, u_draft, u_accept, u_correct, ref_logkappa)
     V = draft.shape[-1]
@@ -475,7 +475,9 @@ def lmhead_backward(hidden, weight, draft_logits, K, D, T, workspace, prm=None,
     on bf16 draft logits) on the same workspace: returns {"d_hidden": [R][H],
     "d_weight": [V][H]} (float32), the M-step gradient of the draft logits
     carried through logits = hidden . weight^T.  Pass False to skip one, or a
-    float32 tensor to write into."""
+    float32 tensor to write into.  Takes R*V bf16 values of scratch from
+    PyTorch's allocator for the call (vsd_lmhead_backward_scratch); without room
+    for them the gradient is made on chip, slower."""
     _need_cuda(hidden, weight, draft_logits)
     V, H = weight.shape
     R = hidden.numel() // H
