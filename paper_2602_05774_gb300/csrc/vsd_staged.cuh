@@ -56,10 +56,13 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
         if (given)
             stream_target_tables<T>(rg, y, V, 0, nch, tab, P.ts.c, policy_evict_first(), P.status);
     }
-    if (!given)
+    if (!given) {
+        // (unaligned rows behind the LM head: that kernel still writes the logits)
+        if (!VEC && P.xtab_given) grid_wait();
         stream_tables<T, VEC, true>(rg, x, y, V, 0, nch, tab, P.ts.c,
                                     P.gnseg ? policy_evict_last() : policy_evict_first(),
                                     policy_evict_first(), P.status);
+    }
     // the kernel before this one (the clearing of the counters, or the LM
     // head) has ended; what was read so far is the call's input
     grid_wait();

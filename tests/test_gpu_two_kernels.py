@@ -80,3 +80,39 @@ def test_persistent_kernel_equals_two_kernels(vsd, V, R, dtype, kind, kl, T):
         for n in ("tokens", "corr_tokens", "logkappa", "weights", "row_stats"):
             m = whole[n].view(2, -1)[i]
             assert torch.equal(m, part[n].reshape(-1)), n
+
+
+@pytest.mark.parametrize("offset", ["target", "grad"])
+def test_lmhead_with_unaligned_rows_waits_for_its_logits(vsd, offset):
+    """Rows that start off a 16-byte boundary, behind the LM head: the row kernel
+    starts before the head's product has ended and must not read the logits
+    until then.  Equal bit for bit to the E-step + M-step on the logits left."""
+    B, K, D, V, H = 32, 8, 8, 32000, 1024
+    R = B * K * D
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    hidden = rnd(R, H).bfloat16()
+    weight = (rnd(V, H) / H ** 0.5).bfloat16()
+    off = lambda want: 1 if offset == want else 0  # noqa: E731
+    target = torch.empty(R * V + 1, dtype=torch.bfloat16, device="cuda")
+    target = target[off("target"):][:R * V].view(R, V).copy_(2 * rnd(R, V))
+    u = [torch.rand(R, device="cuda", generator=g) for _ in range(3)]
+    prm = vsd.params(like=target)
+    for _ in range(3):
+        logits = torch.full((R, V), float("nan"), dtype=torch.bfloat16, device="cuda")
+        res = []
+        for head in (True, False):
+            ws = vsd.new_workspace(vsd.layout(B, K, D, V), "cuda")
+            out = vsd.linear_outputs(B, K, D, V, "cuda", grad=False)
+            buf = torch.empty(R * V + 1, dtype=torch.bfloat16, device="cuda")
+            out["grad"] = buf[off("grad"):][:R * V].view(R, V)
+            if head:
+                vsd.lmhead_estep_mstep(hidden, weight, target, *u, K, D, 1.0, prm=prm,
+                                       workspace=ws, out=out, draft_logits=logits)
+            else:
+                vsd.estep_mstep(logits, target, *u, K, D, 1.0, prm=prm, workspace=ws, out=out)
+            torch.cuda.synchronize()
+            assert vsd.device_status(ws) == (0, 0)
+            res.append(out)
+        for k, want in res[1].items():
+            assert torch.equal(res[0][k], want), k
