@@ -24,6 +24,7 @@
 //                at the row.
 #pragma once
 
+#include <cstddef>
 #include <type_traits>
 
 #include "vsd_common.cuh"
@@ -260,16 +261,26 @@ __device__ __forceinline__ void ring_init(Ring<S>* rg, uint64_t timeout_ns) {
     __syncthreads();
 }
 
-// Dynamic shared memory: [Ring (vector rows only), or MIN bytes if that is
-// more][chunk table].
+// Dynamic shared memory: [Ring (vector rows only)][chunk table].  A kernel that
+// later uses MIN bytes from the start for something else gets the ring moved up
+// so far that those bytes end with the ring's chunk data: the memory of an
+// mbarrier in use may hold nothing else (M-step scratch that reached over the
+// barriers read their words back as its own values, about once in 600 M-steps
+// behind the LM head).
+template <int S, size_t MIN = 0> __host__ __device__ constexpr size_t ring_offset() {
+    constexpr size_t data = sizeof(Ring<S>::data), more = MIN > data ? MIN - data : 0;
+    return (more + 127) / 128 * 128;
+}
 template <int S, size_t MIN = 0> __host__ __device__ constexpr size_t ring_bytes() {
-    return sizeof(Ring<S>) > MIN ? sizeof(Ring<S>) : (MIN + 127) / 128 * 128;
+    return ring_offset<S, MIN>() + sizeof(Ring<S>);
 }
 template <bool VEC, size_t MIN = 0, int S>
 __device__ __forceinline__ void smem_views(unsigned char* dsm, Ring<S>*& rg, float4*& tab,
                                            uint64_t timeout_ns) {
     if (VEC) {
-        rg = reinterpret_cast<Ring<S>*>(dsm);
+        static_assert(ring_offset<S, MIN>() + offsetof(Ring<S>, bar2) >= MIN,
+                      "the barriers lie beyond the bytes used for something else");
+        rg = reinterpret_cast<Ring<S>*>(dsm + ring_offset<S, MIN>());
         tab = reinterpret_cast<float4*>(dsm + ring_bytes<S, MIN>());
         ring_init(rg, timeout_ns);
     } else {

@@ -27,7 +27,8 @@
 namespace vsd {
 
 // Dynamic shared memory: [ring][chunk table]; the M-step's scratch takes the
-// ring's place (vector rows) or follows the table.
+// place of the ring's chunk data, not of its barriers (vector rows), or follows
+// the table.
 inline size_t staged_smem_bytes(int nch, bool vec) {
     return stream_smem_bytes<kRowStages, sizeof(WeightsShared)>(nch, vec) +
            (vec ? 0 : sizeof(WeightsShared));

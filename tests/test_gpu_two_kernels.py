@@ -116,3 +116,30 @@ def test_lmhead_with_unaligned_rows_waits_for_its_logits(vsd, offset):
             res.append(out)
         for k, want in res[1].items():
             assert torch.equal(res[0][k], want), k
+
+
+def test_mstep_scratch_is_its_own(vsd):
+    """The M-step's scratch shares shared memory with the row stream's copies,
+    but not with their barriers: the same call gives the same weights and loss
+    each time (with the barriers' words in the scratch, one call in ten here had
+    a prefix whose zeta held them)."""
+    B, K, D, V, H = 64, 8, 8, 32000, 4096
+    R = B * K * D
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *s: torch.randn(*s, device="cuda", generator=g).bfloat16()  # noqa: E731
+    hidden, weight, target = rnd(R, H), rnd(V, H) / 64, rnd(R, V) * 2
+    u = [torch.rand(R, device="cuda", generator=g) for _ in range(3)]
+    prm = vsd.params(like=target)
+    ws = vsd.new_workspace(vsd.layout(B, K, D, V), "cuda")
+    logits = torch.empty(R, V, dtype=torch.bfloat16, device="cuda")
+    outs = [vsd.linear_outputs(B, K, D, V, "cuda", grad=False) for _ in range(60)]
+    for o in outs:
+        vsd.lmhead_estep_mstep(hidden, weight, target, *u, K, D, 1.0, prm=prm, workspace=ws,
+                               out=o, draft_logits=logits)
+    torch.cuda.synchronize()
+    assert vsd.device_status(ws) == (0, 0)
+    most = torch.stack([o["weights"].view(torch.int32) for o in outs]).mode(dim=0).values
+    assert torch.isfinite(most.view(torch.float32)).all()
+    for o in outs:
+        assert torch.equal(o["weights"].view(torch.int32), most)
+        assert torch.equal(o["loss"], outs[0]["loss"])
