@@ -16,7 +16,7 @@
 // What bounds a single wave of rows (R up to 8 per SM) is the chain of one
 // path: at 768 rows of V = 32000 the row streams 11 us, its tail takes 7, the
 // path's residual draw 11, its epilogue 3, the M-step 9, the counters in
-// between 2, the gradient 14 (69 us a call; 119 on the persistent kernel).
+// between 2, the gradient 14 (65 us a call; 119 on the persistent kernel).
 // Those steps run once per block and are short of instructions as much as of
 // data, so loops in them are kept rolled.
 #pragma once
