@@ -265,7 +265,7 @@ __device__ __forceinline__ void ring_init(Ring<S>* rg, uint64_t timeout_ns) {
 // later uses MIN bytes from the start for something else gets the ring moved up
 // so far that those bytes end with the ring's chunk data: the memory of an
 // mbarrier in use may hold nothing else (M-step scratch that reached over the
-// barriers read their words back as its own values, about once in 600 M-steps
+// barriers read their words back as its own values, about once in 900 M-steps
 // behind the LM head).
 template <int S, size_t MIN = 0> __host__ __device__ constexpr size_t ring_offset() {
     constexpr size_t data = sizeof(Ring<S>::data), more = MIN > data ? MIN - data : 0;

@@ -121,7 +121,7 @@ def test_lmhead_with_unaligned_rows_waits_for_its_logits(vsd, offset):
 def test_mstep_scratch_is_its_own(vsd):
     """The M-step's scratch shares shared memory with the row stream's copies,
     but not with their barriers: the same call gives the same weights and loss
-    each time (with the barriers' words in the scratch, one call in ten here had
+    each time (with the barriers' words in the scratch, about one call in 14 had
     a prefix whose zeta held them)."""
     B, K, D, V, H = 64, 8, 8, 32000, 4096
     R = B * K * D
