@@ -23,7 +23,10 @@
 //
 // Every wait is bounded; a wait that runs out sets VSD_STATUS_TIMEOUT in the
 // status word, and the pair winds down: it waits (again bounded) for its MMAs
-// and copies in flight, then frees its tensor memory.
+// and copies in flight, then frees its tensor memory.  In every case a CTA
+// leaves only when the arrivals of all commits onto its barriers have landed:
+// they come from the tensor core, after the thread that committed went on, and
+// its shared memory may be another block's as soon as it has left.
 #pragma once
 
 #include "vsd_tc.cuh"
@@ -53,6 +56,7 @@ struct Bars {
     uint32_t tmem_base;
     int err;
     uint32_t peer_it;         // CTA 0: stages the other CTA's producer issued
+    uint32_t freed, filled;   // commits the issuer made onto empty[] and acc_full[]
 };
 // [alignment][stages][the epilogue's staging][barriers]
 template <class Epi> constexpr size_t smem_bytes() {
@@ -111,6 +115,9 @@ __device__ __forceinline__ void commit_one(uint64_t* bar) {
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(bar)
                  : "memory");
+}
+__device__ __forceinline__ void store_cluster(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
@@ -370,6 +377,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         mbar_init(&sb->drain, 1);
         sb->err = 0;
         sb->peer_it = 0;
+        sb->freed = sb->filled = 0;
         sb->timeout_ns = timeout_ns;
         mbar_init_fence();
     }
@@ -423,9 +431,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 }
             }
             issued = it;
-            if (rank == 1)
-                asm volatile("st.shared::cluster.u32 [%0], %1;"
-                             :: "r"(map_rank(&sb->peer_it, 0)), "r"(it) : "memory");
+            if (rank == 1) store_cluster(map_rank(&sb->peer_it, 0), it);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer
@@ -467,6 +473,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
             commit_one(&sb->drain);
             wait_phase_drain(&sb->drain, 0, timeout_ns);
+            for (uint32_t r = 0; r < 2; ++r) {  // (lt: tiles whose accumulator was committed)
+                store_cluster(map_rank(&sb->freed, r), it);
+                store_cluster(map_rank(&sb->filled, r), (uint32_t)lt);
+            }
         }
     } else {
         // ------------------------------------------------------ epilogue
@@ -500,6 +510,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     cluster_sync();  // no MMA is in flight any more, nothing more is issued
+    if (threadIdx.x == 0) {
+        // the arrivals of the commits onto this CTA's barriers have landed (the
+        // last phase of each barrier; the earlier ones have been waited for)
+        const uint32_t freed = *(volatile uint32_t*)&sb->freed;
+        const uint32_t filled = *(volatile uint32_t*)&sb->filled;
+        for (uint32_t j = freed > (uint32_t)kStages ? freed - kStages : 0; j < freed; ++j)
+            wait_phase_drain(&sb->empty[j % kStages], (j / kStages) & 1u, timeout_ns);
+        for (uint32_t j = filled > 2u ? filled - 2u : 0; j < filled; ++j)
+            wait_phase_drain(&sb->acc_full[j & 1u], (j >> 1) & 1u, timeout_ns);
+    }
     if (rank == 0 && threadIdx.x == 0) {
         // The copies of the last stages have landed.  (Always so unless a wait
         // ran out; the two producers may then have stopped at different

@@ -61,3 +61,28 @@ def test_backward_tiles_within_bound(vsd, B, K, D, V, H, scratch):
         bound = a.shape[1] * 2.0 ** -24 * (a.abs() @ b.abs()) + 1e-30
         err = (bw[name].double() - a @ b).abs()
         assert bool((err <= bound).all()), "%s off by %g" % (name, float((err - bound).max()))
+
+
+@pytest.mark.parametrize("M,N", [(1, 8), (256, 1024), (300, 1032)])  # 1 tile, a chunk, two units
+@pytest.mark.parametrize("kb", [1, 2, 5, 6, 7, 12, 13])  # K blocks: around the ring's six stages
+def test_every_commit_is_waited_for(vsd, M, N, kb):
+    """The pair leaves once the arrivals of its last commits have landed, at
+    fewer K blocks than the ring has stages, as many, and more; a wait for a
+    phase that never comes would show as its 2 s limit.  Inputs whose partial
+    sums are exact in float32: the float64 product, rounded once."""
+    K = 64 * kb - 8
+    g = torch.Generator(device="cuda").manual_seed(K + M)
+    h = torch.randint(-2, 3, (M, K), generator=g, device="cuda").bfloat16()
+    w = (torch.randint(-64, 65, (N, K), generator=g, device="cuda").float() / 256).bfloat16()
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    vsd.lmhead_logits(h, w, workspace=ws)
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    a.record()
+    got = [vsd.lmhead_logits(h, w, workspace=ws) for _ in range(4)]
+    b.record()
+    torch.cuda.synchronize()
+    assert vsd.device_status(ws) == (0, 0)
+    assert a.elapsed_time(b) < 500
+    want = (h.double() @ w.double().t()).bfloat16()
+    for x in got:
+        assert torch.equal(x, want)
