@@ -107,7 +107,9 @@ typedef struct {
     int32_t test_never_publish; /* test hook, normally 0: if nonzero the fused kernel
                                  never publishes a prefix's M-step, so every gradient
                                  wait runs out after wait_timeout_ns, no gradient row
-                                 is written and VSD_STATUS_TIMEOUT is set            */
+                                 is written and VSD_STATUS_TIMEOUT is set; 2: instead,
+                                 the waits for the rows' copies run out (rows 16-byte
+                                 aligned; results undefined, VSD_STATUS_TIMEOUT)     */
     double kl_weight;  /* VSD (KL) (App., Eq. klv): 0 = none; else loss_b gains
                           kl_weight (1/K) sum over the prefix's rows of the top-K
                           renormalised cross-entropy -sum_{x in top-K of p}

@@ -275,7 +275,8 @@ void set_params(Problem<T>& P, const vsd_params& p) {
     P.zeta_mode = p.zeta_mode;
     P.grad_bf16 = p.grad_dtype == VSD_BF16;
     P.timeout_ns = p.wait_timeout_ns ? p.wait_timeout_ns : kDefaultTimeoutNs;
-    P.inject_wait_fault = p.test_never_publish;
+    P.hold_copies = p.test_never_publish == 2;
+    P.inject_wait_fault = p.test_never_publish && !P.hold_copies;
     P.kl_weight = p.kl_weight;
     P.kl_topk = p.kl_weight != 0.0 ? p.kl_topk : 0;
     P.kl_scale = p.kl_weight / ((double)P.B * (double)P.K * P.ts.Td);

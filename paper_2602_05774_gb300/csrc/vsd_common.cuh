@@ -59,6 +59,12 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
+// A wait that ran out may have had a short limit of the caller's; the copies it
+// leaves in flight are given 2 ms at least to land.
+__device__ __forceinline__ uint64_t drain_ns(uint64_t timeout_ns) {
+    return timeout_ns > 2000000ull ? timeout_ns : 2000000ull;
+}
+
 // ---------------------------------------------------------------- loads
 __device__ __forceinline__ uint64_t policy_evict_first() {
     uint64_t p;

@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
     __shared__ RowShared sh;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     const int r = blockIdx.x;
     row_pass<T, VEC, false, kSampleToken, false>(P, r, rg, tab, sh);
@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kThreads) k_ref_rows(Problem<T> P) {
     __shared__ RowShared sh;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     row_pass<T, VEC, true, kNoToken, true>(P, blockIdx.x, rg, tab, sh);
 }
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
     __shared__ KlRec kslot[kSlots];  // VSD (KL): the top-K terms of a gradient job's row
     Ring<kStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp < kWarps) {  // ------------------------------- streaming warps

@@ -131,7 +131,8 @@ struct Problem {
     double kl_scale;              // kl_weight / (B K T), the gradient factor
     KlRec* klr;                   // [R] the rows' terms
     int grad_bf16;
-    int inject_wait_fault;
+    int inject_wait_fault;        // test hooks: a prefix is never published,
+    int hold_copies;              // the ring's barriers never complete
     uint64_t timeout_ns;
     // workspace
     int* status;
@@ -245,14 +246,15 @@ template <int S> struct Ring {
 };
 
 // Every thread of the block calls it; warps beyond the streaming warps (the
-// fused kernel's control warp) own no ring slots.
+// fused kernel's control warp) own no ring slots.  hold (a test hook): barriers
+// that wait for one arrival more than they get, so that every wait runs out.
 template <int S>
-__device__ __forceinline__ void ring_init(Ring<S>* rg, uint64_t timeout_ns) {
+__device__ __forceinline__ void ring_init(Ring<S>* rg, uint64_t timeout_ns, bool hold) {
     if (threadIdx.x == 0) rg->timeout_ns = timeout_ns;
     if ((threadIdx.x & 31) == 0 && (threadIdx.x >> 5) < kWarps) {
         const int w = threadIdx.x >> 5;
-        for (int st = 0; st < S; ++st) mbar_init(&rg->bar2[w][st], 1);
-        for (int st = 0; st < 2 * S; ++st) mbar_init(&rg->bar1[w][st], 1);
+        for (int st = 0; st < S; ++st) mbar_init(&rg->bar2[w][st], hold ? 2 : 1);
+        for (int st = 0; st < 2 * S; ++st) mbar_init(&rg->bar1[w][st], hold ? 2 : 1);
         rg->pos2[w] = 0;
         rg->pos1[w] = 0;
         rg->broken[w] = 0;
@@ -276,13 +278,13 @@ template <int S, size_t MIN = 0> __host__ __device__ constexpr size_t ring_bytes
 }
 template <bool VEC, size_t MIN = 0, int S>
 __device__ __forceinline__ void smem_views(unsigned char* dsm, Ring<S>*& rg, float4*& tab,
-                                           uint64_t timeout_ns) {
+                                           uint64_t timeout_ns, bool hold) {
     if (VEC) {
         static_assert(ring_offset<S, MIN>() + offsetof(Ring<S>, bar2) >= MIN,
                       "the barriers lie beyond the bytes used for something else");
         rg = reinterpret_cast<Ring<S>*>(dsm + ring_offset<S, MIN>());
         tab = reinterpret_cast<float4*>(dsm + ring_bytes<S, MIN>());
-        ring_init(rg, timeout_ns);
+        ring_init(rg, timeout_ns, hold);
     } else {
         rg = nullptr;
         tab = reinterpret_cast<float4*>(dsm);
@@ -300,6 +302,18 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, int* s
             atomicOr(status, VSD_STATUS_TIMEOUT);
             return false;
         }
+    }
+}
+
+// After a wait that ran out: the copies in flight, slots q0 .. q1 - 1 in order,
+// land before the warp goes on (again bounded), since the ring's memory serves
+// rescans and the M-step and is another block's once this one has ended.
+static __device__ __noinline__ void ring_drain(uint64_t* bars, int ns, int q0, int q1,
+                                               uint64_t timeout_ns) {
+    for (int q = q0; q < q1; ++q) {
+        const uint64_t t0 = global_timer_ns();
+        while (!mbar_try_wait(&bars[q % ns], (uint32_t)(q / ns) & 1u))
+            if (global_timer_ns() - t0 > drain_ns(timeout_ns)) break;
     }
 }
 
@@ -340,13 +354,16 @@ __device__ __forceinline__ void ring_stream(Ring<S>* rg, const T* x, const T* y,
         bulk_g2s(xbuf(slot), x + e0, bytes, bar, polx);
         if (HAS_Y) bulk_g2s(rg->data[warp][slot][1], y + e0, bytes, bar, poly);
     };
-    if (lane == 0)
+    if (lane == 0 && !broken)
         for (int j = 0; j < nj && j < NS; ++j) issue(j);
     for (int j = 0; j < nj; ++j) {
         const int slot = (pos + j) % NS;
         const uint32_t parity = (uint32_t)((pos + j) / NS) & 1u;
-        bool ok = broken ? false : ring_wait(&bars[slot], parity, status, timeout_ns);
-        broken = __any_sync(0xffffffffu, !ok);
+        const bool ok = broken ? false : ring_wait(&bars[slot], parity, status, timeout_ns);
+        if (__any_sync(0xffffffffu, !ok) && !broken) {
+            broken = true;
+            ring_drain(bars, NS, pos + j, pos + min(nj, j + NS), timeout_ns);
+        }
         const int ch = cfirst + j * cstride;
         const int64_t e0 = (int64_t)ch * CE;
         const uint4* sx = xbuf(slot);

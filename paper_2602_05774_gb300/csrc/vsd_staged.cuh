@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
     __shared__ int s_last;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC, sizeof(WeightsShared)>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC, sizeof(WeightsShared)>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     const int r = blockIdx.x, D = P.D, K = P.K, nch = P.nch;
     const int64_t V = P.V;

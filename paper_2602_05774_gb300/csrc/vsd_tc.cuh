@@ -138,7 +138,7 @@ __device__ __forceinline__ void wait_phase_drain(uint64_t* bar, uint32_t parity,
                                                  uint64_t timeout_ns) {
     const uint64_t t0 = global_timer_ns();
     while (!mbar_try_wait(bar, parity))
-        if (global_timer_ns() - t0 > timeout_ns) return;
+        if (global_timer_ns() - t0 > vsd::drain_ns(timeout_ns)) return;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {

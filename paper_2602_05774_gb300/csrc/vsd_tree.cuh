@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1)
     __shared__ RowShared sh;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
     int kids = 0;
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
     __shared__ int s_path, s_best, s_maxd, s_any, s_first;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const vsd_tree_outputs& o = P.tout;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_rows(Pr
     __shared__ RowShared sh;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
     const int64_t V = P.V;
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     __shared__ unsigned char s_acc[1024];
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1134,7 +1134,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_row
     __shared__ SeqCtl ct;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
     const SeqKids kids = seq_kids(reinterpret_cast<unsigned char*>(tab + P.nch), P.N);
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N;
@@ -1171,7 +1171,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     __shared__ RowShared rsh;
     Ring<kRowStages>* rg;
     float4* tab;
-    smem_views<VEC>(dsm, rg, tab, P.timeout_ns);
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     TreeSeqShared& sh = *reinterpret_cast<TreeSeqShared*>(tab + P.nch);
     grid_wait();
     const int N = P.N, b = blockIdx.x, n0 = b * N;

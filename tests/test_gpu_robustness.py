@@ -127,3 +127,38 @@ def test_lattice_output_distribution_is_target(vsd):
     hist = torch.bincount(o["corr_tokens"].long().cpu(), minlength=4).double() / Bn
     assert torch.equal(hist, pp)
     assert o["accept"].double().mean().item() == 0.75
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("wait_ns", [1, 1_000_000])
+def test_row_copies_that_never_complete_are_reported(vsd, dtype, wait_ns):
+    """The row kernels' waits for their copies run out (barriers that wait for an
+    arrival that nothing makes): each block lets its copies land and ends, with
+    the timeout bit in the status word, and the next call is clean.  The waits
+    before the call's counters are cleared are among them (one row: no later
+    block sets the bit again)."""
+    from paper_2602_05774_gb300 import inputs
+    for B, K, D, V in ((1, 1, 1, 4096), (2, 3, 4, 4096)):
+        p = _cuda(inputs.linear_problem(B, K, D, V, dtype, "gauss", seed=9))
+        ws = vsd.new_workspace(vsd.layout(B, K, D, V), "cuda")
+        good = _run(vsd, p, workspace=ws)
+        assert vsd.device_status(ws) == (0, 0)
+        prm = vsd.params(like=p["draft"], wait_timeout_ns=wait_ns, test_never_publish=2,
+                         kl_weight=0.5)
+        _run(vsd, p, prm=prm, workspace=ws)
+        code, bits = vsd.device_status(ws)
+        assert code == 4 and bits & vsd.STATUS_TIMEOUT
+        again = _run(vsd, p, workspace=ws)
+        assert vsd.device_status(ws) == (0, 0)
+        for k in good:
+            assert torch.equal(good[k], again[k]), k
+    p = _cuda(inputs.tree_problem(2, 8, 3, 3, 512, seed=4, dtype=dtype))
+    ws = vsd.new_workspace(vsd.layout(2, V=512, N=8, parent=p["parent"]), "cuda")
+    prm = vsd.params(like=p["draft"], wait_timeout_ns=wait_ns, test_never_publish=2)
+    vsd.tree_estep_mstep(p["draft"], p["target"], p["parent"], p["tokens"], p["u_accept"],
+                         p["u_correct"], 1.0, prm=prm, workspace=ws)
+    code, bits = vsd.device_status(ws)
+    assert code == 4 and bits & vsd.STATUS_TIMEOUT
+    vsd.tree_estep_mstep(p["draft"], p["target"], p["parent"], p["tokens"], p["u_accept"],
+                         p["u_correct"], 1.0, workspace=ws)
+    assert vsd.device_status(ws) == (0, 0)
