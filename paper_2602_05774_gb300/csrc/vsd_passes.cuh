@@ -317,6 +317,13 @@ static __device__ __noinline__ void ring_drain(uint64_t* bars, int ns, int q0, i
     }
 }
 
+// A wait that ran out before grid_wait() may have set the status bit before the
+// kernel in front cleared the word: set again (every warp, after grid_wait()).
+template <int S> __device__ __forceinline__ void ring_report(const Ring<S>* rg, int* status) {
+    if ((threadIdx.x & 31) == 0 && rg->broken[threadIdx.x >> 5])
+        atomicOr(status, VSD_STATUS_TIMEOUT);
+}
+
 // Warp-level stream of this warp's chunks (ch0 + warp, ch0 + warp + kWarps,
 // ... < ch1) of row x (and y) through the ring; consume(ch, bx, by) gets each
 // chunk in registers (positions at or beyond V read as -inf).  Rows must be
@@ -1450,6 +1457,7 @@ __device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, R
     // (a programmatic dependent: what was read so far is the call's input; the
     // workspace is written from here on)
     grid_wait();
+    if constexpr (VEC) ring_report(rg, P.status);
     __syncthreads();
     row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh, rg, pdraw);
 }
