@@ -291,23 +291,9 @@ __device__ __forceinline__ void smem_views(unsigned char* dsm, Ring<S>*& rg, flo
     }
 }
 
-// Bounded wait on a slot; false (and the timeout status bit) if it ran out.
-__device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, int* status,
-                                          uint64_t timeout_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
-    for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (global_timer_ns() - t0 > timeout_ns) {
-            atomicOr(status, VSD_STATUS_TIMEOUT);
-            return false;
-        }
-    }
-}
-
-// After a wait that ran out: the copies in flight, slots q0 .. q1 - 1 in order,
-// land before the warp goes on (again bounded), since the ring's memory serves
-// rescans and the M-step and is another block's once this one has ended.
+// The copies in flight, slots q0 .. q1 - 1 in order, land (or another limit runs
+// out): after a wait that ran out, since the ring's memory serves rescans and the
+// M-step and is another block's once this one has ended.
 static __device__ __noinline__ void ring_drain(uint64_t* bars, int ns, int q0, int q1,
                                                uint64_t timeout_ns) {
     for (int q = q0; q < q1; ++q) {
@@ -316,12 +302,26 @@ static __device__ __noinline__ void ring_drain(uint64_t* bars, int ns, int q0, i
             if (global_timer_ns() - t0 > drain_ns(timeout_ns)) break;
     }
 }
-
-// A wait that ran out before grid_wait() may have set the status bit before the
-// kernel in front cleared the word: set again (every warp, after grid_wait()).
-template <int S> __device__ __forceinline__ void ring_report(const Ring<S>* rg, int* status) {
-    if ((threadIdx.x & 31) == 0 && rg->broken[threadIdx.x >> 5])
-        atomicOr(status, VSD_STATUS_TIMEOUT);
+// Bounded wait for the copies of slot q (NS slots; those up to q1 - 1 are issued).
+// False if it ran out: then they have landed, as far as they do, and the timeout
+// status bit is set, which the kernel in front may be about to clear until it has
+// ended.
+template <int NS>
+__device__ __forceinline__ bool ring_wait(uint64_t* bars, int q, int q1, int* status,
+                                          uint64_t timeout_ns) {
+    uint64_t* bar = &bars[q % NS];
+    const uint32_t parity = (uint32_t)(q / NS) & 1u;
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = global_timer_ns();
+    for (;;) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if (global_timer_ns() - t0 > timeout_ns) {
+            ring_drain(bars, NS, q, q1, timeout_ns);
+            grid_wait();
+            atomicOr(status, VSD_STATUS_TIMEOUT);
+            return false;
+        }
+    }
 }
 
 // Warp-level stream of this warp's chunks (ch0 + warp, ch0 + warp + kWarps,
@@ -365,12 +365,10 @@ __device__ __forceinline__ void ring_stream(Ring<S>* rg, const T* x, const T* y,
         for (int j = 0; j < nj && j < NS; ++j) issue(j);
     for (int j = 0; j < nj; ++j) {
         const int slot = (pos + j) % NS;
-        const uint32_t parity = (uint32_t)((pos + j) / NS) & 1u;
-        const bool ok = broken ? false : ring_wait(&bars[slot], parity, status, timeout_ns);
-        if (__any_sync(0xffffffffu, !ok) && !broken) {
-            broken = true;
-            ring_drain(bars, NS, pos + j, pos + min(nj, j + NS), timeout_ns);
-        }
+        const bool ok = broken ? false
+                               : ring_wait<NS>(bars, pos + j, pos + min(nj, j + NS), status,
+                                               timeout_ns);
+        broken = __any_sync(0xffffffffu, !ok);
         const int ch = cfirst + j * cstride;
         const int64_t e0 = (int64_t)ch * CE;
         const uint4* sx = xbuf(slot);
@@ -1457,7 +1455,6 @@ __device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, R
     // (a programmatic dependent: what was read so far is the call's input; the
     // workspace is written from here on)
     grid_wait();
-    if constexpr (VEC) ring_report(rg, P.status);
     __syncthreads();
     row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh, rg, pdraw);
 }

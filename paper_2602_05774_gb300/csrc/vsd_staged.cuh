@@ -67,7 +67,6 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
     // the kernel before this one (the clearing of the counters, or the LM
     // head) has ended; what was read so far is the call's input
     grid_wait();
-    if constexpr (VEC) ring_report(rg, P.status);
     if (given) {
         const float4* rtab = P.gtab + (int64_t)r * P.nch_ws;
         for (int ch = threadIdx.x; ch < nch; ch += kThreads)
