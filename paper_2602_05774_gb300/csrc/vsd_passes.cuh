@@ -2119,12 +2119,9 @@ __device__ void stream_grad(Ring<S>* rg, const Problem<T>& P, int r, int c0, int
         const float gq = cf.g * rec.izx;  // g / Z
         const bool dense = !(cf.g == 0.f && isfinite(rec.mx));
         const int nkl = KL ? min(max(kl->n, 0), kMaxKlTop) : 0;
-        const int64_t e1 = min(V, (int64_t)c1 * CE);
-        for (int64_t v = (int64_t)c0 * CE + threadIdx.x; v < e1; v += kThreads) {
-            // (rounded steps: no contraction into a fused multiply-add)
-            float o = dense ? __fmul_rn(
-                                  ex2(__fmul_rn(__fsub_rn(elem_value(x, v), rec.mx), P.ts.c)), gq)
-                            : 0.f;
+        const int64_t e0 = (int64_t)c0 * CE + threadIdx.x, e1 = min(V, (int64_t)c1 * CE);
+        // (rounded steps: no contraction into a fused multiply-add)
+        auto put = [&](int64_t v, float o) {
             if (v == cf.t0) o = __fsub_rn(o, cf.c0);
             if (v == cf.t1) o = __fsub_rn(o, cf.c1);
             for (int k = 0; k < nkl; ++k)
@@ -2133,6 +2130,14 @@ __device__ void stream_grad(Ring<S>* rg, const Problem<T>& P, int r, int c0, int
                 g[v] = __float2bfloat16_rn(o);
             else
                 g[v] = o;
+        };
+        // (two loops: a load under a condition would not be issued ahead of the
+        // element before it)
+        if (dense) {
+            for (int64_t v = e0; v < e1; v += kThreads)
+                put(v, __fmul_rn(ex2(__fmul_rn(__fsub_rn(elem_value(x, v), rec.mx), P.ts.c)), gq));
+        } else {
+            for (int64_t v = e0; v < e1; v += kThreads) put(v, 0.f);
         }
     } else {
         constexpr int NP = PV / 2;
