@@ -112,9 +112,12 @@ __device__ __forceinline__ void commit_one(uint64_t* bar) {
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
         :: "r"(smem_u32(bar)) : "memory");
 }
+// Arrive on a barrier of either CTA.  What it hands over is tensor memory, which
+// the tcgen05 fences order; a release at cluster scope would make the warp wait
+// for its global stores too, about a microsecond a tile (M = 4096, N = 128256,
+// K = 256: 583 us with it, 474 now).
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(bar)
-                 : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" :: "r"(bar) : "memory");
 }
 __device__ __forceinline__ void store_cluster(uint32_t addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
@@ -157,23 +160,30 @@ struct Work {
 };
 
 // Chunk order: pairs take units of one 256-row M tile by one 1024-column chunk
-// (four tiles in turn), M tile fastest, so that an epilogue thread can carry
-// its row's statistics over the chunk.
+// (per = kPerChunk tiles in turn), M tile fastest, so that an epilogue thread can
+// carry its row's statistics over the chunk; without statistics a unit is one
+// tile (per = 1), which spreads few units over the pairs (M = 256, K = 4096: N =
+// 8000, 8 units of four tiles on 76 pairs 89 us, 32 of one 36; N = 128256 218, 204).
 struct ChunkOrder {
-    int mt, ntn, nk, nunits, u, nt, step;
+    int mt, ntn, nk, nunits, u, nt, step, per;
     static constexpr int kPerChunk = 1024 / BN;
-    __device__ ChunkOrder(int M, int N, int K, int c, int nc) {
+    __host__ __device__ static long long units(int M, int N, int per) {
+        const int ntn = (N + BN - 1) / BN;
+        return (long long)((M + 2 * BM - 1) / (2 * BM)) * ((ntn + per - 1) / per);
+    }
+    __device__ ChunkOrder(int M, int N, int K, int c, int nc, int per_) {
         mt = (M + 2 * BM - 1) / (2 * BM);
         ntn = (N + BN - 1) / BN;
         nk = (K + BK - 1) / BK;
-        nunits = mt * ((ntn + kPerChunk - 1) / kPerChunk);
+        per = per_;
+        nunits = (int)units(M, N, per);
         u = c;
         nt = 0;
         step = nc;
     }
     __device__ bool next(Work& w) {
         if (u >= nunits) return false;
-        const int t0 = (u / mt) * kPerChunk, t1 = min(t0 + kPerChunk, ntn);
+        const int t0 = (u / mt) * per, t1 = min(t0 + per, ntn);
         w.m0 = (u % mt) * 2 * BM;
         w.n0 = (t0 + nt) * BN;
         w.kb0 = 0;
@@ -232,6 +242,9 @@ struct SplitOrder {
 // small K (d_weight at R = 672, H = 2888, V = 32000: 193 us with them, 114 now).
 struct StoreF32 {
     using Order = SplitOrder;
+    __device__ Order order(int M, int N, int K, int c, int nc) const {
+        return SplitOrder(M, N, K, c, nc);
+    }
     static constexpr int kStaging = 4 * 2 * 4096;
     CUtensorMap map;  // boxes of 32 x 32
     int M, N;
@@ -284,6 +297,12 @@ struct StoreF32 {
 // the hot path): tab[row * stride + chunk].xy = (max, sum 2^{(x - max) c}).
 struct StoreLogits {
     using Order = ChunkOrder;
+    __host__ __device__ static int per_unit(bool stats) {
+        return stats ? ChunkOrder::kPerChunk : 1;
+    }
+    __device__ Order order(int M, int N, int K, int c, int nc) const {
+        return ChunkOrder(M, N, K, c, nc, per_unit(tab != nullptr));
+    }
     static constexpr int kStaging = 0;
     __nv_bfloat16* out;
     int M, N;
@@ -398,7 +417,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            typename Epi::Order order(M, N, K, c, nc);
+            typename Epi::Order order = epi.order(M, N, K, c, nc);
             Work w;
             while (ok && !*(volatile int*)&sb->err && order.next(w)) {
                 const int m0 = w.m0 + (int)rank * BM, n0 = w.n0 + (int)rank * BH;
@@ -439,7 +458,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             uint32_t it = 0;
             int lt = 0;
             bool ok = true;
-            typename Epi::Order order(M, N, K, c, nc);
+            typename Epi::Order order = epi.order(M, N, K, c, nc);
             Work w;
             for (; ok && !*(volatile int*)&sb->err && order.next(w); ++lt) {
                 const int buf = lt & 1;
@@ -482,7 +501,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         // ------------------------------------------------------ epilogue
         const int q = warp & 3;  // TMEM lanes 32q .. 32q + 31
         int lt = 0;
-        typename Epi::Order order(M, N, K, c, nc);
+        typename Epi::Order order = epi.order(M, N, K, c, nc);
         typename Epi::State st;
         epi.init(st, staging, q);
         Work w;
@@ -497,6 +516,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll 1
             for (int cc = 0; cc < BN / 32; ++cc) {
                 uint32_t r[32];
+                __syncwarp();  // (lanes beyond M do not store)
                 tmem_ld32(taddr + 32u * cc, r);
                 epi.columns(st, w, row, w.n0 + 32 * cc, r);
             }

@@ -94,8 +94,8 @@ cudaError_t lmhead_gemm(const void* hidden, const void* weight, int M, int N, in
     auto kern = vsd_g2::k_gemm2<false, false, vsd_g2::StoreLogits>;
     cudaError_t e = ensure_dyn_smem((const void*)kern, vsd_g2::smem_bytes<vsd_g2::StoreLogits>());
     if (e != cudaSuccess) return e;
-    const long long nunits = (long long)((M + 2 * vsd_g2::BM - 1) / (2 * vsd_g2::BM)) *
-                             ((N + 1023) / 1024);
+    const long long nunits = vsd_g2::ChunkOrder::units(
+        M, N, vsd_g2::StoreLogits::per_unit(chunk_tab != nullptr));
     const int pairs = device_sm_count() / 2;
     const int grid = 2 * (int)(nunits < pairs ? nunits : pairs);
     const vsd_g2::StoreLogits epi{static_cast<__nv_bfloat16*>(logits), M, N, chunk_tab,
