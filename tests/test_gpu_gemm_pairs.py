@@ -63,11 +63,13 @@ def test_backward_tiles_within_bound(vsd, B, K, D, V, H, scratch):
         assert bool((err <= bound).all()), "%s off by %g" % (name, float((err - bound).max()))
 
 
-@pytest.mark.parametrize("M,N", [(1, 8), (256, 1024), (300, 1032)])  # 1 tile, a chunk, two units
-@pytest.mark.parametrize("kb", [1, 2, 5, 6, 7, 12, 13])  # K blocks: around the ring's six stages
+# few rows: one tile, several a CTA; pairs: one tile, a chunk, two units
+@pytest.mark.parametrize("M,N", [(1, 8), (128, 40008), (129, 8), (256, 1024), (300, 1032)])
+# K blocks: around the rings' four and six stages; 33: few tiles of few rows on pairs
+@pytest.mark.parametrize("kb", [1, 2, 4, 5, 6, 7, 12, 13, 33])
 def test_every_commit_is_waited_for(vsd, M, N, kb):
     """The pair leaves once the arrivals of its last commits have landed, at
-    fewer K blocks than the ring has stages, as many, and more; a wait for a
+    fewer K blocks than a ring has stages, as many, and more; a wait for a
     phase that never comes would show as its 2 s limit.  Inputs whose partial
     sums are exact in float32: the float64 product, rounded once."""
     K = 64 * kb - 8
