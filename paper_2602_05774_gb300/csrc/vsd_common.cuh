@@ -18,14 +18,13 @@ constexpr int kLoads = 4;                // 16-byte vectors per lane per chunk p
 #define VSD_STAGES 2
 #endif
 constexpr int kStages = VSD_STAGES;      // TMA ring depth per warp, persistent kernel
-// The same, one block per row: 16 KB of ring let eight blocks share an SM, so
-// that more rows stream while others are in their tails (64 heads of 64 rows,
+// One block per row: kRowStages, 16 KB of ring, lets eight blocks share an SM,
+// so that more rows stream while others are in their tails (64 heads of 64 rows,
 // V = 32000: LM head + E/M step 846 us with two stages and six blocks, 828 with
-// one; ten or twelve blocks spill and gain nothing).
-#ifndef VSD_ROW_STAGES
-#define VSD_ROW_STAGES 1
-#endif
-constexpr int kRowStages = VSD_ROW_STAGES;
+// one; ten or twelve blocks spill and gain nothing).  Where long rows are few, a
+// row's own stream bounds the call, and kDeepStages is faster (deep_ring).
+constexpr int kRowStages = 1;
+constexpr int kDeepStages = 2;
 constexpr int kRowBlocks = 8;
 constexpr double kLog2e = 1.4426950408889634073599246810019;
 constexpr double kLn2 = 0.69314718055994530941723212145818;

@@ -8,11 +8,11 @@
 namespace vsd {
 
 // ------------------------------------------------------------ separate kernels
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
@@ -30,11 +30,11 @@ __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
 
 // Rows along supplied greedy reference paths (Algorithm 2's z-bar): per row
 // the target's argmax and log min(1, p/q) there (row_pass with the argmax).
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads) k_ref_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
@@ -428,23 +428,19 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
 // ------------------------------------------------------------ launchers
 template <>
 cudaError_t Launch<VSD_T>::sample(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
-    if (vec) {
-        cudaError_t e = prep(k_sample<VSD_T, true>, smem);
-        if (e) return e;
-        return launch_after(k_sample<VSD_T, true>, P.R, kThreads, smem, s, P);
-    } else {
-        cudaError_t e = prep(k_sample<VSD_T, false>, smem);
-        if (e) return e;
-        return launch_after(k_sample<VSD_T, false>, P.R, kThreads, smem, s, P);
-    }
+    const size_t smem = row_smem_bytes(P.nch, vec, false);
+    auto kern = vec ? k_sample<VSD_T, true, kRowStages> : k_sample<VSD_T, false, kRowStages>;
+    cudaError_t e = prep(kern, smem);
+    if (e) return e;
+    return launch_after(kern, P.R, kThreads, smem, s, P);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::reference(const Problem<VSD_T>& P, bool vec, float* out,
                                      cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
-    auto kern = vec ? k_ref_rows<VSD_T, true> : k_ref_rows<VSD_T, false>;
+    const bool deep = deep_ring(vec, P.nch, P.R, P.nch < 256 ? 4 : 2);
+    const size_t smem = row_smem_bytes(P.nch, vec, deep);
+    auto kern = VSD_BY_RING(k_ref_rows, VSD_T);
     cudaError_t e = prep(kern, smem);
     if (e) return e;
     if ((e = launch_after(kern, P.R, kThreads, smem, s, P))) return e;

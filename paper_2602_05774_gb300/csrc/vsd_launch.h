@@ -63,6 +63,30 @@ template <int S, size_t MIN = 0> inline size_t stream_smem_bytes(int nch, bool v
     return (vec ? ring_bytes<S, MIN>() : 0) + table_smem_bytes(nch);
 }
 
+// Whether a kernel of one block per row takes the ring of kDeepStages: rows of
+// at least 48 chunks (96 KB), all of them resident at per_sm blocks per SM, so
+// that each row's own stream bounds the call.  us, one stage / two stages:
+//   verification, float32: V=65536 R=304 83 / 68, V=128256 R=304 141 / 113, R=608
+//     185 / 167; bf16: V=128256 R=304 87 / 74, R=608 107 / 102, R=4096 396 / 402
+//   E-step + M-step without a gradient, V=128256: float32 R=304 143 / 115, R=608
+//     180 / 172; bf16 R=304 88 / 80, R=608 111 / 119 (per_sm = 2)
+//   reference rows, bf16: V=128256 R=304 50 / 44, R=512 66 / 66; V=524288 R=304
+//     136 / 120, R=512 185 / 204 (per_sm = 2 from 256 chunks on)
+//   trees of 8 nodes, float32, V=128256 R=304: alone 130 / 101, sequential rule
+//     243 / 214, E-step + M-step 207 / 184
+inline bool deep_ring(bool vec, int nch, int64_t rows, int per_sm = 4) {
+    return vec && nch >= 48 && rows <= per_sm * (int64_t)device_sm_count();
+}
+// That kernel's instance (deep, vec: names in the launcher; the further template
+// arguments, each with a comma before it).
+#define VSD_BY_RING(kern, T_, ...)                                   \
+    (deep ? kern<T_, true __VA_ARGS__, kDeepStages>                  \
+          : vec ? kern<T_, true __VA_ARGS__, kRowStages> : kern<T_, false __VA_ARGS__, kRowStages>)
+template <size_t MIN = 0> inline size_t row_smem_bytes(int nch, bool vec, bool deep) {
+    return deep ? stream_smem_bytes<kDeepStages, MIN>(nch, vec)
+                : stream_smem_bytes<kRowStages, MIN>(nch, vec);
+}
+
 // The draft LM head on the tensor cores (vsd_lmhead.cu): logits = hidden .
 // weight^T, bf16 in, fp32 accumulation, bf16 out; status collects timeouts.
 bool lmhead_shape_ok(const void* hidden, const void* weight, const void* logits, int M, int N,

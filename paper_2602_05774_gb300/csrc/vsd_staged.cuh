@@ -29,14 +29,14 @@ namespace vsd {
 // Dynamic shared memory: [ring][chunk table]; the M-step's scratch takes the
 // place of the ring's chunk data, not of its barriers (vector rows), or follows
 // the table.
-inline size_t staged_smem_bytes(int nch, bool vec) {
-    return stream_smem_bytes<kRowStages, sizeof(WeightsShared)>(nch, vec) +
+inline size_t staged_smem_bytes(int nch, bool vec, bool deep) {
+    return row_smem_bytes<sizeof(WeightsShared)>(nch, vec, deep) +
            (vec ? 0 : sizeof(WeightsShared));
 }
 
 // XMODE: kSampleToken the whole E-step + M-step; kGivenToken the verification
 // of given tokens, which ends with the paths.
-template <typename T, bool VEC, bool KL, int XMODE>
+template <typename T, bool VEC, bool KL, int XMODE, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ union {
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
         PathShared path;
     } sh;
     __shared__ int s_last;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC, sizeof(WeightsShared)>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();

@@ -14,12 +14,13 @@ cudaError_t Launch<VSD_T>::grad_rows(const Problem<VSD_T>& P, bool vec, void* gr
 template <>
 cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad, bool grad_bf16,
                                   cudaStream_t s) {
-    const size_t smem = staged_smem_bytes(P.nch, vec);
-    const bool kl = P.kl_topk != 0;
-    auto rows = vec ? (kl ? k_em_rows<VSD_T, true, true, kSampleToken>
-                           : k_em_rows<VSD_T, true, false, kSampleToken>)
-                    : (kl ? k_em_rows<VSD_T, false, true, kSampleToken>
-                          : k_em_rows<VSD_T, false, false, kSampleToken>);
+    // (behind the LM head the smaller block fits beside its CTAs, and streams the
+    // target meanwhile)
+    const bool deep =
+        !P.xtab_given && deep_ring(vec, P.nch, P.R, sizeof(VSD_T) == 2 ? 2 : 4);
+    const size_t smem = staged_smem_bytes(P.nch, vec, deep);
+    auto rows = P.kl_topk ? VSD_BY_RING(k_em_rows, VSD_T, , true, kSampleToken)
+                          : VSD_BY_RING(k_em_rows, VSD_T, , false, kSampleToken);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     if ((e = launch_after(rows, P.R, kThreads, smem, s, P)) || !grad) return e;
@@ -28,9 +29,9 @@ cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad,
 
 template <>
 cudaError_t Launch<VSD_T>::verify(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages, sizeof(WeightsShared)>(P.nch, vec);
-    auto rows = vec ? k_em_rows<VSD_T, true, false, kGivenToken>
-                    : k_em_rows<VSD_T, false, false, kGivenToken>;
+    const bool deep = deep_ring(vec, P.nch, P.R);
+    const size_t smem = row_smem_bytes<sizeof(WeightsShared)>(P.nch, vec, deep);
+    auto rows = VSD_BY_RING(k_em_rows, VSD_T, , false, kGivenToken);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     return launch_after(rows, P.R, kThreads, smem, s, P);

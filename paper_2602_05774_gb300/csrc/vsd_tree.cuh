@@ -61,12 +61,12 @@ static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 //                       the outputs of the tree's nodes.
 // No block waits for another.  The row reads bound the first kernel, a few
 // dependent steps of one row the second.
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1)
     k_tree_verify_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
@@ -94,12 +94,12 @@ struct TreeVerifyNodes {
 };
 inline size_t tree_verify_smem_bytes(int N) { return (size_t)N * 21 + 16; }
 
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
     __shared__ int s_path, s_best, s_maxd, s_any, s_first;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     const int r = blockIdx.x, N = P.N, b = r / N, u = r - b * N, n0 = b * N;
@@ -245,11 +245,11 @@ __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
 // One block per node row: the row pass, then each child's token tested at the
 // row (one thread per child: Eq. 1, each branch alone), and the row's chunk
 // table kept in global memory for the draws.
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
@@ -289,12 +289,12 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_rows(Pr
 // chunk table and one chunk suffice.  Whether u is on an accepted path follows
 // from the acceptance bits of its ancestors, which are all known here; only
 // these few rows are read twice (64 trees of 60 nodes: about 300 of 3840).
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads) k_tree_draws(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ int s_par[1024], s_path;
     __shared__ unsigned char s_acc[1024];
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
@@ -948,8 +948,8 @@ __device__ __forceinline__ float seq_chunk(const uint4 (&bx)[kLoads], const uint
 }
 
 // One read of row r: tab[ch].y = the chunk sums of its masses (block).
-template <typename T, bool VEC>
-__device__ void seq_stream(const Problem<T>& P, int r, Ring<kRowStages>* rg, float4* tab, const SeqMass& sm) {
+template <typename T, bool VEC, int S>
+__device__ void seq_stream(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, const SeqMass& sm) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t V = P.V;
     const T* x = P.draft + (int64_t)r * V;
@@ -989,8 +989,8 @@ __device__ int seq_draw(const Problem<T>& P, int r, const float4* tab, const Tab
 // the others), for every child .la; tlist[r] = the accepted child, 0 if u has
 // no children, -1 if all were rejected, with the correction token in
 // es.corr[r].
-template <typename T, bool VEC>
-__device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, float4* tab, SeqCtl& ct,
+template <typename T, bool VEC, int S>
+__device__ void tree_seq_row(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, SeqCtl& ct,
                              const SeqKids& s) {
     const int N = P.N, b = r / N, u = r - b * N, n0 = b * N;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1127,12 +1127,12 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<kRowStages>* rg, f
 // the reads after a rejection, which come from L2.  64 trees of 60 nodes,
 // V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
 // block per tree, in an fp64 recursion per element over the earlier siblings.
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
     __shared__ SeqCtl ct;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     grid_launch_next();
@@ -1165,11 +1165,11 @@ struct TreeSeqShared {
 };
 
 // One block per tree: the accepted path, and every node's outputs.
-template <typename T, bool VEC>
+template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared rsh;
-    Ring<kRowStages>* rg;
+    Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
     TreeSeqShared& sh = *reinterpret_cast<TreeSeqShared*>(tab + P.nch);

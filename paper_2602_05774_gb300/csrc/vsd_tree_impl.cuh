@@ -11,26 +11,28 @@ namespace vsd {
 // ------------------------------------------------------------ launchers
 template <>
 cudaError_t Launch<VSD_T>::tree(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
-    auto rows = vec ? k_tree_verify_rows<VSD_T, true> : k_tree_verify_rows<VSD_T, false>;
+    const bool deep = deep_ring(vec, P.nch, P.R);
+    const size_t smem = row_smem_bytes(P.nch, vec, deep);
+    auto rows = VSD_BY_RING(k_tree_verify_rows, VSD_T);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
     const size_t sm2 = smem + tree_verify_smem_bytes(P.N);
-    auto nodes = vec ? k_tree_verify<VSD_T, true> : k_tree_verify<VSD_T, false>;
+    auto nodes = VSD_BY_RING(k_tree_verify, VSD_T);
     if ((e = prep(nodes, sm2))) return e;
     return launch_after(nodes, P.R, kThreads, sm2, s, P);
 }
 
 template <>
 cudaError_t Launch<VSD_T>::tree_seq(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec) + seq_smem_bytes(P.N);
-    auto rows = vec ? k_tree_seq_rows<VSD_T, true> : k_tree_seq_rows<VSD_T, false>;
+    const bool deep = deep_ring(vec, P.nch, P.R);
+    const size_t smem = row_smem_bytes(P.nch, vec, deep) + seq_smem_bytes(P.N);
+    auto rows = VSD_BY_RING(k_tree_seq_rows, VSD_T);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
-    const size_t sm2 = stream_smem_bytes<kRowStages>(P.nch, vec) + sizeof(TreeSeqShared);
-    auto seq = vec ? k_tree_seq<VSD_T, true> : k_tree_seq<VSD_T, false>;
+    const size_t sm2 = row_smem_bytes(P.nch, vec, deep) + sizeof(TreeSeqShared);
+    auto seq = VSD_BY_RING(k_tree_seq, VSD_T);
     if ((e = prep(seq, sm2))) return e;
     return launch_after(seq, P.B, kThreads, sm2, s, P);
 }
@@ -39,12 +41,13 @@ template <>
 cudaError_t Launch<VSD_T>::tree_em(const Problem<VSD_T>& P, bool vec,
                                    const vsd_tree_em_outputs& o, void* grad, bool grad_bf16,
                                    cudaStream_t s) {
-    const size_t smem = stream_smem_bytes<kRowStages>(P.nch, vec);
-    auto rows = vec ? k_tree_rows<VSD_T, true> : k_tree_rows<VSD_T, false>;
+    const bool deep = deep_ring(vec, P.nch, P.R);
+    const size_t smem = row_smem_bytes(P.nch, vec, deep);
+    auto rows = VSD_BY_RING(k_tree_rows, VSD_T);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
-    auto draws = vec ? k_tree_draws<VSD_T, true> : k_tree_draws<VSD_T, false>;
+    auto draws = VSD_BY_RING(k_tree_draws, VSD_T);
     if ((e = prep(draws, smem))) return e;
     if ((e = launch_after(draws, P.R, kThreads, smem, s, P))) return e;
     if ((e = prep(k_tree_em<VSD_T>, sizeof(TreeEmShared)))) return e;

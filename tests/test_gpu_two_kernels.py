@@ -143,3 +143,53 @@ def test_mstep_scratch_is_its_own(vsd):
     for o in outs:
         assert torch.equal(o["weights"].view(torch.int32), most)
         assert torch.equal(o["loss"], outs[0]["loss"])
+
+
+def _same_rows(few, many, copies, skip=()):
+    """Every output of `few` equals that of each copy in `many`, bit for bit."""
+    for k, a in few.items():
+        if k in skip or not torch.is_tensor(a):
+            continue
+        b = many[k].reshape(copies, -1)
+        for i in (0, copies // 2, copies - 1):
+            assert torch.equal(b[i], a.reshape(-1)), k
+
+
+@pytest.mark.parametrize("V,dtype", [(24576, "f32"), (50004, "f32"), (49152, "bf16")])
+def test_few_long_rows_equal_many(vsd, V, dtype):
+    """Few rows of at least 48 chunks take the deeper ring, the same rows 64 times
+    over the shallow one: the same results bit for bit."""
+    from paper_2602_05774_gb300 import inputs
+    K, D, n = 5, 2, 64  # 10 rows, 640
+    p = inputs.linear_problem(1, K, D, V, dtype, "gauss", "cuda", seed=V)
+    q = {k: (v.repeat(*([n] + [1] * (v.dim() - 1))) if torch.is_tensor(v) else v)
+         for k, v in p.items()}
+    prm = vsd.params(like=p["draft"], kl_weight=0.5)
+    a, b = _call(vsd, p, 1.0, prm), _call(vsd, q, 1.0, prm)
+    _same_rows(a, b, n, skip=("loss", "grad"))
+    assert torch.equal(b["loss"][:n], a["loss"][:1].expand(n))
+    assert torch.equal(b["grad"].view(n, -1)[n - 1], a["grad"].view(-1) / n)
+    s, t = (vsd.sample_paths(x["draft"], x["u_draft"], K, D, 1.0) for x in (p, q))
+    _same_rows(s, t, n)
+    _same_rows(*(vsd.verify_paths(x["draft"], x["target"], y["tokens"], x["u_accept"],
+                                  x["u_correct"], K, D, 1.0) for x, y in ((p, s), (q, t))), n)
+    r = [dict(r=vsd.reference_logkappa(x["draft"], x["target"], x["draft"].shape[0] // D, D, 1.0))
+         for x in (p, q)]
+    _same_rows(*r, n)
+
+
+@pytest.mark.parametrize("rule", [0, 1])
+def test_few_trees_with_long_rows_equal_many(vsd, rule):
+    from paper_2602_05774_gb300 import inputs
+    V, n = 49160, 80
+    p = {k: (v.cuda() if torch.is_tensor(v) else v)
+         for k, v in inputs.tree_problem(1, 8, 3, 3, V, seed=5).items()}
+    q = {k: (v.repeat(*([n] + [1] * (v.dim() - 1))) if torch.is_tensor(v) else v)
+         for k, v in p.items()}
+    f = lambda x: vsd.verify_tree(x["draft"], x["target"], x["parent"], x["tokens"],  # noqa: E731
+                                  x["u_accept"], x["u_correct"], 1.0, rule=rule)
+    _same_rows(f(p), f(q), n)
+    if rule == 0:
+        f = lambda x: vsd.tree_estep_mstep(x["draft"], x["target"], x["parent"],  # noqa: E731
+                                           x["tokens"], x["u_accept"], x["u_correct"], 1.0)
+        _same_rows(f(p), f(q), n, skip=("loss", "grad"))
