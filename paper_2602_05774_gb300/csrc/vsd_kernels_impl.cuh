@@ -426,10 +426,22 @@ __global__ void __launch_bounds__(kFusedThreads, VSD_FUSED_MIN_BLOCKS)
 }
 
 // ------------------------------------------------------------ launchers
+// Sampling streams one row a block at up to twelve blocks per SM.  Where that many
+// long rows are in turn, their scattered reads cost DRAM bandwidth, and six blocks
+// of twice the depth are faster; shorter rows are bound by their tails.  us, one
+// stage / two stages:
+//   float32  R=4096 V=8000  51 / 53, V=16000  98 / 72, V=49152 272 / 156;
+//            R=1216 (8 per SM) V=49152  57 / 80, R=2048 V=49152 150 / 98
+//   bf16     R=4096 V=32000 70 / 76, V=65536 111 / 115, V=100000 193 / 160
+template <typename T> static bool sample_deep(bool vec, int nch, int64_t rows) {
+    return vec && nch >= (sizeof(T) == 4 ? 48 : 96) && rows > 8 * (int64_t)device_sm_count();
+}
+
 template <>
 cudaError_t Launch<VSD_T>::sample(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
-    const size_t smem = row_smem_bytes(P.nch, vec, false);
-    auto kern = vec ? k_sample<VSD_T, true, kRowStages> : k_sample<VSD_T, false, kRowStages>;
+    const bool deep = sample_deep<VSD_T>(vec, P.nch, P.R);
+    const size_t smem = row_smem_bytes(P.nch, vec, deep);
+    auto kern = VSD_BY_RING(k_sample, VSD_T);
     cudaError_t e = prep(kern, smem);
     if (e) return e;
     return launch_after(kern, P.R, kThreads, smem, s, P);

@@ -178,6 +178,18 @@ def test_few_long_rows_equal_many(vsd, V, dtype):
     _same_rows(*r, n)
 
 
+@pytest.mark.parametrize("V,dtype", [(24580, "f32"), (98312, "bf16")])
+def test_sampling_many_long_rows_equals_few(vsd, V, dtype):
+    """More than eight rows per SM of at least 48 (float32) or 96 chunks are
+    sampled through the deeper ring, fewer through the shallow one."""
+    from paper_2602_05774_gb300 import inputs
+    n = 24
+    p = inputs.linear_problem(1, 64, 1, V, dtype, "gauss", "cuda", seed=V)
+    s, t = (vsd.sample_paths(p["draft"].repeat(m, 1), p["u_draft"].repeat(m), 64, 1, 1.0)
+            for m in (1, n))
+    _same_rows(s, t, n)
+
+
 @pytest.mark.parametrize("rule", [0, 1])
 def test_few_trees_with_long_rows_equal_many(vsd, rule):
     from paper_2602_05774_gb300 import inputs
