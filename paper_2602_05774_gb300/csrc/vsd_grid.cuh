@@ -51,12 +51,12 @@ static inline cudaError_t clear_words(void* ws, size_t bytes, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Launch `kern` as a programmatic dependent of the stream's previous kernel: its
-// blocks may become resident while that kernel's last ones still run, and wait
-// in grid_wait() until it has completed and its writes are visible.
+// Launch `kern`; after: as a programmatic dependent of the stream's previous
+// kernel: its blocks may become resident while that kernel's last ones still run,
+// and wait in grid_wait() until it has completed and its writes are visible.
 template <typename... P, typename... A>
-static cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem,
-                                cudaStream_t s, A... args) {
+static cudaError_t launch(bool after, void (*kern)(P...), unsigned grid, unsigned threads,
+                          size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
@@ -66,8 +66,13 @@ static cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned thre
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = after ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+template <typename K, typename... A>
+static cudaError_t launch_after(K kern, unsigned grid, unsigned threads, size_t smem,
+                                cudaStream_t s, A... args) {
+    return launch(true, kern, grid, threads, smem, s, args...);
 }
 
 }  // namespace vsd

@@ -28,6 +28,46 @@ __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
     }
 }
 
+// Verification of given tokens: the rows, then the paths (accepted length,
+// residual draw, corrected path, log-kappa sums), one block each.  One kernel,
+// the block completing a path running it (k_em_rows), takes over for few
+// unaligned rows only.  us, one kernel / two:
+//   aligned    bf16: V=128256 R=64 64 / 66, R=608 117 / 103, R=4096 416 / 396;
+//              V=32000 R=64 33 / 33, R=4096 150 / 143; V=256 R=32768 339 / 279
+//   unaligned  bf16: V=1001 R=64 23 / 26, R=4096 83 / 66; V=32001 R=64 50 / 52,
+//              R=4096 278 / 247
+// Rows that are not aligned keep more element loads in flight with more registers,
+// which the many short ones lack (S, which means nothing else there: five blocks
+// an SM, four with kDeepStages; bf16 R=4096: V=1001 66 / 73, V=32001 268 / 247).
+template <typename T, bool VEC, int S>
+__global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : S == kDeepStages ? 4 : 5)
+    k_verify_rows(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ RowShared sh;
+    Ring<S>* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
+    grid_launch_next();
+    row_pass<T, VEC, true, kGivenToken, true>(P, blockIdx.x, rg, tab, sh);
+}
+template <typename T, bool VEC, int S>
+__global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1)
+    k_verify_paths(Problem<T> P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ PathShared sh;
+    Ring<S>* rg;
+    float4* tab;
+    smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
+    grid_wait();
+    path_head<T>(P, blockIdx.x, sh);
+    __syncthreads();
+    const int A = sh.A, rA = blockIdx.x * P.D + A;
+    int resid = -1;
+    if (A < P.D && !sh.rec.flags)
+        resid = residual_draw<T, VEC>(P, rA, sh.rec, __ldg(P.u_correct + rA), rg, tab, &sh.resid);
+    path_epilogue<T>(P, blockIdx.x, A, resid);
+}
+
 // Rows along supplied greedy reference paths (Algorithm 2's z-bar): per row
 // the target's argmax and log min(1, p/q) there (row_pass with the argmax).
 template <typename T, bool VEC, int S>
@@ -445,6 +485,28 @@ cudaError_t Launch<VSD_T>::sample(const Problem<VSD_T>& P, bool vec, cudaStream_
     cudaError_t e = prep(kern, smem);
     if (e) return e;
     return launch_after(kern, P.R, kThreads, smem, s, P);
+}
+
+template <>
+cudaError_t Launch<VSD_T>::verify(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
+    const int64_t sms = device_sm_count();
+    if (!vec && P.R <= (P.nch < 16 ? 4 : 2) * sms) return verify_few(P, s);
+    bool deep = deep_ring(vec, P.nch, P.R);
+    size_t smem = row_smem_bytes(P.nch, vec, deep);
+    auto rows = !vec && P.nch >= 12 ? k_verify_rows<VSD_T, false, kDeepStages>
+                                    : VSD_BY_RING(k_verify_rows, VSD_T);
+    cudaError_t e = prep(rows, smem);
+    if (e) return e;
+    if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
+    const int paths = P.B * P.K;
+    deep = deep_ring(vec, P.nch, paths);
+    smem = row_smem_bytes(P.nch, vec, deep);
+    auto kern = VSD_BY_RING(k_verify_paths, VSD_T);
+    if ((e = prep(kern, smem))) return e;
+    // Many long rows: path blocks that are resident early slow the rows down
+    // (V=128256 bf16 R=704: 144 us as dependents, 113 in plain order, R=1024 175
+    // and 147; R=608 103 and 106, V=1000 R=4096 53 and 55).
+    return launch(!(P.nch >= 48 && P.R > 4 * sms), kern, paths, kThreads, smem, s, P);
 }
 
 template <>

@@ -35,7 +35,7 @@ inline size_t staged_smem_bytes(int nch, bool vec, bool deep) {
 }
 
 // XMODE: kSampleToken the whole E-step + M-step; kGivenToken the verification
-// of given tokens, which ends with the paths.
+// of given tokens, which ends with the paths (few unaligned rows).
 template <typename T, bool VEC, bool KL, int XMODE, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -74,8 +74,7 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Prob
                 __ldcg(reinterpret_cast<const float2*>(rtab + ch));
     }
     __syncthreads();
-    row_tail<T, VEC, true, XMODE, true, KL>(
-        P, r, tab, sh.row, rg);
+    row_tail<T, VEC, true, XMODE, true, KL>(P, r, tab, sh.row, rg);
     // the last of n blocks to arrive at a counter
     auto last_of = [&](int* cnt, int n) {
         __syncthreads();
