@@ -530,9 +530,16 @@ cudaError_t Launch<VSD_T>::weights(const Problem<VSD_T>& P, const EStepView& E, 
 template <>
 cudaError_t Launch<VSD_T>::grad(const Problem<VSD_T>& P, bool vec, const float4* rstats,
                                 void* grad, bool grad_bf16, cudaStream_t s) {
-#define VSD_GRAD(V_, G_)                                                        \
-    return launch_after(k_grad<VSD_T, V_, G_>, P.R, kThreads, 0, s, P, rstats, \
-                        reinterpret_cast<G_*>(grad))
+    // As a dependent of the M-step, whose blocks hold few SMs, many gradient rows
+    // are spread over the SMs worse than in plain order.  us, dependent / plain:
+    // V=128256 float32 R=304 68 / 69, R=512 111 / 99, R=1024 181 / 189, R=2048 380 /
+    // 341; bf16 R=4096 384 / 353; V=8000 float32 R=2048 50 / 46, bf16 40 / 42
+    const int64_t sms = device_sm_count();
+    const bool after = !((P.nch >= 128 && P.R > 2 * sms && P.R <= 4 * sms) ||
+                         (P.nch >= 16 && P.R > 8 * sms));
+#define VSD_GRAD(V_, G_)                                                           \
+    return launch(after, k_grad<VSD_T, V_, G_>, P.R, kThreads, 0, s, P, rstats, \
+                  reinterpret_cast<G_*>(grad))
     if (vec && grad_bf16) VSD_GRAD(true, __nv_bfloat16);
     if (vec) VSD_GRAD(true, float);
     if (grad_bf16) VSD_GRAD(false, __nv_bfloat16);
