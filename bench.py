@@ -1,4 +1,4 @@
-"""Benchmark of the fused VSD E-step + M-step (one persistent kernel per step).
+"""Benchmark of the fused VSD E-step + M-step (one vsd_estep_mstep call per step).
 
 Workload (default): vocab128k -- B=32 prefixes x K=16 proposals x D=8 depth,
 V=128256, bf16 draft/target logits (Zipf-shaped target, draft = target +
@@ -91,10 +91,19 @@ def kernel_source_hash():
 
 
 def estep_kernels(R, V, elem, grad=True):
-    """The kernels one vsd_estep_mstep call launches, as the library chooses
-    them (the counters' clearing first)."""
-    chunks = -(-V // (2048 // elem))
-    if chunks <= 64 or not grad or 2 * elem * R * V <= 512 << 20:
+    """The kernels one vsd_estep_mstep call on 16-byte aligned rows launches on a
+    GPU of 152 SMs, by the rule of two_kernels() in csrc/vsd_api.cu (the
+    counters' clearing first)."""
+    nch, sms = -(-V // (2048 // elem)), 152
+    if nch <= 64:
+        two = True
+    elif nch > (288 if elem == 2 else 320) and (R <= sms or R > 2 * sms):
+        two = False
+    elif not grad:
+        two = nch <= 224 or R <= 6 * sms
+    else:
+        two = 2 * elem * R * V <= 512 << 20
+    if two:
         return ["k_clear", "k_em_rows"] + (["k_em_grad"] if grad else [])
     return ["k_clear", "k_fused"]
 

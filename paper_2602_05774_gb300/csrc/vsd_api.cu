@@ -46,19 +46,31 @@ constexpr int kSegChunks = VSD_SEG_CHUNKS;
 #define VSD_GRAD_SEG_CHUNKS 16
 #endif
 constexpr int kGradSegChunks = VSD_GRAD_SEG_CHUNKS;
-// The E-step + M-step runs as two kernels (vsd_staged.cuh) unless rows are long
-// (more chunks than kStagedChunks), their gradient is written and both logit
-// blocks take more than kStagedBytes: then the persistent kernel's overlap of
-// gradients with later rows is worth more than its claims cost.  Measured on
+// Whether the E-step + M-step runs as two kernels (vsd_staged.cuh) or as the
+// persistent one: rows of nch chunks, elem bytes a logit; vec: rows 16-byte
+// aligned; grad: the gradient is written.  The persistent kernel splits a row
+// over several blocks, and overlaps gradients with later rows.  Measured on
 // GB300, us per call, persistent / two kernels:
-//   V=32000 bf16 (32 chunks):  R=64 57 / 49, R=768 119 / 83, R=4096 320 / 258
-//   V=64000 bf16 (63 chunks):  R=768 169 / 120, R=4096 (1.05 GB) 430 / 413
-//   V=128256 bf16 (126):       R=64 113 / 82, R=512 (0.26 GB) 193 / 158,
-//                              R=2048 (1.05 GB) 364 / 422, R=4096 640 / 710
-//   V=64000 float32 (125):     R=512 (0.26 GB) 175 / 139, R=2048 (1.05 GB) 343 / 386
-//   no gradient, V=128256 bf16: R=1024 185 / 172, R=4096 470 / 419
-constexpr int kStagedChunks = 64;
-constexpr size_t kStagedBytes = (size_t)512 << 20;
+//   short rows: V=32000 bf16 (32 chunks)  R=64 57 / 49, R=768 119 / 83, R=4096
+//     320 / 258; V=64000 bf16 (63)  R=768 169 / 120, R=4096 (1.05 GB) 430 / 413
+//   a gradient of many long rows: V=128256 bf16 (126)  R=512 (0.26 GB) 193 / 158,
+//     R=2048 (1.05 GB) 364 / 422, R=4096 640 / 710
+//   without a gradient: V=128256 bf16 R=1024 215 / 172, V=327680 (320) R=1024 340 / 387
+//   few long rows, which two kernels leave to one block each, without a gradient:
+//     bf16 V=262144 (256) R=64 130 / 115, V=327680 R=64 130 / 143, V=393216 (384)
+//     R=64 134 / 157, R=304 256 / 180; float32 V=163840 (320) R=64 126 / 123,
+//     V=196608 (384) R=64 120 / 133, V=524288 (1024) R=64 175 / 304, R=304 391 / 379
+//   rows that are not aligned: bf16 V=262145 (257) R=64 327 / 289, R=512 578 / 412,
+//     V=327681 (321) R=64 321 / 344, R=304 571 / 459; float32 V=327681 (641) R=64
+//     300 / 289, V=458753 (897) R=64 340 / 415, V=393217 (769) R=304 602 / 416
+bool two_kernels(int nch, int64_t R, size_t logit_bytes, size_t elem, bool vec, bool grad) {
+    if (nch <= 64) return true;
+    const int64_t sms = device_sm_count();
+    if (!vec) return nch <= (elem == 2 ? 288 : 704) || R > sms;
+    if (nch > (elem == 2 ? 288 : 320) && (R <= sms || R > 2 * sms)) return false;
+    if (!grad) return nch <= 224 || R <= 6 * sms;
+    return logit_bytes <= (size_t)512 << 20;
+}
 
 // Upper bounds of the chunk count and segment count of a row over both logit
 // dtypes (the smaller float32 chunk gives the larger count).
@@ -436,8 +448,9 @@ vsd_status fused_impl(const void* draft, const void* target, vsd_layout L, float
     cudaError_t e = clear ? clear_counters(ws, L, s) : cudaSuccess;
     if (e != cudaSuccess) return from_cuda(e);
     // (the test hook of the bounded gradient waits needs the kernel that waits)
-    if (!P.inject_wait_fault && (P.nch <= kStagedChunks || !out->grad ||
-                                 2 * sizeof(T) * (size_t)P.R * (size_t)P.V <= kStagedBytes))
+    if (!P.inject_wait_fault &&
+        two_kernels(P.nch, P.R, 2 * sizeof(T) * (size_t)P.R * (size_t)P.V, sizeof(T), vec,
+                    out->grad != nullptr))
         return from_cuda(Launch<T>::staged(P, vec, out->grad, P.grad_bf16, s));
     const int per_sm = Launch<T>::fused_blocks_per_sm(P, vec, P.grad_bf16);
     const int64_t tickets = (int64_t)P.R * (P.nseg + P.gnseg);

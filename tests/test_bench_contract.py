@@ -50,3 +50,23 @@ def test_reference_arm_under_torchrun_prints_once():
                   "--impl", "reference", "--steps", "1", "--warmup", "1"])
     assert len(lines) == 1
     assert json.loads(lines[0])["impl"] == "reference"
+
+
+def test_launch_count_follows_the_librarys_rule():
+    """bench.py restates the rule by which the library takes two kernels or the
+    persistent one; its limits are those of the source."""
+    src = open(os.path.join(ROOT, "paper_2602_05774_gb300", "csrc", "vsd_api.cu")).read()
+    rule = " ".join(src[src.index("bool two_kernels("):].split("}\n")[0].split())
+    for line in ("if (nch <= 64) return true;",
+                 "if (nch > (elem == 2 ? 288 : 320) && (R <= sms || R > 2 * sms)) return false;",
+                 "if (!grad) return nch <= 224 || R <= 6 * sms;",
+                 "return logit_bytes <= (size_t)512 << 20;"):
+        assert line in rule, line
+    sys.path.insert(0, ROOT)
+    import bench
+    two, one = ["k_clear", "k_em_rows", "k_em_grad"], ["k_clear", "k_fused"]
+    for R, V, elem, grad, want in ((4096, 128256, 2, True, one), (4096, 32000, 2, True, two),
+                                   (4096, 128256, 2, False, two[:2]), (512, 128256, 2, True, two),
+                                   (64, 300000, 2, True, one), (256, 300000, 2, False, two[:2]),
+                                   (2048, 262144, 2, False, one), (64, 160000, 4, True, two)):
+        assert bench.estep_kernels(R, V, elem, grad) == want, (R, V, elem, grad)

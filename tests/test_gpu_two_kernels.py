@@ -205,3 +205,28 @@ def test_few_trees_with_long_rows_equal_many(vsd, rule):
         f = lambda x: vsd.tree_estep_mstep(x["draft"], x["target"], x["parent"],  # noqa: E731
                                            x["tokens"], x["u_accept"], x["u_correct"], 1.0)
         _same_rows(f(p), f(q), n, skip=("loss", "grad"))
+
+
+@pytest.mark.parametrize("V,R,n,dtype", [
+    (330000, 64, 4, "bf16"),   # 323 chunks: 64 rows persistent, 256 two kernels
+    (300001, 64, 8, "bf16"),   # 293 chunks, not 16-byte aligned: 64 and 512 rows
+    (361001, 8, 64, "f32"),    # 706 chunks, not aligned: 8 and 512 rows
+    (232000, 320, 4, "bf16"),  # 227 chunks, no gradient: 320 rows two kernels, 1280 persistent
+])
+def test_long_rows_by_either_route(vsd, V, R, n, dtype):
+    """Long rows run on the persistent kernel or as two kernels, by their number:
+    a batch and the same batch n times over, on either side of the line, give
+    the same results bit for bit."""
+    from paper_2602_05774_gb300 import inputs
+    K, D = 8, 1
+    p = inputs.linear_problem(R // K, K, D, V, dtype, "gauss", "cuda", seed=V)
+    q = {k: (v.repeat(*([n] + [1] * (v.dim() - 1))) if torch.is_tensor(v) else v)
+         for k, v in p.items()}
+    grad = R < 320
+    prm = vsd.params(like=p["draft"], kl_weight=0.5 if grad else 0.0,
+                     grad_dtype=torch.float32)
+    a, b = (_call(vsd, x, 1.0, prm, grad=grad) for x in (p, q))
+    _same_rows(a, b, n, skip=("loss", "grad"))
+    assert torch.equal(b["loss"][:-1].view(n, -1)[n - 1], a["loss"][:-1])
+    if grad:  # (a mean over n times the prefixes: an exact factor)
+        assert torch.equal(a["grad"].view(-1) / n, b["grad"].view(n, -1)[n - 1])
