@@ -98,7 +98,7 @@ template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
-    __shared__ int s_path, s_best, s_maxd, s_any, s_first;
+    __shared__ int s_path, s_best, s_maxd, s_any, s_more, s_first;
     Ring<S>* rg;
     float4* tab;
     smem_views<VEC>(dsm, rg, tab, P.timeout_ns, P.hold_copies != 0);
@@ -135,24 +135,36 @@ __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
         }
         return;
     }
+    int* up = t.depth;  // (for now) an accepted node's parent, -1 for a rejected one
     for (int n = tid; n < N; n += kThreads) {
-        t.acc[n] = n ? ld_cg(o.accept + n0 + n) : 1;
+        const int acc = n ? ld_cg(o.accept + n0 + n) : 1;
+        t.acc[n] = acc;
+        up[n] = acc ? t.par[n] : -1;
         if (u == 0) t.la[n] = n ? ld_cg(P.tla + n0 + n) : 0.f;
     }
     __syncthreads();
     if (tid == 0) {
         int x = u;
-        while (x > 0 && t.acc[x]) x = t.par[x];
+        while (x > 0) x = up[x];
         s_path = x == 0;
         s_best = -1;
-        s_maxd = s_any = 0;
+        s_maxd = s_any = s_more = 0;
         s_first = N;
     }
     __syncthreads();
     if (!s_path) return;
-    // each node's depth (-1 below a rejection), the deepest accepted node
-    // (lowest index on ties), u's children
-    for (int n = tid; n < N; n += kThreads) {
+    auto child = [&](int n) {
+        if (n <= u || t.par[n] != u) return;
+        atomicMin(&s_first, n);
+        if (t.acc[n]) s_more = 1;
+        else s_any = 1;
+    };
+    // n's depth (-1 - it below a rejection) and, over the nodes, the deepest
+    // accepted one (lowest index on ties), for the nodes' outputs and for the bonus
+    // token.  Each node walks to the root, so only the root's block and those of
+    // nodes without an accepted child take it (64 chains of 1024 accepted nodes:
+    // 14.7 ms a call with it in every block on an accepted path, 2.8 now).
+    auto walk = [&](int n) {
         int d = 0, ok = 1;
         for (int x = n; x > 0; x = t.par[x]) {
             ok &= t.acc[x];
@@ -161,13 +173,17 @@ __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
         t.depth[n] = ok ? d : -1 - d;
         if (ok) atomicMax(&s_best, (d << 11) | (2047 - n));
         atomicMax(&s_maxd, d);
-        if (n && t.par[n] == u) {
-            atomicMin(&s_first, n);
-            if (!t.acc[n]) s_any = 1;
-        }
+    };
+    for (int n = tid; n < N; n += kThreads) {
+        child(n);
+        if (u == 0) walk(n);
     }
     __syncthreads();
-    const int best = 2047 - (s_best & 2047);
+    if (u && !s_more) {
+        for (int n = tid; n < N; n += kThreads) walk(n);
+        __syncthreads();
+    }
+    const int best = s_best < 0 ? -1 : 2047 - (s_best & 2047);
     if (u == 0) {  // the nodes' outputs; log kappa along each branch (Eq. 2)
         auto depth_of = [&](int n) { return t.depth[n] >= 0 ? t.depth[n] : -1 - t.depth[n]; };
         for (int l = 0; l <= s_maxd; ++l) {
