@@ -165,6 +165,7 @@ struct Problem {
     struct TreeCoef* tcoef;       // [R] each node's gradient terms at its parent's row
     float* tg;                    // [R] each row's dense gradient factor
     int* tbad;                    // [B] the tree failed its checks
+    int read_leaves;              // sequential rule: leaf rows are read with the others
     int* tlist;                   // tree layout: [R] sequential rule: each row's accepted child
     float* tla;                   // tree layout: [R] log alpha of each node's token
     int* resq;                    // [B*K*nseg] residual segment items (path*nseg + seg)
@@ -1062,7 +1063,7 @@ __device__ __forceinline__ RowTask row_task(const Problem<T>& P, int r, const fl
 // rstats[r].
 // vals(which, v, xv, yv) gives the draft and target logits of token v (the
 // draw `which`).
-template <typename T, bool HAS_Y, int XMODE, bool ARGMAX, class Vals>
+template <typename T, bool HAS_Y, int XMODE, bool ARGMAX, bool QUIET = false, class Vals>
 __device__ __forceinline__ void row_finish(const Problem<T>& P, int r, const RowTask& tx,
                                            const RowTask& ty, int ref, int lane, const Vals& vals) {
     const int64_t V = P.V;
@@ -1109,7 +1110,7 @@ __device__ __forceinline__ void row_finish(const Problem<T>& P, int r, const Row
         rec.izy = (HAS_Y && oky) ? 1.f / (float)ty.S.Z : 0.f;
         rec.pad[0] = rec.pad[1] = rec.pad[2] = 0;
         rec.flags = ok ? 0 : 1;
-        if (!ok) atomicOr(P.status, VSD_STATUS_BAD_ROW);
+        if (!ok && !QUIET) atomicOr(P.status, VSD_STATUS_BAD_ROW);
         if (!ok && P.kl_topk) {  // an invalid row has no top-K term
             P.klr[r].n = 0;
             P.klr[r].loss = 0.f;
@@ -1145,7 +1146,8 @@ __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch
 
 // The per-row work once the row's chunk table tab[0..nch) is complete (block):
 // warps 0, 1 and 2 take the three tasks at once, warp 0 then writes the record.
-template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool KL = false, int S>
+template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool KL = false,
+          bool QUIET = false, int S>
 __device__ void row_tail(const Problem<T>& P, int r, const float4* tab, RowShared& sh,
                          Ring<S>* rg, bool pdraw = true) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1163,7 +1165,7 @@ __device__ void row_tail(const Problem<T>& P, int r, const float4* tab, RowShare
         RowTask ty = sh.t[1];
         if (!HAS_Y) ty = RowTask{0.f, TableSum{0, 0, 0.0}, -1, 0.f, 0.f, 0.0};
         const int ref = (HAS_Y && ARGMAX) ? sh.t[2].tok : -1;
-        row_finish<T, HAS_Y, XMODE, ARGMAX>(P, r, sh.t[0], ty, ref, lane,
+        row_finish<T, HAS_Y, XMODE, ARGMAX, QUIET>(P, r, sh.t[0], ty, ref, lane,
                                             [&](int w, int, float& xv, float& yv) {
                                                 xv = sh.t[w].xv;
                                                 yv = sh.t[w].yv;
@@ -1442,8 +1444,9 @@ __device__ void row_tail_warp(const Problem<T>& P, int r, float4* tab, RescanBuf
 // Streams row r of the draft (and, with HAS_Y, of the target) once, then runs
 // row_tail.  XMODE: whether z~ is drawn from q with u_draft, read from
 // given_tokens, or absent (trees).  ARGMAX: locate the greedy reference token.
-// pdraw = false leaves out the draw from p.
-template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, int S>
+// pdraw = false leaves out the draw from p, QUIET the status bit of an invalid
+// row.
+template <typename T, bool VEC, bool HAS_Y, int XMODE, bool ARGMAX, bool QUIET = false, int S>
 __device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, RowShared& sh,
                          bool pdraw = true) {
     const int64_t V = P.V;
@@ -1456,7 +1459,7 @@ __device__ void row_pass(const Problem<T>& P, int r, Ring<S>* rg, float4* tab, R
     // workspace is written from here on)
     grid_wait();
     __syncthreads();
-    row_tail<T, VEC, HAS_Y, XMODE, ARGMAX>(P, r, tab, sh, rg, pdraw);
+    row_tail<T, VEC, HAS_Y, XMODE, ARGMAX, false, QUIET>(P, r, tab, sh, rg, pdraw);
 }
 
 // --------------------------------------------------------------- residual

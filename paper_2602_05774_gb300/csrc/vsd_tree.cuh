@@ -56,8 +56,8 @@ static_assert(sizeof(TreeCoef) == 16, "TreeCoef layout");
 //   k_tree_verify       one block per row, of which most leave at once: at a
 //                       row on an accepted path the rejected children's draws
 //                       (one more read of the row), at the deepest accepted
-//                       node the bonus token (a leaf's row is read here, for
-//                       a draw that the first kernel leaves out), at the root
+//                       node the bonus token (a leaf's row is read here, or
+//                       its chunk table if the first kernel read it), at the root
 //                       the outputs of the tree's nodes.
 // No block waits for another.  The row reads bound the first kernel, a few
 // dependent steps of one row the second.
@@ -81,6 +81,10 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1)
     }
     row_pass<T, VEC, true, kStats, false>(P, r, rg, tab, sh);
     __syncthreads();
+    if (!kids) {  // the table for a bonus token drawn here
+        for (int ch = threadIdx.x; ch < P.nch; ch += kThreads)
+            P.gtab[(int64_t)r * P.nch_ws + ch] = tab[ch];
+    }
     tree_children<T>(P, b, u);
 }
 
@@ -94,7 +98,8 @@ struct TreeVerifyNodes {
 };
 inline size_t tree_verify_smem_bytes(int N) { return (size_t)N * 21 + 16; }
 
-template <typename T, bool VEC, int S>
+// STATS: with row_stats (the first kernel has read every row).
+template <typename T, bool VEC, bool STATS, int S>
 __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ RowShared sh;
@@ -248,6 +253,22 @@ __global__ void __launch_bounds__(kThreads) k_tree_verify(Problem<T> P) {
     }
     if (u == best) {  // the token after the accepted path
         const bool leaf = s_first == N;
+        if (STATS && leaf) {  // its statistics are there, and its chunk table
+            for (int ch = tid; ch < P.nch; ch += kThreads)
+                tab[ch] = ld_cg(P.gtab + (int64_t)r * P.nch_ws + ch);
+            __syncthreads();
+            if (warp == 0) {
+                const float M = table_max(tab, P.nch, 1, lane);
+                const TableSum Sp = table_sum(tab, P.nch, 1, frame_of(M), P.ts.c, lane);
+                int tok = -1;
+                if (!ld_cg(P.rows + r).flags)
+                    tok = warp_sample<T, VEC>(P.draft + (int64_t)r * V, P.target + (int64_t)r * V, V,
+                                              tab, P.nch, 1, M, Sp, __ldg(P.u_correct + r), P.ts.c,
+                                              lane, policy_evict_normal(), warp_chunks(rg));
+                if (lane == 0) o.bonus[b] = tok < V ? tok : -1;
+            }
+            return;
+        }
         if (leaf) {
             row_pass<T, VEC, true, kNoToken, false>(P, r, rg, tab, sh);
             __syncthreads();
@@ -1032,6 +1053,8 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<S>* rg, float4* ta
     }
     __syncthreads();
     const int m = ct.m;
+    if (threadIdx.x == 0 && rec.flags && (m || P.tout.row_stats))
+        atomicOr(P.status, VSD_STATUS_BAD_ROW);
     for (int i = threadIdx.x; i < m; i += kThreads) {
         const int n = n0 + s.kid[i], tok = __ldg(P.given_tokens + n);
         TreeNodeRec nr;
@@ -1137,8 +1160,9 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<S>* rg, float4* ta
     }
 }
 
-// One block per node row (a leaf's row only for the statistics output; the row
-// a bonus token needs is then read by k_tree_seq).
+// One block per node row.  A leaf's row is read for the statistics output, and
+// where the rows are few (read_leaves), since it costs nothing beside the others
+// then; else the row a bonus token needs is read by k_tree_seq.
 // What bounds it: the row reads and row tails (3840 rows of 2 x 64 KB), and
 // the reads after a rejection, which come from L2.  64 trees of 60 nodes,
 // V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
@@ -1158,13 +1182,14 @@ __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_row
     for (int n = u + 1 + threadIdx.x; n < N && !has; n += kThreads)
         has = __ldg(P.parent + (int64_t)b * N + n) == u;
     has = __syncthreads_or(has);
-    if (!has && !P.tout.row_stats) {
+    if (!has && !P.tout.row_stats && !P.read_leaves) {
         grid_wait();
         if (threadIdx.x == 0) P.tlist[r] = 0;
         return;
     }
-    // (a leaf's draw from p may become the bonus token)
-    row_pass<T, VEC, true, kNoToken, false>(P, r, rg, tab, sh, !has);
+    // (a leaf's draw from p may become the bonus token; a leaf read for that alone
+    // sets no status bit here)
+    row_pass<T, VEC, true, kNoToken, false, true>(P, r, rg, tab, sh, !has);
     __syncthreads();
     if (threadIdx.x == 0 && P.tout.row_stats)
         reinterpret_cast<float4*>(P.tout.row_stats)[r] = ld_cg(P.rstats + r);
@@ -1250,7 +1275,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
     }
     __syncthreads();
     const bool leaf = sh.lastkid == 0;
-    if (leaf && !P.tout.row_stats) {  // the leaf's row, for the bonus token
+    if (leaf && !P.tout.row_stats && !P.read_leaves) {  // the leaf's row, for the bonus token
         row_pass<T, VEC, true, kNoToken, false>(P, n0 + best, rg, tab, rsh);
         __syncthreads();
     }
@@ -1258,6 +1283,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_seq(Problem<T> P) {
         o.deepest[b] = best;
         o.accept_len[b] = sh.t.depth[best];
         const int tok = leaf ? ld_cg(P.rows + n0 + best).ps : P.es.corr[n0 + best];
+        if (leaf && ld_cg(P.rows + n0 + best).flags) atomicOr(P.status, VSD_STATUS_BAD_ROW);
         if (!leaf) o.corr_tokens[n0 + sh.lastkid] = tok;
         o.bonus[b] = tok;
     }

@@ -18,13 +18,16 @@ cudaError_t Launch<VSD_T>::tree(const Problem<VSD_T>& P, bool vec, cudaStream_t 
     if (e) return e;
     if ((e = launch_after(rows, P.R, kThreads, smem, s, P))) return e;
     const size_t sm2 = smem + tree_verify_smem_bytes(P.N);
-    auto nodes = VSD_BY_RING(k_tree_verify, VSD_T);
+    auto nodes = P.tout.row_stats ? VSD_BY_RING(k_tree_verify, VSD_T, , true)
+                                  : VSD_BY_RING(k_tree_verify, VSD_T, , false);
     if ((e = prep(nodes, sm2))) return e;
     return launch_after(nodes, P.R, kThreads, sm2, s, P);
 }
 
 template <>
-cudaError_t Launch<VSD_T>::tree_seq(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
+cudaError_t Launch<VSD_T>::tree_seq(const Problem<VSD_T>& P_, bool vec, cudaStream_t s) {
+    Problem<VSD_T> P = P_;
+    P.read_leaves = P.R <= device_sm_count();
     const bool deep = deep_ring(vec, P.nch, P.R);
     const size_t smem = row_smem_bytes(P.nch, vec, deep) + seq_smem_bytes(P.N);
     auto rows = VSD_BY_RING(k_tree_seq_rows, VSD_T);

@@ -64,3 +64,35 @@ def test_deep_accepted_paths(vsd, oracle, parent, noise):
         for n in range(1, len(parent)):
             depth[n] = depth[parent[n]] + 1
         assert (got["accept_len"].cpu().numpy() == depth.max()).all()
+
+
+@pytest.mark.parametrize("rule", [0, 1])
+@pytest.mark.parametrize("copies", [1, 100])  # 3 and 300 rows, fewer and more than SMs
+def test_leaf_rows_early_and_late(vsd, rule, copies):
+    """A root and two leaves, every node accepted, so the bonus token is drawn at
+    the first leaf's row: the same token whether the row is read with the others
+    (row statistics; few rows under the sequential rule) or when it is needed.  A
+    leaf row that enters no result sets no status bit without row statistics."""
+    _, c = _case(1, [-1, 0, 0], 4104, 3, 0.0)
+
+    def run(bad, stats):
+        q = {k: v.repeat(*([copies] + [1] * (v.dim() - 1))) for k, v in c.items()}
+        if bad is not None:
+            q["target"].view(copies, 3, -1)[:, bad, 7] = float("nan")
+        return _verify(vsd, q, stats, rule)
+
+    want, status = run(None, True)
+    assert status == (0, 0) and (want["deepest"] == 1).all()
+    row = torch.softmax(c["target"][1].double(), 0).cumsum(0)
+    tok = int(torch.searchsorted(row, c["u_correct"][0, 1].double().cuda(), right=True))
+    assert (want["bonus"] == tok).all()
+    got, status = run(None, False)
+    assert status == (0, 0)
+    for k in got:
+        assert torch.equal(got[k], want[k]), k
+    got, status = run(2, False)  # the leaf that no output reads
+    assert status == (0, 0) and torch.equal(got["bonus"], want["bonus"])
+    assert run(2, True)[1] == (6, vsd.STATUS_BAD_ROW)
+    for stats in (True, False):
+        got, status = run(1, stats)
+        assert status == (6, vsd.STATUS_BAD_ROW) and (got["bonus"] == -1).all()
