@@ -431,6 +431,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             mma_commit(&sb->drain);
             wait_phase_drain(&sb->drain, 0, timeout_ns);
+            // the arrivals of the last commits have landed too (lt: tiles whose
+            // accumulator was committed)
+            for (uint32_t j = it > (uint32_t)S ? it - S : 0; j < it; ++j)
+                wait_phase_drain(&sb->empty[j % S], (j / S) & 1u, timeout_ns);
+            constexpr uint32_t NB = C::kAccBufs;
+            const uint32_t nt = (uint32_t)lt;
+            for (uint32_t j = nt > NB ? nt - NB : 0; j < nt; ++j)
+                wait_phase_drain(&sb->acc_full[j % NB], (j / NB) & 1u, timeout_ns);
         }
     } else if (warp < 2 + kXWarps) {
         // ------------------------------------------------------ the A operand

@@ -88,3 +88,26 @@ def test_every_commit_is_waited_for(vsd, M, N, kb):
     want = (h.double() @ w.double().t()).bfloat16()
     for x in got:
         assert torch.equal(x, want)
+
+
+@pytest.mark.parametrize("R,V,H", [(16, 40, 64), (128, 168, 520), (300, 1032, 136)])
+def test_backward_on_chip_waits_for_its_commits(vsd, R, V, H):
+    """Without scratch, at few and many K blocks per tile and several tiles: no
+    wait at the end of the kernel is for a phase that never comes (2 s)."""
+    from paper_2602_05774_gb300 import inputs
+    p = inputs.lmhead_problem(R, 1, 1, V, H, "cuda", seed=V)
+    x = inputs.linear_problem(R, 1, 1, V, "bf16", "gauss", "cuda", seed=V)
+    ws = vsd.new_workspace(vsd.layout(R, 1, 1, V), "cuda")
+    prm = vsd.params(like=x["draft"])
+    vsd.estep_mstep(x["draft"], x["target"], x["u_draft"], x["u_accept"], x["u_correct"], 1, 1,
+                    1.0, prm=prm, workspace=ws)
+    dh, dw = torch.empty(R, H, device="cuda"), torch.empty(V, H, device="cuda")
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    for ev in (a, b):  # (the first call loads the kernels)
+        assert vsd.load().vsd_lmhead_backward(
+            p["hidden"].data_ptr(), p["weight"].data_ptr(), H, x["draft"].data_ptr(),
+            vsd.layout(R, 1, 1, V), 1.0, C.byref(prm), dh.data_ptr(), dw.data_ptr(),
+            ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+        ev.record()
+    torch.cuda.synchronize()
+    assert vsd.device_status(ws) == (0, 0) and a.elapsed_time(b) < 500
