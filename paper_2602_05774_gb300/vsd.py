@@ -470,15 +470,19 @@ def lmhead_estep_mstep(hidden, weight, target, u_draft, u_accept, u_correct, K, 
 
 
 def lmhead_backward(hidden, weight, draft_logits, K, D, T, workspace, prm=None,
-                    d_hidden=True, d_weight=True):
+                    d_hidden=True, d_weight=True, scratch=True):
     """The draft LM head's backward after lmhead_estep_mstep() (or estep_mstep()
     on bf16 draft logits) on the same workspace: returns {"d_hidden": [R][H],
     "d_weight": [V][H]} (float32), the M-step gradient of the draft logits
     carried through logits = hidden . weight^T.  Pass False to skip one, or a
-    float32 tensor to write into.  Takes R*V bf16 values of scratch from
-    PyTorch's allocator for the call (vsd_lmhead_backward_scratch); without room
-    for them the gradient is made on chip, slower."""
-    _need_cuda(hidden, weight, draft_logits)
+    float32 tensor to write into.
+    scratch: the R*V bf16 values that the gradient is written to once
+    (vsd_lmhead_backward_scratch).  True takes them from PyTorch's allocator for
+    the call (without room for them the gradient is made on chip); a tensor of at
+    least 2*R*V bytes is used as it is; False makes the gradient on chip, slower,
+    and holds no dense gradient."""
+    _need_cuda(hidden, weight, draft_logits,
+               scratch if torch.is_tensor(scratch) else None)
     V, H = weight.shape
     R = hidden.numel() // H
     lay = layout(R // (K * D), K, D, V)
@@ -490,9 +494,15 @@ def lmhead_backward(hidden, weight, draft_logits, K, D, T, workspace, prm=None,
             res[name] = torch.empty(*shape, dtype=torch.float32, device=dev)
         elif want is not False and want is not None:
             res[name] = want
-    try:  # G in bf16, from the caching allocator; without room for it G is made on chip
-        scratch = torch.empty(R * V, dtype=torch.bfloat16, device=dev) if res else None
-    except torch.OutOfMemoryError:
+    if torch.is_tensor(scratch):
+        if scratch.numel() * scratch.element_size() < 2 * R * V:
+            raise ValueError("scratch too small")
+    elif scratch and res:
+        try:
+            scratch = torch.empty(R * V, dtype=torch.bfloat16, device=dev)
+        except torch.OutOfMemoryError:
+            scratch = None
+    else:
         scratch = None
     _check(_lib().vsd_lmhead_backward_scratch(
         _ptr(hidden), _ptr(weight), H, _ptr(draft_logits), lay, float(T), C.byref(prm),
@@ -625,10 +635,11 @@ class HostLMHeadStep:
     """HostStep for the LM head fused with the E-step + M-step: per call the
     hidden states, target logits and uniforms come from pinned host tensors
     (double-buffered); the LM-head weight stays on the device.  train=True:
-    the draft head's training step, no dense gradient and the LM head's
-    backward (d_hidden, d_weight left on the device)."""
+    the draft head's training step, no dense gradient output and the LM head's
+    backward (d_hidden, d_weight left on the device; scratch as for
+    lmhead_backward)."""
 
-    def __init__(self, weight, B, K, D, V, prm=None, full=True, train=False):
+    def __init__(self, weight, B, K, D, V, prm=None, full=True, train=False, scratch=True):
         self.B, self.K, self.D, self.V = B, K, D, V
         R, H = B * K * D, weight.shape[1]
         self.dev = weight.device
@@ -637,7 +648,7 @@ class HostLMHeadStep:
                                  u=((3, R), torch.float32)), self.dev)
         self.prm = prm or params(grad_dtype=torch.bfloat16)
         gdt = torch.bfloat16 if self.prm.grad_dtype == VSD_BF16 else torch.float32
-        self.train = train
+        self.train, self.scratch = train, scratch
         self.out = linear_outputs(B, K, D, V, self.dev, grad_dtype=gdt, full=full, grad=not train)
         self.ws = new_workspace(layout(B, K, D, V), self.dev)
         self.logits = torch.empty(R, V, dtype=torch.bfloat16, device=self.dev)
@@ -659,7 +670,8 @@ class HostLMHeadStep:
                            out=self.out, draft_logits=self.logits)
         if self.train:
             lmhead_backward(d["hidden"], self.weight, self.logits, self.K, self.D, T, self.ws,
-                            prm=self.prm, d_hidden=self.d_hidden, d_weight=self.d_weight)
+                            prm=self.prm, d_hidden=self.d_hidden, d_weight=self.d_weight,
+                            scratch=self.scratch)
         self.feed.release(s)
         self.loss_host[s].copy_(self.out["loss"], non_blocking=True)
         return self.loss_host[s]

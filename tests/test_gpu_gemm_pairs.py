@@ -111,3 +111,48 @@ def test_backward_on_chip_waits_for_its_commits(vsd, R, V, H):
         ev.record()
     torch.cuda.synchronize()
     assert vsd.device_status(ws) == (0, 0) and a.elapsed_time(b) < 500
+
+
+def test_backward_scratch_is_the_callers_choice(vsd):
+    """scratch=False holds no dense gradient (its R*V bf16 values would dominate
+    here) and gives the bits of the call without scratch; a tensor is used as it
+    is and gives those of the default."""
+    from paper_2602_05774_gb300 import inputs
+    B, K, D, V, H = 16, 8, 4, 32008, 64
+    R = B * K * D
+    p = inputs.lmhead_problem(B, K, D, V, H, "cuda", seed=9)
+    x = inputs.linear_problem(B, K, D, V, "bf16", "gauss", "cuda", seed=9)
+    ws = vsd.new_workspace(vsd.layout(B, K, D, V), "cuda")
+    vsd.estep_mstep(x["draft"], x["target"], x["u_draft"], x["u_accept"], x["u_correct"], K, D,
+                    1.0, workspace=ws, grad=False)
+    dh, dw = torch.empty(R, H, device="cuda"), torch.empty(V, H, device="cuda")
+
+    def run(scratch):
+        dh.fill_(float("nan")), dw.fill_(float("nan"))
+        torch.cuda.synchronize()
+        torch.cuda.reset_peak_memory_stats()
+        before = torch.cuda.memory_allocated()
+        vsd.lmhead_backward(p["hidden"], p["weight"], x["draft"], K, D, 1.0, ws, d_hidden=dh,
+                            d_weight=dw, scratch=scratch)
+        torch.cuda.synchronize()
+        held = torch.cuda.max_memory_allocated() - before
+        return dh.clone(), dw.clone(), held
+
+    *default, held = run(True)
+    assert held >= 2 * R * V
+    *chip, held = run(False)
+    assert held == 0
+    buf = torch.full((R * V,), float("nan"), dtype=torch.bfloat16, device="cuda")
+    *given, held = run(buf)
+    assert held == 0 and torch.isfinite(buf).all()
+    for a, b in zip(default, given):
+        assert torch.equal(a, b)
+    dh2, dw2 = torch.empty_like(dh), torch.empty_like(dw)
+    prm = vsd.params(like=x["draft"])
+    assert vsd.load().vsd_lmhead_backward(
+        p["hidden"].data_ptr(), p["weight"].data_ptr(), H, x["draft"].data_ptr(),
+        vsd.layout(B, K, D, V), 1.0, C.byref(prm), dh2.data_ptr(), dw2.data_ptr(), ws.data_ptr(),
+        ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+    assert torch.equal(chip[0], dh2) and torch.equal(chip[1], dw2)
+    with pytest.raises(ValueError):
+        run(buf[:-1])
