@@ -100,9 +100,10 @@ WsLayout ws_layout(const vsd_layout& L) {
     w.nch_ws = chunks_upper(L.V);
     w.nseg_ws = (w.nch_ws + kSegChunks - 1) / kSegChunks;
     const size_t nseg = (size_t)w.nseg_ws;
-    // residual queue: segments of the paths' residual rows, or a tree's
-    // residual rows (at most one per node)
-    const size_t nq = L.parent ? R : npath * nseg;
+    // the persistent kernel's counters and its queue of the paths' residual
+    // segments (trees have none)
+    const size_t nrow = L.parent ? 0 : R, nres = L.parent ? 0 : npath;
+    const size_t nq = nres * nseg;
     // hot counters on separate 256-byte lines (distinct L2 lines and slices)
     w.status = 0;
     w.ticket = 256;
@@ -115,8 +116,8 @@ WsLayout ws_layout(const vsd_layout& L) {
     w.prefix_cnt = o; o = align256(o + 4 * (size_t)L.B);
     w.ready = o; o = align256(o + 4 * (size_t)L.B);
     w.grad_cnt = o; o = align256(o + 4 * (size_t)L.B);
-    w.row_seg_cnt = o; o = align256(o + 4 * R);
-    w.res_seg_cnt = o; o = align256(o + 4 * npath);
+    w.row_seg_cnt = o; o = align256(o + 4 * nrow);
+    w.res_seg_cnt = o; o = align256(o + 4 * nres);
     w.resq_flag = o; o = align256(o + 4 * nq);
     w.zero_end = o;
     w.rows = o; o = align256(o + sizeof(RowRec) * R);

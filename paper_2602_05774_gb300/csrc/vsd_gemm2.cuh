@@ -18,8 +18,8 @@
 // Measured at R = 4096, H = 4096, V = 32000 (1.07 TFLOP a product, one launch
 // alone): logits 572 us (655 with one CTA per 128 x 256 tile), d_hidden 547 and
 // d_weight 555 from a gradient in memory plus 70 to write it (962 and 1205 with
-// the gradient made on chip for every tile): 1.87 to 1.96 PFLOP/s, cuBLAS's
-// measured rate.  The tensor pipe bounds it.
+// the gradient made on chip for every tile): 1.88 to 1.96 PFLOP/s; cuBLAS ran at
+// 1.91 on this pool.  The tensor pipe bounds it.
 //
 // Every wait is bounded; a wait that runs out sets VSD_STATUS_TIMEOUT in the
 // status word, and the pair winds down: it waits (again bounded) for its MMAs

@@ -40,9 +40,9 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// Tensor map of a row-major bf16 matrix [rows][cols] read in boxes of
-// box_rows x 64 columns with the 128-byte swizzle; out-of-range elements read
-// as zero (they add nothing to a dot product).
+// Tensor map of a row-major bf16 matrix [rows][cols] read in boxes of box_rows x
+// box_cols, swizzled in swizzle_bytes; out-of-range elements read as zero (they
+// add nothing to a dot product).
 bool make_map_box(CUtensorMap* m, const void* base, int rows, int cols, int box_cols,
                   int box_rows, int swizzle_bytes) {
     EncodeTiledFn enc = encode_fn();

@@ -267,9 +267,11 @@ __device__ __forceinline__ void ring_init(Ring<S>* rg, uint64_t timeout_ns, bool
 // Dynamic shared memory: [Ring (vector rows only)][chunk table].  A kernel that
 // later uses MIN bytes from the start for something else gets the ring moved up
 // so far that those bytes end with the ring's chunk data: the memory of an
-// mbarrier in use may hold nothing else (M-step scratch that reached over the
-// barriers read their words back as its own values, about once in 900 M-steps
-// behind the LM head).
+// mbarrier may hold nothing else until it is invalidated.  (With M-step scratch
+// that reached over the barriers, the M-step read barrier words in the place of
+// its own values, about once in 900 M-steps and only behind the LM head; what
+// wrote them then is not known.  The head's blocks could at that time leave
+// before their last barrier arrivals had landed, which they do no more.)
 template <int S, size_t MIN = 0> __host__ __device__ constexpr size_t ring_offset() {
     constexpr size_t data = sizeof(Ring<S>::data), more = MIN > data ? MIN - data : 0;
     return (more + 127) / 128 * 128;
@@ -889,7 +891,6 @@ __device__ __forceinline__ int table_first_max(const float4* tab, int nch, float
 template <typename T>
 __device__ __forceinline__ int first_max_regs(const uint4 (&by)[kLoads], int ch, float M) {
     constexpr int PV = Traits<T>::kPerVec;
-    const int lane = threadIdx.x & 31;
     const int64_t base = (int64_t)ch * chunk_elems<T>();
 #pragma unroll
     for (int k = 0; k < kLoads; ++k) {
@@ -1142,7 +1143,7 @@ struct RowShared {
 // VSD (KL): the row's top-K term of Eq. klv (defined below).
 template <typename T, bool VEC>
 __device__ void kl_select(const Problem<T>& P, int r, const float4* tab, int nch, uint4* buf,
-                          int npair, bool ok, int lane);
+                          bool ok, int lane);
 
 // The per-row work once the row's chunk table tab[0..nch) is complete (block):
 // warps 0, 1 and 2 take the three tasks at once, warp 0 then writes the record.

@@ -3,9 +3,8 @@
 // verification with the sequential sibling rule (lossless multi-draft).
 //
 //   k_tree_rows  one block per node row u: the row pass (tables, statistics,
-//                the target's argmax, a draw from p with u's uniform), then
-//                for every child x of u its token's test at u's row (Eq. 1,
-//                each branch alone).
+//                the target's argmax), then for every child x of u its token's
+//                test at u's row (Eq. 1, each branch alone).
 //   k_tree_draws one block per row with children: the draws their corrected
 //                paths take there, from the residual norm(max(0, p - q)) at
 //                the first rejection, from p below it.
@@ -777,7 +776,7 @@ inline size_t tree_grad_smem_bytes(int N) { return (size_t)N * 4 * sizeof(TreeGr
 template <typename T, bool VEC, typename G>
 __global__ void __launch_bounds__(kThreads) k_tree_grad(Problem<T> P, G* grad) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ int s_n, s_nu;
+    __shared__ int s_n;
     constexpr int PV = Traits<T>::kPerVec;
     const int N = P.N, r = blockIdx.x, b = r / N, u = r - b * N, n0 = b * N;
     TreeGradTerm* tm = reinterpret_cast<TreeGradTerm*>(dsm);  // [2 N] as gathered, then merged
@@ -786,7 +785,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_grad(Problem<T> P, G* grad) {
     G* g = grad + (int64_t)r * V;
     const T* x = P.draft + (int64_t)r * V;
     const int32_t* par = P.parent + (int64_t)n0;
-    if (threadIdx.x == 0) s_n = s_nu = 0;
+    if (threadIdx.x == 0) s_n = 0;
     grid_wait();
     __syncthreads();
     const bool bad = ld_cg(P.tbad + b) != 0;
@@ -921,8 +920,8 @@ __device__ __forceinline__ float2 two_floats(double a) {
     const float h = (float)a;
     return make_float2(h, (float)(a - (double)h));
 }
-// max(0, p - A q): the products are exact inside the multiply-adds, so A in
-// two floats loses nothing of the double.
+// max(0, p - A q) from A in two floats (48 of the double's 53 bits); each product
+// is exact inside its multiply-add, the difference rounded to float twice.
 __device__ __forceinline__ float seq_mass(float p, float q, float ah, float al) {
     return fmaxf(fmaf(-al, q, fmaf(-ah, q, p)), 0.f);
 }
@@ -1165,7 +1164,7 @@ __device__ void tree_seq_row(const Problem<T>& P, int r, Ring<S>* rg, float4* ta
 // then; else the row a bonus token needs is read by k_tree_seq.
 // What bounds it: the row reads and row tails (3840 rows of 2 x 64 KB), and
 // the reads after a rejection, which come from L2.  64 trees of 60 nodes,
-// V = 32000: 0.244 ms a call; 5.46 ms with the rule run along the path by one
+// V = 32000: 210 to 225 us a call; 5.46 ms with the rule run along the path by one
 // block per tree, in an fp64 recursion per element over the earlier siblings.
 template <typename T, bool VEC, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_tree_seq_rows(Problem<T> P) {
