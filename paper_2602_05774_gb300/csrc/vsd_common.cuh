@@ -135,6 +135,15 @@ __device__ __forceinline__ float elem_value(const __nv_bfloat16* row, int64_t v)
     return __uint_as_float(raw_elem(row, v) << 16);
 }
 
+// The same by a coherent load (the element is overwritten later in the kernel).
+__device__ __forceinline__ float elem_value_cg(const float* row, int64_t v) {
+    return __ldcg(row + v);
+}
+__device__ __forceinline__ float elem_value_cg(const __nv_bfloat16* row, int64_t v) {
+    return __uint_as_float(
+        (uint32_t)__ldcg(reinterpret_cast<const unsigned short*>(row) + v) << 16);
+}
+
 // Load chunk c of a row into registers: lane l, vector k holds elements
 // c*CE + k*32*PV + l*PV + [0, PV).  Elements at or beyond V read as -inf.
 template <typename T, bool VEC>

@@ -132,6 +132,17 @@ __global__ void __launch_bounds__(kThreads) k_em_grad(Problem<T> P, G* grad, int
     }
     const float mx = rec.mx, gq = cf.g * rec.izx;  // g / Z
     const bool dense = !(cf.g == 0.f && isfinite(mx));
+    // the logits with sparse terms, before the row is written (the gradient may
+    // take the draft's place)
+    const int j = (int)threadIdx.x - 2;
+    int t = -1;
+    if (j < 0)
+        t = threadIdx.x ? cf.t1 : cf.t0;
+    else if (KL && j < kMaxKlTop)
+        t = ld_cg(&P.klr[r].tok[j]);
+    const bool here = t >= i0 * PV && t < (int64_t)i1 * PV && t < V;
+    const float xt = here && dense ? elem_value_cg(x, t) : 0.f;
+    __syncthreads();
     if constexpr (VEC) {
         const uint64_t pol = policy_evict_first();
         const uint64_t mx2 = f2(mx, mx), c2 = f2(c, c), gq2 = f2(gq, gq);
@@ -176,14 +187,11 @@ __global__ void __launch_bounds__(kThreads) k_em_grad(Problem<T> P, G* grad, int
     // the elements with sparse terms: t0, t1, the top-K tokens
     const int nkl = KL ? min(max(kl.n, 0), kMaxKlTop) : 0;
     if ((int)threadIdx.x < 2 + nkl) {
-        const int j = (int)threadIdx.x - 2;
-        const int t = j >= 0 ? kl.tok[j] : threadIdx.x ? cf.t1 : cf.t0;
-        const bool mine = t >= i0 * PV && t < (int64_t)i1 * PV && t < V &&
-                          !(threadIdx.x >= 1 && t == cf.t0) && !(threadIdx.x >= 2 && t == cf.t1);
+        const bool mine = here && !(threadIdx.x >= 1 && t == cf.t0) &&
+                          !(threadIdx.x >= 2 && t == cf.t1);
         if (mine) {
             // (rounded steps: no contraction into a fused multiply-add)
-            float o = dense ? __fmul_rn(ex2(__fmul_rn(__fsub_rn(elem_value(x, t), mx), c)), gq)
-                            : 0.f;
+            float o = dense ? __fmul_rn(ex2(__fmul_rn(__fsub_rn(xt, mx), c)), gq) : 0.f;
             if (t == cf.t0) o = __fsub_rn(o, cf.c0);
             if (t == cf.t1) o = __fsub_rn(o, cf.c1);
             for (int k = 0; k < nkl; ++k)

@@ -811,6 +811,15 @@ __global__ void __launch_bounds__(kThreads) k_tree_grad(Problem<T> P, G* grad) {
             rank += tm[j].tok < tm[i].tok || (tm[j].tok == tm[i].tok && tm[j].key < tm[i].key);
         srt[rank] = tm[i];
     }
+    // the terms' logits, before the row is written (the gradient may take the
+    // draft's place)
+    __syncthreads();
+    if (dense)
+        for (int i = threadIdx.x; i < nt; i += kThreads) {
+            const int t = srt[i].tok;
+            tm[i].cf = t >= 0 && t < V ? elem_value_cg(x, t) : 0.f;
+        }
+    __syncthreads();
     if constexpr (VEC) {
         constexpr int U = 8, NP = PV / 2;
         const uint64_t pol = policy_evict_first();
@@ -857,7 +866,7 @@ __global__ void __launch_bounds__(kThreads) k_tree_grad(Problem<T> P, G* grad) {
         if ((i && srt[i - 1].tok == t) || t < 0 || t >= V) continue;
         float cf = srt[i].cf;
         for (int j = i + 1; j < nt && srt[j].tok == t; ++j) cf += srt[j].cf;
-        const float val = (dense ? gq * ex2((elem_value(x, t) - mx) * c) : 0.f) - cf;
+        const float val = (dense ? gq * ex2((tm[i].cf - mx) * c) : 0.f) - cf;
         if constexpr (sizeof(G) == 2)
             g[t] = __float2bfloat16_rn(val);
         else

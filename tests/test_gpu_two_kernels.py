@@ -250,3 +250,34 @@ def test_long_rows_by_either_route(vsd, V, R, n, dtype):
     assert torch.equal(b["loss"][:-1].view(n, -1)[n - 1], a["loss"][:-1])
     if grad:  # (a mean over n times the prefixes: an exact factor)
         assert torch.equal(a["grad"].view(-1) / n, b["grad"].view(n, -1)[n - 1])
+
+
+@pytest.mark.parametrize("V,dtype", [(32000, "bf16"), (4099, "f32"), (80000, "bf16")])
+def test_gradient_in_the_drafts_place(vsd, V, dtype):
+    """The gradient may be written over the draft logits: the elements with sparse
+    terms are read before their row is written (linear paths with top-K terms, in
+    one and in several segments a row, and trees)."""
+    from paper_2602_05774_gb300 import inputs
+    B, K, D = 4, 8, 3
+    p = inputs.linear_problem(B, K, D, V, dtype, "spiked", "cuda", seed=V)
+    prm = vsd.params(like=p["draft"], kl_weight=0.5)
+    want = _call(vsd, p, 1.0, prm)
+    out = vsd.linear_outputs(B, K, D, V, "cuda", grad=False, kl=True)
+    out["grad"] = p["draft"]
+    _call(vsd, p, 1.0, prm, out=out)
+    for k in want:
+        assert torch.equal(out[k], want[k]), k
+    q = {k: (v.cuda() if torch.is_tensor(v) else v)
+         for k, v in inputs.tree_problem(B, 24, 4, 4, V, seed=6, dtype=dtype).items()}
+    a = (q["draft"], q["target"], q["parent"], q["tokens"], q["u_accept"], q["u_correct"])
+    want = vsd.tree_estep_mstep(*a, 1.0)
+    import ctypes as C
+    ws = vsd.new_workspace(vsd.layout(B, V=V, N=24, parent=q["parent"]), "cuda")
+    loss = torch.empty(B + 1, device="cuda")
+    st = vsd.TreeEmOutputs(**dict(loss=loss.data_ptr(), grad=q["draft"].data_ptr()))
+    ptr = [t.data_ptr() for t in a]
+    assert vsd.load().vsd_tree_estep_mstep(
+        ptr[0], ptr[1], int(dtype == "bf16"), vsd.layout(B, V=V, N=24, parent=q["parent"]), 1.0,
+        ptr[3], ptr[4], ptr[5], C.byref(vsd.params(like=q["draft"])), C.byref(st), ws.data_ptr(),
+        ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+    assert torch.equal(q["draft"], want["grad"]) and torch.equal(loss, want["loss"])
