@@ -141,7 +141,8 @@ typedef struct {
     float* loss;            /* [B+1] loss_b = -J_b/N_b, then mean over b (Eq. advance)*/
     void* grad;             /* [R][V] d loss / d draft logits, params.grad_dtype;
                                NULL (fused calls): not written, the M-step's
-                               coefficients stay in ws for vsd_lmhead_backward */
+                               coefficients stay in ws for vsd_lmhead_backward.
+                               May be the draft logits' own memory (one dtype) */
     float* kl_loss;         /* [R] the row's top-K term of Eq. klv (with kl_weight)   */
 } vsd_linear_outputs;
 
@@ -231,11 +232,11 @@ vsd_status vsd_weighted_loss_fwd_bwd(const void* draft, vsd_dtype dtype, vsd_lay
 
 /* The fused E-step + M-step (Algorithm 1, both steps, for all prefixes at
  * once; Algorithm 2 as the oracle; Eqs. 1, 2, 11, beta, zeta, advance): two
- * kernels (rows with paths and M-steps, then the gradient), or for long rows
- * with a gradient one persistent kernel, run sampling, verification,
- * utilities, weights, loss and gradient over all prefixes, with the results
- * of vsd_sample_paths, vsd_verify_paths and vsd_weighted_loss_fwd_bwd; which
- * of the two is a matter of speed only.  Arguments as for those
+ * kernels (rows with paths and M-steps, then the gradient), or for long rows,
+ * when they are few, or many with a gradient, one persistent kernel, run
+ * sampling, verification, utilities, weights, loss and gradient over all
+ * prefixes, with the results of vsd_sample_paths, vsd_verify_paths and
+ * vsd_weighted_loss_fwd_bwd; which of the two is a matter of speed only.  Arguments as for those
  * calls: draft, target [R][V] of `dtype`; u_draft, u_accept, u_correct [R];
  * ref_logkappa optional [B][D]; params NULL for the defaults (App. F:
  * w(l) = 1.05^l, tau = 0.2).  Required members of `out`: tokens, accept_len,

@@ -28,12 +28,13 @@ __global__ void __launch_bounds__(kThreads) k_sample(Problem<T> P) {
     }
 }
 
-// Verification of given tokens: the rows, then the paths (accepted length,
-// residual draw, corrected path, log-kappa sums), one block each.  One kernel,
-// the block completing a path running it (k_em_rows), takes over for few
-// unaligned rows only.  us, one kernel / two:
-//   aligned    bf16: V=128256 R=64 64 / 66, R=608 117 / 103, R=4096 416 / 396;
-//              V=32000 R=64 33 / 33, R=4096 150 / 143; V=256 R=32768 339 / 279
+// Verification of given tokens of many rows: the rows, then the paths (accepted
+// length, residual draw, corrected path, log-kappa sums), one block each.  Few rows
+// take one kernel, the block completing a path running it (k_em_rows): as fast on
+// the GPU, and a launch less for the host.  us, one kernel / two:
+//   aligned    bf16: V=4000 R=1024 27 / 29, R=4096 62 / 56; V=32000 R=64 33 / 33, R=1216
+//              64 / 64, R=4096 150 / 143; V=128256 R=64 64 / 66, R=304 76 / 79, R=608
+//              117 / 103, R=4096 416 / 396; V=256 R=32768 339 / 279
 //   unaligned  bf16: V=1001 R=64 23 / 26, R=4096 83 / 66; V=32001 R=64 50 / 52,
 //              R=4096 278 / 247
 // Rows that are not aligned keep more element loads in flight with more registers,
@@ -490,7 +491,8 @@ cudaError_t Launch<VSD_T>::sample(const Problem<VSD_T>& P, bool vec, cudaStream_
 template <>
 cudaError_t Launch<VSD_T>::verify(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
     const int64_t sms = device_sm_count();
-    if (!vec && P.R <= (P.nch < 16 ? 4 : 2) * sms) return verify_few(P, s);
+    if (P.R <= (vec ? (P.nch < 48 ? 8 : 2) : (P.nch < 16 ? 4 : 2)) * sms)
+        return verify_few(P, vec, s);
     bool deep = deep_ring(vec, P.nch, P.R);
     size_t smem = row_smem_bytes(P.nch, vec, deep);
     auto rows = !vec && P.nch >= 12 ? k_verify_rows<VSD_T, false, kDeepStages>

@@ -15,8 +15,8 @@ template <typename T> struct Launch {
     // verification of given tokens (linear paths): rows, accepted lengths, residual
     // draws, corrected paths, log-kappa
     static cudaError_t verify(const Problem<T>& P, bool vec, cudaStream_t s);
-    // the same in one kernel, for few rows that are not 16-byte aligned
-    static cudaError_t verify_few(const Problem<T>& P, cudaStream_t s);
+    // the same in one kernel, for few rows
+    static cudaError_t verify_few(const Problem<T>& P, bool vec, cudaStream_t s);
     // log kappa of supplied greedy reference paths: [B][D] rows -> out [B][D]
     static cudaError_t reference(const Problem<T>& P, bool vec, float* out, cudaStream_t s);
     // tree verification, each branch alone: node rows; then per row the residual

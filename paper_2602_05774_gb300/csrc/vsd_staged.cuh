@@ -1,4 +1,5 @@
-// vsd_staged.cuh -- the E-step + M-step in two kernels, for short rows:
+// vsd_staged.cuh -- the E-step + M-step in two kernels (when: two_kernels() in
+// vsd_api.cu):
 //
 //   k_em_rows  one block per row: the row pass (draws, statistics, the top-K
 //              term of VSD (KL)).  The block completing a path's last row runs
@@ -35,7 +36,7 @@ inline size_t staged_smem_bytes(int nch, bool vec, bool deep) {
 }
 
 // XMODE: kSampleToken the whole E-step + M-step; kGivenToken the verification
-// of given tokens, which ends with the paths (few unaligned rows).
+// of given tokens, which ends with the paths (few rows).
 template <typename T, bool VEC, bool KL, int XMODE, int S>
 __global__ void __launch_bounds__(kThreads, VEC ? kRowBlocks : 1) k_em_rows(Problem<T> P) {
     extern __shared__ __align__(128) unsigned char dsm[];

@@ -28,9 +28,10 @@ cudaError_t Launch<VSD_T>::staged(const Problem<VSD_T>& P, bool vec, void* grad,
 }
 
 template <>
-cudaError_t Launch<VSD_T>::verify_few(const Problem<VSD_T>& P, cudaStream_t s) {
-    const size_t smem = row_smem_bytes(P.nch, false, false);
-    auto rows = k_em_rows<VSD_T, false, false, kGivenToken, kRowStages>;
+cudaError_t Launch<VSD_T>::verify_few(const Problem<VSD_T>& P, bool vec, cudaStream_t s) {
+    const bool deep = deep_ring(vec, P.nch, P.R);
+    const size_t smem = row_smem_bytes<sizeof(WeightsShared)>(P.nch, vec, deep);
+    auto rows = VSD_BY_RING(k_em_rows, VSD_T, , false, kGivenToken);
     cudaError_t e = prep(rows, smem);
     if (e) return e;
     return launch_after(rows, P.R, kThreads, smem, s, P);

@@ -175,12 +175,14 @@ def _same_rows(few, many, copies, skip=()):
             assert torch.equal(b[i], a.reshape(-1)), k
 
 
-@pytest.mark.parametrize("V,dtype", [(24576, "f32"), (50004, "f32"), (49152, "bf16")])
-def test_few_long_rows_equal_many(vsd, V, dtype):
-    """Few rows of at least 48 chunks take the deeper ring, the same rows 64 times
-    over the shallow one: the same results bit for bit."""
+@pytest.mark.parametrize("V,dtype,n", [(24576, "f32", 64), (50004, "f32", 64), (49152, "bf16", 64),
+                                       (4104, "bf16", 128), (4099, "f32", 64)])
+def test_few_rows_equal_many(vsd, V, dtype, n):
+    """Few rows of at least 48 chunks take the deeper ring, and few rows are verified
+    in one kernel; the same rows n times over the shallow ring and two kernels: the
+    same results bit for bit."""
     from paper_2602_05774_gb300 import inputs
-    K, D, n = 5, 2, 64  # 10 rows, 640
+    K, D = 5, 2  # 10 rows; 640, or 1280 of short aligned ones
     p = inputs.linear_problem(1, K, D, V, dtype, "gauss", "cuda", seed=V)
     q = {k: (v.repeat(*([n] + [1] * (v.dim() - 1))) if torch.is_tensor(v) else v)
          for k, v in p.items()}
